@@ -143,10 +143,9 @@ def _as_signflip(case):
     return [(c, "signflip" if k in ("noise20", "bitflip") else k) for c, k in _faults(case) if c > 0]
 
 
-def prepare(case, seed):
-    """The server's inputs on the GPU and the handle it keeps for its model."""
+def _inputs(case, seed):
     w = _workload(case, seed)
-    s = dict(case=case, w=w, z=zeno.from_workload(w))
+    s = dict(case=case, w=w)
     gen = torch.Generator(device=DEVICE)
     gen.manual_seed(seed + 104729)
     if case["call"] == "run":
@@ -172,6 +171,12 @@ def prepare(case, seed):
                  wlabels=torch.randint(0, classes, (w.m, n), generator=gen, device=DEVICE, dtype=torch.int32),
                  faulty=torch.nonzero(~w.honest).flatten().to(torch.int32).to(DEVICE))
     return s
+
+
+def prepare(case, seed):
+    """The server's inputs on the GPU and the handle it keeps for its model."""
+    s = _inputs(case, seed)
+    return dict(s, z=zeno.from_workload(s["w"]))
 
 
 # ---- the calls -------------------------------------------------------------------------------------------
@@ -241,3 +246,124 @@ def tolerance(case):
         # an entry moves by one spacing, 2^-8 of its value
         return {"rel": 1e-3, "max": 2e-2}
     return {"rel": 5e-5}
+
+
+# ---- the same outputs in 64 bits -------------------------------------------------------------------------
+
+def _stored(t, case):
+    """Binary64 values rounded to the storage type of x and V."""
+    return t.to(torch.bfloat16 if case["dtype"] == "bf16" else torch.float32)
+
+
+def _f32(v):
+    return torch.tensor(v, dtype=torch.float32).double().item()      # a scalar as the C interface takes it
+
+
+def _logits(case, p, feats):
+    """Logits of one model, its parameters p as one binary64 vector."""
+    dims, off = _dims(case), 0
+
+    def take(*shape):
+        nonlocal off
+        n = 1
+        for v in shape:
+            n *= v
+        off += n
+        return p[off - n:off].view(shape)
+
+    h = feats
+    if case["model"] == "cnn":
+        chans = dims[1:-1]
+        for l in range(1, len(chans)):
+            W, bias = take(chans[l], chans[l - 1], 3, 3), take(chans[l])
+            h = torch.relu(torch.nn.functional.conv2d(h, W, bias, padding=1))
+            h = torch.nn.functional.max_pool2d(h, 2) if l % 2 == 0 else h
+        h = h.flatten(1)
+        return h @ take(dims[-1], h.shape[1]).t() + take(dims[-1])
+    for l in range(len(dims) - 1):
+        W, bias = take(dims[l + 1], dims[l]), take(dims[l + 1])
+        h = h @ W.t() + bias
+        h = torch.relu(h) if l + 2 < len(dims) else h
+    return h
+
+
+def _exact_scores(case, x, V, feats, targets):
+    g, rho, m, d = _f32(case["gamma"]), _f32(case["rho"]), case["m"], x.numel()
+    if case["model"] == "lsq":              # A x, A v and v . v, a range of columns at a time
+        a0 = torch.zeros(feats.shape[0], dtype=torch.float64, device=DEVICE)
+        av, norms = torch.zeros(feats.shape[0], m, dtype=torch.float64, device=DEVICE), torch.zeros(m, dtype=torch.float64, device=DEVICE)
+        for k in range(0, d, 1 << 22):
+            A, v = feats[:, k:k + (1 << 22)].double(), V[:, k:min(d, k + (1 << 22))].double()
+            a0 += A @ x[k:k + (1 << 22)].double()
+            av += A @ v.t()
+            norms += (v * v).sum(1)
+        r = (a0 - targets.double())[:, None]
+        f0, f = (r * r).mean(0) / 2, ((r - g * av) ** 2).mean(0) / 2
+        return f0 - f - rho * norms
+    x, feats, targets = x.double(), feats.double(), targets.long()
+    f0 = torch.nn.functional.cross_entropy(_logits(case, x, feats), targets)
+    scores = []
+    for i in range(m):
+        v = V[i, :d].double()
+        w = x - g * v
+        if case["dtype"] == "bf16":         # the candidate is itself a bfloat16 model
+            w = w.float().to(torch.bfloat16).double()
+        scores.append(f0 - torch.nn.functional.cross_entropy(_logits(case, w, feats), targets) - rho * (v * v).sum())
+    return torch.stack(scores)
+
+
+def _exact_mean(case, V, scores, d):
+    keep = torch.sort(-scores.float(), stable=True).indices[:case["m"] - case["b"]].tolist()
+    acc = torch.zeros(d, dtype=torch.float64, device=DEVICE)
+    for i in keep:
+        acc += V[i, :d].double()
+    return acc / len(keep)
+
+
+def exact(case, seed):
+    s = _inputs(case, seed)
+    w, call, g, b, m = s["w"], case["call"], _f32(case["gamma"]), case["b"], case["m"]
+    d, V = w.d, w.V
+    if call == "step":
+        scores = _exact_scores(case, w.x, V, w.features, w.targets)
+        return _exact_mean(case, V, scores, d), scores
+    if call == "update":
+        scores = _exact_scores(case, w.x, V, w.features, w.targets)
+        return w.x.double() - g * _exact_mean(case, V, scores, d), scores
+    if call == "run":                       # x is stored between the iterations, the last one is left in 64 bits
+        x, rows = w.x, []
+        for t in range(case["steps"]):
+            rows.append(_exact_scores(case, x, s["V"][t], s["feats"][t], s["labels"][t]))
+            new = x.double() - g * _exact_mean(case, s["V"][t], rows[-1], d)
+            x = _stored(new, case)
+        return new, torch.stack(rows)
+    if call == "iteration":                 # worker i's gradient of softmax regression on its own samples
+        n_in, classes = _dims(case)
+        x = w.x.double()
+        W, bias, n = x[:classes * n_in].view(classes, n_in), x[classes * n_in:], case["worker_batch"]
+        G = torch.empty(m, d, dtype=torch.float64, device=DEVICE)
+        for i in range(m):
+            a = s["wfeats"][i].double()
+            delta = torch.softmax(a @ W.t() + bias, 1)
+            delta[torch.arange(n, device=DEVICE), s["wlabels"][i].long()] -= 1
+            G[i] = torch.cat([(delta.t() @ a / n).flatten(), delta.sum(0) / n])
+        if s["faulty"].numel():
+            G[s["faulty"].long()] = -G[s["faulty"][0].long()]
+        stored = _stored(G, case)
+        scores = _exact_scores(case, w.x, stored, w.features, w.targets)
+        return x - g * _exact_mean(case, stored, scores, d), G, scores
+    if call == "median":
+        out = torch.empty(d, dtype=torch.float64, device=DEVICE)
+        for k in range(0, d, 1 << 20):
+            c = torch.sort(V[:, k:min(d, k + (1 << 20))].double(), 0).values
+            out[k:k + (1 << 20)] = (c[(m - 1) // 2] + c[m // 2]) / 2
+        return out
+    dist = torch.zeros(m, m, dtype=torch.float64, device=DEVICE)
+    for k in range(0, d, 1 << 20):
+        v = V[:, k:min(d, k + (1 << 20))].double()
+        for i in range(m):
+            dist[i] += ((v - v[i]) ** 2).sum(1)
+    dist.fill_diagonal_(float("inf"))       # the m - b - 2 nearest of the others
+    sums = torch.sort(dist, 1).values[:, :m - b - 2].sum(1)
+    k = int(sums.float().argmin())
+    return V[k, :d].double(), torch.tensor([k], dtype=torch.int32, device=DEVICE), sums

@@ -13,7 +13,7 @@ LIB = os.path.join(HERE, "libzeno.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-    "-Xcompiler", "-fPIC", "--shared", "-cudart", "static",
+    "-Xcompiler", "-fPIC", "--threads", "8", "--shared", "-cudart", "static",
     "-I", os.path.join(ROOT, "include"), "-I", CSRC,
 ]
 

@@ -1,12 +1,5 @@
-// The paper's baseline aggregation rules on the same candidate matrix V (Experiments, "Baselines"):
-// the marginal Median and Krum_b.  They share Zeno's inputs and storage types, so a caller can compare
-// the three rules on the same step.
-//
-// Median: out[j] = the one-dimensional median of column j (the middle value of the m sorted entries, the
-// mean of the two middle ones for even m; a NaN entry counts as plus infinity).  One pass over V.  A
-// column is sorted in registers by a bitonic network, 32 values a thread, padded with plus infinity
-// (which leaves the middle ranks where they are); beyond 32 candidates 2, 4, .. 32 neighbouring lanes of
-// a warp share a column and the network's long-range stages exchange values by shuffles.
+// The paper's baseline aggregation rules on the same candidate matrix V (Experiments, "Baselines"): Krum_b here,
+// the marginal Median in zeno_median.cu.
 //
 // Krum: the squared distances ||v_i - v_j||^2 of all pairs, taken as sums of squared differences (not
 // from a Gram matrix: two honest candidates may differ by far less than their norms), then for every
@@ -22,106 +15,6 @@ namespace zeno {
 namespace {
 
 __device__ __forceinline__ float nan_to_inf(float v) { return v != v ? INFINITY : v; }
-
-constexpr int kMedianRegs = 32;               // values of a column one thread holds
-constexpr int kMedianThreads = 128;
-
-__host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }
-
-// Ascending sort of the R * TPC values that TPC neighbouring lanes hold, element e = t * R + i in
-// register i of lane t, by the bitonic network in the form whose comparators all point the same way: a
-// merge of blocks of k elements first compares every element with its mirror image in the block
-// (e ^ (k - 1)), then halves the distance from k / 4 down.  Every index below is a constant once the
-// loops are unrolled, so the values stay in registers; partners R or more elements away sit in another
-// lane and come by shuffle.  With one lane a column, elements from NP on are padding (plus infinity at
-// the top of an ascending network never moves), so comparators that touch them are left out.
-template <int R, int TPC, int NP>
-__device__ __forceinline__ void bitonic_sort_lanes(float (&a)[R], int t) {
-    constexpr int kLogN = ilog2(R) + ilog2(TPC);
-#pragma unroll
-    for (int lk = 1; lk <= kLogN; ++lk) {
-        const int k = 1 << lk;
-        if (k > R) {                          // mirror partner: register R - 1 - i of lane t ^ (k / R - 1)
-            const bool keep_min = (t & (k / (2 * R))) == 0;
-            float o[R];
-#pragma unroll
-            for (int i = 0; i < R; ++i) o[i] = __shfl_xor_sync(0xffffffffu, a[R - 1 - i], k / R - 1);
-#pragma unroll
-            for (int i = 0; i < R; ++i) a[i] = keep_min ? fminf(a[i], o[i]) : fmaxf(a[i], o[i]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < R; ++i) {
-                const int l = i ^ (k - 1);
-                if (l > i && l < NP) {
-                    const float lo = fminf(a[i], a[l]), hi = fmaxf(a[i], a[l]);
-                    a[i] = lo;
-                    a[l] = hi;
-                }
-            }
-        }
-#pragma unroll
-        for (int lj = lk - 2; lj >= 0; --lj) {
-            const int j = 1 << lj;
-            if (j >= R) {
-                const bool keep_min = (t & (j / R)) == 0;
-#pragma unroll
-                for (int i = 0; i < R; ++i) {
-                    const float o = __shfl_xor_sync(0xffffffffu, a[i], j / R);
-                    a[i] = keep_min ? fminf(a[i], o) : fmaxf(a[i], o);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < R; ++i) {
-                    const int l = i ^ j;
-                    if (l > i && l < NP) {
-                        const float lo = fminf(a[i], a[l]), hi = fmaxf(a[i], a[l]);
-                        a[i] = lo;
-                        a[l] = hi;
-                    }
-                }
-            }
-        }
-    }
-}
-
-// A warp takes 32 / TPC neighbouring columns at a time; lane = column * TPC + t holds rows t * R .. of it.
-// With one lane a column the kernel is compiled for its number of candidates, NP = m: the padding, the
-// row bounds and the ranks of the middle values are constants, and the comparators whose results the
-// middle values do not depend on fall away with them.  With more lanes NP = R and m is an argument.
-template <typename T, int TPC, int NP>
-__global__ void __launch_bounds__(kMedianThreads, 4) median_kernel(const T *V, int64_t ldv, int64_t d, int m_arg, float *out) {
-    constexpr int R = kMedianRegs, kCols = 32 / TPC;
-    static_assert(TPC == 1 || NP == R, "padding is only left out when a lane holds the whole column");
-    pdl_wait();
-    pdl_launch_dependents();
-    const int lane = threadIdx.x & 31, t = lane % TPC, c = lane / TPC;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int m = TPC == 1 ? NP : m_arg;
-    const int p0 = (m - 1) / 2, p1 = m / 2;   // ranks of the middle values
-    for (int64_t j0 = warp * kCols; j0 < d; j0 += warps * kCols) {
-        const int64_t j = j0 + c;
-        const bool live = j < d;
-        float a[R];
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            const int row = t * R + i;
-            a[i] = (i < NP && live && row < m) ? nan_to_inf(load_elem(V + (int64_t)row * ldv + j)) : INFINITY;
-        }
-        bitonic_sort_lanes<R, TPC, NP>(a, t);
-        float lo = 0.f, hi = 0.f;
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            if (t * R + i == p0) lo = a[i];
-            if (t * R + i == p1) hi = a[i];
-        }
-        if (TPC > 1) {
-            lo = __shfl_sync(0xffffffffu, lo, (lane & ~(TPC - 1)) | (p0 / R));
-            hi = __shfl_sync(0xffffffffu, hi, (lane & ~(TPC - 1)) | (p1 / R));
-        }
-        if (live && t == 0) out[j] = (m & 1) ? lo : 0.5f * lo + 0.5f * hi;
-    }
-}
 
 // ---- Krum -----------------------------------------------------------------------------------
 
@@ -291,41 +184,6 @@ __global__ void __launch_bounds__(256) copy_row_kernel(const T *V, int64_t ldv, 
         out[j] = load_elem(V + (int64_t)row * ldv + j);
 }
 
-template <typename T, int TPC, int NP>
-cudaError_t launch_median_lanes(Context &c, const T *V, int64_t ldv, int m, float *out, cudaStream_t s) {
-    const int sms = c.sm_count > 0 ? c.sm_count : 148;
-    const int64_t d = c.d;
-    const int per_block = (kMedianThreads / 32) * (32 / TPC);          // columns a block takes at a time
-    const int64_t want = (d + per_block - 1) / per_block, cap = (int64_t)sms * 16;
-    const int blocks = (int)(want < cap ? (want < 1 ? 1 : want) : cap);
-    return launch_chained(median_kernel<T, TPC, NP>, dim3(blocks), dim3(kMedianThreads), 0, s, chain_launches(c), V, ldv, d, m, out);
-}
-
-// the one-lane kernel compiled for exactly m candidates, m = M, M - 1, .. 1
-template <typename T, int M>
-struct MedianOneLane {
-    static cudaError_t launch(Context &c, const T *V, int64_t ldv, int m, float *out, cudaStream_t s) {
-        if (m == M) return launch_median_lanes<T, 1, M>(c, V, ldv, m, out, s);
-        return MedianOneLane<T, M - 1>::launch(c, V, ldv, m, out, s);
-    }
-};
-template <typename T>
-struct MedianOneLane<T, 0> {
-    static cudaError_t launch(Context &, const T *, int64_t, int, float *, cudaStream_t) { return cudaErrorInvalidValue; }
-};
-
-template <typename T>
-cudaError_t launch_median_typed(Context &c, const T *V, int64_t ldv, int m, float *out, cudaStream_t s) {
-    constexpr int R = kMedianRegs;
-    static_assert(R * 32 >= ZENO_MAX_CANDIDATES, "a warp holds the longest column");
-    if (m <= R) return MedianOneLane<T, R>::launch(c, V, ldv, m, out, s);
-    if (m <= R * 2) return launch_median_lanes<T, 2, R>(c, V, ldv, m, out, s);
-    if (m <= R * 4) return launch_median_lanes<T, 4, R>(c, V, ldv, m, out, s);
-    if (m <= R * 8) return launch_median_lanes<T, 8, R>(c, V, ldv, m, out, s);
-    if (m <= R * 16) return launch_median_lanes<T, 16, R>(c, V, ldv, m, out, s);
-    return launch_median_lanes<T, 32, R>(c, V, ldv, m, out, s);
-}
-
 template <typename T>
 cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b, float *out, int32_t *k, float *sums,
                               cudaStream_t s) {
@@ -372,13 +230,6 @@ cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b,
 
 // floats of Krum's workspace for up to m candidates and `blocks` blocks: the blocks' pair sums, then dist[m][m]
 size_t krum_part_floats(int m, int blocks) { return (size_t)blocks * krum_tiles(m) * 16 + (size_t)m * m; }
-
-cudaError_t launch_median(Context &c, const void *V, int64_t ldv, int m, float *out, cudaStream_t s, int *launches) {
-    ++*launches;
-    profile_mark(c, "median", s);
-    if (c.desc.param_dtype == ZENO_BF16) return launch_median_typed(c, static_cast<const __nv_bfloat16 *>(V), ldv, m, out, s);
-    return launch_median_typed(c, static_cast<const float *>(V), ldv, m, out, s);
-}
 
 cudaError_t launch_krum(Context &c, const void *V, int64_t ldv, int m, int b, float *out, int32_t *k, float *sums,
                         cudaStream_t s, int *launches) {

@@ -61,6 +61,32 @@ def test_median_every_network(oracle, dtype):
             assert np.all(np.abs(got[fin] - want[fin]) <= 1.2e-7 * np.maximum(np.abs(want[fin]), 1e-30) + 1e-45), m
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("ldv_pad", [0, 1])         # rows of an odd pitch: bfloat16 columns are read one by one
+def test_median_padded_halves(oracle, dtype, ldv_pad):
+    """Columns of 34 .. 126 candidates, padded to the next compiled size by up to seven infinities of both signs,
+    with real infinities and NaN beside the padding; d = 515 and 516 leave an odd and an even last tile."""
+    for m in (34, 36, 39, 40, 41, 47, 50, 57, 72, 73, 90, 99, 105, 112, 113, 120, 121, 126):
+        d = 515 + m % 2
+        w = syn.make_config(5, d=d, m=m, b=0, n_r=4, n_noise=0, ldv=d + (d + ldv_pad) % 2, seed=3000 + m)
+        V = w.V.to(torch.bfloat16) if dtype == "bf16" else w.V
+        V[:, 7] = float("inf")
+        V[: m // 2 + 1, 8] = float("-inf")
+        V[::3, 9] = float("nan")
+        V[:, d - 1] = torch.arange(m).to(V.dtype)
+        want = oracle.median(int(dtype == "bf16"), syn.to_numpy_params(V), w.ldv, d, m)
+        kind, desc = (0, ((d - 2) // 2, 2) if d % 2 == 0 else (d - 1, 1)) if dtype == "bf16" else (1, (d, 1))
+        with zeno.Zeno(kind, int(dtype == "bf16"), desc, True, m, 4) as z:
+            assert z.d == d
+            got = z.median(V.cuda()).cpu().numpy().astype(np.float64)
+        fin = np.isfinite(want)
+        assert np.array_equal(got[~fin], want[~fin]), m
+        if m % 2 == 1:
+            assert np.array_equal(got, want), m
+        else:                                       # the mean of two stored values formed in binary32: one rounding
+            assert np.all(np.abs(got[fin] - want[fin]) <= 1.2e-7 * np.maximum(np.abs(want[fin]), 1e-30) + 1e-45), m
+
+
 @pytest.mark.parametrize("name", sorted(CASES))
 def test_median_matches_oracle(oracle, name):
     index, ov = CASES[name]

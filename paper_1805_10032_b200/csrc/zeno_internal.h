@@ -348,6 +348,27 @@ __device__ __forceinline__ unsigned long long rank_key(float s, int index) {
     return ((unsigned long long)u << 32) | (unsigned)(0xffffffffu - (unsigned)index);
 }
 
+// Sum, over the 32 lanes, of each of N per-lane values; lane j (< N) ends up holding the total
+// of value j.  Recursive halving: 31 shuffles for N = 32 instead of 160.
+template <int N>
+__device__ __forceinline__ float warp_transpose_reduce(float (&v)[N], int lane) {
+    static_assert(N == 1 || N == 2 || N == 4 || N == 8 || N == 16 || N == 32, "N must be 2^k");
+#pragma unroll
+    for (int s = N / 2; s >= 1; s >>= 1) {
+        const bool upper = (lane & s) != 0;
+#pragma unroll
+        for (int i = 0; i < s; ++i) {
+            float send = upper ? v[i] : v[i + s];
+            float keep = upper ? v[i + s] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+    }
+    float r = v[0];
+#pragma unroll
+    for (int s = N; s < 32; s <<= 1) r += __shfl_xor_sync(0xffffffffu, r, s);
+    return r;
+}
+
 // ReLU that lets a NaN through
 __device__ __forceinline__ float relu_keep_nan(float z) { return (z > 0.f || z != z) ? z : 0.f; }
 

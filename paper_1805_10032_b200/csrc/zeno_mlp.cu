@@ -32,27 +32,6 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
 }
 
-// Sum, over the 32 lanes, of each of N per-lane values; lane j (< N) ends up holding the total
-// of value j.  Recursive halving: 31 shuffles for N = 32 instead of 160.
-template <int N>
-__device__ __forceinline__ float warp_transpose_reduce(float (&v)[N], int lane) {
-    static_assert(N == 1 || N == 2 || N == 4 || N == 8 || N == 16 || N == 32, "N must be 2^k");
-#pragma unroll
-    for (int s = N / 2; s >= 1; s >>= 1) {
-        const bool upper = (lane & s) != 0;
-#pragma unroll
-        for (int i = 0; i < s; ++i) {
-            float send = upper ? v[i] : v[i + s];
-            float keep = upper ? v[i + s] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-        }
-    }
-    float r = v[0];
-#pragma unroll
-    for (int s = N; s < 32; s <<= 1) r += __shfl_xor_sync(0xffffffffu, r, s);
-    return r;
-}
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int s = 16; s >= 1; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);

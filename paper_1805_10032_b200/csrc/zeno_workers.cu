@@ -7,9 +7,8 @@
 //   inject_faults_kernel                                  the bit-flipping failure (negated gradient, the
 //                                                         first faulty row copied over the others) and the
 //                                                         failure model's scaled gradient eps * v.
-// These kernels build the step's INPUT (the candidate matrix V); they are not on the scoring path.  One
-// block per worker; the sizes they are meant for are the paper's (a hundred samples per worker, a model of
-// a few thousand parameters).
+// These kernels build the step's INPUT (the candidate matrix V); they are not on the scoring path.  The sizes
+// they are meant for are the paper's (a hundred samples per worker, a model of a few thousand parameters).
 #include <math.h>
 
 #include "zeno_internal.h"
@@ -20,6 +19,7 @@ namespace {
 
 constexpr int kWThreads = 256;
 constexpr int kWMaxClasses = 32;
+constexpr int kWMaxSmem = 224 * 1024;         // one class pads to four: 12,288 samples' delta and the sums need 200 KB
 
 __device__ __forceinline__ float block_sum(float v, float *scratch) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -37,73 +37,205 @@ template <typename T> __device__ __forceinline__ void store_elem(T *p, float v);
 template <> __device__ __forceinline__ void store_elem<float>(float *p, float v) { *p = v; }
 template <> __device__ __forceinline__ void store_elem<__nv_bfloat16>(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 
-// Softmax regression, worker w = blockIdx.x: samples feats[w][n][in], labels[w][n].
+// Softmax regression, worker w = blockIdx.y: samples feats[w][n][in], labels[w][n].
 //   delta[j][c] = (softmax(W a_j + b)[c] - [c == label_j]) / n;  dW[c][k] = sum_j delta[j][c] a_j[k];  db[c] = sum_j delta[j][c]
-// dynamic shared memory: delta [n][classes].
-template <typename T>
-__global__ void __launch_bounds__(kWThreads) worker_grad_softmax_kernel(const T *x, int in, int classes, int has_bias,
-                                                                         const float *feats, const int32_t *labels, int n,
-                                                                         const int32_t *flip, T *V, int64_t ldv) {
-    extern __shared__ float delta[];
-    const int w = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// A cluster of eight blocks works for one worker: block r takes an eighth of the samples' logits and leaves their
+// delta in the shared memory of all eight, then every block takes an eighth of the input indices of dW.  Latency is
+// all there is (20 workers of 100 samples x 784 inputs read 6 MB, 1 us): one block a worker, with its samples one
+// after another in a warp, left 128 SMs idle and took 500 us for those sizes where this takes 22 us.
+// dynamic shared memory: delta [n][pitch] (pitch: classes rounded up to 4), then the sample groups' sums.
+constexpr int kWCluster = 8;
+constexpr int kWGradWarps = 8;
+constexpr int kWSamples = 2;                  // samples a warp takes at a time: the weights are read once for both
+
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// address, in the cluster's shared window, of this block's shared variable p as block `rank` has it
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, unsigned rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+// CM: classes the registers are sized for, a multiple of 4
+template <typename T, int CM>
+__global__ void __launch_bounds__(kWGradWarps * 32, 2)
+worker_grad_softmax_kernel(const T *x, int in, int classes, int has_bias, const float *feats, const int32_t *labels, int n,
+                           const int32_t *flip, T *V, int64_t ldv) {
+    extern __shared__ __align__(16) float delta[];
+    constexpr int S = kWSamples, CR = CM <= 4 ? 4 : CM <= 16 ? 16 : 32;
+    const int w = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rank = (int)cluster_rank();
+    const int pitch = (classes + 3) & ~3;
+    float *sums = delta + (size_t)n * pitch;
+    pdl_wait();                               // no early trigger: what follows reads V through the read-only path
     const float *a = feats + (int64_t)w * n * in;
     const int32_t *lab = labels + (int64_t)w * n;
     const bool flipped = flip != nullptr && flip[w] != 0;
     T *out = V + (int64_t)w * ldv;
-    // logits: one warp per sample, lanes stride the input index
-    for (int j = warp; j < n; j += kWThreads / 32) {
-        float z[kWMaxClasses];
+    const int cls = lane & (CR - 1);
+    const float bias = has_bias && cls < classes ? load_elem(x + (int64_t)classes * in + cls) : 0.f;
+    cluster_barrier();                        // every block of the cluster runs: their shared memory may be written
+    // logits of this block's samples: a warp takes S of them, lanes stride the input index
+    const int per_block = (n + kWCluster - 1) / kWCluster;
+    const int j_end = min(n, (rank + 1) * per_block);
+    for (int j0 = rank * per_block + warp * S; j0 < j_end; j0 += kWGradWarps * S) {
+        float z[S][CM];
 #pragma unroll
-        for (int c = 0; c < kWMaxClasses; ++c) z[c] = 0.f;
+        for (int q = 0; q < S; ++q)
+#pragma unroll
+            for (int c = 0; c < CM; ++c) z[q][c] = 0.f;
+#pragma unroll(CM <= 12 ? 4 : 1)
         for (int k = lane; k < in; k += 32) {
-            const float av = a[(int64_t)j * in + k];
+            float av[S];
 #pragma unroll
-            for (int c = 0; c < kWMaxClasses; ++c)
-                if (c < classes) z[c] = fmaf(load_elem(x + (int64_t)c * in + k), av, z[c]);
-        }
-        float zmax = -INFINITY;
+            for (int q = 0; q < S; ++q) av[q] = __ldg(a + (int64_t)min(j0 + q, j_end - 1) * in + k);
 #pragma unroll
-        for (int c = 0; c < kWMaxClasses; ++c) {
-            if (c < classes) {
+            for (int c = 0; c < CM; ++c) {
+                if (c < classes) {
+                    const float wv = load_elem(x + (int64_t)c * in + k);
 #pragma unroll
-                for (int s = 16; s >= 1; s >>= 1) z[c] += __shfl_xor_sync(0xffffffffu, z[c], s);
-                if (has_bias) z[c] += load_elem(x + (int64_t)classes * in + c);
-                zmax = fmaxf(zmax, z[c]);
+                    for (int q = 0; q < S; ++q) z[q][c] = fmaf(wv, av[q], z[q][c]);
+                }
             }
         }
-        float se = 0.f;
 #pragma unroll
-        for (int c = 0; c < kWMaxClasses; ++c)
-            if (c < classes) se += expf(z[c] - zmax);
-        int label = lab[j];
-        if (flipped) label = classes - 1 - label;
-        if (lane == 0) {
+        for (int q = 0; q < S; ++q) {
+            // lane c (and its copies CR lanes apart) collects class c, so that a class costs one exponential
+            float v[CR];
 #pragma unroll
-            for (int c = 0; c < kWMaxClasses; ++c)
-                if (c < classes) delta[j * classes + c] = (expf(z[c] - zmax) / se - (c == label ? 1.f : 0.f)) / (float)n;
+            for (int c = 0; c < CR; ++c) v[c] = c < CM ? z[q][c < CM ? c : 0] : 0.f;
+            const float zc = warp_transpose_reduce<CR>(v, lane) + bias;
+            const int j = j0 + q;
+            if (j >= j_end) break;
+            float zmax = cls < classes ? zc : -INFINITY;
+#pragma unroll
+            for (int s = CR / 2; s >= 1; s >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, s));
+            const float e = cls < classes ? expf(zc - zmax) : 0.f;
+            float se = e;
+#pragma unroll
+            for (int s = CR / 2; s >= 1; s >>= 1) se += __shfl_xor_sync(0xffffffffu, se, s);
+            int label = __ldg(lab + j);
+            if (flipped) label = classes - 1 - label;
+            const float dj = cls < classes ? (e / se - (cls == label ? 1.f : 0.f)) / (float)n : 0.f;
+            if (cls < pitch)                  // the copies share the cluster's blocks between them
+                for (int r = lane / CR; r < kWCluster; r += 32 / CR) cluster_store(cluster_addr(delta + (size_t)j * pitch + cls, r), dj);
         }
     }
-    __syncthreads();
-    // dW: a thread per input index k, all classes in registers; samples in order
-    for (int k = threadIdx.x; k < in; k += kWThreads) {
-        float g[kWMaxClasses];
+    cluster_barrier();
+    // dW: this block's chunks of 32 input indices, a lane per index, all classes in registers.  With fewer chunks
+    // than warps, groups of warps share a chunk and split the samples; their sums are added in group order.
+    const int chunks = (in + 31) / 32, per = (chunks + kWCluster - 1) / kWCluster;
+    const int first = rank * per, mine = min(per, chunks - first);
+    const int groups = per >= kWGradWarps ? 1 : kWGradWarps / per;
+    const int group = per >= kWGradWarps ? 0 : warp / per;
+    const int step = groups > 1 ? per : kWGradWarps;
+    const int js = (n + groups - 1) / groups;
+    for (int t = groups > 1 ? warp % per : warp; t < per; t += step) {      // one turn if groups share the chunks
+        const int k = (first + t) * 32 + lane;
+        const bool ok = group < groups && t < mine && k < in;
+        float g[CM];
 #pragma unroll
-        for (int c = 0; c < kWMaxClasses; ++c) g[c] = 0.f;
-        for (int j = 0; j < n; ++j) {
-            const float av = a[(int64_t)j * in + k];
+        for (int c = 0; c < CM; ++c) g[c] = 0.f;
+        if (ok) {
+            const int j1 = min(n, (group + 1) * js);
+#pragma unroll 8
+            for (int j = group * js; j < j1; ++j) {
+                const float av = __ldg(a + (int64_t)j * in + k);
+                const float4 *dj = reinterpret_cast<const float4 *>(delta + (size_t)j * pitch);
 #pragma unroll
-            for (int c = 0; c < kWMaxClasses; ++c)
-                if (c < classes) g[c] = fmaf(delta[j * classes + c], av, g[c]);
+                for (int c4 = 0; c4 < CM / 4; ++c4) {
+                    if (4 * c4 < pitch) {
+                        const float4 d4 = dj[c4];
+                        g[4 * c4] = fmaf(d4.x, av, g[4 * c4]);
+                        g[4 * c4 + 1] = fmaf(d4.y, av, g[4 * c4 + 1]);
+                        g[4 * c4 + 2] = fmaf(d4.z, av, g[4 * c4 + 2]);
+                        g[4 * c4 + 3] = fmaf(d4.w, av, g[4 * c4 + 3]);
+                    }
+                }
+            }
         }
+        if (groups > 1) {
+            if (ok && group > 0) {
 #pragma unroll
-        for (int c = 0; c < kWMaxClasses; ++c)
-            if (c < classes) store_elem(out + (int64_t)c * in + k, g[c]);
+                for (int c = 0; c < CM; ++c)
+                    if (c < classes) sums[(((group - 1) * per + t) * classes + c) * 32 + lane] = g[c];
+            }
+            __syncthreads();
+            if (ok && group == 0) {
+                for (int q = 0; q + 1 < groups; ++q)
+#pragma unroll
+                    for (int c = 0; c < CM; ++c)
+                        if (c < classes) g[c] += sums[((q * per + t) * classes + c) * 32 + lane];
+            }
+        }
+        if (ok && group == 0) {
+#pragma unroll
+            for (int c = 0; c < CM; ++c)
+                if (c < classes) store_elem(out + (int64_t)c * in + k, g[c]);
+        }
     }
-    if (has_bias && threadIdx.x < classes) {
-        float g = 0.f;
-        for (int j = 0; j < n; ++j) g += delta[j * classes + threadIdx.x];
-        store_elem(out + (int64_t)classes * in + threadIdx.x, g);
+    if (has_bias && rank == kWCluster - 1) {  // the block with the fewest input indices
+        for (int c = warp; c < classes; c += kWGradWarps) {
+            float g = 0.f;
+            for (int j = lane; j < n; j += 32) g += delta[(size_t)j * pitch + c];
+#pragma unroll
+            for (int s = 16; s >= 1; s >>= 1) g += __shfl_xor_sync(0xffffffffu, g, s);
+            if (lane == 0) store_elem(out + (int64_t)classes * in + c, g);
+        }
     }
+}
+
+inline size_t worker_grad_smem(int in, int classes, int n) {
+    const int per = ((in + 31) / 32 + kWCluster - 1) / kWCluster;
+    const int groups = per >= kWGradWarps ? 1 : kWGradWarps / per;
+    return ((size_t)n * ((classes + 3) & ~3) + (size_t)(groups - 1) * per * classes * 32) * sizeof(float);
+}
+
+template <typename T, int CM>
+cudaError_t launch_softmax(Context &c, const T *x, int in, int classes, const float *feats, const int32_t *labels, int n,
+                           int m, const int32_t *flip, T *V, int64_t ldv, cudaStream_t s) {
+    const size_t smem = worker_grad_smem(in, classes, n);
+    static PerDeviceOnce attr_set;
+    if (attr_set.need(c.device)) {
+        cudaError_t e = cudaFuncSetAttribute(worker_grad_softmax_kernel<T, CM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kWMaxSmem);
+        if (e != cudaSuccess) return e;
+        attr_set.mark(c.device);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kWCluster, m);
+    cfg.blockDim = dim3(kWGradWarps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kWCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chain_launches(c) ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, worker_grad_softmax_kernel<T, CM>, x, in, classes, (int)c.desc.has_bias, feats, labels, n, flip,
+                              V, ldv);
+}
+
+template <typename T>
+cudaError_t launch_softmax_classes(Context &c, const T *x, int in, int classes, const float *feats, const int32_t *labels, int n,
+                                   int m, const int32_t *flip, T *V, int64_t ldv, cudaStream_t s) {
+    if (classes <= 4) return launch_softmax<T, 4>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
+    if (classes <= 12) return launch_softmax<T, 12>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
+    return launch_softmax<T, kWMaxClasses>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
 }
 
 // Least squares, worker w = blockIdx.x: A[w][n][d], y[w][n]:  r_j = a_j . x - y_j;  grad[k] = sum_j a_j[k] r_j / n.
@@ -134,13 +266,15 @@ __global__ void __launch_bounds__(kWThreads) worker_grad_lsq_kernel(const float 
 template <typename T>
 __global__ void __launch_bounds__(256) inject_faults_kernel(T *V, int64_t ldv, int64_t d, const int32_t *faulty, int n_faulty,
                                                             int m, int mode, float eps) {
+    pdl_wait();                               // no early trigger: what follows reads V through the read-only path
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < d; k += (int64_t)gridDim.x * blockDim.x) {
         if (mode == 0) {
-            const int f0 = faulty[0];
+            const int f0 = __ldg(faulty);
             if (f0 < 0 || f0 >= m) continue;
             const float v = -load_elem(V + (int64_t)f0 * ldv + k);
+#pragma unroll 4
             for (int f = 0; f < n_faulty; ++f) {
-                const int row = faulty[f];
+                const int row = __ldg(faulty + f);
                 if (row >= 0 && row < m) store_elem(V + (int64_t)row * ldv + k, v);
             }
         } else {
@@ -172,17 +306,12 @@ cudaError_t launch_worker_gradients(Context &c, const void *x, const float *feat
         return cudaGetLastError();
     }
     const int in = (int)c.desc.dims[0], classes = (int)c.desc.dims[1];
-    const size_t smem = (size_t)n * classes * sizeof(float);
+    const int32_t *labels = static_cast<const int32_t *>(targets);
     if (c.desc.param_dtype == ZENO_BF16)
-        worker_grad_softmax_kernel<__nv_bfloat16><<<m, kWThreads, smem, s>>>(static_cast<const __nv_bfloat16 *>(x), in, classes,
-                                                                            c.desc.has_bias, features,
-                                                                            static_cast<const int32_t *>(targets), n, flip,
-                                                                            static_cast<__nv_bfloat16 *>(V), ldv);
-    else
-        worker_grad_softmax_kernel<float><<<m, kWThreads, smem, s>>>(static_cast<const float *>(x), in, classes, c.desc.has_bias,
-                                                                    features, static_cast<const int32_t *>(targets), n, flip,
-                                                                    static_cast<float *>(V), ldv);
-    return cudaGetLastError();
+        return launch_softmax_classes(c, static_cast<const __nv_bfloat16 *>(x), in, classes, features, labels, n, m, flip,
+                                      static_cast<__nv_bfloat16 *>(V), ldv, s);
+    return launch_softmax_classes(c, static_cast<const float *>(x), in, classes, features, labels, n, m, flip,
+                                  static_cast<float *>(V), ldv, s);
 }
 
 cudaError_t launch_inject_faults(Context &c, void *V, int64_t ldv, int m, const int32_t *faulty, int n_faulty, int mode,
@@ -193,10 +322,10 @@ cudaError_t launch_inject_faults(Context &c, void *V, int64_t ldv, int m, const 
     int64_t want = (c.d + 255) / 256;
     const int blocks = (int)(want < (int64_t)sms * 8 ? (want < 1 ? 1 : want) : (int64_t)sms * 8);
     if (c.desc.param_dtype == ZENO_BF16)
-        inject_faults_kernel<<<blocks, 256, 0, s>>>(static_cast<__nv_bfloat16 *>(V), ldv, c.d, faulty, n_faulty, m, mode, eps);
-    else
-        inject_faults_kernel<<<blocks, 256, 0, s>>>(static_cast<float *>(V), ldv, c.d, faulty, n_faulty, m, mode, eps);
-    return cudaGetLastError();
+        return launch_chained(inject_faults_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, s, chain_launches(c),
+                              static_cast<__nv_bfloat16 *>(V), ldv, c.d, faulty, n_faulty, m, mode, eps);
+    return launch_chained(inject_faults_kernel<float>, dim3(blocks), dim3(256), 0, s, chain_launches(c), static_cast<float *>(V),
+                          ldv, c.d, faulty, n_faulty, m, mode, eps);
 }
 
 }  // namespace zeno

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_1805_10032_b200 import synthetic as syn
 from paper_1805_10032_b200 import zeno
 
 import parity as P
@@ -50,6 +51,31 @@ def test_softmax_regression_worker_gradients_and_label_flipping(oracle):
         want = oracle.worker_gradient(MLP, F32, dims, True, x.numpy(), feats[i].numpy(), labels[i].numpy(),
                                       flip=bool(flip[i]))
         assert P.rel_l2(Vh[i, :d].numpy(), want) <= 2e-6, i
+
+
+# one and many chunks of 32 inputs a block, fewer samples than blocks, one class up to the most, both limits of n
+@pytest.mark.parametrize("n_w,dims,bias", [(1, (5, 1), True), (3, (31, 4), False), (9, (257, 5), True), (33, (300, 12), True),
+                                           (17, (1029, 13), False), (100, (64, 32), True), (12288, (6, 1), True),
+                                           (384, (4100, 32), True)])
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_softmax_worker_gradients_over_the_sizes(oracle, n_w, dims, bias, dtype):
+    g = torch.Generator().manual_seed(n_w)
+    m, d = 3, dims[0] * dims[1] + (dims[1] if bias else 0)
+    x = torch.randn(d, generator=g) * 0.1
+    x = x.to(torch.bfloat16) if dtype else x
+    feats = torch.randn(m, n_w, dims[0], generator=g)
+    labels = torch.randint(0, dims[1], (m, n_w), generator=g, dtype=torch.int32)
+    V = torch.full((m, d + 3), float("nan"), device="cuda", dtype=x.dtype)
+    with zeno.Zeno(MLP, dtype, dims, bias, m_max=m, n_r_max=4) as z:
+        z.worker_gradients(x.cuda(), feats.cuda(), labels.cuda(), V)
+        torch.cuda.synchronize()
+    Vh = V.float().cpu()
+    assert torch.isnan(Vh[:, d:]).all()
+    for i in range(m):
+        want = oracle.worker_gradient(MLP, dtype, dims, bias, syn.to_numpy_params(x), feats[i].numpy(), labels[i].numpy())
+        # binary32 logits and sums (2e-6, as above), then one rounding to the storage type (2^-9 of an entry);
+        # one class: the gradient is zero
+        assert np.linalg.norm(Vh[i, :d].numpy() - want) <= (2e-6 + (2.0 ** -9 if dtype else 0.0)) * np.linalg.norm(want), i
 
 
 def test_least_squares_worker_gradients(oracle):

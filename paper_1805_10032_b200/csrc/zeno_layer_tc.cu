@@ -760,15 +760,31 @@ cudaError_t launch_typed(Context &c, const LayerTcLaunch &l, cudaStream_t s) {
     // sit behind the ring
     const int zq_bytes = HEAD ? 4 * ((l.head->classes + 1) & ~1) * l.n_pad * 4 : 0;
     const int budget = HEAD ? kLSmemBudget - 10 * 1024 : kLSmemBudget;
-    // the activation ring gets kBStages stages, the weight ring (whose tiles come from HBM) the rest
-    a.b_stages = layer_tc_b_stages(l.n_pad);
-    a.stages = (budget - 1024 - zq_bytes - a.b_stages * b_bytes) / stage_bytes;
-    if (a.stages > kLMaxStages) a.stages = kLMaxStages;
-    if (a.stages < 2) return cudaErrorInvalidConfiguration;
     const int acc_cols = Tr::kAccPerPad * l.n_pad;
     a.n_sets = 2 * acc_cols + 2 * Tr::kACols <= kLTmemCols ? 2 : 1;
     a.n_abufs = (kLTmemCols - a.n_sets * acc_cols) / Tr::kACols;
     if (a.n_abufs > kLMaxABufs) a.n_abufs = kLMaxABufs;
+    // the activation ring gets its stages, the weight ring (whose tiles come from HBM) the rest
+    a.b_stages = layer_tc_b_stages(l.n_pad);
+    auto weight_stages = [&] {
+        const int fit = (budget - 1024 - zq_bytes - a.b_stages * b_bytes) / stage_bytes;
+        return fit > kLMaxStages ? kLMaxStages : fit;
+    };
+    a.stages = weight_stages();
+    // A barrier tells only whether the phase of the given parity was the last to complete, so a waiter must be at
+    // most one phase behind.  With an odd number of stages the two converter sets take turns on every stage, and a
+    // set can wait for a load before the stage's previous one, the other set's, has landed (loads complete in any
+    // order): it would take the phase before that for the one awaited, read stale data and release the stage twice.
+    // What a set knows is that its last A buffer was free, so every k-block up to two and n_abufs before the
+    // present one has been converted: an odd ring has to be at least that long.
+    while (a.stages == 3 && a.stages <= a.n_abufs + 1 && a.b_stages > 2) {
+        --a.b_stages;                       // four stages of weights instead of three are worth one of activations
+        a.stages = weight_stages();
+    }
+    if ((a.stages & 1) && a.stages <= a.n_abufs + 1) {
+        if (a.stages >= 5) a.n_abufs = a.stages - 2; else --a.stages;
+    }
+    if (a.stages < 2) return cudaErrorInvalidConfiguration;
     a.Hout = l.Hout;
     a.Hsplit = l.Hsplit_out;
     a.relu = LINEAR ? 0 : l.relu;          // LINEAR: raw products, the combine kernel activates

@@ -68,6 +68,21 @@ SHRUNK = {
 }
 
 
+# padded sample counts that would leave the layer kernel an odd ring of weight stages shorter than its A buffers and
+# two, on which a converter set could overtake the other one's load
+@pytest.mark.parametrize("n_r", [17, 33, 64, 83, 100, 128])
+def test_weight_rings_of_every_padded_sample_count(oracle, n_r):
+    w = syn.make_config(2, dims=(400, 160, 632, 368, 10), m=32, b=12, n_r=n_r, faults=[(12, "noise200")])
+    P.run_step_parity(oracle, w)
+    x, V, feats, tgt = P.to_device(w)
+    with zeno.from_workload(w) as z:
+        first = z.step(x, V, feats, tgt, w.gamma, w.rho, w.b)
+        for _ in range(50):
+            again = z.step(x, V, feats, tgt, w.gamma, w.rho, w.b)
+            assert all(torch.equal(a, b) for a, b in zip(first, again))
+        z.check_device_status()
+
+
 @pytest.mark.parametrize("name", sorted(SHRUNK))
 def test_step_matches_oracle_on_shrunk_workloads(oracle, name):
     index, ov = SHRUNK[name]

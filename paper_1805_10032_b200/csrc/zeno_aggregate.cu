@@ -9,6 +9,7 @@
 // (one fused multiply-add in binary32, rounded to the storage type of x), so that the step costs no
 // further pass over x; out may then be NULL.
 #include "zeno_internal.h"
+#include "zeno_tail.cuh"
 
 namespace zeno {
 
@@ -88,9 +89,9 @@ __device__ __forceinline__ void store_param(__nv_bfloat16 *p, float v) { *p = __
 // A row that is not to be added (beyond k, or an index outside [0, m)) is read from row 0 instead,
 // so that the load needs no branch, and its value is dropped.
 template <typename T, int B, Load L>
-__global__ void __launch_bounds__(256) aggregate_vec_kernel(const T *V, int64_t ldv, int64_t d, int m,
-                                                             const int32_t *idx, int k, float *out, T *xu,
-                                                             float gamma) {
+__global__ void __launch_bounds__(kRankMax) aggregate_vec_kernel(const T *V, int64_t ldv, int64_t d, int m,
+                                                             const int32_t *idx, RankArgs rank, int k, float *out,
+                                                             T *xu, float gamma) {
     constexpr int E = Group<T>::kElems;
     __shared__ int64_t rows_s[ZENO_MAX_CANDIDATES];
     pdl_wait();
@@ -98,7 +99,7 @@ __global__ void __launch_bounds__(256) aggregate_vec_kernel(const T *V, int64_t 
     // through the read-only path) must not become resident before x is final: no early trigger then, the
     // dependents start when this grid has completed.
     if (!xu) pdl_launch_dependents();
-    stage_rows(idx, k, m, ldv, rows_s);
+    if (rank.on) rank_rows(rank, m, k, ldv, rows_s); else stage_rows(idx, k, m, ldv, rows_s);
     const int64_t groups = d / E;            // whole groups; the d % E tail columns follow below
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < groups;
          g += (int64_t)gridDim.x * blockDim.x) {
@@ -152,16 +153,16 @@ __global__ void __launch_bounds__(256) aggregate_vec_kernel(const T *V, int64_t 
 
 // Any ldv >= d, any d: one element per thread.
 template <typename T>
-__global__ void __launch_bounds__(256) aggregate_scalar_kernel(const T *V, int64_t ldv, int64_t d,
-                                                                int m, const int32_t *idx, int k,
-                                                                float *out, T *xu, float gamma) {
+__global__ void __launch_bounds__(kRankMax) aggregate_scalar_kernel(const T *V, int64_t ldv, int64_t d,
+                                                                int m, const int32_t *idx, RankArgs rank,
+                                                                int k, float *out, T *xu, float gamma) {
     __shared__ int64_t rows_s[ZENO_MAX_CANDIDATES];
     pdl_wait();
     // With the in-place update the next kernel on the stream (the next step's first kernel, which reads x
     // through the read-only path) must not become resident before x is final: no early trigger then, the
     // dependents start when this grid has completed.
     if (!xu) pdl_launch_dependents();
-    stage_rows(idx, k, m, ldv, rows_s);
+    if (rank.on) rank_rows(rank, m, k, ldv, rows_s); else stage_rows(idx, k, m, ldv, rows_s);
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < d;
          j += (int64_t)gridDim.x * blockDim.x) {
         float acc = 0.f;
@@ -177,16 +178,16 @@ __global__ void __launch_bounds__(256) aggregate_scalar_kernel(const T *V, int64
 
 template <typename T, int B>
 cudaError_t launch_vec(const Context &c, int blocks, bool plain, const T *V, int64_t ldv, int m, const int32_t *idx,
-                       int k, float *out, T *xu, float gamma, cudaStream_t s) {
+                       const RankArgs &rank, int k, float *out, T *xu, float gamma, cudaStream_t s) {
     if (plain)
         return launch_chained(aggregate_vec_kernel<T, B, Load::kPlain>, dim3(blocks), dim3(256), 0, s, chain_launches(c),
-                              V, ldv, c.d, m, idx, k, out, xu, gamma);
+                              V, ldv, c.d, m, idx, rank, k, out, xu, gamma);
     return launch_chained(aggregate_vec_kernel<T, B, Load::kStreaming>, dim3(blocks), dim3(256), 0, s, chain_launches(c),
-                          V, ldv, c.d, m, idx, k, out, xu, gamma);
+                          V, ldv, c.d, m, idx, rank, k, out, xu, gamma);
 }
 
 template <typename T>
-cudaError_t launch_typed(const Context &c, const T *V, int64_t ldv, int m, const int32_t *idx, int k,
+cudaError_t launch_typed(const Context &c, const T *V, int64_t ldv, int m, const int32_t *idx, const RankArgs &rank, int k,
                          float *out, T *xu, float gamma, bool aligned, cudaStream_t s) {
     const int sms = c.sm_count > 0 ? c.sm_count : 148;
     const int64_t d = c.d;
@@ -200,30 +201,32 @@ cudaError_t launch_typed(const Context &c, const T *V, int64_t ldv, int m, const
         // selected rows of more than four L2 capacities: plain loads; below: streaming loads
         const bool plain = (double)k * (double)d * sizeof(T) > 4.0 * 126.0 * 1024 * 1024;
         // rows in flight per thread: the largest of 8, 6, 5, 4 that divides k (no ragged last batch), else 6
-        if (k % 8 == 0) return launch_vec<T, 8>(c, blocks, plain, V, ldv, m, idx, k, out, xu, gamma, s);
-        if (k % 6 == 0) return launch_vec<T, 6>(c, blocks, plain, V, ldv, m, idx, k, out, xu, gamma, s);
-        if (k % 5 == 0) return launch_vec<T, 5>(c, blocks, plain, V, ldv, m, idx, k, out, xu, gamma, s);
-        if (k % 4 == 0) return launch_vec<T, 4>(c, blocks, plain, V, ldv, m, idx, k, out, xu, gamma, s);
-        return launch_vec<T, 6>(c, blocks, plain, V, ldv, m, idx, k, out, xu, gamma, s);
+        if (k % 8 == 0) return launch_vec<T, 8>(c, blocks, plain, V, ldv, m, idx, rank, k, out, xu, gamma, s);
+        if (k % 6 == 0) return launch_vec<T, 6>(c, blocks, plain, V, ldv, m, idx, rank, k, out, xu, gamma, s);
+        if (k % 5 == 0) return launch_vec<T, 5>(c, blocks, plain, V, ldv, m, idx, rank, k, out, xu, gamma, s);
+        if (k % 4 == 0) return launch_vec<T, 4>(c, blocks, plain, V, ldv, m, idx, rank, k, out, xu, gamma, s);
+        return launch_vec<T, 6>(c, blocks, plain, V, ldv, m, idx, rank, k, out, xu, gamma, s);
     }
     const int64_t want = (d + 255) / 256;
     int blocks = (int)(want < cap ? want : cap);
     if (blocks < 1) blocks = 1;
     return launch_chained(aggregate_scalar_kernel<T>, dim3(blocks), dim3(256), 0, s, chain_launches(c), V, ldv, d, m,
-                          idx, k, out, xu, gamma);
+                          idx, rank, k, out, xu, gamma);
 }
 
 }  // namespace
 
 cudaError_t launch_aggregate(Context &c, const void *V, int64_t ldv, int m,
-                             const int32_t *idx, int k, float *out, void *xu, float gamma, bool aligned,
+                             const int32_t *idx, const RankArgs *rank_in, int k, float *out, void *xu, float gamma, bool aligned,
                              cudaStream_t s, int *launches) {
+    RankArgs rank = {};
+    if (rank_in) rank = *rank_in;
     ++*launches;
     profile_mark(c, "aggregate", s);
     if (c.desc.param_dtype == ZENO_BF16)
-        return launch_typed(c, static_cast<const __nv_bfloat16 *>(V), ldv, m, idx, k, out, static_cast<__nv_bfloat16 *>(xu),
+        return launch_typed(c, static_cast<const __nv_bfloat16 *>(V), ldv, m, idx, rank, k, out, static_cast<__nv_bfloat16 *>(xu),
                             gamma, aligned, s);
-    return launch_typed(c, static_cast<const float *>(V), ldv, m, idx, k, out, static_cast<float *>(xu), gamma, aligned, s);
+    return launch_typed(c, static_cast<const float *>(V), ldv, m, idx, rank, k, out, static_cast<float *>(xu), gamma, aligned, s);
 }
 
 }  // namespace zeno

@@ -125,7 +125,7 @@ zeno_status check_common(const Context *c, const void *V, int64_t ldv, int32_t m
 // cross-entropy and the scoring tail as for the dense models.
 zeno_status enqueue_score_cnn(Context *c, const void *x, const void *V, int64_t ldv, int32_t m, const zeno_batch *batch,
                               float gamma, float rho, float *scores, float *loss_buf, float *norms, int keep,
-                              int32_t *idx, bool *ranked, bool aligned, cudaStream_t s, int *launches) {
+                              int32_t *idx, zeno::RankArgs *rank, bool aligned, cudaStream_t s, int *launches) {
     const int n_r = batch->n_r, L = c->desc.n_layers, lc = L - 1;
     const int classes = (int)c->desc.dims[lc + 2];
     zeno::TailArgs tail;
@@ -142,6 +142,7 @@ zeno_status enqueue_score_cnn(Context *c, const void *x, const void *V, int64_t 
     tail.idx = idx;
     tail.keep = keep;
     tail.ticket = c->tickets;
+    tail.defer = rank != nullptr;
     int side = (int)c->desc.dims[0];
     cudaError_t e = cudaSuccess;
     for (int l = 0; l < lc; ++l) {
@@ -202,18 +203,23 @@ zeno_status enqueue_score_cnn(Context *c, const void *x, const void *V, int64_t 
         e = zeno::launch_mlp_loss(*c, c->act[lc & 1], static_cast<const int32_t *>(batch->targets), n_r, m, classes,
                                   loss_buf, tail, s, launches);
         if (e != cudaSuccess) return fail_cuda(c, e);
+        if (rank && zeno::mlp_loss_groups(n_r, classes) > 1) {
+            rank->loss_sum = c->loss_part;
+            rank->groups = zeno::mlp_loss_groups(n_r, classes);
+        }
     }
-    *ranked = keep > 0;
     return ZENO_OK;
 }
 
 // keep > 0 asks for the ranking as well (idx[0..keep)); *ranked tells whether the scoring pass
-// delivered it (the MLP tail does) or a separate select launch is still needed.
+// delivered it (the MLP tail does) or a separate select launch is still needed.  rank_in != NULL: the averaging
+// kernel that follows scores and ranks (softmax losses, up to kRankMax candidates); it is filled in and switched on.
 zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv, int32_t m,
                           const zeno_batch *batch, float gamma, float rho, float *scores,
-                          float *losses, float *norms, int keep, int32_t *idx, bool *ranked,
+                          float *losses, float *norms, int keep, int32_t *idx, bool *ranked, zeno::RankArgs *rank_in,
                           cudaStream_t s, int *launches) {
     *ranked = false;
+    zeno::RankArgs *rank = m <= zeno::kRankMax && c->desc.kind != ZENO_LOSS_LEAST_SQUARES ? rank_in : nullptr;
     zeno_status st = check_common(c, V, ldv, m);
     if (st != ZENO_OK) return st;
     if (!x || !batch || !batch->features || !batch->targets || !scores) return ZENO_ERR_INVALID_ARG;
@@ -224,6 +230,16 @@ zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv,
     const bool aligned = score_rows_aligned(*c, x, V, ldv, batch->features);
     float *loss_buf = losses ? losses : c->losses;
     cudaError_t e = cudaSuccess;
+    if (rank) {
+        rank->on = 1;
+        rank->loss_sum = c->loss_sum;
+        rank->groups = 1;
+        rank->norm_tot = c->norms;
+        rank->rho = rho;
+        rank->n_r = n_r;
+        rank->scores = scores;
+        rank->idx = idx;
+    }
 
     if (c->desc.kind == ZENO_LOSS_LEAST_SQUARES) {
         zeno::LsqArgs a;
@@ -241,8 +257,9 @@ zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv,
         return e == cudaSuccess ? ZENO_OK : fail_cuda(c, e);
     }
 
+    if (keep > 0) *ranked = true;          // the tail of the pass, or the averaging kernel
     if (c->desc.kind == ZENO_LOSS_SOFTMAX_CNN)
-        return enqueue_score_cnn(c, x, V, ldv, m, batch, gamma, rho, scores, loss_buf, norms, keep, idx, ranked, aligned, s, launches);
+        return enqueue_score_cnn(c, x, V, ldv, m, batch, gamma, rho, scores, loss_buf, norms, keep, idx, rank, aligned, s, launches);
 
     const int L = c->desc.n_layers;
     zeno::TailArgs tail;
@@ -259,6 +276,7 @@ zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv,
     tail.idx = idx;
     tail.keep = keep;
     tail.ticket = c->tickets;
+    tail.defer = rank != nullptr;
     const float *xf = static_cast<const float *>(x);
     const float *Vf = static_cast<const float *>(V);
     const int classes = (int)c->desc.dims[L];
@@ -349,7 +367,6 @@ zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv,
             e = zeno::launch_layer_tc(*c, t, s, launches);
             if (e != cudaSuccess) return fail_cuda(c, e);
             if (with_head) {
-                *ranked = keep > 0;
                 return ZENO_OK;
             }
             if (t.linear) {
@@ -424,8 +441,11 @@ zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv,
         e = zeno::launch_mlp_loss(*c, c->act[(L - 1) & 1], static_cast<const int32_t *>(batch->targets),
                                   n_r, m, classes, loss_buf, tail, s, launches);
         if (e != cudaSuccess) return fail_cuda(c, e);
+        if (rank && zeno::mlp_loss_groups(n_r, classes) > 1) {
+            rank->loss_sum = c->loss_part;
+            rank->groups = zeno::mlp_loss_groups(n_r, classes);
+        }
     }
-    *ranked = keep > 0;
     return ZENO_OK;
 }
 
@@ -439,11 +459,11 @@ zeno_status enqueue_select(Context *c, const float *scores, int32_t m, int32_t b
 
 // xu: NULL, or the parameter vector that takes Algorithm 1's update in the same pass (out may then be NULL)
 zeno_status enqueue_aggregate(Context *c, const void *V, int64_t ldv, int32_t m, const int32_t *idx,
-                              int32_t k, float *out, void *xu, float gamma, cudaStream_t s, int *launches) {
+                              const zeno::RankArgs *rank, int32_t k, float *out, void *xu, float gamma, cudaStream_t s, int *launches) {
     zeno_status st = check_common(c, V, ldv, m);
     if (st != ZENO_OK) return st;
     if (!idx || (!out && !xu) || k < 1 || k > m) return ZENO_ERR_INVALID_ARG;
-    cudaError_t e = zeno::launch_aggregate(*c, V, ldv, m, idx, k, out, xu, gamma,
+    cudaError_t e = zeno::launch_aggregate(*c, V, ldv, m, idx, rank && rank->on ? rank : nullptr, k, out, xu, gamma,
                                            aggregate_rows_aligned(*c, V, ldv, out, xu), s, launches);
     return e == cudaSuccess ? ZENO_OK : fail_cuda(c, e);
 }
@@ -673,7 +693,7 @@ zeno_status zeno_score(zeno_handle h, const void *x, const void *V, int64_t ldv,
     profile_begin(h);
     bool ranked = false;
     zeno_status st = enqueue_score(h, x, V, ldv, m, batch, gamma, rho, scores, losses, norms, 0, nullptr,
-                                   &ranked, static_cast<cudaStream_t>(stream), &launches);
+                                   &ranked, nullptr, static_cast<cudaStream_t>(stream), &launches);
     profile_end(h, static_cast<cudaStream_t>(stream));
     h->last_launches = st == ZENO_OK ? launches : 0;
     return st;
@@ -701,7 +721,7 @@ zeno_status zeno_aggregate(zeno_handle h, const void *V, int64_t ldv, int32_t m,
     if (guard.err != cudaSuccess) return fail_cuda(h, guard.err);
     int launches = 0;
     profile_begin(h);
-    zeno_status st = enqueue_aggregate(h, V, ldv, m, idx, k, out, nullptr, 0.f, static_cast<cudaStream_t>(stream),
+    zeno_status st = enqueue_aggregate(h, V, ldv, m, idx, nullptr, k, out, nullptr, 0.f, static_cast<cudaStream_t>(stream),
                                        &launches);
     profile_end(h, static_cast<cudaStream_t>(stream));
     h->last_launches = st == ZENO_OK ? launches : 0;
@@ -845,10 +865,11 @@ zeno_status zeno_step(zeno_handle h, const void *x, const void *V, int64_t ldv, 
     int launches = 0;
     profile_begin(h);
     bool ranked = false;
+    zeno::RankArgs rank = {};
     zeno_status st = enqueue_score(h, x, V, ldv, m, batch, gamma, rho, score_buf, nullptr, nullptr, m - b,
-                                   idx_buf, &ranked, s, &launches);
+                                   idx_buf, &ranked, &rank, s, &launches);
     if (st == ZENO_OK && !ranked) st = enqueue_select(h, score_buf, m, b, idx_buf, s, &launches);
-    if (st == ZENO_OK) st = enqueue_aggregate(h, V, ldv, m, idx_buf, m - b, out, nullptr, 0.f, s, &launches);
+    if (st == ZENO_OK) st = enqueue_aggregate(h, V, ldv, m, idx_buf, &rank, m - b, out, nullptr, 0.f, s, &launches);
     profile_end(h, s);
     h->last_launches = st == ZENO_OK ? launches : 0;
     return st;
@@ -868,11 +889,12 @@ zeno_status zeno_step_update(zeno_handle h, void *x, const void *V, int64_t ldv,
     int launches = 0;
     profile_begin(h);
     bool ranked = false;
+    zeno::RankArgs rank = {};
     zeno_status st = enqueue_score(h, x, V, ldv, m, batch, gamma, rho, score_buf, nullptr, nullptr, m - b,
-                                   idx_buf, &ranked, s, &launches);
+                                   idx_buf, &ranked, &rank, s, &launches);
     if (st == ZENO_OK && !ranked) st = enqueue_select(h, score_buf, m, b, idx_buf, s, &launches);
     // the scoring pass has read x by the time the average is formed: the update goes in place
-    if (st == ZENO_OK) st = enqueue_aggregate(h, V, ldv, m, idx_buf, m - b, out, x, gamma, s, &launches);
+    if (st == ZENO_OK) st = enqueue_aggregate(h, V, ldv, m, idx_buf, &rank, m - b, out, x, gamma, s, &launches);
     profile_end(h, s);
     h->last_launches = st == ZENO_OK ? launches : 0;
     return st;
@@ -903,10 +925,11 @@ zeno_status zeno_run(zeno_handle h, void *x, const void *V, int64_t ldv, int64_t
         float *score_buf = scores ? scores + (size_t)t * m : h->scores;
         int32_t *idx_buf = idx ? idx + (size_t)t * (m - b) : h->idx;
         bool ranked = false;
+        zeno::RankArgs rank = {};
         st = enqueue_score(h, x, Vt, ldv, m, &batch, gamma, rho, score_buf, nullptr, nullptr, m - b, idx_buf, &ranked,
-                           s, &launches);
+                           &rank, s, &launches);
         if (st == ZENO_OK && !ranked) st = enqueue_select(h, score_buf, m, b, idx_buf, s, &launches);
-        if (st == ZENO_OK) st = enqueue_aggregate(h, Vt, ldv, m, idx_buf, m - b, nullptr, x, gamma, s, &launches);
+        if (st == ZENO_OK) st = enqueue_aggregate(h, Vt, ldv, m, idx_buf, &rank, m - b, nullptr, x, gamma, s, &launches);
     }
     profile_end(h, s);
     h->last_launches = st == ZENO_OK ? launches : 0;
@@ -965,10 +988,11 @@ zeno_status zeno_step_host(zeno_handle h, const void *x, const void *V, int64_t 
     int launches = 0;
     profile_begin(h);
     bool ranked = false;
+    zeno::RankArgs rank = {};
     zeno_status st = enqueue_score(h, dx, dV, ldv, m, &batch, gamma, rho, h->scores, nullptr, nullptr, m - b,
-                                   h->idx, &ranked, s, &launches);
+                                   h->idx, &ranked, &rank, s, &launches);
     if (st == ZENO_OK && !ranked) st = enqueue_select(h, h->scores, m, b, h->idx, s, &launches);
-    if (st == ZENO_OK) st = enqueue_aggregate(h, dV, ldv, m, h->idx, m - b, dout, nullptr, 0.f, s, &launches);
+    if (st == ZENO_OK) st = enqueue_aggregate(h, dV, ldv, m, h->idx, &rank, m - b, dout, nullptr, 0.f, s, &launches);
     profile_end(h, s);
     if (st != ZENO_OK) {
         h->last_launches = 0;

@@ -121,6 +121,23 @@ struct TailArgs {
     int32_t *idx;       // used if keep > 0
     int keep;           // m - b, or 0: no ranking wanted
     unsigned *ticket;   // zero between launches
+    int defer;          // leave it at loss_sum and norm_tot: the averaging kernel scores and ranks
+};
+
+// The score and the ranking formed at the head of every block of the averaging kernel, from what the scoring
+// pass left.  A pass that ends in one block's ticket, score and sort puts about 3 us of dependent loads and
+// barriers between two kernels of a step; here the same loads take the place of the one for the row indices.
+// Up to kRankMax candidates (a thread each), where counting the better ones costs m shared-memory reads.
+constexpr int kRankMax = 256;
+struct RankArgs {
+    int on;                    // 0: the row indices are given
+    const double *loss_sum;    // [m+1][groups] sums of the models' sample losses
+    int groups;
+    const float *norm_tot;     // [m]
+    float rho;
+    int n_r;
+    float *scores;             // [m] and
+    int32_t *idx;              // [m - b], written by the first block
 };
 
 // One dense layer of all m+1 models (candidate 0 is x itself).
@@ -171,6 +188,7 @@ cudaError_t launch_lsq_from_sums(Context &c, const double *sums, int m, int n_r,
                                  float rho, float *losses, float *norms, float *scores, cudaStream_t s,
                                  int *launches);
 bool mlp_can_fuse_loss(int out, int n_r);
+int mlp_loss_groups(int n_r, int classes);   // blocks per model of the loss kernel
 // Warp-MMA version of the layer kernel (16-byte aligned rows, in % 8 == 0).
 cudaError_t launch_mlp_layer_mma(Context &c, const LayerArgs &a, cudaStream_t s, int *launches);
 int mlp_mma_norm_slots(int out);
@@ -181,8 +199,9 @@ cudaError_t launch_lsq_score(Context &c, const LsqArgs &a, const float *y, float
 cudaError_t launch_select(Context &c, const float *scores, int m, int b, int32_t *idx, cudaStream_t s,
                           int *launches);
 // xu != NULL: the parameter vector to update in the same pass, xu <- xu - gamma out (out may be NULL)
+// rank: how the rows are found (idx is not read then), or NULL
 cudaError_t launch_aggregate(Context &c, const void *V, int64_t ldv, int m,
-                             const int32_t *idx, int k, float *out, void *xu, float gamma, bool aligned,
+                             const int32_t *idx, const RankArgs *rank, int k, float *out, void *xu, float gamma, bool aligned,
                              cudaStream_t s, int *launches);
 
 // One convolutional layer (3 x 3, stride 1, zero padding 1, ReLU, optionally followed by a 2 x 2 max
@@ -310,6 +329,27 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// The same with the grid's x blocks grouped into clusters of `cluster`.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_clustered(void (*kernel)(KArgs...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                    bool overlap, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t hi16_in_low) {
     return __uint_as_float(hi16_in_low << 16);
 }
@@ -367,6 +407,26 @@ __device__ __forceinline__ float warp_transpose_reduce(float (&v)[N], int lane) 
 #pragma unroll
     for (int s = N; s < 32; s <<= 1) r += __shfl_xor_sync(0xffffffffu, r, s);
     return r;
+}
+
+// ---- thread-block clusters
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();                             // .aligned: the warp has to arrive as one
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// address, in the cluster's shared window, of this block's shared variable p as block `rank` has it
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, unsigned rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
 // ReLU that lets a NaN through

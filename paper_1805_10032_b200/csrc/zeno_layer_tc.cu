@@ -638,7 +638,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 if (head_last) {                       // uniform in the group; rewritten only after the barriers below
                     __threadfence();
                     head_finish_model<T>(a, model, zq, g);
-                    if (g == 0) {
+                    if (g == 0 && !a.head.tail.defer) {
                         const unsigned tk = atomicAdd(a.head.tail.ticket, 1u);
                         if (tk == (unsigned)a.m) {
                             *a.head.tail.ticket = 0;

@@ -9,9 +9,9 @@
 // the next 128 columns are issued before the current ones are consumed; the layer's input
 // activations are staged through shared memory, double buffered.
 //
-// A small last layer (mlp_head_kernel) runs as one block per model and also evaluates the
-// cross-entropy; the block that finishes last (a ticket, no waiting) then forms the scores and the
-// ranking, so the whole tail of the scoring pass costs no extra launch.
+// A small last layer (mlp_head_kernel) runs as one cluster of blocks per model and also evaluates the
+// cross-entropy.  In a step the averaging kernel forms the scores and the ranking from the losses; in a call that
+// ends with the scores the block that finishes last (a ticket, no waiting) does, so neither costs a launch.
 #include "zeno_internal.h"
 #include "zeno_tail.cuh"
 
@@ -221,28 +221,35 @@ __global__ void __launch_bounds__(kLayerWarps * 32, 1) mlp_layer_kernel(LayerArg
 }
 
 // The last layer when it is small (out <= 32 classes and n_r <= 32 samples, or out <= 16 and
-// n_r <= 64): one block per model
-// computes all of the model's logits, its cross-entropy, and -- in the block that finishes last --
-// the scores and the ranking.  The block first forms w = x - gamma v for the layer's rows in
-// shared memory (coalesced loads, v^2 accumulated on the way) next to the model's input
-// activations; then warp q multiplies samples SPW q .. SPW q + SPW - 1 against all rows, lanes
-// striding k.
+// n_r <= 64): a cluster of blocks per model computes all of the model's logits and its cross-entropy.
+// Block r of the cluster takes a slice of the input range: it forms w = x - gamma v for its columns of the layer's
+// rows in shared memory (coalesced loads, v^2 accumulated on the way) next to its columns of the model's input
+// activations; warp q multiplies samples SPW q .. SPW q + SPW - 1 against all rows, lanes striding k; the partial
+// logits go to the first block's shared memory, which adds them up and takes the loss, a warp per sample.
+// The work is a chain of latencies (784 x 10 of 21 models: 0.7 MB), so the slices are short enough for all of a
+// block's loads to be in flight at once and everything else a block needs is requested with them.
 template <typename T, int OUT_T, int SPW, bool VEC>
-__global__ void __launch_bounds__(256, 1) mlp_head_kernel(LayerArgs a) {
-    constexpr int KC = 512;                      // k-extent staged per pass
-    constexpr int NS = 8 * SPW;                  // samples a block can hold
+__global__ void __launch_bounds__(256) mlp_head_kernel(LayerArgs a, int cluster, int kslice, int KC) {
+    constexpr int NS = 8 * SPW;                  // samples a cluster can hold
+    constexpr int kRows = OUT_T / 8;             // rows a warp stages
+    constexpr int kMaxIter = 4;                  // KC / 128 at most
     extern __shared__ __align__(16) float smem_dyn[];
-    float(*ws)[KC] = reinterpret_cast<float(*)[KC]>(smem_dyn);                  // [OUT_T][KC]
-    float(*hs)[KC] = reinterpret_cast<float(*)[KC]>(smem_dyn + OUT_T * KC);     // [NS][KC]
-    __shared__ float zl[32][NS + 1];
+    float *ws = smem_dyn;                                            // [OUT_T][KC]
+    float *hs = ws + OUT_T * KC;                                     // [NS][KC]
+    float *zp = hs + NS * KC;                                        // [cluster][NS][OUT_T], the first block's is used
+    float *np = zp + cluster * NS * OUT_T;                           // [cluster][8] sums of v^2, likewise
+    __shared__ double loss_s[NS];
 
     // The weights are inputs of the whole call: unless this is the call's first kernel (what precedes it
     // on the stream may then still be producing x or V), they are read while the kernel that produces the
     // activations is still running.
     if (a.first_in_call) pdl_wait();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c = blockIdx.x;
+    const int rank = (int)cluster_rank();
+    const int c = blockIdx.x / cluster;
     const int K = a.in;
+    const int k0 = rank * kslice, k1 = min(K, k0 + kslice);
     const bool has_v = c > 0;
     const T *xw = static_cast<const T *>(a.x) + a.offW;
     const T *vbase = static_cast<const T *>(a.V) + (has_v ? (int64_t)(c - 1) * a.ldv : 0);
@@ -255,154 +262,192 @@ __global__ void __launch_bounds__(256, 1) mlp_head_kernel(LayerArgs a) {
 #pragma unroll
         for (int q = 0; q < SPW; ++q) acc[o][q] = 0.f;
     float nrm = 0.f;
-    // bias of the rows this lane ends up with after the reduction: requested now, used at the end
-    constexpr int kBatches = OUT_T * SPW / 32;
-    float bias_x[kBatches], bias_v[kBatches];
+    // the first block's: a lane's bias entry and the warp's labels, requested now, used at the end
+    float bias_x = 0.f, bias_v = 0.f;
+    int lab[SPW];
 #pragma unroll
-    for (int bi = 0; bi < kBatches; ++bi) {
-        const int o = bi * (32 / SPW) + lane / SPW;
-        const bool ok = a.offB >= 0 && o < a.out;
-        bias_x[bi] = ok ? load_elem(static_cast<const T *>(a.x) + a.offB + o) : 0.f;
-        bias_v[bi] = ok && has_v ? load_elem(vbase + a.offB + o) : 0.f;
+    for (int q = 0; q < SPW; ++q) lab[q] = 0;
+    if (rank == 0) {
+        if (a.offB >= 0 && lane < a.out) {
+            bias_x = load_elem(static_cast<const T *>(a.x) + a.offB + lane);
+            if (has_v) bias_v = load_elem(vbase + a.offB + lane);
+            if (warp == 0) nrm = bias_v * bias_v;
+        }
+#pragma unroll
+        for (int q = 0; q < SPW; ++q)
+            if (warp + 8 * q < a.n_r) lab[q] = __ldg(a.labels + warp + 8 * q);
     }
 
-    // w = x - gamma v of the layer's rows for the chunk starting at kb (zero beyond the rows / K)
+    // w = x - gamma v of the layer's rows for the columns from kb on (zero beyond the rows and the slice)
     auto stage_weights = [&](int kb) {
         if (VEC) {
             // all of a thread's loads are issued before the first is used
-            constexpr int kPerThread = OUT_T * (KC / 4) / 256;
-            float xv[kPerThread][4], vv[kPerThread][4];
+            float xv[kRows * kMaxIter][4], vv[kRows * kMaxIter][4];
 #pragma unroll
-            for (int u = 0; u < kPerThread; ++u) {
-                const int t = threadIdx.x + u * 256;
-                const int o = t / (KC / 4), kk = (t % (KC / 4)) * 4;
+            for (int u = 0; u < kRows * kMaxIter; ++u) {
+                const int o = warp + 8 * (u / kMaxIter), kk = (u % kMaxIter) * 128 + 4 * lane;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) xv[u][e] = vv[u][e] = 0.f;
-                if (o < a.out && kb + kk < K) {
+                if (o < a.out && kk < KC && kb + kk < k1) {
                     load_vec4(xw + (int64_t)o * K + kb + kk, xv[u]);
                     if (has_v) load_vec4(vw + (int64_t)o * K + kb + kk, vv[u]);
                 }
             }
 #pragma unroll
-            for (int u = 0; u < kPerThread; ++u) {
-                const int t = threadIdx.x + u * 256;
-                const int o = t / (KC / 4), kk = (t % (KC / 4)) * 4;
-                float w4[4];
+            for (int u = 0; u < kRows * kMaxIter; ++u) {
+                const int o = warp + 8 * (u / kMaxIter), kk = (u % kMaxIter) * 128 + 4 * lane;
+                if (kk < KC) {
+                    float w4[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    w4[e] = candidate_param<T>(xv[u][e], vv[u][e], a.gamma);
-                    nrm = fmaf(vv[u][e], vv[u][e], nrm);
+                    for (int e = 0; e < 4; ++e) {
+                        w4[e] = candidate_param<T>(xv[u][e], vv[u][e], a.gamma);
+                        nrm = fmaf(vv[u][e], vv[u][e], nrm);
+                    }
+                    *reinterpret_cast<float4 *>(ws + o * KC + kk) = make_float4(w4[0], w4[1], w4[2], w4[3]);
                 }
-                *reinterpret_cast<float4 *>(&ws[o][kk]) = make_float4(w4[0], w4[1], w4[2], w4[3]);
             }
         } else {
-            for (int t = threadIdx.x; t < OUT_T * KC; t += 256) {
-                const int o = t / KC, kk = t % KC;
-                float w = 0.f;
-                if (o < a.out && kb + kk < K) {
-                    const float xv = load_elem(xw + (int64_t)o * K + kb + kk);
-                    const float vv = has_v ? load_elem(vw + (int64_t)o * K + kb + kk) : 0.f;
-                    w = candidate_param<T>(xv, vv, a.gamma);
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+                const int o = warp + 8 * r;
+#pragma unroll 8
+                for (int kk = lane; kk < KC; kk += 32) {
+                    float xv = 0.f, vv = 0.f;
+                    if (o < a.out && kb + kk < k1) {
+                        xv = load_elem(xw + (int64_t)o * K + kb + kk);
+                        if (has_v) vv = load_elem(vw + (int64_t)o * K + kb + kk);
+                    }
+                    ws[o * KC + kk] = candidate_param<T>(xv, vv, a.gamma);
                     nrm = fmaf(vv, vv, nrm);
                 }
-                ws[o][kk] = w;
             }
         }
     };
-    // the model's input activations for the chunk (asynchronous copies on the vector path)
+    // the model's input activations for the same columns (asynchronous copies on the vector path)
     auto stage_acts = [&](int kb) {
-        if (VEC) {
-            for (int t = threadIdx.x; t < NS * (KC / 4); t += 256) {
-                const int j = t / (KC / 4), kk = (t % (KC / 4)) * 4;
-                const bool ok = j < a.n_r && kb + kk < K;
-                cp_async16(&hs[j][kk], ok ? hin + (int64_t)j * K + kb + kk : a.Hin, ok);
-            }
-            cp_async_commit();
-        } else {
-            for (int t = threadIdx.x; t < NS * KC; t += 256) {
-                const int j = t / KC, kk = t % KC;
-                hs[j][kk] = (j < a.n_r && kb + kk < K) ? __ldg(hin + (int64_t)j * K + kb + kk) : 0.f;
+#pragma unroll
+        for (int q = 0; q < SPW; ++q) {
+            const int j = warp + 8 * q;
+            if (VEC) {
+                for (int kk = 4 * lane; kk < KC; kk += 128) {
+                    const bool ok = j < a.n_r && kb + kk < k1;
+                    cp_async16(hs + j * KC + kk, ok ? hin + (int64_t)j * K + kb + kk : a.Hin, ok);
+                }
+            } else {
+#pragma unroll 8
+                for (int kk = lane; kk < KC; kk += 32)
+                    hs[j * KC + kk] = (j < a.n_r && kb + kk < k1) ? __ldg(hin + (int64_t)j * K + kb + kk) : 0.f;
             }
         }
+        if (VEC) cp_async_commit();
     };
 
-    stage_weights(0);
+    if (k0 < k1) stage_weights(k0);
     pdl_wait();
     pdl_launch_dependents();
-    for (int kb = 0; kb < K; kb += KC) {
-        if (kb > 0) __syncthreads();
+    for (int kb = k0; kb < k1; kb += KC) {
+        if (kb > k0) __syncthreads();
         stage_acts(kb);                 // in flight while the weights are formed
-        if (kb > 0) stage_weights(kb);
+        if (kb > k0) stage_weights(kb);
         if (VEC) cp_async_wait<0>();
         __syncthreads();
         // warp q: its SPW samples against every row; lane l takes k = 4l + 128 i
+        if (warp * SPW < a.n_r) {
 #pragma unroll 1
-        for (int i = 0; i < KC / 128; ++i) {
-            if (kb + i * 128 >= K) break;
-            const int kk = i * 128 + 4 * lane;
-            float4 h4[SPW];
+            for (int kk = 4 * lane; kk < KC; kk += 128) {
+                if (kb + kk - 4 * lane >= k1) break;
+                float4 h4[SPW];
 #pragma unroll
-            for (int q = 0; q < SPW; ++q) h4[q] = *reinterpret_cast<const float4 *>(&hs[warp * SPW + q][kk]);
+                for (int q = 0; q < SPW; ++q) h4[q] = *reinterpret_cast<const float4 *>(hs + (warp * SPW + q) * KC + kk);
 #pragma unroll
-            for (int o = 0; o < OUT_T; ++o) {
-                const float4 w4 = *reinterpret_cast<const float4 *>(&ws[o][kk]);
+                for (int o = 0; o < OUT_T; ++o) {
+                    const float4 w4 = *reinterpret_cast<const float4 *>(ws + o * KC + kk);
 #pragma unroll
-                for (int q = 0; q < SPW; ++q) {
-                    acc[o][q] = fmaf(w4.x, h4[q].x, acc[o][q]);
-                    acc[o][q] = fmaf(w4.y, h4[q].y, acc[o][q]);
-                    acc[o][q] = fmaf(w4.z, h4[q].z, acc[o][q]);
-                    acc[o][q] = fmaf(w4.w, h4[q].w, acc[o][q]);
+                    for (int q = 0; q < SPW; ++q) {
+                        acc[o][q] = fmaf(w4.x, h4[q].x, acc[o][q]);
+                        acc[o][q] = fmaf(w4.y, h4[q].y, acc[o][q]);
+                        acc[o][q] = fmaf(w4.z, h4[q].z, acc[o][q]);
+                        acc[o][q] = fmaf(w4.w, h4[q].w, acc[o][q]);
+                    }
                 }
             }
         }
     }
-
-    // lane totals: 32 (row, sample) pairs at a time; lane l receives pair l of the batch
-    constexpr int kRowsPerBatch = 32 / SPW;
+    // the earlier layers' partial sums of v^2 of this candidate
+    if (rank == 0 && has_v) {
+        for (int l = 0; l + 1 < a.tail.used.layers; ++l) {
+            const float *src = a.tail.normpart + (int64_t)(c - 1) * a.tail.np_slots + a.tail.used.base[l];
+            const int count = a.tail.used.count[l];
+            for (int t0 = threadIdx.x; t0 < count; t0 += 4 * 256) {
+                float v[4];
 #pragma unroll
-    for (int ob = 0; ob < OUT_T; ob += kRowsPerBatch) {
-        float v[32];
-#pragma unroll
-        for (int o = 0; o < kRowsPerBatch; ++o)
-#pragma unroll
-            for (int q = 0; q < SPW; ++q) v[o * SPW + q] = acc[ob + o][q];
-        float z = warp_transpose_reduce<32>(v, lane);
-        const int o = ob + lane / SPW, j = warp * SPW + lane % SPW;
-        if (o < a.out && j < a.n_r) {
-            if (a.offB >= 0) z += candidate_param<T>(bias_x[ob / kRowsPerBatch], bias_v[ob / kRowsPerBatch], a.gamma);
-            if (a.relu) z = relu_keep_nan(z);
-            zl[o][j] = z;
+                for (int u = 0; u < 4; ++u) v[u] = t0 + u * 256 < count ? __ldcg(src + t0 + u * 256) : 0.f;
+                nrm += (v[0] + v[1]) + (v[2] + v[3]);
+            }
         }
     }
-    // ||v||^2 of this layer's rows and bias entries: one slot per warp
-    if (has_v) {
-        if (a.offB >= 0 && threadIdx.x < a.out) {
-            const float bv = load_elem(vbase + a.offB + threadIdx.x);
-            nrm = fmaf(bv, bv, nrm);
+
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");     // every block runs: its shared memory may be written
+    // lane totals, N (row, sample) pairs at a time; lane l receives pair l of the batch
+    constexpr int N = OUT_T * SPW < 32 ? OUT_T * SPW : 32, kRowsPerBatch = N / SPW;
+    if (warp * SPW < a.n_r) {
+        const uint32_t dst = cluster_addr(zp + (size_t)rank * NS * OUT_T, 0);
+#pragma unroll
+        for (int ob = 0; ob < OUT_T; ob += kRowsPerBatch) {
+            float v[N];
+#pragma unroll
+            for (int o = 0; o < kRowsPerBatch; ++o)
+#pragma unroll
+                for (int q = 0; q < SPW; ++q) v[o * SPW + q] = acc[ob + o][q];
+            const float z = warp_transpose_reduce<N>(v, lane);
+            const int o = ob + lane / SPW, j = warp * SPW + lane % SPW;
+            if (lane < N && o < a.out && j < a.n_r) cluster_store(dst + 4 * (j * OUT_T + o), z);
         }
-        nrm = warp_sum(nrm);
-        if (lane == 0) a.normpart[(int64_t)(c - 1) * a.np_slots + a.np_base + warp] = nrm;
+    }
+    nrm = warp_sum(nrm);
+    if (lane == 0) cluster_store(cluster_addr(np + rank * 8 + warp, 0), nrm);
+    cluster_barrier();
+    if (rank != 0) return;
+    // the loss of the samples warp, warp + 8, ..: a lane per class (logits and their differences in double: the
+    // score is a difference of losses that agree in several digits)
+    const double bias = a.offB >= 0 ? (double)candidate_param<T>(bias_x, bias_v, a.gamma) : 0.0;
+#pragma unroll
+    for (int q = 0; q < SPW; ++q) {
+        const int j = warp + 8 * q;
+        if (j >= a.n_r) break;
+        double z = 0.0;
+        if (lane < a.out) {
+            for (int r = 0; r < cluster; ++r) z += (double)zp[(r * NS + j) * OUT_T + lane];
+            z += bias;
+        }
+        double zmax = lane < a.out ? z : -INFINITY;      // not rounded: a logit of 1e10 is 512 from its float
+#pragma unroll
+        for (int s = 16; s >= 1; s >>= 1) zmax = fmax(zmax, __shfl_xor_sync(0xffffffffu, zmax, s));
+        const float dz = (float)(z - zmax);
+        const float se = warp_sum(lane < a.out ? expf(dz) : 0.f);           // a NaN logit makes se NaN
+        int l = lab[q];
+        if (l < 0 || l >= a.out) l = 0;
+        const double zl = __shfl_sync(0xffffffffu, z, l);
+        if (lane == 0) loss_s[j] = (zmax - zl) + (double)logf(se);
     }
     __syncthreads();
-    if (has_v) block_norm_total(a.tail, c - 1);          // all layers' partials of this candidate
     if (warp == 0) {
         double l = 0.0;
-        for (int j = lane; j < a.n_r; j += 32) {
-            float zmax = -INFINITY;
-            for (int o = 0; o < a.out; ++o) zmax = fmaxf(zmax, zl[o][j]);
-            float se = 0.f;
-            for (int o = 0; o < a.out; ++o) se += expf(zl[o][j] - zmax);   // a NaN logit makes se NaN
-            int lab = a.labels[j];
-            if (lab < 0 || lab >= a.out) lab = 0;
-            l += (double)((zmax - zl[lab][j]) + logf(se));
-        }
+        for (int j = lane; j < a.n_r; j += 32) l += loss_s[j];
         l = warp_sum(l);
         if (lane == 0) {
             a.tail.loss_sum[c] = l;
             a.losses[c] = (float)(l / (double)a.n_r);
         }
+    } else if (warp == 1 && has_v) {
+        float nv = 0.f;
+        for (int t = lane; t < cluster * 8; t += 32) nv += np[t];
+        nv = warp_sum(nv);
+        if (lane == 0) a.tail.norm_tot[c - 1] = nv;
     }
-    if (take_last_ticket(a.tail.ticket, gridDim.x)) finalize_and_select(a.tail);
+    if (a.tail.defer) return;
+    if (take_last_ticket(a.tail.ticket, gridDim.x / cluster)) finalize_and_select(a.tail);
 }
 
 // Per model: mean over the samples of log-sum-exp(z) - z[label].  G blocks per model (block g takes
@@ -444,6 +489,7 @@ __global__ void __launch_bounds__(256) mlp_loss_kernel(const float *logits, cons
         }
     }
     if (c > 0 && g == 0) block_norm_total(tail, c - 1);
+    if (tail.defer) return;
     if (take_last_ticket(tail.ticket, gridDim.x)) {
         if (G > 1) {
             for (int i = threadIdx.x; i <= tail.m; i += blockDim.x) {
@@ -489,15 +535,33 @@ int mlp_norm_slots(int out) {
 bool mlp_can_fuse_loss(int out, int n_r) { return (out <= 32 && n_r <= 32) || (out <= 16 && n_r <= 64); }
 
 template <typename T, bool VEC>
-cudaError_t launch_head(const LayerArgs &a, cudaStream_t s, bool overlap) {
+cudaError_t launch_head(Context &c, const LayerArgs &a, cudaStream_t s) {
+    // blocks per model: as many as leave a slice of 128 columns and are resident at once (two to an SM up to 16 x 16
+    // logits, one beyond: the accumulators).  A second wave costs more than the longer slice (101 models of 512 x 10,
+    // 64 samples: 21 us with one block a model, 29 with two)
+    const int sms = c.sm_count > 0 ? c.sm_count : 148;
+    const int room = a.out <= 16 && a.n_r <= 16 ? 2 * sms : sms;
+    int cluster = 1;
+    while (cluster < 8 && a.in / (2 * cluster) >= 128 && (a.m + 1) * 2 * cluster <= room) cluster *= 2;
+    const int kslice = ((a.in + cluster - 1) / cluster + 3) / 4 * 4;
+    const int KC = kslice >= 512 ? 512 : (kslice + 127) / 128 * 128;
     auto go = [&](auto kernel, int out_t, int ns) {
-        const size_t smem = sizeof(float) * (size_t)(out_t + ns) * 512;
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        return launch_chained(kernel, dim3(a.m + 1), dim3(256), smem, s, overlap, a);
+        const size_t smem = sizeof(float) * ((size_t)(out_t + ns) * KC + (size_t)cluster * (ns * out_t + 8));
+        if (smem > 36 * 1024) {                  // 48 KB less the static part, the sort of the tail among it
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        return launch_clustered(kernel, cluster, dim3(cluster * (a.m + 1)), dim3(256), smem, s, chain_launches(c), a, cluster, kslice,
+                                KC);
     };
-    if (a.n_r > 32) return go(mlp_head_kernel<T, 16, 8, VEC>, 16, 64);
-    if (a.out <= 16) return go(mlp_head_kernel<T, 16, 4, VEC>, 16, 32);
+    if (a.out <= 16) {
+        if (a.n_r <= 8) return go(mlp_head_kernel<T, 16, 1, VEC>, 16, 8);
+        if (a.n_r <= 16) return go(mlp_head_kernel<T, 16, 2, VEC>, 16, 16);
+        if (a.n_r <= 32) return go(mlp_head_kernel<T, 16, 4, VEC>, 16, 32);
+        return go(mlp_head_kernel<T, 16, 8, VEC>, 16, 64);
+    }
+    if (a.n_r <= 8) return go(mlp_head_kernel<T, 32, 1, VEC>, 32, 8);
+    if (a.n_r <= 16) return go(mlp_head_kernel<T, 32, 2, VEC>, 32, 16);
     return go(mlp_head_kernel<T, 32, 4, VEC>, 32, 32);
 }
 
@@ -507,8 +571,8 @@ cudaError_t launch_mlp_layer(Context &c, const LayerArgs &a, bool aligned, cudaS
     profile_mark(c, a.fuse_loss ? "mlp_head_loss_tail" : "mlp_layer", s);
     if (a.fuse_loss) {
         if (c.desc.param_dtype == ZENO_BF16)
-            return aligned ? launch_head<__nv_bfloat16, true>(a, s, chain_launches(c)) : launch_head<__nv_bfloat16, false>(a, s, chain_launches(c));
-        return aligned ? launch_head<float, true>(a, s, chain_launches(c)) : launch_head<float, false>(a, s, chain_launches(c));
+            return aligned ? launch_head<__nv_bfloat16, true>(c, a, s) : launch_head<__nv_bfloat16, false>(c, a, s);
+        return aligned ? launch_head<float, true>(c, a, s) : launch_head<float, false>(c, a, s);
     }
     if (c.desc.param_dtype == ZENO_BF16)
         return aligned ? launch_layer_nrt<__nv_bfloat16, true>(a, s, chain_launches(c))
@@ -516,14 +580,18 @@ cudaError_t launch_mlp_layer(Context &c, const LayerArgs &a, bool aligned, cudaS
     return aligned ? launch_layer_nrt<float, true>(a, s, chain_launches(c)) : launch_layer_nrt<float, false>(a, s, chain_launches(c));
 }
 
+// enough blocks to spread a large batch of wide logits over the SMs
+int mlp_loss_groups(int n_r, int classes) {
+    if ((int64_t)n_r * classes < 16384) return 1;
+    return n_r >= 64 ? 8 : n_r >= 32 ? 4 : 2;
+}
+
 cudaError_t launch_mlp_loss(Context &c, const float *logits, const int32_t *labels, int n_r,
                             int m, int classes, float *losses, const TailArgs &tail, cudaStream_t s,
                             int *launches) {
     ++*launches;
     profile_mark(c, "mlp_loss_tail", s);
-    // enough blocks to spread a large batch of wide logits over the SMs
-    int G = 1;
-    if ((int64_t)n_r * classes >= 16384) G = n_r >= 64 ? 8 : n_r >= 32 ? 4 : 2;
+    const int G = mlp_loss_groups(n_r, classes);
     return launch_chained(mlp_loss_kernel, dim3((m + 1) * G), dim3(256), 0, s, chain_launches(c), logits, labels, n_r,
                           classes, losses, c.loss_part, G, tail);
 }

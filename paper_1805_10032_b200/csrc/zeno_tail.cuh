@@ -55,6 +55,36 @@ __device__ __forceinline__ void block_norm_total(const TailArgs &t, int i) {
     }
 }
 
+// Called by ALL threads of a block of at least kRankMax threads: rows_s[r] = element offset of the row with the
+// r-th highest score, r < k.  Candidate i's rank is the number of candidates with a higher key.
+__device__ __forceinline__ void rank_rows(const RankArgs &r, int m, int k, int64_t ldv, int64_t *rows_s) {
+    __shared__ unsigned long long keys[kRankMax];
+    const int i = threadIdx.x;
+    unsigned long long key = 0ull;
+    if (i < m) {
+        double s0 = 0.0, si = 0.0;
+        for (int q = 0; q < r.groups; ++q) {
+            s0 += __ldcg(r.loss_sum + q);
+            si += __ldcg(r.loss_sum + (int64_t)(1 + i) * r.groups + q);
+        }
+        const float sc = (float)((s0 - si) * (1.0 / (double)r.n_r) - (double)r.rho * (double)__ldcg(r.norm_tot + i));
+        if (blockIdx.x == 0) r.scores[i] = sc;
+        key = rank_key(sc, i);
+        keys[i] = key;
+    }
+    __syncthreads();
+    if (i < m) {
+        int rank = 0;
+#pragma unroll 8
+        for (int j = 0; j < m; ++j) rank += keys[j] > key;
+        if (rank < k) {
+            rows_s[rank] = (int64_t)i * ldv;
+            if (blockIdx.x == 0) r.idx[rank] = i;
+        }
+    }
+    __syncthreads();
+}
+
 // One block, any size.  norms[i] = the per-candidate totals left by block_norm_total;
 // scores[i] = f_0 - f_i - rho norms[i]; if keep > 0, idx[0..keep) = the candidates with the
 // highest scores in rank order (bitonic sort of the packed keys in shared memory).

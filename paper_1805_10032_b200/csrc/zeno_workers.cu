@@ -48,24 +48,6 @@ constexpr int kWCluster = 8;
 constexpr int kWGradWarps = 8;
 constexpr int kWSamples = 2;                  // samples a warp takes at a time: the weights are read once for both
 
-__device__ __forceinline__ unsigned cluster_rank() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// address, in the cluster's shared window, of this block's shared variable p as block `rank` has it
-__device__ __forceinline__ uint32_t cluster_addr(const void *p, unsigned rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ void cluster_store(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-
 // CM: classes the registers are sized for, a multiple of 4
 template <typename T, int CM>
 __global__ void __launch_bounds__(kWGradWarps * 32, 2)
@@ -212,22 +194,8 @@ cudaError_t launch_softmax(Context &c, const T *x, int in, int classes, const fl
         if (e != cudaSuccess) return e;
         attr_set.mark(c.device);
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kWCluster, m);
-    cfg.blockDim = dim3(kWGradWarps * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kWCluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = chain_launches(c) ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, worker_grad_softmax_kernel<T, CM>, x, in, classes, (int)c.desc.has_bias, feats, labels, n, flip,
-                              V, ldv);
+    return launch_clustered(worker_grad_softmax_kernel<T, CM>, kWCluster, dim3(kWCluster, m), dim3(kWGradWarps * 32), smem, s,
+                            chain_launches(c), x, in, classes, (int)c.desc.has_bias, feats, labels, n, flip, V, ldv);
 }
 
 template <typename T>

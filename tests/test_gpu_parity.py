@@ -68,6 +68,32 @@ SHRUNK = {
 }
 
 
+# the small last layer over its limits: one to eight blocks a model, slices with remainders, rows of any alignment,
+# every compiled number of classes and samples; candidates up to and beyond what the averaging kernel ranks itself
+@pytest.mark.parametrize("dims,n_r,m,dtype,pad", [
+    ((33, 2), 1, 5, "f32", 1), ((250, 10), 9, 7, "f32", 0), ((517, 16), 33, 20, "bf16", 0), ((1028, 17), 8, 9, "f32", 0),
+    ((1029, 32), 32, 37, "f32", 1), ((4100, 10), 16, 20, "bf16", 4), ((4100, 16), 64, 20, "f32", 4), ((784, 31), 17, 36, "bf16", 1),
+    ((784, 10), 4, 149, "f32", 0), ((60, 10), 4, 256, "f32", 0), ((60, 10), 4, 257, "f32", 0)])
+def test_small_last_layer_over_its_limits(oracle, dims, n_r, m, dtype, pad):
+    d = dims[0] * dims[1] + dims[1]
+    b = m // 3
+    w = syn.make_config(1, dims=dims, n_r=n_r, m=m, b=b, dtype=dtype, ldv=d + pad, faults=[(b, "signflip")])
+    P.run_step_parity(oracle, w)
+
+
+def test_small_last_layer_with_huge_logits(oracle):
+    """Noise candidates of a deep model whose logits reach 1e10, where neighbouring binary32 values are 1,024 apart:
+    their losses stay finite and they are dropped."""
+    w = syn.make_config(2, dims=(432, 448, 280, 834, 10), m=64, b=25, n_r=3, faults=[(25, "noise200")])
+    P.run_step_parity(oracle, w)
+    x, V, feats, tgt = P.to_device(w)
+    with zeno.from_workload(w) as z:
+        _, scores, idx = z.step(x, V, feats, tgt, w.gamma, w.rho, w.b)
+        _, losses, _ = z.score(x, V, feats, tgt, w.gamma, w.rho)
+    assert torch.isfinite(scores).all() and losses.max().item() > 1e9
+    assert w.honest[idx.cpu().long()].all()
+
+
 # padded sample counts that would leave the layer kernel an odd ring of weight stages shorter than its A buffers and
 # two, on which a converter set could overtake the other one's load
 @pytest.mark.parametrize("n_r", [17, 33, 64, 83, 100, 128])

@@ -145,7 +145,15 @@ zeno_status enqueue_score_cnn(Context *c, const void *x, const void *V, int64_t 
     tail.defer = rank != nullptr;
     int side = (int)c->desc.dims[0];
     cudaError_t e = cudaSuccess;
-    for (int l = 0; l < lc; ++l) {
+    if (c->cnn_net.layers) {
+        for (int l = 0; l < lc; ++l) {
+            tail.used.base[l] = c->np_base[l];
+            tail.used.count[l] = zeno::cnn_norm_slots((int)c->desc.dims[l + 2]);
+        }
+        e = zeno::launch_cnn_tc(*c, c->cnn_net, x, V, ldv, batch->features, n_r, m, gamma, c->act[(lc - 1) & 1], s, launches);
+        if (e != cudaSuccess) return fail_cuda(c, e);
+    }
+    for (int l = c->cnn_net.layers; l < lc; ++l) {
         zeno::CnnLayerArgs a;
         a.x = x;
         a.V = V;
@@ -606,6 +614,12 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
         c->np_slots = slots;
         act_elems = rows * (size_t)n_r_max * (size_t)widest;
         norm_elems = (size_t)m_max * (size_t)slots;
+        // the tensor-core layers index a layer's pixels, over all samples and planes, in 32 bits
+        int64_t most = 0;
+        for (int l = 0; l < lc; ++l) most = desc->dims[l + 1] > most ? desc->dims[l + 1] : most;
+        most = desc->dims[lc + 1] > most ? desc->dims[lc + 1] : most;
+        if (c->use_tc && ((int64_t)n_r_max + 2) * (desc->dims[0] + 1) * (desc->dims[0] + 1) * (most + 8) < ((int64_t)1 << 31))
+            zeno::cnn_tc_layout(*c, &c->cnn_net);
     } else {
         c->lsq_slabs = zeno::lsq_slab_count(*c);
         lsq_elems = ((size_t)c->lsq_slabs + 1) * rows * ((size_t)n_r_max + 1);
@@ -630,7 +644,16 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     const size_t krum_elems = m_max <= ZENO_KRUM_MAX_M ? zeno::krum_part_floats(m_max, c->krum_blocks) : 0;
     const size_t at_krum = reserve(krum_elems, 4), at_krums = reserve(m_max, 4);
 
+    // last, because a handle can do without it: with no room for it the convolutional layers run on the CUDA cores
+    const size_t without_cnn = bytes;
+    const size_t at_cnn = reserve((size_t)c->cnn_net.floats, 4);
+
     e = cudaMalloc(&c->arena, bytes);
+    if (e != cudaSuccess && c->cnn_net.layers) {
+        cudaGetLastError();
+        c->cnn_net.layers = 0;
+        e = cudaMalloc(&c->arena, without_cnn);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete c;
@@ -656,7 +679,12 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     c->head_tickets = reinterpret_cast<unsigned *>(base + at_headt);
     c->krum_part = krum_elems ? reinterpret_cast<float *>(base + at_krum) : nullptr;
     c->krum_sums = reinterpret_cast<float *>(base + at_krums);
+    if (c->cnn_net.layers) c->cnn_ws = reinterpret_cast<float *>(base + at_cnn);
     e = cudaMemset(c->dev_status, 0, sizeof(int));
+    // the padding of the planes and of the weights' operands is zero from here on; a first call may be on a stream
+    // that does not wait for the default one
+    if (e == cudaSuccess && c->cnn_net.layers) e = cudaMemset(c->cnn_ws, 0, (size_t)c->cnn_net.floats * 4);
+    if (e == cudaSuccess && c->cnn_net.layers) e = cudaStreamSynchronize(nullptr);
     if (e == cudaSuccess) e = cudaMemset(c->tickets, 0, ticket_elems * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(c->head_tickets, 0, rows * sizeof(unsigned));
     if (e != cudaSuccess) {

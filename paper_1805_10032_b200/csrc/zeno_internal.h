@@ -41,6 +41,19 @@ constexpr int kStreamTcMinKR = 128;
 // Which norm-partial slots a call filled: per layer (first slot, count).
 struct NormSlots { int base[ZENO_MAX_LAYERS]; int count[ZENO_MAX_LAYERS]; int layers; };
 
+// One convolutional layer on the tensor cores: sizes, and the places of its parts in the workspace of these layers
+// (offsets and strides in floats).
+struct CnnTcLayer {
+    int side, cin, cout, first, pool;
+    int groups, stages, nks, n, nblk, rows, lead;
+    int64_t px, in, in_model, w, w_model, bias, bias_model;
+};
+struct CnnTcNet {
+    int layers;              // 0: the layers run on the CUDA cores
+    int64_t z, floats;
+    CnnTcLayer layer[ZENO_MAX_LAYERS];
+};
+
 struct Context {
     zeno_model_desc desc;
     int64_t d;
@@ -52,6 +65,8 @@ struct Context {
     int np_base[ZENO_MAX_LAYERS];   // first norm-partial slot of layer l
     int np_slots;                   // norm-partial slots per candidate
     int64_t cnn_flat;               // convolutional network: inputs of its dense layer
+    CnnTcNet cnn_net;
+    float *cnn_ws;                  // the tensor-core layers' inputs, weights and unpooled planes
     void *arena;                    // the one device allocation everything below is carved from
     float *act[2];                  // activations [m_max+1][n_r_max][widest layer output]
     double *loss_part;              // [m_max + 1][8] per-block sums of the sample losses
@@ -224,6 +239,10 @@ struct CnnLayerArgs {
 bool cnn_side_ok(int side);
 int cnn_norm_slots(int cout);
 cudaError_t launch_cnn_conv(Context &c, const CnnLayerArgs &a, cudaStream_t s, int *launches);
+// The same layers on the tensor cores (zeno_cnn_tc.cu): all of them, the dense layer's input into `flat`.
+void cnn_tc_layout(const Context &c, CnnTcNet *net);
+cudaError_t launch_cnn_tc(Context &c, const CnnTcNet &net, const void *x, const void *V, int64_t ldv, const float *features,
+                          int n_r, int m, float gamma, float *flat, cudaStream_t s, int *launches);
 
 // Tensor-core stream for the first layer (fp32 storage).
 bool stream_tc_plan(int sms, int K, int out, int n_r, int m, StreamTcPlan *p);

@@ -43,6 +43,35 @@ def test_step_matches_oracle(oracle, name):
     assert r["agg_err"] <= P.AGG_RTOL
 
 
+# one tile and many, a pair of tiles half empty, more than 64 output planes (two items), up to four input planes (paired
+# taps) and more, sides whose lines end inside a tile, planes that are no multiple of a group, unaligned rows
+@pytest.mark.parametrize("dims,n_r,dtype", [((2, 1, 1, 1, 2), 1, "f32"), ((4, 5, 3, 70, 3), 2, "bf16"), ((28, 1, 5, 13, 10), 3, "f32"),
+                                            ((32, 4, 66, 130, 7), 2, "f32"), ((14, 3, 33, 10, 10), 17, "f32"),
+                                            ((30, 2, 8, 20, 11), 5, "bf16"), ((16, 9, 16, 16, 40, 40, 43), 6, "f32")])
+def test_tensor_core_layers_over_their_limits(oracle, dims, n_r, dtype):
+    d = syn.param_count("cnn", dims)
+    w = syn.make_config(6, dims=dims, n_r=n_r, dtype=dtype, m=5, b=2, faults=[(2, "signflip")], ldv=d + (d + 1) % 2)
+    P.run_step_parity(oracle, w)
+
+
+def test_fewer_samples_and_candidates_than_the_handle_was_made_for(oracle):
+    """The padding stays zero and nothing of a larger call is read by a smaller one."""
+    w = syn.make_config(6, dims=(16, 3, 8, 8, 12, 12, 10), m=9, b=3, n_r=11, faults=[(3, "signflip")])
+    x, V, f, t = P.to_device(w)
+    with zeno.from_workload(w) as z, zeno.Zeno(zeno.LOSS_SOFTMAX_CNN, zeno.F32, w.dims, True, 4, 3) as small:
+        z.score(x, V * float("nan"), f, t, w.gamma, w.rho)
+        got = z.score(x, V[:4], f[:3].contiguous(), t[:3], w.gamma, w.rho)
+        want = small.score(x, V[:4], f[:3].contiguous(), t[:3], w.gamma, w.rho)
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+def test_cuda_core_layers(oracle, monkeypatch):
+    """The kernel that serves without tensor cores."""
+    monkeypatch.setenv("ZENO_DISABLE_TENSOR_CORES", "1")
+    w = syn.make_config(6, dims=(16, 3, 9, 17, 20, 33, 10), m=5, b=2, n_r=6, faults=[(2, "signflip")])
+    P.run_step_parity(oracle, w)
+
+
 def test_kernels_of_the_step():
     w = syn.make_config(6, dims=(16, 3, 8, 8, 12, 12, 10), m=5, b=2, n_r=4, faults=[(2, "signflip")])
     x, V, f, t = P.to_device(w)

@@ -9,10 +9,6 @@
 
 namespace zeno {
 
-// Rows of V (and x) handled per warp in the CUDA-core kernels.
-constexpr int kRowsPerWarp = 4;
-// Warps per block in the layer kernel; one block covers kRowsPerWarp * kLayerWarps output rows.
-constexpr int kLayerWarps = 8;
 // Number of k-slabs the least-squares stream is cut into is at most this.
 constexpr int kMaxSlabs = 1024;
 // Most kernels one call can enqueue (layers + loss + finalize + select + aggregate).

@@ -81,6 +81,19 @@ def test_small_last_layer_over_its_limits(oracle, dims, n_r, m, dtype, pad):
     P.run_step_parity(oracle, w)
 
 
+# the layer kernel for rows of any alignment: one row tile and several, slices with remainders, one to eight blocks a tile,
+# every compiled number of samples, several sample tiles, no bias
+@pytest.mark.parametrize("dims,n_r,m,dtype,bias", [
+    ((65, 3, 2), 1, 3, "f32", True), ((63, 64, 5), 8, 4, "f32", False), ((1029, 65, 11), 9, 5, "f32", True),
+    ((2051, 37, 129, 10), 19, 6, "f32", True), ((515, 301, 40), 25, 37, "f32", True), ((130, 131, 33), 33, 20, "bf16", True),
+    ((4100, 43, 43), 70, 7, "bf16", True), ((257, 67, 101), 128, 5, "f32", True)])
+def test_layers_of_unaligned_rows(oracle, dims, n_r, m, dtype, bias):
+    d = syn.param_count("mlp", dims, bias)
+    b = m // 3
+    w = syn.make_config(2, dims=dims, n_r=n_r, m=m, b=b, dtype=dtype, has_bias=bias, ldv=d + (d + 1) % 2, faults=[(b, "signflip")] if b else [])
+    P.run_step_parity(oracle, w)
+
+
 def test_small_last_layer_with_huge_logits(oracle):
     """Noise candidates of a deep model whose logits reach 1e10, where neighbouring binary32 values are 1,024 apart:
     their losses stay finite and they are dropped."""

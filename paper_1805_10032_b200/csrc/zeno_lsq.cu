@@ -11,6 +11,7 @@
 #include <mutex>
 
 #include "zeno_internal.h"
+#include "zeno_tail.cuh"
 
 namespace zeno {
 
@@ -197,35 +198,53 @@ __global__ void __launch_bounds__(LsqShape<NRT, RB>::kMaxWarps * 32, 1) lsq_stre
     }
 }
 
-// One block.  Sums the slab partials in slab order (double), then
+// Sums the slab partials in double, a block per 32 entries: its eight warps take every eighth slab and their sums are
+// added in warp order.  The block that finishes last (a ticket, no waiting) forms
 //   residual r_j = (A x)_j - y_j,  f_0 = sum r_j^2 / (2 n_r),
 //   f_i = sum (r_j - gamma (A v_i)_j)^2 / (2 n_r),  score_i = f_0 - f_i - rho ||v_i||^2.
-__global__ void __launch_bounds__(1024) lsq_finish_kernel(const float *part, int slabs, int m,
-                                                           int n_r, const float *y, float gamma,
-                                                           float rho, float *losses, float *norms,
-                                                           float *scores, float *sums /*[m+1][n_r+1]*/) {
-    const int rows = m + 1, stride = n_r + 1;
-    for (int t = threadIdx.x; t < rows * stride; t += blockDim.x) {
-        double acc = 0.0;
-        for (int s = 0; s < slabs; ++s) acc += (double)part[(int64_t)s * rows * stride + t];
-        sums[t] = (float)acc;
+// One block over all entries and slabs took 40 us for 65 x 17 sums of 148 slabs, a chain of 148 loads per thread.
+constexpr int kFinishWarps = 8;
+__global__ void __launch_bounds__(kFinishWarps * 32) lsq_finish_kernel(const float *part, int slabs, int m, int n_r, const float *y,
+                                                                       float gamma, float rho, float *losses, float *norms,
+                                                                       float *scores, float *sums /*[m+1][n_r+1]*/,
+                                                                       unsigned *ticket) {
+    const int rows = m + 1, stride = n_r + 1, n = rows * stride;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double warp_s[kFinishWarps][32];
+    const int t = blockIdx.x * 32 + lane;
+    double acc = 0.0;
+    if (t < n) {
+#pragma unroll 4
+        for (int s = warp; s < slabs; s += kFinishWarps) acc += (double)__ldcg(part + (int64_t)s * n + t);
     }
+    warp_s[warp][lane] = acc;
     __syncthreads();
+    if (warp == 0 && t < n) {
+        double tot = 0.0;
+#pragma unroll
+        for (int w = 0; w < kFinishWarps; ++w) tot += warp_s[w][lane];
+        sums[t] = (float)tot;
+    }
+    if (!take_last_ticket(ticket, gridDim.x)) return;
     // the losses stay in double until the score is formed: f_0 - f_i cancels many digits
     __shared__ double f_s[ZENO_MAX_CANDIDATES + 1];
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+    for (int r = warp; r < rows; r += kFinishWarps) {                // a warp a model, lanes over the samples
         double f = 0.0;
-        for (int j = 0; j < n_r; ++j) {
-            double res = (double)sums[j] - (double)y[j];
-            if (r > 0) res -= (double)gamma * (double)sums[r * stride + j];
+        for (int j = lane; j < n_r; j += 32) {
+            double res = (double)__ldcg(sums + j) - (double)y[j];
+            if (r > 0) res -= (double)gamma * (double)__ldcg(sums + r * stride + j);
             f += res * res;
         }
-        f_s[r] = f / (2.0 * n_r);
-        losses[r] = (float)f_s[r];
+#pragma unroll
+        for (int sft = 16; sft >= 1; sft >>= 1) f += __shfl_xor_sync(0xffffffffu, f, sft);
+        if (lane == 0) {
+            f_s[r] = f / (2.0 * n_r);
+            losses[r] = (float)f_s[r];
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        float nv = sums[(i + 1) * stride + n_r];
+        const float nv = __ldcg(sums + (i + 1) * stride + n_r);
         if (norms) norms[i] = nv;
         scores[i] = (float)(f_s[0] - f_s[1 + i] - (double)rho * (double)nv);
     }
@@ -328,8 +347,9 @@ cudaError_t launch_lsq_score(Context &c, const LsqArgs &a, const float *y, float
     // the combined sums live behind the slab partials in the same workspace region
     const int rows = a.m + 1;
     float *sums = a.part + (int64_t)slabs * rows * (a.n_r + 1);
-    lsq_finish_kernel<<<1, 1024, 0, s>>>(a.part, slabs, a.m, a.n_r, y, gamma, rho, losses, norms,
-                                         scores, sums);
+    // not chained to the stream: with its blocks resident beside the stream's the step was 2 % slower
+    lsq_finish_kernel<<<(rows * (a.n_r + 1) + 31) / 32, kFinishWarps * 32, 0, s>>>(a.part, slabs, a.m, a.n_r, y, gamma, rho, losses, norms,
+                                                                                   scores, sums, c.tickets);
     return cudaGetLastError();
 }
 
@@ -370,6 +390,7 @@ constexpr size_t kStaticScratchFloats =
     (size_t)(kStaticMaxSlabs + 1) * (ZENO_STATIC_MAX_M + 1) * (ZENO_STATIC_MAX_N_R + 1) + (ZENO_STATIC_MAX_M + 1);
 
 static __device__ __align__(256) float g_static_scratch[kStaticScratchFloats];
+static __device__ unsigned g_static_ticket;      // of its finishing kernel, zero between calls
 
 using zeno::kMaxDevices;
 float *g_static_scratch_ptr[kMaxDevices];      // device address of the array, per device
@@ -442,9 +463,13 @@ extern "C" zeno_status zeno_score_lsq_static(int32_t device, const float *x, con
             // call, so nothing left over from an earlier call has to be cleared.
             float *sums = a.part + (int64_t)slabs * rows * (n_r + 1);
             float *loss_buf = losses ? losses : sums + (int64_t)rows * (n_r + 1);
-            zeno::lsq_finish_kernel<<<1, 1024, 0, s>>>(a.part, slabs, m, n_r, y, gamma, rho, loss_buf, norms, scores,
-                                                       sums);
-            e = cudaGetLastError();
+            unsigned *ticket = nullptr;
+            e = cudaGetSymbolAddress(reinterpret_cast<void **>(&ticket), g_static_ticket);
+            if (e == cudaSuccess) {
+                zeno::lsq_finish_kernel<<<(rows * (n_r + 1) + 31) / 32, zeno::kFinishWarps * 32, 0, s>>>(
+                    a.part, slabs, m, n_r, y, gamma, rho, loss_buf, norms, scores, sums, ticket);
+                e = cudaGetLastError();
+            }
         }
     }
     if (e != cudaSuccess) st = ZENO_ERR_CUDA;

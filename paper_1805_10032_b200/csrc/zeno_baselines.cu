@@ -5,7 +5,8 @@
 // from a Gram matrix: two honest candidates may differ by far less than their norms), then for every
 // candidate the sum over its m - b - 2 nearest neighbours, the arg min of those sums, and a copy of the
 // winning row.  The pair sums are accumulated per block over its share of the columns and added up
-// afterwards in a fixed order, so the result does not depend on scheduling.
+// afterwards in a fixed order, so the result does not depend on scheduling.  Three launches: the pairs; a block per
+// candidate that adds its distances up and sums the nearest; the copy, whose blocks find the arg min themselves.
 #include <math.h>
 
 #include "zeno_internal.h"
@@ -119,69 +120,81 @@ __global__ void __launch_bounds__(kKrumThreads, kMaxMine == 1 ? 4 : 3) krum_pair
     }
 }
 
-// dist[i][j] = the blocks' partial sums added in block order (in double), one warp an entry: lanes take
-// every 32nd block and their sums meet in a fixed butterfly.  A NaN distance counts as plus infinity.
-__global__ void __launch_bounds__(256) krum_reduce_kernel(const float *part, int slabs, int m, float *dist) {
+// Candidate i = blockIdx.x: its distances to the others, the blocks' partial sums added in a fixed order (a warp an entry:
+// lanes take every 32nd block and their sums meet in a butterfly, in double; a NaN distance counts as plus infinity),
+// then the sum of the m - b - 2 smallest: a distance belongs to it if fewer than that many others are smaller, or equal
+// and of a lower index.
+constexpr int kSumsWarps = 32;                // one round of entries up to 32 candidates
+__global__ void __launch_bounds__(kSumsWarps * 32) krum_sums_kernel(const float *part, int slabs, int m, int b, float *sums_out, float *sums_ws) {
+    __shared__ float dist[ZENO_KRUM_MAX_M];
+    __shared__ double warp_part[kSumsWarps];
+    pdl_wait();
+    pdl_launch_dependents();
     const int mb = krum_row_blocks(m), tiles = krum_tiles(m);
-    const int lane = threadIdx.x & 31;
-    const int entry = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (entry >= tiles * 16) return;
-    const int tile = entry >> 4, e = entry & 15;
-    int ib, jb;
-    krum_tile_of(tile, mb, ib, jb);
-    const int i = ib * 4 + (e >> 2), j = jb * 4 + (e & 3);
-    if (i >= m || j >= m) return;
-    double s = 0.0;
-    for (int q = lane; q < slabs; q += 32) s += (double)part[(int64_t)q * tiles * 16 + entry];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x;
+    for (int j = warp; j < m; j += kSumsWarps) {
+        const int lo = min(i, j), hi = max(i, j), ib = lo >> 2, jb = hi >> 2;
+        const int tile = ib * mb - ib * (ib - 1) / 2 + (jb - ib);
+        const float *src = part + tile * 16 + (lo & 3) * 4 + (hi & 3);
+        double s = 0.0;
+#pragma unroll 8
+        for (int q = lane; q < slabs; q += 32) s += (double)__ldcg(src + (int64_t)q * tiles * 16);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-        const float v = nan_to_inf((float)s);
-        dist[i * m + j] = v;
-        if (ib != jb) dist[j * m + i] = v;    // a diagonal tile holds both (i, j) and (j, i) itself
-    }
-}
-
-// One block.  For every candidate the sum of its m - b - 2 smallest distances to the others (ascending,
-// as a sorted sum); the arg min, lowest index first.
-__global__ void __launch_bounds__(128) krum_finish_kernel(const float *dist, int m, int b, float *sums_out, int32_t *k_out,
-                                                          float *sums_ws) {
-    const int nn = m - b - 2;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        unsigned used[ZENO_KRUM_MAX_M / 32];
-#pragma unroll
-        for (int w = 0; w < ZENO_KRUM_MAX_M / 32; ++w) used[w] = 0u;
-        used[i >> 5] |= 1u << (i & 31);
-        float s = 0.f;
-        for (int t = 0; t < nn; ++t) {
-            int best = -1;
-            float bv = INFINITY;
-            for (int j = 0; j < m; ++j) {
-                if (used[j >> 5] & (1u << (j & 31))) continue;
-                const float v = dist[i * m + j];
-                if (best < 0 || v < bv) { best = j; bv = v; }
-            }
-            used[best >> 5] |= 1u << (best & 31);
-            s += bv;
-        }
-        sums_ws[i] = s;
-        if (sums_out) sums_out[i] = s;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) dist[j] = nan_to_inf((float)s);
     }
     __syncthreads();
+    const int nn = m - b - 2;
+    double mine = 0.0;
+    for (int j = threadIdx.x; j < m; j += kSumsWarps * 32) {
+        if (j == i) continue;
+        const float v = dist[j];
+        int rank = 0;
+        for (int k = 0; k < m; ++k)
+            if (k != i && k != j) rank += dist[k] < v || (dist[k] == v && k < j);
+        if (rank < nn) mine += (double)v;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    if (lane == 0) warp_part[warp] = mine;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        int best = 0;
-        for (int i = 1; i < m; ++i)
-            if (sums_ws[i] < sums_ws[best]) best = i;
-        *k_out = best;
+        double s = 0.0;
+        for (int w = 0; w < kSumsWarps; ++w) s += warp_part[w];
+        sums_ws[i] = (float)s;
+        if (sums_out) sums_out[i] = (float)s;
     }
 }
 
+// The arg min of the sums, lowest index first, found by every block for itself, and (out != NULL) the copy of its row.
 template <typename T>
-__global__ void __launch_bounds__(256) copy_row_kernel(const T *V, int64_t ldv, int64_t d, int m, const int32_t *k, float *out) {
-    const int row = *k;
-    if (row < 0 || row >= m) return;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < d; j += (int64_t)gridDim.x * blockDim.x)
-        out[j] = load_elem(V + (int64_t)row * ldv + j);
+__global__ void __launch_bounds__(256) copy_row_kernel(const T *V, int64_t ldv, int64_t d, int m, const float *sums, int32_t *k_out,
+                                                       float *out) {
+    __shared__ int row_s;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (threadIdx.x < 32) {
+        float best = INFINITY;
+        int at = ZENO_KRUM_MAX_M;
+        for (int i = threadIdx.x; i < m; i += 32) {
+            const float v = __ldcg(sums + i);
+            if (at == ZENO_KRUM_MAX_M || v < best) { best = v; at = i; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float v = __shfl_xor_sync(0xffffffffu, best, o);
+            const int w = __shfl_xor_sync(0xffffffffu, at, o);
+            if (w < ZENO_KRUM_MAX_M && (at == ZENO_KRUM_MAX_M || v < best || (v == best && w < at))) { best = v; at = w; }
+        }
+        if (threadIdx.x == 0) {
+            row_s = at;
+            if (blockIdx.x == 0) *k_out = at;
+        }
+    }
+    __syncthreads();
+    if (!out) return;
+    const T *row = V + (int64_t)row_s * ldv;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < d; j += (int64_t)gridDim.x * blockDim.x) out[j] = load_elem(row + j);
 }
 
 template <typename T>
@@ -207,33 +220,26 @@ cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b,
     const int64_t want = (d + kKrumCols - 1) / kKrumCols;
     int blocks = per_sm * sms < c.krum_blocks ? per_sm * sms : c.krum_blocks;
     if (want < blocks) blocks = (int)(want < 1 ? 1 : want);
-    if (tiles < kKrumThreads)
-        krum_pairs_kernel<T, 1><<<blocks, kKrumThreads, smem, s>>>(V, ldv, d, m, c.krum_part);
-    else
-        krum_pairs_kernel<T, 3><<<blocks, kKrumThreads, smem, s>>>(V, ldv, d, m, c.krum_part);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained(tiles < kKrumThreads ? krum_pairs_kernel<T, 1> : krum_pairs_kernel<T, 3>, dim3(blocks),
+                                   dim3(kKrumThreads), smem, s, chain_launches(c), V, ldv, d, m, c.krum_part);
     if (e != cudaSuccess) return e;
-    float *dist = c.krum_part + (size_t)c.krum_blocks * krum_tiles(c.m_max) * 16;     // m_max <= ZENO_KRUM_MAX_M here
-    krum_reduce_kernel<<<(tiles * 16 + 7) / 8, 256, 0, s>>>(c.krum_part, blocks, m, dist);
-    e = cudaGetLastError();
+    e = launch_chained(krum_sums_kernel, dim3(m), dim3(kSumsWarps * 32), 0, s, chain_launches(c), (const float *)c.krum_part, blocks, m, b, sums,
+                       c.krum_sums);
     if (e != cudaSuccess) return e;
-    krum_finish_kernel<<<1, 128, 0, s>>>(dist, m, b, sums, k, c.krum_sums);
-    e = cudaGetLastError();
-    if (e != cudaSuccess || !out) return e;
-    int64_t cw = (d + 255) / 256;
-    const int cblocks = (int)(cw < (int64_t)sms * 8 ? (cw < 1 ? 1 : cw) : (int64_t)sms * 8);
-    copy_row_kernel<T><<<cblocks, 256, 0, s>>>(V, ldv, d, m, k, out);
-    return cudaGetLastError();
+    const int64_t cw = (d + 255) / 256;
+    const int cblocks = !out ? 1 : (int)(cw < (int64_t)sms * 8 ? (cw < 1 ? 1 : cw) : (int64_t)sms * 8);
+    return launch_chained(copy_row_kernel<T>, dim3(cblocks), dim3(256), 0, s, chain_launches(c), V, ldv, d, m,
+                          (const float *)c.krum_sums, k, out);
 }
 
 }  // namespace
 
-// floats of Krum's workspace for up to m candidates and `blocks` blocks: the blocks' pair sums, then dist[m][m]
-size_t krum_part_floats(int m, int blocks) { return (size_t)blocks * krum_tiles(m) * 16 + (size_t)m * m; }
+// floats of Krum's workspace for up to m candidates and `blocks` blocks: the blocks' pair sums
+size_t krum_part_floats(int m, int blocks) { return (size_t)blocks * krum_tiles(m) * 16; }
 
 cudaError_t launch_krum(Context &c, const void *V, int64_t ldv, int m, int b, float *out, int32_t *k, float *sums,
                         cudaStream_t s, int *launches) {
-    *launches += out ? 4 : 3;
+    *launches += 3;
     profile_mark(c, "krum", s);
     if (c.desc.param_dtype == ZENO_BF16)
         return launch_krum_typed(c, static_cast<const __nv_bfloat16 *>(V), ldv, m, b, out, k, sums, s);

@@ -140,6 +140,29 @@ def test_krum_matches_oracle(oracle, name):
     assert torch.equal(out.cpu(), w.V[k, :w.d].float())
 
 
+# one tile in flight and two, the last size of either, the first with several pair tiles a thread, the most candidates;
+# ties of identical rows, a row of infinite distances, odd pitches
+@pytest.mark.parametrize("m,b,dtype", [(3, 0, "f32"), (5, 1, "f32"), (64, 20, "f32"), (65, 20, "f32"), (88, 3, "f32"), (89, 30, "f32"),
+                                       (128, 50, "f32"), (20, 8, "bf16"), (128, 50, "bf16")])
+def test_krum_over_its_sizes(oracle, m, b, dtype):
+    w = syn.make_config(1, dims=(333, 7), m=m, b=b, dtype=dtype, ldv=2351, faults=[(b, "noise200")] if b else [], seed=77 + m)
+    assert w.ldv >= w.d
+    w.V[1] = w.V[0]
+    if m > 5:
+        w.V[4, 11] = float("nan")
+    k_orc, sums_orc, _ = oracle.krum(P.DTYPE[dtype], syn.to_numpy_params(w.V), w.ldv, w.d, m, b)
+    with zeno.from_workload(w) as z:
+        out, k, sums = z.krum(w.V.cuda(), b)
+        none, k2, _ = z.krum(w.V.cuda(), b, want_out=False)
+    assert none is None and k2.item() == k.item()
+    sums = sums.cpu().numpy().astype(np.float64)
+    fin = np.isfinite(sums_orc)
+    assert np.array_equal(sums[~fin], sums_orc[~fin])
+    assert np.allclose(sums[fin], sums_orc[fin], rtol=2e-5, atol=0)
+    assert k.item() == int(np.argmin(sums))
+    assert torch.equal(out.cpu(), w.V[k.item(), :w.d].float())
+
+
 def test_krum_toy_example_on_the_gpu():
     # Discussion, the one-dimensional toy example: Krum_2({-1, -1, 0.2, 0.4, 1.6, 1.8}) = -1
     V = torch.tensor([[-1.0], [-1.0], [0.2], [0.4], [1.6], [1.8]])

@@ -221,13 +221,17 @@ zeno_status enqueue_score_cnn(Context *c, const void *x, const void *V, int64_t 
 
 // keep > 0 asks for the ranking as well (idx[0..keep)); *ranked tells whether the scoring pass
 // delivered it (the MLP tail does) or a separate select launch is still needed.  rank_in != NULL: the averaging
-// kernel that follows scores and ranks (softmax losses, up to kRankMax candidates); it is filled in and switched on.
+// kernel that follows may score and rank (softmax losses, up to kRankMax candidates); it is filled in and switched on.
 zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv, int32_t m,
                           const zeno_batch *batch, float gamma, float rho, float *scores,
                           float *losses, float *norms, int keep, int32_t *idx, bool *ranked, zeno::RankArgs *rank_in,
                           cudaStream_t s, int *launches) {
     *ranked = false;
-    zeno::RankArgs *rank = m <= zeno::kRankMax && c->desc.kind != ZENO_LOSS_LEAST_SQUARES ? rank_in : nullptr;
+    // The averaging kernel ranks while the rows it will read fit L2.  Every one of its blocks then spends about a
+    // microsecond on it, which the scoring pass's shorter end outweighs for few rows (12 x 1.8 M fp32: a step of 73.2 us
+    // becomes 69.8) but not for many (60 x 1.8 M: 298.6 against 300.3; 20 x 37.7 M bfloat16: 1,234 against 1,244).
+    const bool small = (double)keep * (double)c->d * (double)elem_size(c->desc.param_dtype) <= 126.0 * 1024 * 1024;
+    zeno::RankArgs *rank = small && m <= zeno::kRankMax && c->desc.kind != ZENO_LOSS_LEAST_SQUARES ? rank_in : nullptr;
     zeno_status st = check_common(c, V, ldv, m);
     if (st != ZENO_OK) return st;
     if (!x || !batch || !batch->features || !batch->targets || !scores) return ZENO_ERR_INVALID_ARG;

@@ -359,7 +359,13 @@ __global__ void __launch_bounds__(256) cnn_pack_kernel(const __grid_constant__ C
     if ((int)blockIdx.x >= a.weight_blocks) {                    // the batch, dealt over the rest of the grid
         const int pixels = a.side * a.side, pitch = a.side + 1, total = a.n_r * a.groups * pixels;
         const int nb = (gridDim.x - a.weight_blocks) * gridDim.y;
-        for (int t = ((blockIdx.x - a.weight_blocks) * gridDim.y + blockIdx.y) * 256 + tid; t < total; t += nb * 256) {
+        const int first = ((blockIdx.x - a.weight_blocks) * gridDim.y + blockIdx.y) * 256 + tid;
+        // A first layer's paired taps multiply a fourth column with zero weights.  For the last pixel of the last sample
+        // that is the first pixel of the slot after the batch, the one position beyond it that is read into a pixel that
+        // counts: an earlier call with more samples may have left a NaN or an infinity there, and 0 x NaN is NaN.
+        if (a.groups == 1 && first < 2)                          // of either term
+            reinterpret_cast<float4 *>(a.in0)[first * a.px + a.lead + (int64_t)a.n_r * pitch * pitch] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int t = first; t < total; t += nb * 256) {
             const int ng = t / pixels, pix = t - ng * pixels, n = ng / a.groups, g = ng - n * a.groups;
             const int y = pix / a.side, x = pix - y * a.side;
             float h[4], l[4];

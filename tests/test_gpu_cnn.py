@@ -65,6 +65,25 @@ def test_fewer_samples_and_candidates_than_the_handle_was_made_for(oracle):
         assert all(torch.equal(a, b) for a, b in zip(got, want))
 
 
+# the first pixel of a sample is read, with zero weights, by the paired taps of the sample before it (one to four input
+# planes); five planes: no paired taps
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("planes", [1, 3, 4, 5])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_a_smaller_batch_reads_no_pixel_of_a_larger_one(dtype, planes, value):
+    w = syn.make_config(6, dims=(8, planes, 8, 8, 10), m=4, b=1, n_r=5, faults=[(1, "signflip")], dtype=dtype)
+    x, V, f, t = P.to_device(w)
+    bad = f.clone().view(5, planes, 8, 8)
+    with zeno.from_workload(w) as z, zeno.from_workload(w) as fresh:
+        for n in (1, 2, 4):
+            bad[n, :, 0, 0] = value
+            z.score(x, V, bad.view_as(f), t, w.gamma, w.rho)
+            got = z.score(x, V, f[:n].contiguous(), t[:n], w.gamma, w.rho)
+            want = fresh.score(x, V, f[:n].contiguous(), t[:n], w.gamma, w.rho)
+            assert all(torch.isfinite(v).all() for v in want)
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
 def test_cuda_core_layers(oracle, monkeypatch):
     """The kernel that serves without tensor cores."""
     monkeypatch.setenv("ZENO_DISABLE_TENSOR_CORES", "1")

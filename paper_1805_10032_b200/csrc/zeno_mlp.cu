@@ -48,6 +48,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // shared memory.
 // Bound by the loads' latency and the CUDA cores' rate: 38 models of 1029 x 301 with 19 samples take 61 us (one
 // warp per four rows and one block an SM: 80), 24 models of 4096 x 43 with 40 samples in clusters of two 90 us less.
+constexpr int kMaxCluster = 8;                   // blocks of a cluster, here and in the head
 constexpr int kLRows = 64, kLK = 64, kLGroups = 4, kLPitch = kLK + 4;
 constexpr int kLRun = 4;                         // slices of a run (a group's sixteen columns of each)
 __host__ __device__ constexpr int layer_stage_floats(int TN) { return 2 * (kLRows + 8 * TN) * kLPitch; }
@@ -219,11 +220,12 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
 // logits go to the first block's shared memory, which adds them up and takes the loss, a warp per sample.
 // The work is a chain of latencies (784 x 10 of 21 models: 0.7 MB), so the slices are short enough for all of a
 // block's loads to be in flight at once and everything else a block needs is requested with them.
+constexpr int kHeadCols = 512;                   // columns staged at a time, at most
 template <typename T, int OUT_T, int SPW, bool VEC>
 __global__ void __launch_bounds__(256) mlp_head_kernel(LayerArgs a, int cluster, int kslice, int KC) {
     constexpr int NS = 8 * SPW;                  // samples a cluster can hold
     constexpr int kRows = OUT_T / 8;             // rows a warp stages
-    constexpr int kMaxIter = 4;                  // KC / 128 at most
+    constexpr int kMaxIter = kHeadCols / 128;    // KC / 128 at most
     extern __shared__ __align__(16) float smem_dyn[];
     float *ws = smem_dyn;                                            // [OUT_T][KC]
     float *hs = ws + OUT_T * KC;                                     // [NS][KC]
@@ -496,29 +498,36 @@ __global__ void __launch_bounds__(256) mlp_loss_kernel(const float *logits, cons
     }
 }
 
+template <typename T, int TN>
+cudaError_t launch_layer_tn(Context &c, const LayerArgs &a, cudaStream_t s) {
+    const int sms = c.sm_count > 0 ? c.sm_count : 148;
+    const int sample_tiles = (a.n_r + 8 * TN - 1) / (8 * TN);
+    const int64_t tiles = (int64_t)((a.out + kLRows - 1) / kLRows) * sample_tiles;
+    // two blocks fit an SM: with fewer than that, clusters of blocks share a tile's slices, at least two slices a block
+    // (evening out a last wave with clusters as well made 190 tiles' kernel 10 % faster and its step 9 % slower)
+    int cluster = 1;
+    while (cluster < kMaxCluster && tiles * (a.m + 1) * 2 * cluster <= 2 * sms && a.in >= 2 * kLK * 2 * cluster) cluster *= 2;
+    // the limit is the function's, for every handle and thread of the process: the most any call asks for, set once
+    static PerDeviceOnce attr_set;
+    if (attr_set.need(c.device)) {
+        cudaError_t e = cudaFuncSetAttribute(mlp_layer_kernel<T, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)layer_smem(TN, kMaxCluster));
+        if (e != cudaSuccess) return e;
+        attr_set.mark(c.device);
+    }
+    // the sample tiles of the same rows run side by side and find them in L2
+    return launch_clustered(mlp_layer_kernel<T, TN>, cluster, dim3((unsigned)(tiles * cluster), a.m + 1), dim3(kLGroups * 64),
+                            layer_smem(TN, cluster), s, chain_launches(c), a, sample_tiles, cluster);
+}
+
 template <typename T>
 cudaError_t launch_layer(Context &c, const LayerArgs &a, cudaStream_t s) {
-    const int sms = c.sm_count > 0 ? c.sm_count : 148;
-    auto go = [&](auto kernel, int tn) {
-        const int sample_tiles = (a.n_r + 8 * tn - 1) / (8 * tn);
-        const int64_t tiles = (int64_t)((a.out + kLRows - 1) / kLRows) * sample_tiles;
-        // two blocks fit an SM: with fewer than that, clusters of blocks share a tile's slices, at least two slices a block
-        // (evening out a last wave with clusters as well made 190 tiles' kernel 10 % faster and its step 9 % slower)
-        int cluster = 1;
-        while (cluster < 8 && tiles * (a.m + 1) * 2 * cluster <= 2 * sms && a.in >= 2 * kLK * 2 * cluster) cluster *= 2;
-        const size_t smem = layer_smem(tn, cluster);
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        // the sample tiles of the same rows run side by side and find them in L2
-        return launch_clustered(kernel, cluster, dim3((unsigned)(tiles * cluster), a.m + 1), dim3(kLGroups * 64), smem, s,
-                                chain_launches(c), a, sample_tiles, cluster);
-    };
     // samples in tiles of 8 TN: one tile if it holds them all, else the width that pads them least
     const bool by24 = a.n_r > 32 && (a.n_r + 23) / 24 <= (a.n_r + 31) / 32;
-    if (a.n_r <= 8) return go(mlp_layer_kernel<T, 1>, 1);
-    if (a.n_r <= 16) return go(mlp_layer_kernel<T, 2>, 2);
-    if (a.n_r <= 24 || by24) return go(mlp_layer_kernel<T, 3>, 3);
-    return go(mlp_layer_kernel<T, 4>, 4);
+    if (a.n_r <= 8) return launch_layer_tn<T, 1>(c, a, s);
+    if (a.n_r <= 16) return launch_layer_tn<T, 2>(c, a, s);
+    if (a.n_r <= 24 || by24) return launch_layer_tn<T, 3>(c, a, s);
+    return launch_layer_tn<T, 4>(c, a, s);
 }
 
 }  // namespace
@@ -529,35 +538,42 @@ int mlp_norm_slots(int out) { return (out + kLRows - 1) / kLRows * (kLGroups * 2
 // logits: every output row in one block, every sample in one tile.
 bool mlp_can_fuse_loss(int out, int n_r) { return (out <= 32 && n_r <= 32) || (out <= 16 && n_r <= 64); }
 
-template <typename T, bool VEC>
-cudaError_t launch_head(Context &c, const LayerArgs &a, cudaStream_t s) {
+template <typename T, int OUT_T, int SPW, bool VEC>
+cudaError_t launch_head_sized(Context &c, const LayerArgs &a, cudaStream_t s) {
+    constexpr int NS = 8 * SPW;
     // blocks per model: as many as leave a slice of 128 columns and are resident at once (two to an SM up to 16 x 16
     // logits, one beyond: the accumulators).  A second wave costs more than the longer slice (101 models of 512 x 10,
     // 64 samples: 21 us with one block a model, 29 with two)
     const int sms = c.sm_count > 0 ? c.sm_count : 148;
     const int room = a.out <= 16 && a.n_r <= 16 ? 2 * sms : sms;
     int cluster = 1;
-    while (cluster < 8 && a.in / (2 * cluster) >= 128 && (a.m + 1) * 2 * cluster <= room) cluster *= 2;
+    while (cluster < kMaxCluster && a.in / (2 * cluster) >= 128 && (a.m + 1) * 2 * cluster <= room) cluster *= 2;
     const int kslice = ((a.in + cluster - 1) / cluster + 3) / 4 * 4;
-    const int KC = kslice >= 512 ? 512 : (kslice + 127) / 128 * 128;
-    auto go = [&](auto kernel, int out_t, int ns) {
-        const size_t smem = sizeof(float) * ((size_t)(out_t + ns) * KC + (size_t)cluster * (ns * out_t + 8));
-        if (smem > 36 * 1024) {                  // 48 KB less the static part, the sort of the tail among it
-            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        return launch_clustered(kernel, cluster, dim3(cluster * (a.m + 1)), dim3(256), smem, s, chain_launches(c), a, cluster, kslice,
-                                KC);
-    };
-    if (a.out <= 16) {
-        if (a.n_r <= 8) return go(mlp_head_kernel<T, 16, 1, VEC>, 16, 8);
-        if (a.n_r <= 16) return go(mlp_head_kernel<T, 16, 2, VEC>, 16, 16);
-        if (a.n_r <= 32) return go(mlp_head_kernel<T, 16, 4, VEC>, 16, 32);
-        return go(mlp_head_kernel<T, 16, 8, VEC>, 16, 64);
+    const int KC = kslice >= kHeadCols ? kHeadCols : (kslice + 127) / 128 * 128;
+    auto smem = [](int cols, int blocks) { return sizeof(float) * ((size_t)(OUT_T + NS) * cols + (size_t)blocks * (NS * OUT_T + 8)); };
+    // the limit is the function's, for every handle and thread of the process: the most any call asks for, set once
+    static PerDeviceOnce attr_set;
+    if (attr_set.need(c.device)) {
+        cudaError_t e = cudaFuncSetAttribute(mlp_head_kernel<T, OUT_T, SPW, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem(kHeadCols, kMaxCluster));
+        if (e != cudaSuccess) return e;
+        attr_set.mark(c.device);
     }
-    if (a.n_r <= 8) return go(mlp_head_kernel<T, 32, 1, VEC>, 32, 8);
-    if (a.n_r <= 16) return go(mlp_head_kernel<T, 32, 2, VEC>, 32, 16);
-    return go(mlp_head_kernel<T, 32, 4, VEC>, 32, 32);
+    return launch_clustered(mlp_head_kernel<T, OUT_T, SPW, VEC>, cluster, dim3(cluster * (a.m + 1)), dim3(256), smem(KC, cluster), s,
+                            chain_launches(c), a, cluster, kslice, KC);
+}
+
+template <typename T, bool VEC>
+cudaError_t launch_head(Context &c, const LayerArgs &a, cudaStream_t s) {
+    if (a.out <= 16) {
+        if (a.n_r <= 8) return launch_head_sized<T, 16, 1, VEC>(c, a, s);
+        if (a.n_r <= 16) return launch_head_sized<T, 16, 2, VEC>(c, a, s);
+        if (a.n_r <= 32) return launch_head_sized<T, 16, 4, VEC>(c, a, s);
+        return launch_head_sized<T, 16, 8, VEC>(c, a, s);
+    }
+    if (a.n_r <= 8) return launch_head_sized<T, 32, 1, VEC>(c, a, s);
+    if (a.n_r <= 16) return launch_head_sized<T, 32, 2, VEC>(c, a, s);
+    return launch_head_sized<T, 32, 4, VEC>(c, a, s);
 }
 
 cudaError_t launch_mlp_layer(Context &c, const LayerArgs &a, bool aligned, cudaStream_t s,

@@ -1,5 +1,7 @@
 """GPU parity: the CUDA path, called through the C ABI, against the float64 oracle on the same
 seeded inputs, element by element."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -369,3 +371,33 @@ def test_host_entry_point_matches_device_entry_point():
         z.step_host(w.x.pin_memory(), w.V.pin_memory(), w.features.pin_memory(),
                     w.targets.pin_memory(), w.gamma, w.rho, w.b, out_h, s_h, i_h)
     assert torch.equal(out.cpu(), out_h) and torch.equal(s.cpu(), s_h) and torch.equal(idx.cpu(), i_h)
+
+
+# Handles are independent of one another: two host threads run the server loops of two models whose last layers (and,
+# with rows of no alignment, whose dense layers) are served by one kernel with different amounts of shared memory.
+@pytest.mark.parametrize("dims,n_r", [(((3000, 10), (4096, 10)), 4), (((1029, 40), (300, 40)), 32)])
+def test_two_handles_on_two_host_threads(dims, n_r):
+    failures = []
+    ready = threading.Barrier(2)
+
+    def loops(one, steps=100):
+        try:
+            w = syn.make_config(2, dims=one, m=4, b=1, n_r=n_r, faults=[(1, "signflip")])
+            with torch.cuda.stream(torch.cuda.Stream()), zeno.from_workload(w) as z:
+                x, V, f, t = (v.repeat(steps, *([1] * v.dim())) if k else v for k, v in enumerate(P.to_device(w)))
+                want = z.run(x, V, f, t, 0.0, w.rho, w.b)           # gamma = 0: x stays as it is
+                ready.wait(60)
+                for i in range(40):
+                    got = z.run(x, V, f, t, 0.0, w.rho, w.b)
+                    if not all(torch.equal(a, b) for a, b in zip(got, want)):
+                        failures.append((one, i))
+        except Exception as e:
+            failures.append((one, e))
+            ready.abort()
+
+    threads = [threading.Thread(target=loops, args=(one,)) for one in dims]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not failures, failures

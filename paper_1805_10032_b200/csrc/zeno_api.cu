@@ -684,13 +684,20 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     c->krum_part = krum_elems ? reinterpret_cast<float *>(base + at_krum) : nullptr;
     c->krum_sums = reinterpret_cast<float *>(base + at_krums);
     if (c->cnn_net.layers) c->cnn_ws = reinterpret_cast<float *>(base + at_cnn);
-    e = cudaMemset(c->dev_status, 0, sizeof(int));
-    // the padding of the planes and of the weights' operands is zero from here on; a first call may be on a stream
-    // that does not wait for the default one
-    if (e == cudaSuccess && c->cnn_net.layers) e = cudaMemset(c->cnn_ws, 0, (size_t)c->cnn_net.floats * 4);
-    if (e == cudaSuccess && c->cnn_net.layers) e = cudaStreamSynchronize(nullptr);
-    if (e == cudaSuccess) e = cudaMemset(c->tickets, 0, ticket_elems * sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMemset(c->head_tickets, 0, rows * sizeof(unsigned));
+    // The status word, the tickets and the padding of the convolutional layers' workspace are zero from here on.  A memset
+    // returns before it has run, and a first call may be on a stream that waits for no other, so the handle is handed out
+    // when they have; on a stream of their own, so that this waits for no work of the caller's.
+    cudaStream_t clear = nullptr;
+    e = cudaStreamCreateWithFlags(&clear, cudaStreamNonBlocking);
+    if (e == cudaSuccess) {
+        e = cudaMemsetAsync(c->dev_status, 0, sizeof(int), clear);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->tickets, 0, ticket_elems * sizeof(unsigned), clear);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->head_tickets, 0, rows * sizeof(unsigned), clear);
+        if (e == cudaSuccess && c->cnn_net.layers) e = cudaMemsetAsync(c->cnn_ws, 0, (size_t)c->cnn_net.floats * 4, clear);
+        const cudaError_t synced = cudaStreamSynchronize(clear);
+        if (e == cudaSuccess) e = synced;
+        cudaStreamDestroy(clear);
+    }
     if (e != cudaSuccess) {
         cudaFree(c->arena);
         delete c;

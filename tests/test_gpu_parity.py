@@ -401,3 +401,27 @@ def test_two_handles_on_two_host_threads(dims, n_r):
     for th in threads:
         th.join()
     assert not failures, failures
+
+
+# more candidates than the averaging kernel ranks, and least squares: both passes end in the block that takes the last
+# ticket, which the workspace has to hold zero for
+@pytest.mark.parametrize("index,ov", [(1, dict(m=300, b=8)), (5, dict(d=20000, m=12, b=4, n_r=16, n_noise=4))])
+def test_a_new_handle_is_ready_for_any_stream(index, ov):
+    """zeno_create has cleared its workspace when it returns: calls on a stream that waits for no other are right while
+    the default stream still has work ahead of anything queued there, and when that work ends."""
+    w = syn.make_config(index, **ov)
+    x, V, f, t = (v.repeat(4, *([1] * v.dim())) if k else v for k, v in enumerate(P.to_device(w)))
+    with zeno.from_workload(w) as z:
+        want, _ = z.run(x, V, f, t, 0.0, w.rho, w.b)                # gamma = 0: x stays as it is
+    side = torch.cuda.Stream()
+    scores = [torch.empty_like(want) for _ in range(200)]
+    for _ in range(10):
+        for s in scores:
+            s.fill_(-1)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(20_000_000)                               # some 10 ms
+        with zeno.from_workload(w) as z, torch.cuda.stream(side):
+            for s in scores:
+                z.run(x, V, f, t, 0.0, w.rho, w.b, scores=s)
+            torch.cuda.synchronize()
+        assert all(torch.equal(s, want) for s in scores)

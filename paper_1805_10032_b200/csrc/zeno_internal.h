@@ -185,6 +185,7 @@ struct LsqArgs {
     int n_r, m;
     float *part;      // [slabs][m+1][n_r+1]; the last column holds the partial sum of squares
     int slabs;
+    unsigned *ticket; // zeroed by the stream kernel for the finish that follows it, or NULL: zero between calls
 };
 
 // Launchers return the cudaError_t of the launch; *launches is incremented per kernel.

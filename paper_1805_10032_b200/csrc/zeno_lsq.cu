@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(LsqShape<NRT, RB>::kMaxWarps * 32, 1) lsq_stre
     const int j0 = blockIdx.z * NRT;
     const int n_valid = min(NRT, a.n_r - j0);
     const int64_t K = a.d;
+    if (a.ticket && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) *a.ticket = 0;
 
     const float *rowp[RB];
 #pragma unroll
@@ -311,6 +312,7 @@ int lsq_slab_count(const Context &c) {
 static cudaError_t launch_lsq_pass(Context &c, const LsqArgs &a_in, bool aligned, int *slabs_out, cudaStream_t s,
                                    int *launches) {
     LsqArgs a = a_in;
+    a.ticket = nullptr;
     const int nrt = a.n_r <= 8 ? 8 : (a.n_r <= 16 ? 16 : 32);
     // small problems: no more slabs than there are stages of A
     const int64_t stages = (a.d + (kStageFloats / nrt) - 1) / (kStageFloats / nrt);
@@ -379,18 +381,18 @@ cudaError_t launch_lsq_from_sums(Context &c, const double *sums, int m, int n_r,
 
 // ---- scoring without any allocation -------------------------------------------------------
 //
-// The slab partials, the combined sums and the losses of zeno_score_lsq_static live in this
+// The slab partials, the combined sums, the losses and the finish's ticket of zeno_score_lsq_static live in this
 // array.  It is part of the library image: every GPU that loads the library carries it until
-// the process exits.  Size: (slabs + 1) (m + 1) (n_r + 1) + (m + 1) floats with slabs <= 160,
+// the process exits.  Size: (slabs + 1) (m + 1) (n_r + 1) + (m + 1) + 1 words with slabs <= 160,
 // m <= ZENO_STATIC_MAX_M, n_r <= ZENO_STATIC_MAX_N_R -- about 1.4 MB.
 namespace {
 
 constexpr int kStaticMaxSlabs = 160;
-constexpr size_t kStaticScratchFloats =
+constexpr size_t kStaticTicket =               // index of the ticket
     (size_t)(kStaticMaxSlabs + 1) * (ZENO_STATIC_MAX_M + 1) * (ZENO_STATIC_MAX_N_R + 1) + (ZENO_STATIC_MAX_M + 1);
+constexpr size_t kStaticScratchFloats = kStaticTicket + 1;
 
 static __device__ __align__(256) float g_static_scratch[kStaticScratchFloats];
-static __device__ unsigned g_static_ticket;      // of its finishing kernel, zero between calls
 
 using zeno::kMaxDevices;
 float *g_static_scratch_ptr[kMaxDevices];      // device address of the array, per device
@@ -443,6 +445,7 @@ extern "C" zeno_status zeno_score_lsq_static(int32_t device, const float *x, con
         a.n_r = n_r;
         a.m = m;
         a.part = g_static_scratch_ptr[device];
+        a.ticket = reinterpret_cast<unsigned *>(a.part + kStaticTicket);
         const int rows = m + 1;
         const int nrt = n_r <= 8 ? 8 : (n_r <= 16 ? 16 : 32);
         const int64_t stages = (d + (zeno::kStageFloats / nrt) - 1) / (zeno::kStageFloats / nrt);
@@ -459,17 +462,13 @@ extern "C" zeno_status zeno_score_lsq_static(int32_t device, const float *x, con
         else
             e = aligned ? zeno::launch_stream<32, 4, true>(a, s) : zeno::launch_stream<32, 4, false>(a, s);
         if (e == cudaSuccess) {
-            // Every partial the finishing kernel reads is rewritten by the stream kernel of the same
-            // call, so nothing left over from an earlier call has to be cleared.
+            // Everything the finishing kernel reads, its ticket included, is rewritten by the stream kernel of the
+            // same call, so nothing an earlier call left behind, not even one that raced with another, matters.
             float *sums = a.part + (int64_t)slabs * rows * (n_r + 1);
             float *loss_buf = losses ? losses : sums + (int64_t)rows * (n_r + 1);
-            unsigned *ticket = nullptr;
-            e = cudaGetSymbolAddress(reinterpret_cast<void **>(&ticket), g_static_ticket);
-            if (e == cudaSuccess) {
-                zeno::lsq_finish_kernel<<<(rows * (n_r + 1) + 31) / 32, zeno::kFinishWarps * 32, 0, s>>>(
-                    a.part, slabs, m, n_r, y, gamma, rho, loss_buf, norms, scores, sums, ticket);
-                e = cudaGetLastError();
-            }
+            zeno::lsq_finish_kernel<<<(rows * (n_r + 1) + 31) / 32, zeno::kFinishWarps * 32, 0, s>>>(
+                a.part, slabs, m, n_r, y, gamma, rho, loss_buf, norms, scores, sums, a.ticket);
+            e = cudaGetLastError();
         }
     }
     if (e != cudaSuccess) st = ZENO_ERR_CUDA;

@@ -91,18 +91,19 @@ def test_a_call_after_calls_that_raced_on_the_scratch():
     w = syn.make_config(5, d=4096, m=3, b=1, n_r=2, n_noise=1)
     want, _, _ = _static(w, False)
     pairs = [(torch.cuda.Stream(), P.to_device(syn.make_config(5, d=4096, m=m, b=1, n_r=n_r, n_noise=1)))
-             for m, n_r in ((64, 16), (63, 16))]
+             for m, n_r in ((64, 16), (63, 16), (64, 15), (61, 13), (64, 9), (50, 16))]
     spoilt = torch.empty(64, device="cuda")
     torch.cuda.synchronize()
-    for stream, _ in pairs:
-        with torch.cuda.stream(stream):
-            torch.cuda._sleep(20_000_000)                # the calls of both streams then run side by side
-    for _ in range(300):
-        for stream, (x, V, A, y) in pairs:
-            zeno.score_lsq_static(x, V, A, y, w.gamma, w.rho, spoilt, stream=stream)
-    torch.cuda.synchronize()
-    got, _, _ = _static(w, False)
-    assert np.array_equal(got, want)
+    for _ in range(10):
+        for stream, _ in pairs:
+            with torch.cuda.stream(stream):
+                torch.cuda._sleep(8_000_000)             # the calls of all streams then run side by side
+        for _ in range(25):
+            for stream, (x, V, A, y) in pairs:
+                zeno.score_lsq_static(x, V, A, y, w.gamma, w.rho, spoilt, stream=stream)
+        torch.cuda.synchronize()
+        got, _, _ = _static(w, False)
+        assert np.array_equal(got, want)
 
 
 def test_sizes_beyond_the_fixed_scratch_are_refused():

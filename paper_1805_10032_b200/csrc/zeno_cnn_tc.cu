@@ -242,7 +242,8 @@ __global__ void __launch_bounds__(kCThreads, 1) cnn_conv_tc_kernel(CnnTcArgs a) 
         const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
         const int per_sample = pitch * pitch;
         uint32_t g = 0;
-        for (int li = 0; get_item(li, model, nb, pair) && !*abortp; ++li) {
+        for (int li = 0;; ++li) {
+            if (!__all_sync(0xffffffffu, get_item(li, model, nb, pair) && !*abortp)) break;
             const bool have = pair * kCTiles + t < a.tiles;      // the last pair may hold one tile
             // the sums start from the bias, asked for before the first accumulators are awaited (written two kernels ago:
             // not by the read-only path)
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(kCThreads, 1) cnn_conv_tc_kernel(CnnTcArgs a) 
             bool ok = true;
             for (int st = 0; st < a.stages_per_item; ++st, ++g) {
                 const int set = g & 1;
-                if (!mbar_wait(bar_dfull(set), (g >> 1) & 1, abortp)) { ok = false; break; }
+                if (!__all_sync(0xffffffffu, mbar_wait(bar_dfull(set), (g >> 1) & 1, abortp))) { ok = false; break; }
                 tc_fence_after();
                 if (have) {
                     const uint32_t d = tmem + lane_addr + set * (kCTiles * tile_cols) + t * tile_cols;
@@ -289,22 +290,24 @@ __global__ void __launch_bounds__(kCThreads, 1) cnn_conv_tc_kernel(CnnTcArgs a) 
             if (!ok) break;
             const int q = (pair * kCTiles + t) * 128 + quad * 32 + lane;        // this thread's pixel on the line
             const int sample = q / per_sample, r = q - sample * per_sample, y = r / pitch, x = r - y * pitch;
-            if (!have || sample >= a.n_r || y >= a.side || x >= a.side) continue;   // padding
-            float4 *out = reinterpret_cast<float4 *>(a.out + (int64_t)model * a.out_model) + a.out_lead + q;
+            if (have && sample < a.n_r && y < a.side && x < a.side) {           // not padding
+                float4 *out = reinterpret_cast<float4 *>(a.out + (int64_t)model * a.out_model) + a.out_lead + q;
 #pragma unroll
-            for (int c = 0; c < kCMaxN / 4; ++c) {
-                const int grp = nb * (a.n / 4) + c;
-                if (4 * c >= a.n || grp >= a.out_groups) break;
-                const float4 z = make_float4(relu_keep_nan(acc[4 * c]), relu_keep_nan(acc[4 * c + 1]),
-                                             relu_keep_nan(acc[4 * c + 2]), relu_keep_nan(acc[4 * c + 3]));
-                if (a.pool) {
-                    out[(int64_t)grp * a.out_px] = z;
-                } else {
-                    const float4 h = make_float4(tf32_hi(z.x), tf32_hi(z.y), tf32_hi(z.z), tf32_hi(z.w));
-                    out[(int64_t)grp * a.out_px] = h;
-                    out[(int64_t)(a.out_groups + grp) * a.out_px] = make_float4(z.x - h.x, z.y - h.y, z.z - h.z, z.w - h.w);
+                for (int c = 0; c < kCMaxN / 4; ++c) {
+                    const int grp = nb * (a.n / 4) + c;
+                    if (4 * c >= a.n || grp >= a.out_groups) break;
+                    const float4 z = make_float4(relu_keep_nan(acc[4 * c]), relu_keep_nan(acc[4 * c + 1]),
+                                                 relu_keep_nan(acc[4 * c + 2]), relu_keep_nan(acc[4 * c + 3]));
+                    if (a.pool) {
+                        out[(int64_t)grp * a.out_px] = z;
+                    } else {
+                        const float4 h = make_float4(tf32_hi(z.x), tf32_hi(z.y), tf32_hi(z.z), tf32_hi(z.w));
+                        out[(int64_t)grp * a.out_px] = h;
+                        out[(int64_t)(a.out_groups + grp) * a.out_px] = make_float4(z.x - h.x, z.y - h.y, z.z - h.z, z.w - h.w);
+                    }
                 }
             }
+            __syncwarp();                                        // the next item's first tcgen05.ld is the whole warp's
         }
     }
 

@@ -77,7 +77,7 @@ __device__ __forceinline__ void drain_mmas(uint32_t bar) {
 __device__ __forceinline__ void wait_for_nothing(uint32_t bar, volatile int *abort_flag) {
     if (abort_flag[1] == 0) (void)__all_sync(0xffffffffu, mbar_wait(bar, 0, abort_flag));
 }
-// Status word of a block that gave up: kernel id (1 first-layer stream, 2 layer, 3 least squares) in
+// Status word of a block that gave up: kernel id (1 first-layer stream, 2 layer, 3 least squares, 4 convolution) in
 // bits 24-27, the index of the barrier within the block's barrier array in bits 1-16, the awaited
 // parity in bit 0.  Never zero.
 __device__ __forceinline__ int wait_code(int kernel_id, int flag, uint32_t bars_base) {

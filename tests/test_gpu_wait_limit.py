@@ -33,6 +33,9 @@ CASES = {
     "first_layer_stream": (1, 2, dict(dims=(520, 200, 136, 10), n_r=21, m=6, b=2, faults=[(2, "noise200")])),
     "layer": (2, 4, dict(dims=(264, 136, 72, 50), m=9, b=3, n_r=19, faults=[(3, "signflip")])),
     "least_squares": (3, 5, dict(d=70000, m=13, b=5, n_r=16, n_noise=5)),
+    # a first layer of up to four planes (paired taps) and a wider one, either storage type
+    "convolution": (4, 6, dict(dims=(16, 3, 8, 8, 12, 12, 10), m=5, b=2, n_r=4, faults=[(2, "signflip")])),
+    "convolution_wide_bf16": (4, 6, dict(dims=(8, 9, 16, 72, 10), m=5, b=2, n_r=7, faults=[(2, "signflip")], dtype="bf16")),
 }
 
 
@@ -49,7 +52,7 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_the_context_usable(oracle, 
             z.check_device_status()
         assert e.value.status == zeno.ERR_TIMEOUT
         code = z.last_wait_code
-        assert (code >> 24) & 0xf in (1, 2, 3)          # a tensor-core kernel of this step
+        assert (code >> 24) & 0xf in (1, 2, 3, 4)       # a tensor-core kernel of this step
         if name != "first_layer_stream":                # (that step also runs a layer kernel after the stream)
             assert (code >> 24) & 0xf == kernel_id
         assert 0 <= ((code >> 1) & 0xffff) < 64         # an index into that kernel's barrier array

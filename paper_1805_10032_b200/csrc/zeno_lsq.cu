@@ -203,42 +203,62 @@ __global__ void __launch_bounds__(LsqShape<NRT, RB>::kMaxWarps * 32, 1) lsq_stre
 // added in warp order.  The block that finishes last (a ticket, no waiting) forms
 //   residual r_j = (A x)_j - y_j,  f_0 = sum r_j^2 / (2 n_r),
 //   f_i = sum (r_j - gamma (A v_i)_j)^2 / (2 n_r),  score_i = f_0 - f_i - rho ||v_i||^2.
-// One block over all entries and slabs took 40 us for 65 x 17 sums of 148 slabs, a chain of 148 loads per thread.
-constexpr int kFinishWarps = 8;
-__global__ void __launch_bounds__(kFinishWarps * 32) lsq_finish_kernel(const float *part, int slabs, int m, int n_r, const float *y,
+// One block over all entries and slabs took 40 us for 65 x 17 sums of 148 slabs, a chain of 148 loads per thread; up to
+// kFinishAlone slabs one block of 1,024 threads does it all, as the tickets cost 2-4 us more than the loads.
+constexpr int kFinishWarps = 8, kFinishAlone = 8;
+__global__ void __launch_bounds__(1024) lsq_finish_kernel(const float *part, int slabs, int m, int n_r, const float *y,
                                                                        float gamma, float rho, float *losses, float *norms,
                                                                        float *scores, float *sums /*[m+1][n_r+1]*/,
                                                                        unsigned *ticket) {
     const int rows = m + 1, stride = n_r + 1, n = rows * stride;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ double warp_s[kFinishWarps][32];
-    const int t = blockIdx.x * 32 + lane;
-    double acc = 0.0;
-    if (t < n) {
+    if (slabs <= kFinishAlone) {
+        for (int t = threadIdx.x; t < n; t += blockDim.x) {
+            double acc = 0.0;
 #pragma unroll 4
-        for (int s = warp; s < slabs; s += kFinishWarps) acc += (double)__ldcg(part + (int64_t)s * n + t);
-    }
-    warp_s[warp][lane] = acc;
-    __syncthreads();
-    if (warp == 0 && t < n) {
-        double tot = 0.0;
+            for (int s = 0; s < slabs; ++s) acc += (double)__ldcg(part + (int64_t)s * n + t);
+            sums[t] = (float)acc;
+        }
+        __syncthreads();
+    } else {
+        const int t = blockIdx.x * 32 + lane;
+        double acc = 0.0;
+        if (t < n) {
+#pragma unroll 4
+            for (int s = warp; s < slabs; s += kFinishWarps) acc += (double)__ldcg(part + (int64_t)s * n + t);
+        }
+        warp_s[warp][lane] = acc;
+        __syncthreads();
+        if (warp == 0 && t < n) {
+            double tot = 0.0;
 #pragma unroll
-        for (int w = 0; w < kFinishWarps; ++w) tot += warp_s[w][lane];
-        sums[t] = (float)tot;
+            for (int w = 0; w < kFinishWarps; ++w) tot += warp_s[w][lane];
+            sums[t] = (float)tot;
+        }
+        if (!take_last_ticket(ticket, gridDim.x)) return;
     }
-    if (!take_last_ticket(ticket, gridDim.x)) return;
     // the losses stay in double until the score is formed: f_0 - f_i cancels many digits
     __shared__ double f_s[ZENO_MAX_CANDIDATES + 1];
-    for (int r = warp; r < rows; r += kFinishWarps) {                // a warp a model, lanes over the samples
+    // a lane a model, four beyond eight samples: a warp a model left 501 models of 4 samples 63 rounds of loads and
+    // shuffles, 35 us
+    const int lanes = n_r <= 8 ? 1 : 4, first = threadIdx.x % lanes;
+    for (int r0 = 0; r0 < rows; r0 += (int)blockDim.x / lanes) {
+        const int r = r0 + threadIdx.x / lanes;
         double f = 0.0;
-        for (int j = lane; j < n_r; j += 32) {
-            double res = (double)__ldcg(sums + j) - (double)y[j];
-            if (r > 0) res -= (double)gamma * (double)__ldcg(sums + r * stride + j);
-            f += res * res;
+        if (r < rows) {
+#pragma unroll 8
+            for (int j = first; j < n_r; j += lanes) {
+                double res = (double)__ldcg(sums + j) - (double)__ldg(y + j);
+                if (r > 0) res -= (double)gamma * (double)__ldcg(sums + r * stride + j);
+                f += res * res;
+            }
         }
-#pragma unroll
-        for (int sft = 16; sft >= 1; sft >>= 1) f += __shfl_xor_sync(0xffffffffu, f, sft);
-        if (lane == 0) {
+        if (lanes > 1) {
+            f += __shfl_xor_sync(0xffffffffu, f, 2);
+            f += __shfl_xor_sync(0xffffffffu, f, 1);
+        }
+        if (r < rows && first == 0) {
             f_s[r] = f / (2.0 * n_r);
             losses[r] = (float)f_s[r];
         }
@@ -284,6 +304,14 @@ __global__ void __launch_bounds__(1024) lsq_from_sums_kernel(const double *sums 
         if (norms) norms[i] = (float)nv;
         scores[i] = (float)(f_s[0] - f_s[1 + i] - (double)rho * nv);
     }
+}
+
+// not chained to the stream: with its blocks resident beside the stream's the step was 2 % slower
+void launch_finish(const float *part, int slabs, int m, int n_r, const float *y, float gamma, float rho, float *losses, float *norms,
+                   float *scores, float *sums, unsigned *ticket, cudaStream_t s) {
+    const int blocks = slabs <= kFinishAlone ? 1 : ((m + 1) * (n_r + 1) + 31) / 32;
+    lsq_finish_kernel<<<blocks, slabs <= kFinishAlone ? 1024 : kFinishWarps * 32, 0, s>>>(part, slabs, m, n_r, y, gamma, rho, losses, norms,
+                                                                                          scores, sums, ticket);
 }
 
 template <int NRT, int RB, bool VEC>
@@ -349,9 +377,7 @@ cudaError_t launch_lsq_score(Context &c, const LsqArgs &a, const float *y, float
     // the combined sums live behind the slab partials in the same workspace region
     const int rows = a.m + 1;
     float *sums = a.part + (int64_t)slabs * rows * (a.n_r + 1);
-    // not chained to the stream: with its blocks resident beside the stream's the step was 2 % slower
-    lsq_finish_kernel<<<(rows * (a.n_r + 1) + 31) / 32, kFinishWarps * 32, 0, s>>>(a.part, slabs, a.m, a.n_r, y, gamma, rho, losses, norms,
-                                                                                   scores, sums, c.tickets);
+    launch_finish(a.part, slabs, a.m, a.n_r, y, gamma, rho, losses, norms, scores, sums, c.tickets, s);
     return cudaGetLastError();
 }
 
@@ -466,8 +492,7 @@ extern "C" zeno_status zeno_score_lsq_static(int32_t device, const float *x, con
             // same call, so nothing an earlier call left behind, not even one that raced with another, matters.
             float *sums = a.part + (int64_t)slabs * rows * (n_r + 1);
             float *loss_buf = losses ? losses : sums + (int64_t)rows * (n_r + 1);
-            zeno::lsq_finish_kernel<<<(rows * (n_r + 1) + 31) / 32, zeno::kFinishWarps * 32, 0, s>>>(
-                a.part, slabs, m, n_r, y, gamma, rho, loss_buf, norms, scores, sums, a.ticket);
+            zeno::launch_finish(a.part, slabs, m, n_r, y, gamma, rho, loss_buf, norms, scores, sums, a.ticket, s);
             e = cudaGetLastError();
         }
     }

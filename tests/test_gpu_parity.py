@@ -203,6 +203,13 @@ def test_lsq_unaligned(oracle):
     P.run_step_parity(oracle, w)
 
 
+# the finish: one block or many, one lane or four per model, fewer and more models than a block's lanes
+@pytest.mark.parametrize("d,n_r,m", [(500, 1, 1), (500, 8, 300), (3001, 9, 260), (20000, 8, 257), (20000, 33, 65), (70001, 9, 70)])
+def test_lsq_finish_over_its_splits(oracle, d, n_r, m):
+    w = syn.make_config(5, d=d, m=m, b=m // 3, n_r=n_r, n_noise=m // 3)
+    P.run_step_parity(oracle, w)
+
+
 def test_no_bias_model(oracle):
     w = syn.make_config(2, dims=(96, 24, 10), n_r=6, m=5, b=1, faults=[(1, "noise200")],
                         has_bias=False)

@@ -8,7 +8,9 @@
 // min(a[i], b[H - 1 - i]), so the value of rank H - 1 is the largest of those and the value of rank H the
 // smallest of max(a[i], b[H - 1 - i]).  A column of fewer than 2 H values is padded with equally many minus
 // and plus infinities (one more plus infinity when the number is odd), which leaves the middle where it is.
-// bfloat16 columns go two to a thread, compared in pairs by the packed minimum and maximum.
+// Up to 12 candidates, where the loads are what it waits for, bfloat16 columns go two to a thread, compared in pairs by
+// the packed minimum and maximum (1.8 M columns of 5: 8.3 us against 10.8 with one); beyond, the packed comparisons are
+// the slower ones (100: 717 us against 232, and 19.0 against 6.5 for 7,960 columns, which then fill half as many SMs).
 //
 // Beyond 128 candidates 8, 16 or 32 neighbouring lanes of a warp share a column, 32 values each, sorted by a
 // bitonic network whose long-range stages exchange values by shuffles.
@@ -22,17 +24,19 @@ namespace {
 
 constexpr int kMedianThreads = 128;
 constexpr int kMedianMaxHalf = 64;            // values in each half of a column one thread holds
+constexpr int kMedianTwoColsHalf = 6;         // bfloat16: halves up to which a thread takes two columns
 
 __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }
 
 __device__ __forceinline__ float nan_to_inf(float v) { return v != v ? INFINITY : v; }
 
-// What a register of the one-thread kernel holds: one binary32 column, or two bfloat16 columns.
-template <typename T> struct Cols;
-template <> struct Cols<float> {
+// What a register of the one-thread kernel holds: one column in binary32, or two bfloat16 columns.
+template <typename T>
+struct OneCol {
+    using Elem = T;
     using Reg = float;
     static constexpr int kCols = 1;
-    static __device__ __forceinline__ Reg load(const float *p, bool, bool) { return __ldg(p); }
+    static __device__ __forceinline__ Reg load(const T *p, bool, bool) { return load_elem(p); }
     static __device__ __forceinline__ Reg all(float v) { return v; }
     static __device__ __forceinline__ Reg min(Reg a, Reg b) { return fminf(a, b); }
     static __device__ __forceinline__ Reg max(Reg a, Reg b) { return fmaxf(a, b); }
@@ -44,7 +48,8 @@ template <> struct Cols<float> {
         *out = odd ? lo : 0.5f * lo + 0.5f * hi;
     }
 };
-template <> struct Cols<__nv_bfloat16> {
+struct TwoCols {
+    using Elem = __nv_bfloat16;
     using Reg = __nv_bfloat162;
     static constexpr int kCols = 2;
     // whole: both columns exist and their four bytes may be read at once
@@ -108,10 +113,10 @@ __host__ __device__ constexpr int median_blocks_per_sm(int H) {
 // Bound by the comparisons: minimum and maximum issue at half the rate of an addition, so a column of 100
 // costs about 1,700 half-rate instructions where reading it costs 100 loads.  100 x 1.8 M binary32 values take
 // 241 us (114 us of memory time); the whole column sorted over four lanes with shuffles took 934 us.
-template <typename T, int H>
+template <typename C, int H>
 __global__ void __launch_bounds__(kMedianThreads, median_blocks_per_sm(H))
-median_select_kernel(const T *V, int64_t ldv, int64_t d, int m, int pairs, float *out) {
-    using C = Cols<T>;
+median_select_kernel(const typename C::Elem *V, int64_t ldv, int64_t d, int m, int pairs, float *out) {
+    using T = typename C::Elem;
     using Reg = typename C::Reg;
     constexpr int kTile = kMedianThreads * C::kCols;
     constexpr int kSlack = H <= 16 ? 1 : 7;       // most padding values
@@ -260,29 +265,38 @@ cudaError_t launch_lanes(Context &c, const T *V, int64_t ldv, int m, float *out,
 
 // the one-thread kernel whose halves hold just m values: every H up to 16, then steps of four (a finer step
 // would save at most 6 % of the comparisons and quadruple the kernels)
-template <typename T, int H>
+template <typename C, int H>
 struct MedianSelect {
+    using T = typename C::Elem;
     static cudaError_t launch(Context &c, const T *V, int64_t ldv, int m, float *out, cudaStream_t s) {
         constexpr int kSmaller = H > 16 ? H - 4 : H - 1;
-        if (m <= 2 * kSmaller) return MedianSelect<T, kSmaller>::launch(c, V, ldv, m, out, s);
+        if (m <= 2 * kSmaller) return MedianSelect<C, kSmaller>::launch(c, V, ldv, m, out, s);
         const int sms = c.sm_count > 0 ? c.sm_count : 148;
-        const int64_t d = c.d, tile = kMedianThreads * Cols<T>::kCols;
+        const int64_t d = c.d, tile = kMedianThreads * C::kCols;
         const int64_t want = (d + tile - 1) / tile, cap = (int64_t)sms * median_blocks_per_sm(H) * 8;
         const int blocks = (int)(want < cap ? want : cap);
         const int pairs = ldv % 2 == 0 && reinterpret_cast<uintptr_t>(V) % 4 == 0;
-        return launch_chained(median_select_kernel<T, H>, dim3(blocks), dim3(kMedianThreads), 0, s, chain_launches(c), V, ldv, d, m,
+        return launch_chained(median_select_kernel<C, H>, dim3(blocks), dim3(kMedianThreads), 0, s, chain_launches(c), V, ldv, d, m,
                               pairs, out);
     }
 };
-template <typename T>
-struct MedianSelect<T, 0> {
-    static cudaError_t launch(Context &, const T *, int64_t, int, float *, cudaStream_t) { return cudaErrorInvalidValue; }
+template <typename C>
+struct MedianSelect<C, 0> {
+    static cudaError_t launch(Context &, const typename C::Elem *, int64_t, int, float *, cudaStream_t) { return cudaErrorInvalidValue; }
 };
+
+cudaError_t launch_select(Context &c, const float *V, int64_t ldv, int m, float *out, cudaStream_t s) {
+    return MedianSelect<OneCol<float>, kMedianMaxHalf>::launch(c, V, ldv, m, out, s);
+}
+cudaError_t launch_select(Context &c, const __nv_bfloat16 *V, int64_t ldv, int m, float *out, cudaStream_t s) {
+    if (m <= 2 * kMedianTwoColsHalf) return MedianSelect<TwoCols, kMedianTwoColsHalf>::launch(c, V, ldv, m, out, s);
+    return MedianSelect<OneCol<__nv_bfloat16>, kMedianMaxHalf>::launch(c, V, ldv, m, out, s);
+}
 
 template <typename T>
 cudaError_t launch_typed(Context &c, const T *V, int64_t ldv, int m, float *out, cudaStream_t s) {
     static_assert(kMedianRegs * 32 >= ZENO_MAX_CANDIDATES, "a warp holds the longest column");
-    if (m <= 2 * kMedianMaxHalf) return MedianSelect<T, kMedianMaxHalf>::launch(c, V, ldv, m, out, s);
+    if (m <= 2 * kMedianMaxHalf) return launch_select(c, V, ldv, m, out, s);
     if (m <= kMedianRegs * 8) return launch_lanes<T, 8>(c, V, ldv, m, out, s);
     if (m <= kMedianRegs * 16) return launch_lanes<T, 16>(c, V, ldv, m, out, s);
     return launch_lanes<T, 32>(c, V, ldv, m, out, s);

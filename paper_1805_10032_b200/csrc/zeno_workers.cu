@@ -39,26 +39,30 @@ template <> __device__ __forceinline__ void store_elem<__nv_bfloat16>(__nv_bfloa
 
 // Softmax regression, worker w = blockIdx.y: samples feats[w][n][in], labels[w][n].
 //   delta[j][c] = (softmax(W a_j + b)[c] - [c == label_j]) / n;  dW[c][k] = sum_j delta[j][c] a_j[k];  db[c] = sum_j delta[j][c]
-// A cluster of eight blocks works for one worker: block r takes an eighth of the samples' logits and leaves their
-// delta in the shared memory of all eight, then every block takes an eighth of the input indices of dW.  Latency is
-// all there is (20 workers of 100 samples x 784 inputs read 6 MB, 1 us): one block a worker, with its samples one
-// after another in a warp, left 128 SMs idle and took 500 us for those sizes where this takes 22 us.
+// A cluster of blocks works for one worker: block r takes its share of the samples' logits and leaves their delta in the
+// shared memory of all of them, then every block takes its share of the input indices of dW.  Latency is all there is
+// (20 workers of 100 samples x 784 inputs read 6 MB, 1 us): one block a worker, with its samples one after another in a
+// warp, left 128 SMs idle and took 500 us for those sizes where this takes 22 us.  A block with fewer samples than its
+// warps take at a time splits their input range over the warps (256 workers of one sample x 3072 inputs, 20 classes:
+// 28 us, 1,750 before; one block a worker: 186).
 // dynamic shared memory: delta [n][pitch] (pitch: classes rounded up to 4), then the sample groups' sums.
-constexpr int kWCluster = 8;
+constexpr int kWCluster = 8;                  // blocks of a worker's cluster at most
 constexpr int kWGradWarps = 8;
 constexpr int kWSamples = 2;                  // samples a warp takes at a time: the weights are read once for both
 
-// CM: classes the registers are sized for, a multiple of 4
-template <typename T, int CM>
+// CM: classes the registers are sized for, a multiple of 4.  SPLIT: the kernel for few samples, whose clusters may be of
+// fewer than kWCluster blocks.
+template <typename T, int CM, bool SPLIT>
 __global__ void __launch_bounds__(kWGradWarps * 32, 2)
 worker_grad_softmax_kernel(const T *x, int in, int classes, int has_bias, const float *feats, const int32_t *labels, int n,
                            const int32_t *flip, T *V, int64_t ldv) {
     extern __shared__ __align__(16) float delta[];
     constexpr int S = kWSamples, CR = CM <= 4 ? 4 : CM <= 16 ? 16 : 32;
     const int w = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rank = (int)cluster_rank();
+    const int rank = (int)cluster_rank(), cluster = SPLIT ? (int)gridDim.x : kWCluster;
     const int pitch = (classes + 3) & ~3;
     float *sums = delta + (size_t)n * pitch;
+    __shared__ float part_z[SPLIT ? kWGradWarps : 1][S][CR];
     pdl_wait();                               // no early trigger: what follows reads V through the read-only path
     const float *a = feats + (int64_t)w * n * in;
     const int32_t *lab = labels + (int64_t)w * n;
@@ -67,42 +71,80 @@ worker_grad_softmax_kernel(const T *x, int in, int classes, int has_bias, const 
     const int cls = lane & (CR - 1);
     const float bias = has_bias && cls < classes ? load_elem(x + (int64_t)classes * in + cls) : 0.f;
     cluster_barrier();                        // every block of the cluster runs: their shared memory may be written
-    // logits of this block's samples: a warp takes S of them, lanes stride the input index
-    const int per_block = (n + kWCluster - 1) / kWCluster;
+    // logits of this block's samples: a warp takes S of them, lanes stride the input index; with fewer of them than warps
+    // a sample's warps (warp, warp + units, ..) deal the input range out
+    const int per_block = (n + cluster - 1) / cluster;
     const int j_end = min(n, (rank + 1) * per_block);
-    for (int j0 = rank * per_block + warp * S; j0 < j_end; j0 += kWGradWarps * S) {
+    const int units = (per_block + S - 1) / S, parts = SPLIT && units < kWGradWarps ? kWGradWarps / units : 1;
+    const int part = parts > 1 ? warp / units : 0;
+    // one turn if warps share samples, and then all of them take it
+    for (int u = parts > 1 ? warp % units : warp; u < units; u += kWGradWarps) {
+        const int j0 = rank * per_block + u * S;
+        if (!SPLIT && j0 >= j_end) break;
         float z[S][CM];
 #pragma unroll
         for (int q = 0; q < S; ++q)
 #pragma unroll
             for (int c = 0; c < CM; ++c) z[q][c] = 0.f;
-#pragma unroll(CM <= 12 ? 4 : 1)
-        for (int k = lane; k < in; k += 32) {
-            float av[S];
+        if (!SPLIT && CM <= 12) {
+#pragma unroll 4
+            for (int k = lane; k < in; k += 32) {
+                float av[S];
 #pragma unroll
-            for (int q = 0; q < S; ++q) av[q] = __ldg(a + (int64_t)min(j0 + q, j_end - 1) * in + k);
+                for (int q = 0; q < S; ++q) av[q] = __ldg(a + (int64_t)min(j0 + q, j_end - 1) * in + k);
 #pragma unroll
-            for (int c = 0; c < CM; ++c) {
-                if (c < classes) {
-                    const float wv = load_elem(x + (int64_t)c * in + k);
+                for (int c = 0; c < CM; ++c) {
+                    if (c < classes) {
+                        const float wv = load_elem(x + (int64_t)c * in + k);
 #pragma unroll
-                    for (int q = 0; q < S; ++q) z[q][c] = fmaf(wv, av[q], z[q][c]);
+                        for (int q = 0; q < S; ++q) z[q][c] = fmaf(wv, av[q], z[q][c]);
+                    }
                 }
             }
-        }
+        } else if (!SPLIT || (j0 < j_end && part < parts)) {
+            // of more classes the conditions become branches, each with a load to wait for: beyond the classes the last
+            // one's weight again, its product dropped
+#pragma unroll(CM <= 12 ? 4 : 1)
+            for (int k = part * 32 + lane; k < in; k += parts * 32) {
+                float av[S], wv[CM];
 #pragma unroll
-        for (int q = 0; q < S; ++q) {
-            // lane c (and its copies CR lanes apart) collects class c, so that a class costs one exponential
+                for (int q = 0; q < S; ++q) av[q] = __ldg(a + (int64_t)min(j0 + q, j_end - 1) * in + k);
+#pragma unroll
+                for (int c = 0; c < CM; ++c) wv[c] = load_elem(x + (int64_t)min(c, classes - 1) * in + k);
+#pragma unroll
+                for (int c = 0; c < CM; ++c)
+#pragma unroll
+                    for (int q = 0; q < S; ++q) z[q][c] = fmaf(wv[c], av[q], z[q][c]);
+            }
+        }
+        // lane c (and its copies CR lanes apart) collects class c, so that a class costs one exponential
+        auto collect = [&](int q) {
             float v[CR];
 #pragma unroll
             for (int c = 0; c < CR; ++c) v[c] = c < CM ? z[q][c < CM ? c : 0] : 0.f;
-            const float zc = warp_transpose_reduce<CR>(v, lane) + bias;
+            return warp_transpose_reduce<CR>(v, lane);
+        };
+        if (SPLIT && parts > 1) {
+#pragma unroll
+            for (int q = 0; q < S; ++q) part_z[warp][q][cls] = collect(q);
+            __syncthreads();
+            if (part > 0) break;
+        }
+#pragma unroll
+        for (int q = 0; q < S; ++q) {
+            float zj;
+            if (SPLIT && parts > 1) {
+                zj = bias;
+                for (int p = 0; p < parts; ++p) zj += part_z[warp + p * units][q][cls];
+            } else {
+                zj = collect(q) + bias;
+            }
             const int j = j0 + q;
             if (j >= j_end) break;
-            float zmax = cls < classes ? zc : -INFINITY;
+            float zmax = cls < classes ? zj : -INFINITY;
 #pragma unroll
             for (int s = CR / 2; s >= 1; s >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, s));
-            const float e = cls < classes ? expf(zc - zmax) : 0.f;
+            const float e = cls < classes ? expf(zj - zmax) : 0.f;
             float se = e;
 #pragma unroll
             for (int s = CR / 2; s >= 1; s >>= 1) se += __shfl_xor_sync(0xffffffffu, se, s);
@@ -110,13 +152,13 @@ worker_grad_softmax_kernel(const T *x, int in, int classes, int has_bias, const 
             if (flipped) label = classes - 1 - label;
             const float dj = cls < classes ? (e / se - (cls == label ? 1.f : 0.f)) / (float)n : 0.f;
             if (cls < pitch)                  // the copies share the cluster's blocks between them
-                for (int r = lane / CR; r < kWCluster; r += 32 / CR) cluster_store(cluster_addr(delta + (size_t)j * pitch + cls, r), dj);
+                for (int r = lane / CR; r < cluster; r += 32 / CR) cluster_store(cluster_addr(delta + (size_t)j * pitch + cls, r), dj);
         }
     }
     cluster_barrier();
     // dW: this block's chunks of 32 input indices, a lane per index, all classes in registers.  With fewer chunks
     // than warps, groups of warps share a chunk and split the samples; their sums are added in group order.
-    const int chunks = (in + 31) / 32, per = (chunks + kWCluster - 1) / kWCluster;
+    const int chunks = (in + 31) / 32, per = (chunks + cluster - 1) / cluster;
     const int first = rank * per, mine = min(per, chunks - first);
     const int groups = per >= kWGradWarps ? 1 : kWGradWarps / per;
     const int group = per >= kWGradWarps ? 0 : warp / per;
@@ -166,7 +208,7 @@ worker_grad_softmax_kernel(const T *x, int in, int classes, int has_bias, const 
                 if (c < classes) store_elem(out + (int64_t)c * in + k, g[c]);
         }
     }
-    if (has_bias && rank == kWCluster - 1) {  // the block with the fewest input indices
+    if (has_bias && rank == cluster - 1) {    // the block with the fewest input indices
         for (int c = warp; c < classes; c += kWGradWarps) {
             float g = 0.f;
             for (int j = lane; j < n; j += 32) g += delta[(size_t)j * pitch + c];
@@ -177,25 +219,38 @@ worker_grad_softmax_kernel(const T *x, int in, int classes, int has_bias, const 
     }
 }
 
-inline size_t worker_grad_smem(int in, int classes, int n) {
-    const int per = ((in + 31) / 32 + kWCluster - 1) / kWCluster;
+inline size_t worker_grad_smem(int in, int classes, int n, int cluster) {
+    const int per = ((in + 31) / 32 + cluster - 1) / cluster;
     const int groups = per >= kWGradWarps ? 1 : kWGradWarps / per;
     return ((size_t)n * ((classes + 3) & ~3) + (size_t)(groups - 1) * per * classes * 32) * sizeof(float);
 }
 
-template <typename T, int CM>
-cudaError_t launch_softmax(Context &c, const T *x, int in, int classes, const float *feats, const int32_t *labels, int n,
-                           int m, const int32_t *flip, T *V, int64_t ldv, cudaStream_t s) {
-    const size_t smem = worker_grad_smem(in, classes, n);
+template <typename T, int CM, bool SPLIT>
+cudaError_t launch_softmax_split(Context &c, const T *x, int in, int classes, const float *feats, const int32_t *labels, int n,
+                                 int m, const int32_t *flip, T *V, int64_t ldv, cudaStream_t s) {
+    // fewer blocks a worker where two an SM do not hold them all and they would have no samples for their warps: further
+    // waves of blocks with little to do cost more than they bring
+    const int sms = c.sm_count > 0 ? c.sm_count : 148;
+    int cluster = kWCluster;
+    while (SPLIT && cluster > 1 && m * cluster > 2 * sms && n < kWGradWarps * kWSamples * cluster) cluster /= 2;
+    const size_t smem = worker_grad_smem(in, classes, n, cluster);
     static PerDeviceOnce attr_set;
     if (attr_set.need(c.device)) {
-        cudaError_t e = cudaFuncSetAttribute(worker_grad_softmax_kernel<T, CM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(worker_grad_softmax_kernel<T, CM, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              kWMaxSmem);
         if (e != cudaSuccess) return e;
         attr_set.mark(c.device);
     }
-    return launch_clustered(worker_grad_softmax_kernel<T, CM>, kWCluster, dim3(kWCluster, m), dim3(kWGradWarps * 32), smem, s,
+    return launch_clustered(worker_grad_softmax_kernel<T, CM, SPLIT>, cluster, dim3(cluster, m), dim3(kWGradWarps * 32), smem, s,
                             chain_launches(c), x, in, classes, (int)c.desc.has_bias, feats, labels, n, flip, V, ldv);
+}
+
+// up to 64 samples eight blocks leave at least every second warp without any
+template <typename T, int CM>
+cudaError_t launch_softmax(Context &c, const T *x, int in, int classes, const float *feats, const int32_t *labels, int n,
+                           int m, const int32_t *flip, T *V, int64_t ldv, cudaStream_t s) {
+    if (n <= kWCluster * kWGradWarps * kWSamples / 2) return launch_softmax_split<T, CM, true>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
+    return launch_softmax_split<T, CM, false>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
 }
 
 template <typename T>
@@ -203,6 +258,7 @@ cudaError_t launch_softmax_classes(Context &c, const T *x, int in, int classes, 
                                    int m, const int32_t *flip, T *V, int64_t ldv, cudaStream_t s) {
     if (classes <= 4) return launch_softmax<T, 4>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
     if (classes <= 12) return launch_softmax<T, 12>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
+    if (classes <= 20) return launch_softmax<T, 20>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
     return launch_softmax<T, kWMaxClasses>(c, x, in, classes, feats, labels, n, m, flip, V, ldv, s);
 }
 

@@ -78,6 +78,30 @@ def test_softmax_worker_gradients_over_the_sizes(oracle, n_w, dims, bias, dtype)
         assert np.linalg.norm(Vh[i, :d].numpy() - want) <= (2e-6 + (2.0 ** -9 if dtype else 0.0)) * np.linalg.norm(want), i
 
 
+# few samples, whose input range a block's warps share, and clusters of four, two and one blocks; the most samples of
+# that kernel and one more
+@pytest.mark.parametrize("m,n_w,dims", [(40, 1, (100, 13)), (75, 17, (33, 20)), (160, 33, (65, 21)), (300, 2, (700, 32)),
+                                        (300, 64, (31, 10)), (300, 65, (31, 10))])
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_softmax_worker_gradients_of_many_workers(oracle, m, n_w, dims, dtype):
+    g = torch.Generator().manual_seed(m)
+    d = dims[0] * dims[1] + dims[1]
+    x = torch.randn(d, generator=g) * 0.1
+    x = x.to(torch.bfloat16) if dtype else x
+    feats = torch.randn(m, n_w, dims[0], generator=g)
+    labels = torch.randint(0, dims[1], (m, n_w), generator=g, dtype=torch.int32)
+    V = torch.full((m, d + 3), float("nan"), device="cuda", dtype=x.dtype)
+    with zeno.Zeno(MLP, dtype, dims, True, m_max=m, n_r_max=4) as z:
+        z.worker_gradients(x.cuda(), feats.cuda(), labels.cuda(), V)
+        torch.cuda.synchronize()
+    Vh = V.float().cpu()
+    assert torch.isnan(Vh[:, d:]).all() and torch.isfinite(Vh[:, :d]).all()
+    for i in (0, 1, m // 2, m - 2, m - 1):
+        want = oracle.worker_gradient(MLP, dtype, dims, True, syn.to_numpy_params(x), feats[i].numpy(), labels[i].numpy())
+        # as over the sizes above
+        assert np.linalg.norm(Vh[i, :d].numpy() - want) <= (2e-6 + (2.0 ** -9 if dtype else 0.0)) * np.linalg.norm(want), i
+
+
 def test_least_squares_worker_gradients(oracle):
     g = torch.Generator().manual_seed(3)
     d, m, n_w = 5003, 6, 9

@@ -8,6 +8,8 @@
 // A small last layer (mlp_head_kernel) runs as one cluster of blocks per model and also evaluates the
 // cross-entropy.  In a step the averaging kernel forms the scores and the ranking from the losses; in a call that
 // ends with the scores the block that finishes last (a ticket, no waiting) does, so neither costs a launch.
+#include <type_traits>
+
 #include "zeno_internal.h"
 #include "zeno_tail.cuh"
 
@@ -37,31 +39,55 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 
-// One dense layer of all models, rows of any alignment.  A block takes 64 output rows of one model and 8 TN samples and
+// One dense layer of all models, rows of any alignment.  A block takes 8 R output rows of one model and 8 TN samples and
 // stages slices of 64 input columns in shared memory -- w = x - gamma v formed on the way, v^2 accumulated, all of the
 // next slice's loads in flight during the present one's arithmetic.  Its four groups of 64 threads take sixteen of the
-// columns each and their sums are added at the end, so that few rows still have eight warps at work on every 64 of
-// them; a thread holds 8 rows x TN samples and reads four columns of each at a time (8 + TN 16-byte reads for 32 TN
-// multiplications).  A warp loads 32 neighbouring columns of one row, which needs no alignment and touches two lines.
+// columns each and their sums are added at the end, so that few rows still have eight warps at work on every 8 R of
+// them; a thread holds R rows x TN samples and reads four columns of each at a time (R + TN 16-byte reads for 4 R TN
+// multiplications).  R = 8, or 4 for layers of up to 32 rows, which then take up to 64 samples at a time instead of 32.
+// VEC (rows aligned to four elements): a load takes four columns of a row, half a warp a row's slice; else a warp loads
+// 32 neighbouring columns of one row, which needs no alignment and touches two lines.
 // The products are summed in runs of 64 columns that are then added to the total, so rounding errors stay those of
 // short sums.  Where that leaves SMs idle a cluster of blocks deals the slices out and meets in the first one's
 // shared memory.
 // Bound by the loads' latency and the CUDA cores' rate: 38 models of 1029 x 301 with 19 samples take 61 us (one
-// warp per four rows and one block an SM: 80), 24 models of 4096 x 43 with 40 samples in clusters of two 90 us less.
+// warp per four rows and one block an SM: 80).  A whole pass with VEC and without: 101 models of 2500 x 2000 in bfloat16,
+// 4 samples, 892 us and 3,381; with R = 4 and 8: 61 models of 3001 x 20 x 3, 200 samples, 181 us and 309.
 constexpr int kMaxCluster = 8;                   // blocks of a cluster, here and in the head
-constexpr int kLRows = 64, kLK = 64, kLGroups = 4, kLPitch = kLK + 4;
+constexpr int kLK = 64, kLGroups = 4, kLPitch = kLK + 4;
 constexpr int kLRun = 4;                         // slices of a run (a group's sixteen columns of each)
-__host__ __device__ constexpr int layer_stage_floats(int TN) { return 2 * (kLRows + 8 * TN) * kLPitch; }
-__host__ __device__ constexpr int layer_red_floats(int TN) { return kLRows * (8 * TN + 1); }
-inline size_t layer_smem(int TN, int cluster) {
-    const int stage = layer_stage_floats(TN), red = kLGroups * layer_red_floats(TN);
-    return sizeof(float) * ((size_t)(stage > red ? stage : red) + (cluster > 1 ? cluster * (layer_red_floats(TN) + 8) : 0));
+constexpr int kLFewRows = 32;                    // layers of up to so many rows: R = 4
+__host__ __device__ constexpr int layer_stage_floats(int R, int TN) { return 2 * (8 * R + 8 * TN) * kLPitch; }
+__host__ __device__ constexpr int layer_red_floats(int R, int TN) { return 8 * R * (8 * TN + 1); }
+__host__ __device__ constexpr int layer_own_floats(int R, int TN) {
+    return layer_stage_floats(R, TN) > kLGroups * layer_red_floats(R, TN) ? layer_stage_floats(R, TN) : kLGroups * layer_red_floats(R, TN);
+}
+inline size_t layer_smem(int R, int TN, int cluster) {
+    return sizeof(float) * ((size_t)layer_own_floats(R, TN) + (cluster > 1 ? cluster * (layer_red_floats(R, TN) + 8) : 0));
 }
 
-template <typename T, int TN>
+// elements as they lie in memory: one, or four
+template <typename T> struct RawOf;
+template <> struct RawOf<float> { using One = float; using Four = float4; };
+template <> struct RawOf<__nv_bfloat16> { using One = unsigned short; using Four = uint2; };
+__device__ __forceinline__ float raw_to_float(float v) { return v; }
+__device__ __forceinline__ float raw_to_float(unsigned short v) { return bf16_bits_to_float(v); }
+__device__ __forceinline__ float4 raw_to_float4(float4 v) { return v; }
+__device__ __forceinline__ float4 raw_to_float4(uint2 v) {
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                       __uint_as_float(v.y & 0xffff0000u));
+}
+
+template <typename T, int R, int TN, bool VEC>
 __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a, int sample_tiles, int cluster) {
-    constexpr int BN = 8 * TN, kRed = layer_red_floats(TN);
-    constexpr int kStage = layer_stage_floats(TN) > kLGroups * kRed ? layer_stage_floats(TN) : kLGroups * kRed;
+    constexpr int kRows = 8 * R, BN = 8 * TN, kRed = layer_red_floats(R, TN), kOwn = layer_own_floats(R, TN);
+    // Loads with no condition around them, entries beyond the rows or columns taken from elsewhere in the layer and dropped
+    // when they are staged: every conditional bfloat16 load became a branch with a wait of its own (21 models of
+    // 1345 x 1000, 4 samples: 217 us a pass against 102).  Binary32 loads stay conditional, and so do bfloat16 ones beside the
+    // registers of more samples: the masks and the spills cost more there (10 to 20 %).
+    constexpr bool kFree = VEC || (is_bf16<T>::value && TN <= 2);
+    using Raw = typename std::conditional<VEC, typename RawOf<T>::Four, typename std::conditional<kFree, typename RawOf<T>::One, float>::type>::type;
+    constexpr int kLoads = VEC ? R / 2 : 2 * R;  // of x and of v, a thread and slice
     extern __shared__ __align__(16) float smem_dyn[];
     pdl_wait();
     pdl_launch_dependents();
@@ -70,7 +96,7 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
     const int rank = cluster > 1 ? (int)cluster_rank() : 0;
     const int c = blockIdx.y;                    // model: 0 = x, 1+i = x - gamma v_i
     const int tile = blockIdx.x / cluster, row_tile = tile / sample_tiles, sample_tile = tile - row_tile * sample_tiles;
-    const int row0 = row_tile * kLRows, j0 = sample_tile * BN;
+    const int row0 = row_tile * kRows, j0 = sample_tile * BN;
     const int K = a.in;
     const bool has_v = c > 0;
     const T *xw = static_cast<const T *>(a.x) + a.offW;
@@ -79,23 +105,42 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
     const float *hin = a.Hin + (int64_t)c * a.hin_cand_stride;
     const int tx = t & 7, ty = t >> 3;           // this thread's rows tx + 8 r and samples ty + 8 n
 
-    float acc[8][TN], tot[8][TN];
+    float acc[R][TN], tot[R][TN];
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int n = 0; n < TN; ++n) acc[r][n] = tot[r][n] = 0.f;
     float nrm = 0.f;
-    float xr[16], vr[16], hr[2 * TN];
-    auto load = [&](int kt) {                    // rows and samples warp + 8 r, columns lane and lane + 32 of the slice
+    Raw xr[kLoads], vr[kLoads];
+    float hr[2 * TN];
+    // VEC: rows 2 warp + (lane >> 4) + 16 u, columns from 4 (lane & 15) on; else rows warp + 8 r, columns lane and lane + 32
+    const int vrow = 2 * warp + (lane >> 4), vcol = 4 * (lane & 15);
+    auto load = [&](int kt) {
+        if constexpr (VEC) {
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = kt * kLK + h * 32 + lane, o = row0 + warp + 8 * r;
-                const bool ok = k < K && o < a.out;
-                xr[2 * r + h] = ok ? load_elem(xw + (int64_t)o * K + k) : 0.f;
-                vr[2 * r + h] = ok && has_v ? load_elem(vw + (int64_t)o * K + k) : 0.f;
+            for (int u = 0; u < R / 2; ++u) {
+                const int k = kt * kLK + vcol;
+                const int64_t at = (int64_t)min(row0 + vrow + 16 * u, a.out - 1) * K + (k < K ? k : 0);
+                xr[u] = __ldg(reinterpret_cast<const Raw *>(xw + at));
+                vr[u] = __ldg(reinterpret_cast<const Raw *>(vw + at));         // of model 0 a row that is dropped
             }
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int k = kt * kLK + h * 32 + lane, o = row0 + warp + 8 * r;
+                    if constexpr (kFree) {
+                        const int64_t at = (int64_t)min(o, a.out - 1) * K + min(k, K - 1);
+                        xr[2 * r + h] = __ldg(reinterpret_cast<const Raw *>(xw + at));
+                        vr[2 * r + h] = __ldg(reinterpret_cast<const Raw *>(vw + at));
+                    } else {
+                        const bool ok = k < K && o < a.out;
+                        xr[2 * r + h] = ok ? load_elem(xw + (int64_t)o * K + k) : 0.f;
+                        vr[2 * r + h] = ok && has_v ? load_elem(vw + (int64_t)o * K + k) : 0.f;
+                    }
+                }
+        }
 #pragma unroll
         for (int r = 0; r < TN; ++r)
 #pragma unroll
@@ -104,15 +149,40 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
                 hr[2 * r + h] = k < K && j < a.n_r ? __ldg(hin + (int64_t)j * K + k) : 0.f;
             }
     };
-    auto store = [&](int b) {
-        float *ws = smem_dyn + b * (kLRows + BN) * kLPitch, *hs = ws + kLRows * kLPitch;
+    auto store = [&](int b, int kt) {
+        float *ws = smem_dyn + b * (kRows + BN) * kLPitch, *hs = ws + kRows * kLPitch;
+        if constexpr (VEC) {
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                nrm = fmaf(vr[2 * r + h], vr[2 * r + h], nrm);
-                ws[(warp + 8 * r) * kLPitch + h * 32 + lane] = candidate_param<T>(xr[2 * r + h], vr[2 * r + h], a.gamma);
+            for (int u = 0; u < R / 2; ++u) {
+                const bool ok = kt * kLK + vcol < K && row0 + vrow + 16 * u < a.out;
+                const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 x = ok ? raw_to_float4(xr[u]) : zero, v = ok && has_v ? raw_to_float4(vr[u]) : zero;
+                nrm = fmaf(v.x, v.x, nrm);
+                nrm = fmaf(v.y, v.y, nrm);
+                nrm = fmaf(v.z, v.z, nrm);
+                nrm = fmaf(v.w, v.w, nrm);
+                *reinterpret_cast<float4 *>(ws + (vrow + 16 * u) * kLPitch + vcol) =
+                    make_float4(candidate_param<T>(x.x, v.x, a.gamma), candidate_param<T>(x.y, v.y, a.gamma),
+                                candidate_param<T>(x.z, v.z, a.gamma), candidate_param<T>(x.w, v.w, a.gamma));
             }
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float x, v;
+                    if constexpr (kFree) {
+                        const bool ok = kt * kLK + h * 32 + lane < K && row0 + warp + 8 * r < a.out;
+                        x = ok ? raw_to_float(xr[2 * r + h]) : 0.f;
+                        v = ok && has_v ? raw_to_float(vr[2 * r + h]) : 0.f;
+                    } else {
+                        x = xr[2 * r + h];
+                        v = vr[2 * r + h];
+                    }
+                    nrm = fmaf(v, v, nrm);
+                    ws[(warp + 8 * r) * kLPitch + h * 32 + lane] = candidate_param<T>(x, v, a.gamma);
+                }
+        }
 #pragma unroll
         for (int r = 0; r < TN; ++r)
 #pragma unroll
@@ -121,20 +191,20 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
     const int slices = (K + kLK - 1) / kLK;
     if (rank < slices) {
         load(rank);
-        store(0);
+        store(0, rank);
         __syncthreads();
         int b = 0, run = 0;
         for (int kt = rank; kt < slices; kt += cluster, b ^= 1) {
             const bool more = kt + cluster < slices;
             if (more) load(kt + cluster);
-            const float *ws = smem_dyn + b * (kLRows + BN) * kLPitch + g * 16, *hs = ws + kLRows * kLPitch;
+            const float *ws = smem_dyn + b * (kRows + BN) * kLPitch + g * 16, *hs = ws + kRows * kLPitch;
 #pragma unroll
             for (int k = 0; k < 16; k += 4) {
                 float4 h[TN];
 #pragma unroll
                 for (int n = 0; n < TN; ++n) h[n] = *reinterpret_cast<const float4 *>(hs + (ty + 8 * n) * kLPitch + k);
 #pragma unroll
-                for (int r = 0; r < 8; ++r) {
+                for (int r = 0; r < R; ++r) {
                     const float4 w = *reinterpret_cast<const float4 *>(ws + (tx + 8 * r) * kLPitch + k);
 #pragma unroll
                     for (int n = 0; n < TN; ++n) {
@@ -148,7 +218,7 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
             if (++run == kLRun || !more) {
                 run = 0;
 #pragma unroll
-                for (int r = 0; r < 8; ++r)
+                for (int r = 0; r < R; ++r)
 #pragma unroll
                     for (int n = 0; n < TN; ++n) {
                         tot[r][n] += acc[r][n];
@@ -156,37 +226,38 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
                     }
             }
             if (more) {
-                store(b ^ 1);
+                store(b ^ 1, kt + cluster);
                 __syncthreads();
             }
         }
     }
     // the groups' sums, in group order
     __syncthreads();
-    float *red = smem_dyn;                                           // [kLGroups][kLRows][BN + 1]
+    float *red = smem_dyn;                                           // [kLGroups][kRows][BN + 1]
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int n = 0; n < TN; ++n) red[g * kRed + (tx + 8 * r) * (BN + 1) + ty + 8 * n] = tot[r][n];
     __syncthreads();
-    const int o = row0 + t;
+    constexpr int kStep = kLGroups * 64 / kRows;                     // a thread finishes one row's samples n0, n0 + kStep, ..
+    const int row = R == 8 ? t : tid % kRows, n0 = R == 8 ? g : tid / kRows, o = row0 + row;
     float bx = 0.f, bv = 0.f;
     if (rank == 0 && o < a.out && a.offB >= 0) {
         bx = load_elem(static_cast<const T *>(a.x) + a.offB + o);
         if (has_v) bv = load_elem(vbase + a.offB + o);
     }
-    if (g == 0) nrm = fmaf(bv, bv, nrm);
+    if (n0 == 0) nrm = fmaf(bv, bv, nrm);
     nrm = warp_sum(nrm);
-    float *parts = smem_dyn + kStage;                                // [cluster][kRed + 8], the first block's is used
+    float *parts = smem_dyn + kOwn;                                  // [cluster][kRed + 8], the first block's is used
     if (cluster > 1) {
         __syncwarp();
         asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         const uint32_t dst = cluster_addr(parts + rank * (kRed + 8), 0);
-        for (int n = g; n < BN; n += kLGroups) {
+        for (int n = n0; n < BN; n += kStep) {
             float z = 0.f;
 #pragma unroll
-            for (int u = 0; u < kLGroups; ++u) z += red[u * kRed + t * (BN + 1) + n];
-            cluster_store(dst + 4 * (t * (BN + 1) + n), z);
+            for (int u = 0; u < kLGroups; ++u) z += red[u * kRed + row * (BN + 1) + n];
+            cluster_store(dst + 4 * (row * (BN + 1) + n), z);
         }
         if (lane == 0) cluster_store(dst + 4 * (kRed + warp), nrm);
         cluster_barrier();
@@ -195,13 +266,13 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
         for (int r = 0; r < cluster; ++r) nrm += parts[r * (kRed + 8) + kRed + warp];
     }
     const float bias = candidate_param<T>(bx, bv, a.gamma);
-    for (int n = g; n < BN; n += kLGroups) {
+    for (int n = n0; n < BN; n += kStep) {
         float z = 0.f;
         if (cluster > 1) {
-            for (int r = 0; r < cluster; ++r) z += parts[r * (kRed + 8) + t * (BN + 1) + n];
+            for (int r = 0; r < cluster; ++r) z += parts[r * (kRed + 8) + row * (BN + 1) + n];
         } else {
 #pragma unroll
-            for (int u = 0; u < kLGroups; ++u) z += red[u * kRed + t * (BN + 1) + n];
+            for (int u = 0; u < kLGroups; ++u) z += red[u * kRed + row * (BN + 1) + n];
         }
         if (a.offB >= 0) z += bias;
         if (a.relu) z = relu_keep_nan(z);
@@ -498,11 +569,11 @@ __global__ void __launch_bounds__(256) mlp_loss_kernel(const float *logits, cons
     }
 }
 
-template <typename T, int TN>
-cudaError_t launch_layer_tn(Context &c, const LayerArgs &a, cudaStream_t s) {
+template <typename T, int R, int TN, bool VEC>
+cudaError_t launch_layer_tiles(Context &c, const LayerArgs &a, cudaStream_t s) {
     const int sms = c.sm_count > 0 ? c.sm_count : 148;
     const int sample_tiles = (a.n_r + 8 * TN - 1) / (8 * TN);
-    const int64_t tiles = (int64_t)((a.out + kLRows - 1) / kLRows) * sample_tiles;
+    const int64_t tiles = (int64_t)((a.out + 8 * R - 1) / (8 * R)) * sample_tiles;
     // two blocks fit an SM: with fewer than that, clusters of blocks share a tile's slices, at least two slices a block
     // (evening out a last wave with clusters as well made 190 tiles' kernel 10 % faster and its step 9 % slower)
     int cluster = 1;
@@ -510,29 +581,35 @@ cudaError_t launch_layer_tn(Context &c, const LayerArgs &a, cudaStream_t s) {
     // the limit is the function's, for every handle and thread of the process: the most any call asks for, set once
     static PerDeviceOnce attr_set;
     if (attr_set.need(c.device)) {
-        cudaError_t e = cudaFuncSetAttribute(mlp_layer_kernel<T, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)layer_smem(TN, kMaxCluster));
+        cudaError_t e = cudaFuncSetAttribute(mlp_layer_kernel<T, R, TN, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)layer_smem(R, TN, kMaxCluster));
         if (e != cudaSuccess) return e;
         attr_set.mark(c.device);
     }
     // the sample tiles of the same rows run side by side and find them in L2
-    return launch_clustered(mlp_layer_kernel<T, TN>, cluster, dim3((unsigned)(tiles * cluster), a.m + 1), dim3(kLGroups * 64),
-                            layer_smem(TN, cluster), s, chain_launches(c), a, sample_tiles, cluster);
+    return launch_clustered(mlp_layer_kernel<T, R, TN, VEC>, cluster, dim3((unsigned)(tiles * cluster), a.m + 1), dim3(kLGroups * 64),
+                            layer_smem(R, TN, cluster), s, chain_launches(c), a, sample_tiles, cluster);
 }
 
-template <typename T>
+// samples in tiles of 8 TN: one tile if it holds them all, else the width that pads them least
+template <typename T, bool VEC>
 cudaError_t launch_layer(Context &c, const LayerArgs &a, cudaStream_t s) {
-    // samples in tiles of 8 TN: one tile if it holds them all, else the width that pads them least
+    if (a.out <= kLFewRows) {
+        if (a.n_r <= 8) return launch_layer_tiles<T, 4, 1, VEC>(c, a, s);
+        if (a.n_r <= 16) return launch_layer_tiles<T, 4, 2, VEC>(c, a, s);
+        if (a.n_r <= 32) return launch_layer_tiles<T, 4, 4, VEC>(c, a, s);
+        return launch_layer_tiles<T, 4, 8, VEC>(c, a, s);
+    }
     const bool by24 = a.n_r > 32 && (a.n_r + 23) / 24 <= (a.n_r + 31) / 32;
-    if (a.n_r <= 8) return launch_layer_tn<T, 1>(c, a, s);
-    if (a.n_r <= 16) return launch_layer_tn<T, 2>(c, a, s);
-    if (a.n_r <= 24 || by24) return launch_layer_tn<T, 3>(c, a, s);
-    return launch_layer_tn<T, 4>(c, a, s);
+    if (a.n_r <= 8) return launch_layer_tiles<T, 8, 1, VEC>(c, a, s);
+    if (a.n_r <= 16) return launch_layer_tiles<T, 8, 2, VEC>(c, a, s);
+    if (a.n_r <= 24 || by24) return launch_layer_tiles<T, 8, 3, VEC>(c, a, s);
+    return launch_layer_tiles<T, 8, 4, VEC>(c, a, s);
 }
 
 }  // namespace
 
-int mlp_norm_slots(int out) { return (out + kLRows - 1) / kLRows * (kLGroups * 2); }
+int mlp_norm_slots(int out) { return (out + 63) / 64 * (kLGroups * 2); }      // a slot per warp of every row tile
 
 // The cross-entropy can ride on the last layer's launch when one block sees all of a model's
 // logits: every output row in one block, every sample in one tile.
@@ -585,8 +662,9 @@ cudaError_t launch_mlp_layer(Context &c, const LayerArgs &a, bool aligned, cudaS
             return aligned ? launch_head<__nv_bfloat16, true>(c, a, s) : launch_head<__nv_bfloat16, false>(c, a, s);
         return aligned ? launch_head<float, true>(c, a, s) : launch_head<float, false>(c, a, s);
     }
-    if (c.desc.param_dtype == ZENO_BF16) return launch_layer<__nv_bfloat16>(c, a, s);
-    return launch_layer<float>(c, a, s);
+    if (c.desc.param_dtype == ZENO_BF16)
+        return aligned ? launch_layer<__nv_bfloat16, true>(c, a, s) : launch_layer<__nv_bfloat16, false>(c, a, s);
+    return aligned ? launch_layer<float, true>(c, a, s) : launch_layer<float, false>(c, a, s);
 }
 
 // enough blocks to spread a large batch of wide logits over the SMs

@@ -96,6 +96,22 @@ def test_layers_of_unaligned_rows(oracle, dims, n_r, m, dtype, bias):
     P.run_step_parity(oracle, w)
 
 
+# the same kernel on rows aligned to four elements (four columns a load), and with half its rows a tile (layers of up to 32
+# rows, up to 64 samples a tile): columns that end inside a slice and inside a load's reach, one and several slices, one
+# row, 32 and 33, every compiled number of samples, clusters
+@pytest.mark.parametrize("dims,n_r,m", [((4, 36, 4), 1, 3), ((68, 100, 4), 8, 4), ((324, 148, 100), 16, 5), ((260, 68, 36), 24, 21),
+                                        ((132, 132, 64), 33, 20), ((516, 4, 4), 9, 7), ((1028, 32, 4), 65, 5), ((60, 28, 8), 64, 30),
+                                        ((2052, 12, 4), 31, 4)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("pad", [0, 1])
+def test_layers_of_rows_aligned_to_four(oracle, dims, n_r, m, dtype, pad):
+    d = syn.param_count("mlp", dims, True)
+    assert d % 4 == 0                                   # pad = 0: the aligned kernel, 1: that for any rows
+    b = m // 3
+    w = syn.make_config(2, dims=dims, n_r=n_r, m=m, b=b, dtype=dtype, ldv=d + pad, faults=[(b, "signflip")])
+    P.run_step_parity(oracle, w)
+
+
 def test_small_last_layer_with_huge_logits(oracle):
     """Noise candidates of a deep model whose logits reach 1e10, where neighbouring binary32 values are 1,024 apart:
     their losses stay finite and they are dropped."""

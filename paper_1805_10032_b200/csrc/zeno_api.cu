@@ -530,13 +530,11 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     c->spin_limit = zeno::kSpinLimit;
 
     DeviceGuard guard(device);
-    cudaDeviceProp prop;
-    cudaError_t e = guard.err != cudaSuccess ? guard.err : cudaGetDeviceProperties(&prop, device);
+    cudaError_t e = guard.err != cudaSuccess ? guard.err : cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) {
         delete c;
         return ZENO_ERR_CUDA;
     }
-    c->sm_count = prop.multiProcessorCount;
 
     const size_t rows = (size_t)m_max + 1;
     size_t act_elems = 0, norm_elems = 0, lsq_elems = 0, tc_elems = 0, ticket_elems = 1, split_elems = 0;

@@ -112,6 +112,13 @@ int64_t zeno_param_count(const zeno_model_desc *desc);
  * workspace for up to m_max candidates and n_r_max server samples.
  * INVALID_ARG: NULL arguments, m_max outside [1, ZENO_MAX_CANDIDATES], n_r_max < 1,
  * bad layer sizes.  UNSUPPORTED: unknown kind/dtype, least squares with bfloat16.
+ * Device memory of a convolutional network (S_l: side of the planes layer l reads, flat: inputs of the dense layer),
+ * about: 4 (m_max + 1) n_r_max (flat + classes) bytes, and for the convolutional layers, per model and sample,
+ * 8 sum_{l>1} C_{l-1} (S_l + 1)^2 + 4 max_{l even} C_l (S_l + 1)^2 bytes -- for as many of the m_max + 1 models as 4 GiB
+ * hold (at least one); more are taken in groups.  (32 x 32 x 3 -> 32, 32, 64, 64: 0.66 MB a model and sample; a few MB
+ * a model for its weights and the lines' ends.)  With no room for that, or with the environment variable
+ * ZENO_DISABLE_TENSOR_CORES set, the layers run on the CUDA cores, in 8 (m_max + 1) n_r_max max_l C_l S^2 bytes (S: the
+ * side after the layer's pooling).
  * WORKSPACE / CUDA: allocation failed (the handle is not created). */
 zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m_max,
                         int32_t n_r_max, int32_t device);

@@ -633,7 +633,6 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
         bytes += round_up(elems * esz, kAlign);
         return at;
     };
-    const size_t at_act0 = reserve(act_elems, 4), at_act1 = reserve(act_elems, 4);
     const size_t at_norm = reserve(norm_elems, 4), at_lsq = reserve(lsq_elems, 4);
     const size_t at_loss = reserve(rows, 4), at_norms = reserve(m_max, 4);
     const size_t at_scores = reserve(m_max, 4), at_idx = reserve(m_max, 4);
@@ -646,15 +645,27 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     const size_t krum_elems = m_max <= ZENO_KRUM_MAX_M ? zeno::krum_part_floats(m_max, c->krum_blocks) : 0;
     const size_t at_krum = reserve(krum_elems, 4), at_krums = reserve(m_max, 4);
 
-    // last, because a handle can do without it: with no room for it the convolutional layers run on the CUDA cores
-    const size_t without_cnn = bytes;
-    const size_t at_cnn = reserve((size_t)c->cnn_net.floats, 4);
-
-    e = cudaMalloc(&c->arena, bytes);
-    if (e != cudaSuccess && c->cnn_net.layers) {
-        cudaGetLastError();
-        c->cnn_net.layers = 0;
-        e = cudaMalloc(&c->arena, without_cnn);
+    // Last what depends on where convolutional layers run: on the tensor cores, in a workspace of their own, beside which
+    // only the dense layer's input and the logits are kept; with no room for that, on the CUDA cores, between two buffers
+    // of the widest layer's size like any other model's layers.
+    const size_t without_acts = bytes;
+    size_t at_act[2], at_cnn = 0;
+    e = cudaErrorMemoryAllocation;
+    if (c->cnn_net.layers) {
+        const int lc = desc->n_layers - 1;
+        at_act[(lc - 1) & 1] = reserve(rows * (size_t)n_r_max * (size_t)c->cnn_flat, 4);
+        at_act[lc & 1] = reserve(rows * (size_t)n_r_max * (size_t)desc->dims[lc + 2], 4);
+        at_cnn = reserve((size_t)c->cnn_net.floats, 4);
+        e = cudaMalloc(&c->arena, bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            c->cnn_net.layers = 0;
+        }
+    }
+    if (!c->cnn_net.layers) {
+        bytes = without_acts;
+        for (size_t &at : at_act) at = reserve(act_elems, 4);
+        e = cudaMalloc(&c->arena, bytes);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -662,8 +673,7 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
         return ZENO_ERR_WORKSPACE;
     }
     char *base = static_cast<char *>(c->arena);
-    c->act[0] = reinterpret_cast<float *>(base + at_act0);
-    c->act[1] = reinterpret_cast<float *>(base + at_act1);
+    for (int i = 0; i < 2; ++i) c->act[i] = reinterpret_cast<float *>(base + at_act[i]);
     c->normpart = reinterpret_cast<float *>(base + at_norm);
     c->lsq_part = reinterpret_cast<float *>(base + at_lsq);
     c->losses = reinterpret_cast<float *>(base + at_loss);

@@ -398,7 +398,8 @@ struct CnnPackArgs {
     const float *features;
     float *in0;                    // [2][groups][px][4]
     int64_t px;
-    int lead, side, planes, groups, n_r, layers, weight_blocks;
+    int lead, side, planes, groups, n_r, weight_blocks;
+    int first_model;               // of this launch; the workspace counts from it
     float *normpart;
     int np_slots;
     CnnPackLayer layer[ZENO_MAX_LAYERS];
@@ -439,10 +440,10 @@ __global__ void __launch_bounds__(256) cnn_pack_kernel(const __grid_constant__ C
     int li = 0, blk = blockIdx.x;
     while (blk >= a.layer[li].blocks) blk -= a.layer[li++].blocks;
     const CnnPackLayer &L = a.layer[li];
-    const int c = blockIdx.y;
-    const bool has_v = c > 0;
+    const int c = blockIdx.y, model = a.first_model + c;
+    const bool has_v = model > 0;
     const T *xp = static_cast<const T *>(a.x);
-    const T *vp = static_cast<const T *>(a.V) + (has_v ? (int64_t)(c - 1) * a.ldv : 0);
+    const T *vp = static_cast<const T *>(a.V) + (has_v ? (int64_t)(model - 1) * a.ldv : 0);
     float nrm = 0.f;
     // consecutive threads: the four planes of a group, then the output planes, so that the stores are contiguous
     for (int t = tid; t < (L.cin + 3) / 4 * 64; t += 256) {
@@ -483,7 +484,7 @@ __global__ void __launch_bounds__(256) cnn_pack_kernel(const __grid_constant__ C
     if (has_v) {                                                 // one slot per warp
 #pragma unroll
         for (int s = 16; s >= 1; s >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, s);
-        if ((tid & 31) == 0) a.normpart[(int64_t)(c - 1) * a.np_slots + L.np_base + blk * 8 + (tid >> 5)] = nrm;
+        if ((tid & 31) == 0) a.normpart[(int64_t)(model - 1) * a.np_slots + L.np_base + blk * 8 + (tid >> 5)] = nrm;
     }
 }
 
@@ -544,8 +545,9 @@ cudaError_t launch_conv(Context &c, const CnnTcArgs &a, int nb, int blocks, size
 
 }  // namespace
 
-// Sizes of layer l of a handle's network, and where its parts lie in the workspace (floats from its start).
-void cnn_tc_layout(const Context &c, CnnTcNet *net) {
+// Sizes of the layers of a handle's network, and where their parts lie in a workspace for `models` models (floats from
+// its start).
+static void layout_models(const Context &c, int models, CnnTcNet *net) {
     const zeno_model_desc &d = c.desc;
     const int lc = d.n_layers - 1;
     const bool bf16 = d.param_dtype == ZENO_BF16;
@@ -558,6 +560,7 @@ void cnn_tc_layout(const Context &c, CnnTcNet *net) {
     int side = (int)d.dims[0];
     int64_t z_most = 0;
     net->layers = lc;
+    net->models = models;
     for (int l = 0; l < lc; ++l) {
         CnnTcLayer &L = net->layer[l];
         L.side = side;
@@ -575,19 +578,37 @@ void cnn_tc_layout(const Context &c, CnnTcNet *net) {
         L.lead = side + 2;
         L.px = L.lead + (int64_t)(c.n_r_max + 1) * (side + 1) * (side + 1) + kCTiles * 128 + side + 3;
         L.in_model = 2 * (int64_t)L.groups * L.px * 4;
-        L.in = take(L.in_model * (l == 0 ? 1 : c.m_max + 1));
+        L.in = take(L.in_model * (l == 0 ? 1 : models));
         L.w_model = (int64_t)L.nblk * L.stages * L.nks * 2 * L.rows * 4;
-        L.w = take(L.w_model * (c.m_max + 1));
+        L.w = take(L.w_model * models);
         L.bias_model = (int64_t)L.nblk * L.n;
-        L.bias = take(L.bias_model * (c.m_max + 1));
+        L.bias = take(L.bias_model * models);
         if (L.pool) {
-            const int64_t z = (int64_t)(L.cout + 3) / 4 * L.px * 4 * (c.m_max + 1);
+            const int64_t z = (int64_t)(L.cout + 3) / 4 * L.px * 4 * models;
             if (z > z_most) z_most = z;
             side /= 2;
         }
     }
     net->z = take(z_most);
     net->floats = off;
+}
+
+// As many models as 4 GiB hold, at least one, so that a large handle leaves the memory to the caller's candidates: 101
+// models of 32 x 32 x 3 -> 32, 32, 64, 64 with 128 samples would take 8.4 GB (the CUDA-core layers' buffers: 3.4).  A
+// group's uneven last wave and the gaps between its kernels are what it costs: their step takes 6.66 ms in two groups,
+// with 512 MiB and groups of six models 7.76.
+constexpr int64_t kCWorkspaceFloats = (int64_t)1 << 30;
+void cnn_tc_layout(const Context &c, CnnTcNet *net) {
+    layout_models(c, c.m_max + 1, net);
+    if (net->floats <= kCWorkspaceFloats) return;
+    CnnTcNet one, two;
+    layout_models(c, 1, &one);
+    layout_models(c, 2, &two);
+    const int64_t more = (kCWorkspaceFloats - one.floats) / (two.floats - one.floats);
+    const int most = more < 0 ? 1 : 1 + (int)more;
+    if (most > c.m_max) return;
+    const int groups = (c.m_max + most) / most;                      // of evenly many models
+    layout_models(c, (c.m_max + groups) / groups, net);
 }
 
 cudaError_t launch_cnn_tc(Context &c, const CnnTcNet &net, const void *x, const void *V, int64_t ldv, const float *features,
@@ -607,7 +628,6 @@ cudaError_t launch_cnn_tc(Context &c, const CnnTcNet &net, const void *x, const 
     p.planes = net.layer[0].cin;
     p.groups = net.layer[0].groups;
     p.n_r = n_r;
-    p.layers = net.layers;
     p.normpart = c.normpart;
     p.np_slots = c.np_slots;
     for (int l = 0; l < net.layers; ++l) {
@@ -631,80 +651,89 @@ cudaError_t launch_cnn_tc(Context &c, const CnnTcNet &net, const void *x, const 
         p.weight_blocks += q.blocks;
     }
     const int64_t batch = (int64_t)n_r * p.groups * p.side * p.side;
-    int fx = (int)((batch + 256LL * (m + 1) - 1) / (256LL * (m + 1)));
-    const int fx_cap = 8 * sms / (m + 1) + 1;
-    if (fx > fx_cap) fx = fx_cap;
-    ++*launches;
-    profile_mark(c, "cnn_conv3x3", s);          // with the first layer
-    const dim3 pack_grid(p.weight_blocks + fx, m + 1);
-    cudaError_t e = bf16 ? launch_chained(cnn_pack_kernel<__nv_bfloat16>, pack_grid, dim3(256), 0, s, chain_launches(c), p)
-                         : launch_chained(cnn_pack_kernel<float>, pack_grid, dim3(256), 0, s, chain_launches(c), p);
-    if (e != cudaSuccess) return e;
-    for (int l = 0; l < net.layers; ++l) {
-        const CnnTcLayer &L = net.layer[l];
-        const CnnTcLayer *next = l + 1 < net.layers ? &net.layer[l + 1] : nullptr;
-        CnnTcArgs a = {};
-        a.in = c.cnn_ws + L.in;
-        a.in_model = l == 0 ? 0 : L.in_model;
-        a.px = L.px;
-        a.w = c.cnn_ws + L.w;
-        a.bias = c.cnn_ws + L.bias;
-        a.w_model = L.w_model;
-        a.bias_model = L.bias_model;
-        a.pool = L.pool;
-        const int z_groups = (L.cout + 3) / 4;
-        if (L.pool) {
-            a.out = c.cnn_ws + net.z;
-            a.out_model = (int64_t)z_groups * L.px * 4;
-            a.out_px = L.px;
-            a.out_groups = z_groups;
-            a.out_lead = L.lead;
-        } else {
-            a.out = c.cnn_ws + next->in;
-            a.out_model = next->in_model;
-            a.out_px = next->px;
-            a.out_groups = next->groups;
-            a.out_lead = next->lead;
+    const CnnTcLayer &last = net.layer[net.layers - 1];
+    const int64_t flat_model = (int64_t)n_r * last.cout * (last.side / 2) * (last.side / 2);
+    for (int first = 0; first <= m; first += net.models) {
+        const int models = std::min(net.models, m + 1 - first);
+        int fx = 0;                                  // the batch is packed once, with the first group's weights
+        if (first == 0) {
+            fx = (int)((batch + 256LL * models - 1) / (256LL * models));
+            const int fx_cap = 8 * sms / models + 1;
+            if (fx > fx_cap) fx = fx_cap;
         }
-        a.groups = L.groups;
-        a.stages_per_item = L.stages;
-        a.debias = bf16 ? 3.2e-8f : 6.1e-8f;              // for kCDrain steps, see the top of the file
-        a.nblk = L.nblk;
-        a.side = L.side;
-        a.n_r = n_r;
-        a.models = m + 1;
-        a.tiles = (int)(((int64_t)n_r * (L.side + 1) * (L.side + 1) + 127) / 128);
-        a.tile_pairs = (a.tiles + kCTiles - 1) / kCTiles;
-        a.lead = L.lead;
-        a.plane_bytes = (kCTiles * 128 + 2 * (L.side + 2) + 1) * 16;      // the paired taps of a first layer reach one further
-        a.a_bytes = (L.first ? 2 : 4) * a.plane_bytes;
-        a.b_bytes = L.nks * 2 * L.rows * 16;
-        a.stage_bytes = round_up_int(a.a_bytes + a.b_bytes, 128);
-        a.ring = (kCSmem - 1024) / a.stage_bytes;
-        if (a.ring > kCMaxStages) a.ring = kCMaxStages;
-        a.status = c.dev_status;
-        a.spin_limit = c.spin_limit;
-        const int items = a.models * a.nblk * a.tile_pairs;
-        const int rounds = (items + sms - 1) / sms, blocks = (items + rounds - 1) / rounds;
+        p.first_model = first;
         ++*launches;
-        if (l > 0) profile_mark(c, "cnn_conv3x3", s);
-        // more than half of an SM's shared memory, so that no SM holds two of the kernel's blocks, of which the second would
-        // wait for the first one's tensor memory while other SMs idle (two layers of 16 planes, 640 images: 59 us against 51)
-        const size_t smem = std::max((size_t)a.ring * a.stage_bytes, (size_t)116 * 1024);
-        e = bf16 ? (L.first ? launch_conv<true, true>(c, a, L.n / 16, blocks, smem, s) : launch_conv<true, false>(c, a, L.n / 16, blocks, smem, s))
-                 : (L.first ? launch_conv<false, true>(c, a, L.n / 16, blocks, smem, s) : launch_conv<false, false>(c, a, L.n / 16, blocks, smem, s));
+        profile_mark(c, "cnn_conv3x3", s);          // with the first layer
+        const dim3 pack_grid(p.weight_blocks + fx, models);
+        cudaError_t e = bf16 ? launch_chained(cnn_pack_kernel<__nv_bfloat16>, pack_grid, dim3(256), 0, s, chain_launches(c), p)
+                             : launch_chained(cnn_pack_kernel<float>, pack_grid, dim3(256), 0, s, chain_launches(c), p);
         if (e != cudaSuccess) return e;
-        if (!L.pool) continue;
-        const int total = n_r * z_groups * (L.side / 2) * (L.side / 2);
-        int bx = (total + 255) / 256;
-        const int cap = 16 * sms / (m + 1) + 1;
-        if (bx > cap) bx = cap;
-        ++*launches;
-        e = launch_chained(cnn_pool_kernel, dim3(bx, m + 1), dim3(256), 0, s, chain_launches(c), (const float *)a.out, a.out_model,
-                           a.out_px, L.lead, L.side, L.cout, z_groups, n_r, next ? c.cnn_ws + next->in : nullptr,
-                           next ? next->in_model : 0, next ? next->px : 0, next ? next->groups : 0, next ? next->lead : 0,
-                           next ? nullptr : flat);
-        if (e != cudaSuccess) return e;
+        for (int l = 0; l < net.layers; ++l) {
+            const CnnTcLayer &L = net.layer[l];
+            const CnnTcLayer *next = l + 1 < net.layers ? &net.layer[l + 1] : nullptr;
+            CnnTcArgs a = {};
+            a.in = c.cnn_ws + L.in;
+            a.in_model = l == 0 ? 0 : L.in_model;
+            a.px = L.px;
+            a.w = c.cnn_ws + L.w;
+            a.bias = c.cnn_ws + L.bias;
+            a.w_model = L.w_model;
+            a.bias_model = L.bias_model;
+            a.pool = L.pool;
+            const int z_groups = (L.cout + 3) / 4;
+            if (L.pool) {
+                a.out = c.cnn_ws + net.z;
+                a.out_model = (int64_t)z_groups * L.px * 4;
+                a.out_px = L.px;
+                a.out_groups = z_groups;
+                a.out_lead = L.lead;
+            } else {
+                a.out = c.cnn_ws + next->in;
+                a.out_model = next->in_model;
+                a.out_px = next->px;
+                a.out_groups = next->groups;
+                a.out_lead = next->lead;
+            }
+            a.groups = L.groups;
+            a.stages_per_item = L.stages;
+            a.debias = bf16 ? 3.2e-8f : 6.1e-8f;              // for kCDrain steps, see the top of the file
+            a.nblk = L.nblk;
+            a.side = L.side;
+            a.n_r = n_r;
+            a.models = models;
+            a.tiles = (int)(((int64_t)n_r * (L.side + 1) * (L.side + 1) + 127) / 128);
+            a.tile_pairs = (a.tiles + kCTiles - 1) / kCTiles;
+            a.lead = L.lead;
+            a.plane_bytes = (kCTiles * 128 + 2 * (L.side + 2) + 1) * 16;      // the paired taps of a first layer reach one further
+            a.a_bytes = (L.first ? 2 : 4) * a.plane_bytes;
+            a.b_bytes = L.nks * 2 * L.rows * 16;
+            a.stage_bytes = round_up_int(a.a_bytes + a.b_bytes, 128);
+            a.ring = (kCSmem - 1024) / a.stage_bytes;
+            if (a.ring > kCMaxStages) a.ring = kCMaxStages;
+            a.status = c.dev_status;
+            a.spin_limit = c.spin_limit;
+            const int items = a.models * a.nblk * a.tile_pairs;
+            const int rounds = (items + sms - 1) / sms, blocks = (items + rounds - 1) / rounds;
+            ++*launches;
+            if (l > 0) profile_mark(c, "cnn_conv3x3", s);
+            // more than half of an SM's shared memory, so that no SM holds two of the kernel's blocks, of which the second would
+            // wait for the first one's tensor memory while other SMs idle (two layers of 16 planes, 640 images: 59 us against 51)
+            const size_t smem = std::max((size_t)a.ring * a.stage_bytes, (size_t)116 * 1024);
+            e = bf16 ? (L.first ? launch_conv<true, true>(c, a, L.n / 16, blocks, smem, s) : launch_conv<true, false>(c, a, L.n / 16, blocks, smem, s))
+                     : (L.first ? launch_conv<false, true>(c, a, L.n / 16, blocks, smem, s) : launch_conv<false, false>(c, a, L.n / 16, blocks, smem, s));
+            if (e != cudaSuccess) return e;
+            if (!L.pool) continue;
+            const int total = n_r * z_groups * (L.side / 2) * (L.side / 2);
+            int bx = (total + 255) / 256;
+            const int cap = 16 * sms / models + 1;
+            if (bx > cap) bx = cap;
+            ++*launches;
+            e = launch_chained(cnn_pool_kernel, dim3(bx, models), dim3(256), 0, s, chain_launches(c), (const float *)a.out, a.out_model,
+                               a.out_px, L.lead, L.side, L.cout, z_groups, n_r, next ? c.cnn_ws + next->in : nullptr,
+                               next ? next->in_model : 0, next ? next->px : 0, next ? next->groups : 0, next ? next->lead : 0,
+                               next ? nullptr : flat + first * flat_model);
+            if (e != cudaSuccess) return e;
+        }
     }
     return cudaSuccess;
 }

@@ -46,6 +46,7 @@ struct CnnTcLayer {
 };
 struct CnnTcNet {
     int layers;              // 0: the layers run on the CUDA cores
+    int models;              // models the workspace holds: a call with more takes them in groups
     int64_t z, floats;
     CnnTcLayer layer[ZENO_MAX_LAYERS];
 };

@@ -65,6 +65,27 @@ def test_fewer_samples_and_candidates_than_the_handle_was_made_for(oracle):
         assert all(torch.equal(a, b) for a, b in zip(got, want))
 
 
+def test_models_in_groups():
+    """More models than the convolutional workspace holds (4 GiB) are taken in groups: every candidate's loss, norm and
+    score as a handle for fewer candidates gives them; and what the two handles take of the device's memory."""
+    w = syn.make_config(6, dims=(32, 3, 32, 32, 10), m=99, b=4, n_r=128, faults=[(4, "signflip")])
+    x, V, f, t = P.to_device(w)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    with zeno.from_workload(w) as z, zeno.Zeno(zeno.LOSS_SOFTMAX_CNN, zeno.F32, w.dims, True, 25, 128) as few:
+        used = free - torch.cuda.mem_get_info()[0]
+        scores, losses, norms = z.score(x, V, f, t, w.gamma, w.rho)
+        for i in range(0, 99, 25):
+            part = few.score(x, V[i:i + 25], f, t, w.gamma, w.rho)
+            # the dense layer deals its 8,192 inputs out to more blocks where there are fewer models: other partial sums
+            for got, want in zip(part, (scores[i:i + 25], torch.cat([losses[:1], losses[1 + i:26 + i]]), norms[i:i + 25])):
+                assert torch.allclose(got, want, rtol=2e-6, atol=0)
+        z.check_device_status()
+    # all models at once: 5.3 GB and 1.4 GB, beside them 0.5 GB of the dense layer's input
+    assert used < 4 * 2 ** 30 + 2.1e9, used
+
+
 # the first pixel of a sample is read, with zero weights, by the paired taps of the sample before it (one to four input
 # planes); five planes: no paired taps
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])

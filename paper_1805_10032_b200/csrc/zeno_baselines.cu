@@ -15,8 +15,6 @@ namespace zeno {
 
 namespace {
 
-__device__ __forceinline__ float nan_to_inf(float v) { return v != v ? INFINITY : v; }
-
 // ---- Krum -----------------------------------------------------------------------------------
 
 constexpr int kKrumThreads = 256;

@@ -446,6 +446,9 @@ __device__ __forceinline__ void cluster_store(uint32_t addr, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
+// the baseline rules' reading of a NaN entry
+__device__ __forceinline__ float nan_to_inf(float v) { return v != v ? INFINITY : v; }
+
 // ReLU that lets a NaN through
 __device__ __forceinline__ float relu_keep_nan(float z) { return (z > 0.f || z != z) ? z : 0.f; }
 

@@ -28,8 +28,6 @@ constexpr int kMedianTwoColsHalf = 6;         // bfloat16: halves up to which a 
 
 __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }
 
-__device__ __forceinline__ float nan_to_inf(float v) { return v != v ? INFINITY : v; }
-
 // What a register of the one-thread kernel holds: one column in binary32, or two bfloat16 columns.
 template <typename T>
 struct OneCol {

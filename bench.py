@@ -65,14 +65,14 @@ def measured_peaks():
 # scaled by the parameters processed (reads x 16, the slab writes as they are).
 _CSRC = "paper_1805_10032_b200/csrc/"
 NCU_TRAFFIC = {
-    ("0:lsq_tc", 5): {"bytes": 2.1751e+10, "sources": ["zeno_lsq_tc.cu", "zeno_tc.cuh"], "sha256_16": "1f142f64bf1a0db1"},
+    ("0:lsq_tc", 5): {"bytes": 2.1751e+10, "sources": ["zeno_lsq_tc.cu", "zeno_tc.cuh"], "sha256_16": "5f290bc1cb436ea1"},
     ("1:layer_tc", 4): {"bytes": 1.4225e+09, "sources": ["zeno_layer_tc.cu", "zeno_tc.cuh"], "sha256_16": "f0b30a6b2bae6de9"},
     ("2:layer_tc", 4): {"bytes": 1.4892e+09, "sources": ["zeno_layer_tc.cu", "zeno_tc.cuh"], "sha256_16": "f0b30a6b2bae6de9"},
     ("3:layer_tc", 4): {"bytes": 3.6208e+08, "sources": ["zeno_layer_tc.cu", "zeno_tc.cuh"], "sha256_16": "f0b30a6b2bae6de9"},
     ("5:aggregate", 4): {"bytes": 1.6506e+09, "sources": ["zeno_aggregate.cu"], "sha256_16": "d4ebd34a19b63638"},
     ("1:layer_tc", 3): {"bytes": 6.5876e+08, "sources": ["zeno_layer_tc.cu", "zeno_tc.cuh"], "sha256_16": "f0b30a6b2bae6de9"},
     ("3:layer_tc", 3): {"bytes": 1.3774e+08, "sources": ["zeno_layer_tc.cu", "zeno_tc.cuh"], "sha256_16": "f0b30a6b2bae6de9"},
-    ("0:stream_tf32x3", 2): {"bytes": 1.3695e+08, "sources": ["zeno_stream_tc.cu", "zeno_tc.cuh"], "sha256_16": "bfb9d41675540c43"},
+    ("0:stream_tf32x3", 2): {"bytes": 1.3695e+08, "sources": ["zeno_stream_tc.cu", "zeno_tc.cuh"], "sha256_16": "29cebb6ae28093f2"},
     ("2:layer_tc_head", 2): {"bytes": 2.5343e+07, "sources": ["zeno_layer_tc.cu", "zeno_tc.cuh"], "sha256_16": "f0b30a6b2bae6de9"},
 }
 

@@ -70,7 +70,6 @@ inline size_t layer_smem(int R, int TN, int cluster) {
 template <typename T> struct RawOf;
 template <> struct RawOf<float> { using One = float; using Four = float4; };
 template <> struct RawOf<__nv_bfloat16> { using One = unsigned short; using Four = uint2; };
-__device__ __forceinline__ float raw_to_float(float v) { return v; }
 __device__ __forceinline__ float raw_to_float(unsigned short v) { return bf16_bits_to_float(v); }
 __device__ __forceinline__ float4 raw_to_float4(float4 v) { return v; }
 __device__ __forceinline__ float4 raw_to_float4(uint2 v) {
@@ -598,6 +597,7 @@ cudaError_t launch_layer(Context &c, const LayerArgs &a, cudaStream_t s) {
         if (a.n_r <= 8) return launch_layer_tiles<T, 4, 1, VEC>(c, a, s);
         if (a.n_r <= 16) return launch_layer_tiles<T, 4, 2, VEC>(c, a, s);
         if (a.n_r <= 32) return launch_layer_tiles<T, 4, 4, VEC>(c, a, s);
+        if (a.n_r <= 48) return launch_layer_tiles<T, 4, 3, VEC>(c, a, s);
         return launch_layer_tiles<T, 4, 8, VEC>(c, a, s);
     }
     const bool by24 = a.n_r > 32 && (a.n_r + 23) / 24 <= (a.n_r + 31) / 32;

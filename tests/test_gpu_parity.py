@@ -100,7 +100,7 @@ def test_layers_of_unaligned_rows(oracle, dims, n_r, m, dtype, bias):
 # rows, up to 64 samples a tile): columns that end inside a slice and inside a load's reach, one and several slices, one
 # row, 32 and 33, every compiled number of samples, clusters
 @pytest.mark.parametrize("dims,n_r,m", [((4, 36, 4), 1, 3), ((68, 100, 4), 8, 4), ((324, 148, 100), 16, 5), ((260, 68, 36), 24, 21),
-                                        ((132, 132, 64), 33, 20), ((516, 4, 4), 9, 7), ((1028, 32, 4), 65, 5), ((60, 28, 8), 64, 30),
+                                        ((132, 132, 64), 33, 20), ((516, 4, 4), 9, 7), ((136, 20, 4), 33, 20), ((1028, 32, 4), 65, 5), ((60, 28, 8), 64, 30),
                                         ((2052, 12, 4), 31, 4)])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("pad", [0, 1])

@@ -17,103 +17,188 @@ namespace {
 
 // ---- Krum -----------------------------------------------------------------------------------
 
-constexpr int kKrumThreads = 256;
-constexpr int kKrumCols = 128;                // columns staged per tile
-constexpr int kKrumPitch = kKrumCols + 1;     // row pitch in floats: rows of a tile start in different banks
+// The rows are taken in blocks of B, their number rounded up to even, and a warp holds one tile of pairs in registers: B x B
+// pairs of two different blocks, or the 2 x B (B - 1) / 2 pairs inside the blocks 2 w and 2 w + 1.  A lane owns a column: it
+// reads 2 B values of a staged tile of columns (neighbouring lanes, neighbouring words) for up to B x B differences and
+// multiplications, and keeps its sums to the end.  Every tile's lanes take the same columns in the same order, so identical
+// rows get identical distances.  With more tiles than a block has warps, gridDim.y blocks share a stretch of columns, each
+// staging the row blocks its tiles name; with fewer, groups of warps split the columns.
+// The rows come by asynchronous copies, three stages, 16 bytes at a time where rows are aligned, else 4.
+// Bound by issue: of 20 rows a column costs 190 differences and 190 multiplications, 0.74 of the schedulers' slots are taken,
+// 0.6 of them by these.  1.8 M columns: 20 rows 48 us (4 x 4 tiles a thread from shared memory: 104), 64 rows 401 (580), 100 rows
+// 1,080 (1,280).  Two columns an instruction (packed additions and multiplications, blocks of 5 and 7 rows): 54, 810 and 2,240
+// us; the packed instructions take the arithmetic pipe twice as long each.
+constexpr int kKrumThreads = 256, kKrumWarps = kKrumThreads / 32;
+constexpr int kKrumStages = 3;
+constexpr int kKrumBlocksPerSm = 2;
+constexpr int kKrumMaxBlocks = 16;            // row blocks
+constexpr int kKrumMaxTiles = kKrumMaxBlocks * kKrumMaxBlocks / 2;
+constexpr int kKrumPad = 8;                   // entries between staged rows: rows stay aligned to 16 bytes
+constexpr int kKrumMaxRows = 128;             // staged by a block
 
-__host__ __device__ inline int krum_row_blocks(int m) { return (m + 3) / 4; }
-__host__ __device__ inline int krum_tiles(int m) { const int mb = krum_row_blocks(m); return mb * (mb + 1) / 2; }
-// groups of threads that share the pair tiles and split a tile's columns between them
-__host__ __device__ inline int krum_groups(int m) { const int t = krum_tiles(m); return t >= kKrumThreads ? 1 : kKrumThreads / t; }
-// shared memory of the pair kernel: the staged rows, or the groups' sums when those need more
-inline size_t krum_pairs_smem(int m) {
-    const size_t rows = (size_t)krum_row_blocks(m) * 4 * kKrumPitch, red = (size_t)krum_groups(m) * krum_tiles(m) * 16;
-    return (rows > red ? rows : red) * sizeof(float);
+struct KrumPlan {
+    int B, nb;                                // rows of a block, blocks
+    int tiles, ny, per_y;                     // tiles of pairs; blocks that share them; tiles of each
+    unsigned used[kKrumMaxTiles / kKrumWarps];                 // row blocks a block of blocks y reads
+    unsigned char ia[kKrumMaxTiles], ib[kKrumMaxTiles];        // a tile's blocks; diag: the pairs inside them
+    unsigned char diag[kKrumMaxTiles];
+    unsigned char at[kKrumMaxBlocks][kKrumMaxBlocks];          // the tile of two blocks
+};
+
+// columns staged at a time: as many as leave room for two blocks an SM (three stages of 28, 70 and 128 binary32 rows)
+inline int krum_cols(int rows, int entry_bytes) { return rows * entry_bytes <= 28 * 4 ? 256 : rows * entry_bytes <= 70 * 4 ? 128 : 64; }
+
+__device__ __forceinline__ void krum_copy(uint32_t dst, const void *src, bool valid, bool wide) {
+    if (wide)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ float krum_value(const float *p) { return *p; }
+__device__ __forceinline__ float krum_value(const __nv_bfloat16 *p) {
+    return bf16_bits_to_float(*reinterpret_cast<const unsigned short *>(p));
 }
 
-// tile index -> (ib, jb) with ib <= jb, row by row of the upper triangle of blocks of four rows
-__device__ __forceinline__ void krum_tile_of(int tile, int mb, int &ib, int &jb) {
-    ib = 0;
-    int left = tile;
-    while (left >= mb - ib) { left -= mb - ib; ++ib; }
-    jb = ib + left;
-}
-
-// part[block][tile][4][4]: sums of squared differences of the 4 x 4 pairs (i, j) of a tile over the
-// columns this block took.  With fewer tiles than threads, groups of threads split a staged tile's
-// columns and their sums are added in group order before they are written.
-// kMaxMine: pair tiles a thread may hold (1 while the tiles are fewer than the threads; 528 tiles at m = 128
-// over 256 threads need 3).
-template <typename T, int kMaxMine>
-__global__ void __launch_bounds__(kKrumThreads, kMaxMine == 1 ? 4 : 3) krum_pairs_kernel(const T *V, int64_t ldv, int64_t d, int m, float *part) {
-    extern __shared__ float rows[];           // [m rounded up to 4][kKrumPitch], then [groups][tiles][16]
+// part[block][tile][B * B]: sums of squared differences of a tile's pairs over the columns this block took.
+template <typename T, int B, int C, bool WIDE>
+__global__ void __launch_bounds__(kKrumThreads, kKrumBlocksPerSm)
+krum_pairs_kernel(const T *V, int64_t ldv, int64_t d, int m, const __grid_constant__ KrumPlan plan, float *part) {
+    constexpr int kPitch = C + kKrumPad, kPairs = B * (B - 1) / 2;
+    constexpr int E = (WIDE ? 16 : 4) / (int)sizeof(T), kChunks = C / E;          // entries of a copy, copies of a row
+    constexpr bool kHalves = !WIDE && sizeof(T) == 2;             // rows may start in the second half of 4 bytes
+    extern __shared__ __align__(16) uint8_t krum_smem[];
+    __shared__ const T *row_at[kKrumMaxRows];                     // where a staged row's copies start, or NULL
+    __shared__ unsigned char late[kKrumMaxRows];                  // entries of them before the row's first
+    T *stage0 = reinterpret_cast<T *>(krum_smem);
     pdl_wait();
     pdl_launch_dependents();
-    const int mb = krum_row_blocks(m), tiles = krum_tiles(m), groups = krum_groups(m);
-    const int m4 = mb * 4;
-    const int tid = threadIdx.x;
-    const bool shared_tiles = tiles < kKrumThreads;                 // one tile a thread, groups of threads
-    const int group = tid / tiles < groups ? tid / tiles : -1;      // threads beyond groups * tiles idle
-    const int n_mine = shared_tiles ? (group >= 0 ? 1 : 0) : (tiles - tid + kKrumThreads - 1) / kKrumThreads;
-    float acc[kMaxMine][16];
-#pragma unroll
-    for (int q = 0; q < kMaxMine; ++q)
-#pragma unroll
-        for (int e = 0; e < 16; ++e) acc[q][e] = 0.f;
-    for (int64_t j0 = (int64_t)blockIdx.x * kKrumCols; j0 < d; j0 += (int64_t)gridDim.x * kKrumCols) {
-        __syncthreads();
-#pragma unroll 8
-        for (int t = tid; t < m4 * kKrumCols; t += kKrumThreads) {
-            const int r = t / kKrumCols, c = t - r * kKrumCols;
-            rows[r * kKrumPitch + c] = (r < m && j0 + c < d) ? load_elem(V + (int64_t)r * ldv + j0 + c) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < kMaxMine; ++q) {
-            if (q >= n_mine) break;
-            const int tile = shared_tiles ? tid - group * tiles : tid + q * kKrumThreads;
-            int ib, jb;
-            krum_tile_of(tile, mb, ib, jb);
-            const float *ri = rows + ib * 4 * kKrumPitch, *rj = rows + jb * 4 * kKrumPitch;
-            const int c0 = shared_tiles ? group : 0, cs = shared_tiles ? groups : 1;
-#pragma unroll(kMaxMine == 1 ? 4 : 1)
-            for (int c = c0; c < kKrumCols; c += cs) {
-                float a[4], b[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    a[u] = ri[u * kKrumPitch + c];
-                    b[u] = rj[u * kKrumPitch + c];
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) {
-                        const float df = a[u] - b[w];
-                        acc[q][u * 4 + w] = fmaf(df, df, acc[q][u * 4 + w]);
-                    }
-            }
-        }
-    }
-    float *dst = part + (int64_t)blockIdx.x * tiles * 16;
-    if (!shared_tiles) {
-#pragma unroll
-        for (int q = 0; q < kMaxMine; ++q) {
-            if (q >= n_mine) break;
-            float *o = dst + (tid + q * kKrumThreads) * 16;
-#pragma unroll
-            for (int e = 0; e < 16; e += 4) *reinterpret_cast<float4 *>(o + e) = make_float4(acc[q][e], acc[q][e + 1], acc[q][e + 2], acc[q][e + 3]);
-        }
-        return;
-    }
-    __syncthreads();                          // the staged rows are done with: the groups' sums take their place
-    if (group >= 0) {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) rows[tid * 16 + e] = acc[0][e];       // tid = group * tiles + tile
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned used = plan.used[blockIdx.y];
+    const int rows = __popc(used) * B, stage = rows * kPitch;
+    // this warp's tile and its share of the columns
+    const int groups = plan.per_y <= kKrumWarps / 2 ? kKrumWarps / plan.per_y : 1;
+    const int group = warp / plan.per_y, mine = warp - group * plan.per_y, tile = blockIdx.y * plan.per_y + mine;
+    const bool busy = group < groups && tile < plan.tiles;
+    const int ia = busy ? plan.ia[tile] : 0, ib = busy ? plan.ib[tile] : 0;
+    const bool diag = busy && plan.diag[tile];
+    const bool odd_base = kHalves && (reinterpret_cast<uintptr_t>(V) & 2), odd_pitch = kHalves && (ldv & 1);
+    auto half = [&](int row) { return (int)(odd_base != (odd_pitch && (row & 1))); };
+
+    for (int r = threadIdx.x; r < rows; r += kKrumThreads) {
+        unsigned left = used;
+        for (int skip = r / B; skip > 0; --skip) left &= left - 1;
+        const int row = (__ffs(left) - 1) * B + r % B;
+        row_at[r] = row < m ? V + (int64_t)row * ldv - half(row) : nullptr;
+        late[r] = (unsigned char)half(row);
     }
     __syncthreads();
-    for (int t = tid; t < tiles * 16; t += kKrumThreads) {
+    for (int r = warp; r < rows; r += kKrumWarps)                 // rows beyond m are and stay zero
+        if (!row_at[r])
+            for (int s = 0; s < kKrumStages; ++s)
+                for (int c = lane; c < kPitch; c += 32) stage0[s * stage + r * kPitch + c] = T(0.f);
+    const int64_t tiles_c = (d + C - 1) / C;
+    auto load = [&](int64_t ct, int s) {
+        const int64_t j0 = ct * C;
+        const bool last = j0 + C > d;
+        const int q = threadIdx.x % kChunks * E, r0 = threadIdx.x / kChunks;      // kChunks divides the threads
+        uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage0 + s * stage + r0 * kPitch + q);
+        for (int r = r0; r < rows; r += kKrumThreads / kChunks, dst += kKrumThreads / kChunks * kPitch * (int)sizeof(T)) {
+            const T *row = row_at[r];
+            if (!row) continue;
+            const bool ok = !last || j0 + q - (kHalves ? late[r] : 0) < d;         // beyond the columns nothing is read
+            krum_copy(dst, ok ? row + j0 + q : row, ok, WIDE);
+        }
+        if (kHalves && (int)threadIdx.x < rows && late[threadIdx.x]) {             // the last entry of rows that start half a word late
+            const T *row = row_at[threadIdx.x];
+            const bool ok = j0 + C - 1 < d;
+            if (row) krum_copy((uint32_t)__cvta_generic_to_shared(stage0 + s * stage + threadIdx.x * kPitch + C), ok ? row + j0 + C : row, ok, false);
+        }
+    };
+    float acc[B * B];
+#pragma unroll
+    for (int e = 0; e < B * B; ++e) acc[e] = 0.f;
+    // the tile's two blocks of rows within a stage; of bfloat16 rows with an odd pitch every other one starts an entry later
+    const int sa = __popc(used & ((1u << ia) - 1)) * B, sb = __popc(used & ((1u << ib) - 1)) * B;
+    const int a_even = sa * kPitch + half(ia * B), a_odd = sa * kPitch + half(ia * B + 1);
+    const int b_even = sb * kPitch + half(ib * B), b_odd = sb * kPitch + half(ib * B + 1);
+
+    int64_t ct = blockIdx.x;
+    for (int s = 0; s < kKrumStages - 1; ++s) {
+        if (ct + (int64_t)s * gridDim.x < tiles_c) load(ct + (int64_t)s * gridDim.x, s);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    int s = 0;
+    for (; ct < tiles_c; ct += gridDim.x) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kKrumStages - 2) : "memory");
+        __syncthreads();                      // the stage has landed for every thread; the one before is free
+        const int64_t next = ct + (int64_t)(kKrumStages - 1) * gridDim.x;
+        if (next < tiles_c) load(next, s == 0 ? kKrumStages - 1 : s - 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        T *st = stage0 + s * stage;
+        if (ct * C + C > d) {                 // beyond the columns whatever the copies brought counts as zero
+            const int left = (int)(d - ct * C);
+            for (int r = warp; r < rows; r += kKrumWarps)
+                for (int c = left + late[r] + lane; c < kPitch; c += 32) st[r * kPitch + c] = T(0.f);
+            __syncthreads();
+        }
+        if (busy) {
+#pragma unroll 1
+            for (int c = group * 32 + lane; c < C; c += groups * 32) {
+                auto value = [&](int even, int odd, int r) { return krum_value(st + (kHalves && (r & 1) ? odd : even) + r * kPitch + c); };
+                float a[B];
+#pragma unroll
+                for (int r = 0; r < B; ++r) a[r] = value(a_even, a_odd, r);
+                if (!diag) {
+#pragma unroll
+                    for (int q = 0; q < B; ++q) {
+                        const float b = value(b_even, b_odd, q);
+#pragma unroll
+                        for (int r = 0; r < B; ++r) {
+                            const float df = a[r] - b;
+                            acc[q * B + r] = fmaf(df, df, acc[q * B + r]);
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        if (t == 1) {
+#pragma unroll
+                            for (int r = 0; r < B; ++r) a[r] = value(b_even, b_odd, r);
+                        }
+#pragma unroll
+                        for (int q = 1; q < B; ++q)
+#pragma unroll
+                            for (int r = 0; r < q; ++r) {
+                                const float df = a[r] - a[q];
+                                float &sum = acc[t * kPairs + q * (q - 1) / 2 + r];
+                                sum = fmaf(df, df, sum);
+                            }
+                    }
+                }
+            }
+        }
+        if (++s == kKrumStages) s = 0;
+    }
+    // the lanes' sums, 32 pairs at a time (lane l receives pair l of the batch), then the groups'
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    float *red = reinterpret_cast<float *>(krum_smem);             // [group][tile of the block][B * B]
+    if (busy) {
+#pragma unroll
+        for (int e0 = 0; e0 < B * B; e0 += 32) {
+            float v[32];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] = e0 + e < B * B ? acc[e0 + e < B * B ? e0 + e : 0] : 0.f;
+            const float sum = warp_transpose_reduce<32>(v, lane);
+            if (e0 + lane < B * B) red[warp * B * B + e0 + lane] = sum;
+        }
+    }
+    __syncthreads();
+    const int here = min(plan.per_y, plan.tiles - (int)blockIdx.y * plan.per_y) * B * B;
+    float *dst = part + ((int64_t)blockIdx.x * plan.tiles + blockIdx.y * plan.per_y) * (B * B);
+    for (int t = threadIdx.x; t < here; t += kKrumThreads) {
         float sum = 0.f;
-        for (int g = 0; g < groups; ++g) sum += rows[g * tiles * 16 + t];
+        for (int g = 0; g < groups; ++g) sum += red[g * plan.per_y * B * B + t];
         dst[t] = sum;
     }
 }
@@ -123,20 +208,21 @@ __global__ void __launch_bounds__(kKrumThreads, kMaxMine == 1 ? 4 : 3) krum_pair
 // then the sum of the m - b - 2 smallest: a distance belongs to it if fewer than that many others are smaller, or equal
 // and of a lower index.
 constexpr int kSumsWarps = 32;                // one round of entries up to 32 candidates
-__global__ void __launch_bounds__(kSumsWarps * 32) krum_sums_kernel(const float *part, int slabs, int m, int b, float *sums_out, float *sums_ws) {
+__global__ void __launch_bounds__(kSumsWarps * 32) krum_sums_kernel(const float *part, int slabs, int m, int b,
+                                                                    const __grid_constant__ KrumPlan plan, float *sums_out, float *sums_ws) {
     __shared__ float dist[ZENO_KRUM_MAX_M];
     __shared__ double warp_part[kSumsWarps];
     pdl_wait();
     pdl_launch_dependents();
-    const int mb = krum_row_blocks(m), tiles = krum_tiles(m);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x, B = plan.B;
+    const int64_t slab = (int64_t)plan.tiles * B * B;
     for (int j = warp; j < m; j += kSumsWarps) {
-        const int lo = min(i, j), hi = max(i, j), ib = lo >> 2, jb = hi >> 2;
-        const int tile = ib * mb - ib * (ib - 1) / 2 + (jb - ib);
-        const float *src = part + tile * 16 + (lo & 3) * 4 + (hi & 3);
+        const int lo = min(i, j), hi = max(i, j), ia = lo / B, ib = hi / B, r = lo - ia * B, q = hi - ib * B;
+        const int e = ia != ib ? q * B + r : (ia & 1) * (B * (B - 1) / 2) + q * (q - 1) / 2 + r;
+        const float *src = part + (int64_t)plan.at[ia][ib] * B * B + (i == j ? 0 : e);
         double s = 0.0;
-#pragma unroll 8
-        for (int q = lane; q < slabs; q += 32) s += (double)__ldcg(src + (int64_t)q * tiles * 16);
+#pragma unroll 4
+        for (int q = lane; q < slabs; q += 32) s += (double)__ldcg(src + q * slab);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) dist[j] = nan_to_inf((float)s);
@@ -195,33 +281,102 @@ __global__ void __launch_bounds__(256) copy_row_kernel(const T *V, int64_t ldv, 
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < d; j += (int64_t)gridDim.x * blockDim.x) out[j] = load_elem(row + j);
 }
 
+int krum_grid_x(const KrumPlan &p, int sms) {
+    const int x = kKrumBlocksPerSm * sms / p.ny;
+    return x < 1 ? 1 : x;
+}
+
+// Rows in blocks of B: the B that pads m to an even number of blocks with the fewest rows, the largest of those that tie.
+KrumPlan krum_plan(int m) {
+    KrumPlan p = {};
+    int best = 1 << 30;
+    for (int B : {3, 5, 7, 8, 10}) {
+        const int nb = (m + 2 * B - 1) / (2 * B) * 2;
+        if (nb > kKrumMaxBlocks || nb * B > best || (nb > 2 && B < 7)) continue;
+        best = nb * B;
+        p.B = B;
+        p.nb = nb;
+    }
+    p.tiles = p.nb * p.nb / 2;
+    p.ny = (p.tiles + kKrumWarps - 1) / kKrumWarps;
+    p.per_y = (p.tiles + p.ny - 1) / p.ny;
+    // neighbouring tiles share row blocks: two of the one against four of the other
+    int n = 0;
+    for (int i0 = 0; i0 < p.nb; i0 += 2)
+        for (int j0 = 0; j0 < p.nb; j0 += 4)
+            for (int i = i0; i < i0 + 2 && i < p.nb; ++i)
+                for (int j = j0; j < j0 + 4 && j < p.nb; ++j) {
+                    if (i >= j) continue;
+                    const bool diag = j == i + 1 && (i & 1) == 0;              // these two blocks have a tile of either kind
+                    for (int k = 0; k < (diag ? 2 : 1); ++k) {
+                        p.ia[n] = (unsigned char)i;
+                        p.ib[n] = (unsigned char)j;
+                        p.diag[n] = (unsigned char)k;
+                        if (k) p.at[i][i] = p.at[j][j] = (unsigned char)n;
+                        else p.at[i][j] = (unsigned char)n;
+                        p.used[n / p.per_y] |= 1u << i | 1u << j;
+                        ++n;
+                    }
+                }
+    return p;
+}
+
+template <typename T, int B, int C, bool WIDE>
+cudaError_t launch_pairs_cols(Context &c, const KrumPlan &p, int rows, const T *V, int64_t ldv, int m, cudaStream_t s, int *blocks) {
+    auto smem = [](int r) {
+        const size_t stages = (size_t)kKrumStages * r * (C + kKrumPad) * sizeof(T), red = sizeof(float) * kKrumWarps * B * B;
+        return red > stages ? red : stages;
+    };
+    static PerDeviceOnce attr_set;
+    if (attr_set.need(c.device)) {
+        cudaError_t e = cudaFuncSetAttribute(krum_pairs_kernel<T, B, C, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem(C == 256 ? 28 * 4 / (int)sizeof(T) : C == 128 ? 70 * 4 / (int)sizeof(T) : kKrumMaxRows));
+        if (e != cudaSuccess) return e;
+        attr_set.mark(c.device);
+    }
+    const int64_t want = (c.d + C - 1) / C;
+    *blocks = krum_grid_x(p, c.sm_count > 0 ? c.sm_count : 148);
+    if (want < *blocks) *blocks = (int)want;
+    return launch_chained(krum_pairs_kernel<T, B, C, WIDE>, dim3(*blocks, p.ny), dim3(kKrumThreads), smem(rows), s, chain_launches(c), V, ldv,
+                          c.d, m, p, c.krum_part);
+}
+
+template <typename T, int B, bool WIDE>
+cudaError_t launch_pairs(Context &c, const KrumPlan &p, const T *V, int64_t ldv, int m, cudaStream_t s, int *blocks) {
+    int rows = 0;
+    for (int y = 0; y < p.ny; ++y) {
+        int n = 0;
+        for (unsigned u = p.used[y]; u; u &= u - 1) n += B;
+        if (n > rows) rows = n;
+    }
+    const int cols = krum_cols(rows, sizeof(T));
+    if (cols == 256) return launch_pairs_cols<T, B, 256, WIDE>(c, p, rows, V, ldv, m, s, blocks);
+    if (B >= 7 && cols == 128) return launch_pairs_cols<T, B < 7 ? 7 : B, 128, WIDE>(c, p, rows, V, ldv, m, s, blocks);
+    return launch_pairs_cols<T, B < 7 ? 7 : B, 64, WIDE>(c, p, rows, V, ldv, m, s, blocks);
+}
+
+template <typename T, bool WIDE>
+cudaError_t launch_pairs_of(Context &c, const KrumPlan &p, const T *V, int64_t ldv, int m, cudaStream_t s, int *blocks) {
+    switch (p.B) {
+        case 3: return launch_pairs<T, 3, WIDE>(c, p, V, ldv, m, s, blocks);
+        case 5: return launch_pairs<T, 5, WIDE>(c, p, V, ldv, m, s, blocks);
+        case 7: return launch_pairs<T, 7, WIDE>(c, p, V, ldv, m, s, blocks);
+        case 8: return launch_pairs<T, 8, WIDE>(c, p, V, ldv, m, s, blocks);
+        default: return launch_pairs<T, 10, WIDE>(c, p, V, ldv, m, s, blocks);
+    }
+}
+
 template <typename T>
 cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b, float *out, int32_t *k, float *sums,
                               cudaStream_t s) {
     const int64_t d = c.d;
     const int sms = c.sm_count > 0 ? c.sm_count : 148;
-    const int tiles = krum_tiles(m);
-    const size_t smem = krum_pairs_smem(m);
-    static PerDeviceOnce attr_set;
-    if (attr_set.need(c.device)) {
-        cudaError_t e = cudaFuncSetAttribute(krum_pairs_kernel<T, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)krum_pairs_smem(ZENO_KRUM_MAX_M));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(krum_pairs_kernel<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)krum_pairs_smem(ZENO_KRUM_MAX_M));
-        if (e != cudaSuccess) return e;
-        attr_set.mark(c.device);
-    }
-    // as many blocks as stay resident (shared memory, 2048 threads an SM), within what the partials were sized for
-    int per_sm = (int)((200u << 10) / smem);
-    per_sm = per_sm > 8 ? 8 : (per_sm < 1 ? 1 : per_sm);
-    const int64_t want = (d + kKrumCols - 1) / kKrumCols;
-    int blocks = per_sm * sms < c.krum_blocks ? per_sm * sms : c.krum_blocks;
-    if (want < blocks) blocks = (int)(want < 1 ? 1 : want);
-    cudaError_t e = launch_chained(tiles < kKrumThreads ? krum_pairs_kernel<T, 1> : krum_pairs_kernel<T, 3>, dim3(blocks),
-                                   dim3(kKrumThreads), smem, s, chain_launches(c), V, ldv, d, m, c.krum_part);
+    const KrumPlan p = krum_plan(m);
+    int blocks = 0;
+    const bool wide = reinterpret_cast<uintptr_t>(V) % 16 == 0 && (ldv * (int64_t)sizeof(T)) % 16 == 0;
+    cudaError_t e = wide ? launch_pairs_of<T, true>(c, p, V, ldv, m, s, &blocks) : launch_pairs_of<T, false>(c, p, V, ldv, m, s, &blocks);
     if (e != cudaSuccess) return e;
-    e = launch_chained(krum_sums_kernel, dim3(m), dim3(kSumsWarps * 32), 0, s, chain_launches(c), (const float *)c.krum_part, blocks, m, b, sums,
+    e = launch_chained(krum_sums_kernel, dim3(m), dim3(kSumsWarps * 32), 0, s, chain_launches(c), (const float *)c.krum_part, blocks, m, b, p, sums,
                        c.krum_sums);
     if (e != cudaSuccess) return e;
     const int64_t cw = (d + 255) / 256;
@@ -232,8 +387,16 @@ cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b,
 
 }  // namespace
 
-// floats of Krum's workspace for up to m candidates and `blocks` blocks: the blocks' pair sums
-size_t krum_part_floats(int m, int blocks) { return (size_t)blocks * krum_tiles(m) * 16; }
+// floats of Krum's workspace for up to m_max candidates: the blocks' sums of every tile's pairs
+size_t krum_part_floats(int m_max, int sms) {
+    size_t most = 0;
+    for (int m = 1; m <= m_max; ++m) {
+        const KrumPlan p = krum_plan(m);
+        const size_t need = (size_t)krum_grid_x(p, sms) * p.tiles * p.B * p.B;
+        if (need > most) most = need;
+    }
+    return most;
+}
 
 cudaError_t launch_krum(Context &c, const void *V, int64_t ldv, int m, int b, float *out, int32_t *k, float *sums,
                         cudaStream_t s, int *launches) {

@@ -87,7 +87,6 @@ struct Context {
     // Krum: per-block partial sums of the pairs' squared distances, and the candidates' sums
     float *krum_part;               // NULL when m_max is beyond ZENO_KRUM_MAX_M
     float *krum_sums;               // [m_max]
-    int krum_blocks;                // blocks the partials were sized for
     void *host_stage;               // device copies of host inputs (zeno_step_host), grown on demand
     void *tmap_cache;               // encoded tensor maps of the tensor-core kernels (host memory, malloc'ed), or NULL
     size_t host_stage_bytes;
@@ -296,7 +295,7 @@ cudaError_t launch_split_acts(Context &c, const float *H, int models, int n_r, i
                               int *launches);
 
 // The paper's baseline aggregation rules on the same V (zeno_baselines.cu).
-size_t krum_part_floats(int m, int blocks);
+size_t krum_part_floats(int m_max, int sms);
 cudaError_t launch_median(Context &c, const void *V, int64_t ldv, int m, float *out, cudaStream_t s, int *launches);
 cudaError_t launch_krum(Context &c, const void *V, int64_t ldv, int m, int b, float *out, int32_t *k, float *sums,
                         cudaStream_t s, int *launches);

@@ -163,6 +163,29 @@ def test_krum_over_its_sizes(oracle, m, b, dtype):
     assert torch.equal(out.cpu(), w.V[k.item(), :w.d].float())
 
 
+# the last size of every block of rows and the first of the next, one stretch of columns and several, copies of 16 and of 4
+# bytes, bfloat16 rows that start in either half of 4 bytes
+@pytest.mark.parametrize("m", [3, 6, 7, 10, 11, 14, 15, 16, 17, 20, 21, 28, 29, 40, 42, 43, 70, 71, 96, 97, 100, 112, 113, 120, 121])
+@pytest.mark.parametrize("dtype,d,pad", [("f32", 2346, 2), ("f32", 515, 0), ("bf16", 2346, 6), ("bf16", 515, 0), ("bf16", 1026, 0)])
+def test_krum_over_its_tiles(oracle, m, dtype, d, pad):
+    w = syn.make_config(5, d=d, m=m, b=0, n_r=2, n_noise=0, ldv=d + pad, seed=500 + m)
+    V = w.V.to(torch.bfloat16) if dtype == "bf16" else w.V
+    V[:, d:] = float("nan")
+    V[m - 1] = V[0]                                 # identical rows of two blocks: equal distances, the lower index wins
+    V[m // 2, d - 1] += 3
+    b = min(m // 3, m - 3)
+    _, sums_orc, _ = oracle.krum(int(dtype == "bf16"), syn.to_numpy_params(V), w.ldv, d, m, b)
+    kind, desc = (0, ((d - 2) // 2, 2) if d % 2 == 0 else (d - 1, 1)) if dtype == "bf16" else (1, (d, 1))
+    with zeno.Zeno(kind, int(dtype == "bf16"), desc, True, m, 4) as z:
+        assert z.d == d
+        out, k, sums = z.krum(V.cuda(), b)
+    sums = sums.cpu().numpy().astype(np.float64)
+    # sums of d squares in binary32: relative error below d / lanes * 2^-24, far within
+    assert np.allclose(sums, sums_orc, rtol=2e-5, atol=0)
+    assert k.item() == int(np.argmin(sums))
+    assert torch.equal(out.cpu(), V[k.item(), :d].float())
+
+
 def test_krum_toy_example_on_the_gpu():
     # Discussion, the one-dimensional toy example: Krum_2({-1, -1, 0.2, 0.4, 1.6, 1.8}) = -1
     V = torch.tensor([[-1.0], [-1.0], [0.2], [0.4], [1.6], [1.8]])

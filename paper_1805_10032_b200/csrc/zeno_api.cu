@@ -642,6 +642,8 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     const size_t at_losspart = reserve(rows * 8, 8), at_losssum = reserve(rows, 8);
     const size_t at_headz = reserve(head_elems, 4), at_headt = reserve(rows, 4);
     const size_t krum_elems = m_max <= ZENO_KRUM_MAX_M ? zeno::krum_part_floats(m_max, c->sm_count > 0 ? c->sm_count : 148) : 0;
+    const int64_t loop_elems = zeno::loop_workspace(*desc, c->d, device);
+    const size_t at_loop = reserve((size_t)loop_elems, 4);
     const size_t at_krum = reserve(krum_elems, 4), at_krums = reserve(m_max, 4);
 
     // Last what depends on where convolutional layers run: on the tensor cores, in a workspace of their own, beside which
@@ -688,6 +690,7 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     c->act_split[1] = base + at_split1;
     c->head_zpart = head_elems ? reinterpret_cast<float *>(base + at_headz) : nullptr;
     c->head_tickets = reinterpret_cast<unsigned *>(base + at_headt);
+    c->loop_ws = loop_elems ? reinterpret_cast<float *>(base + at_loop) : nullptr;
     c->krum_part = krum_elems ? reinterpret_cast<float *>(base + at_krum) : nullptr;
     c->krum_sums = reinterpret_cast<float *>(base + at_krums);
     if (c->cnn_net.layers) c->cnn_ws = reinterpret_cast<float *>(base + at_cnn);
@@ -961,6 +964,14 @@ zeno_status zeno_run(zeno_handle h, void *x, const void *V, int64_t ldv, int64_t
     int launches = 0;
     profile_begin(h);
     zeno_status st = ZENO_OK;
+    if (isfinite(gamma) && isfinite(rho) && rho >= 0.f && zeno::loop_usable(*h, m, n_r, steps)) {
+        cudaError_t e = zeno::launch_loop(*h, static_cast<float *>(x), static_cast<const float *>(V), ldv, step_stride_v, m, features,
+                                          static_cast<const int32_t *>(targets), n_r, steps, gamma, rho, m - b, scores, idx, s, &launches);
+        profile_end(h, s);
+        if (e != cudaSuccess) return fail_cuda(h, e);
+        h->last_launches = launches;
+        return ZENO_OK;
+    }
     for (int32_t t = 0; t < steps && st == ZENO_OK; ++t) {
         // iteration t of Algorithm 1's server loop: its own candidates and its own batch, the x of iteration t - 1
         const void *Vt = static_cast<const char *>(V) + (size_t)t * (size_t)step_stride_v * esz;

@@ -87,6 +87,7 @@ struct Context {
     // Krum: per-block partial sums of the pairs' squared distances, and the candidates' sums
     float *krum_part;               // NULL when m_max is beyond ZENO_KRUM_MAX_M
     float *krum_sums;               // [m_max]
+    float *loop_ws;                 // the server loop's products of many iterations, or NULL
     void *host_stage;               // device copies of host inputs (zeno_step_host), grown on demand
     void *tmap_cache;               // encoded tensor maps of the tensor-core kernels (host memory, malloc'ed), or NULL
     size_t host_stage_bytes;
@@ -293,6 +294,13 @@ int layer_tc_norm_slots(int out);
 cudaError_t launch_layer_tc(Context &c, const LayerTcLaunch &l, cudaStream_t s, int *launches);
 cudaError_t launch_split_acts(Context &c, const float *H, int models, int n_r, int K, void *out, cudaStream_t s,
                               int *launches);
+
+// The server loop of a small binary32 softmax regression in two launches (zeno_loop.cu).  Shorter loops are as many steps.
+constexpr int kLoopMinSteps = 4;
+int64_t loop_workspace(const zeno_model_desc &desc, int64_t d, int device);
+bool loop_usable(const Context &c, int m, int n_r, int steps);
+cudaError_t launch_loop(Context &c, float *x, const float *V, int64_t ldv, int64_t stride_v, int m, const float *features, const int32_t *labels,
+                        int n_r, int steps, float gamma, float rho, int keep, float *scores, int32_t *idx, cudaStream_t s, int *launches);
 
 // The paper's baseline aggregation rules on the same V (zeno_baselines.cu).
 size_t krum_part_floats(int m_max, int sms);

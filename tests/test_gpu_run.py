@@ -83,6 +83,50 @@ def test_server_loop_matches_the_chained_oracle(oracle, name):
     assert not torch.equal(x.cpu(), w.x)
 
 
+# the loop of a small binary32 softmax regression: features staged whole and by stretch, a stretch with several classes and a
+# class over several stretches, one and two copies of the candidates, more candidates than warps, one class and the most,
+# samples of one and several passes, rows of every alignment, no bias, more iterations than the products of one launch
+@pytest.mark.parametrize("dims,n_r,m,bias,pad,steps", [
+    ((784, 10), 4, 20, True, 2, 5), ((33, 2), 1, 1, True, 1, 4), ((32, 32), 9, 5, True, 0, 4), ((40, 3), 64, 12, False, 0, 4),
+    ((517, 16), 13, 31, True, 1, 4), ((600, 11), 5, 70, True, 3, 4), ((1023, 31), 4, 7, True, 1, 4), ((300, 1), 2, 16, True, 0, 4),
+    ((4096, 4), 8, 15, True, 0, 4), ((20, 32), 6, 200, True, 0, 30), ((20, 5), 3, 200, True, 0, 4)])
+def test_two_launch_loop_over_its_limits(oracle, dims, n_r, m, bias, pad, steps):
+    b = m // 3
+    ov = dict(dims=dims, n_r=n_r, m=m, b=b, has_bias=bias, ldv=syn.param_count("mlp", dims, bias) + pad, faults=[(b, "signflip")] if b else [])
+    ws = [syn.make_config(1, seed=900 + t, **ov) for t in range(steps)]
+    w = ws[0]
+    x = w.x.cuda().clone()
+    with zeno.from_workload(w) as z:
+        scores, idx = z.run(x, torch.stack([s.V for s in ws]).cuda(), torch.stack([s.features for s in ws]).cuda(),
+                            torch.stack([s.targets for s in ws]).cuda(), w.gamma, w.rho, w.b)
+        assert z.last_launch_count == (4 if steps == 30 else 2)
+    gamma, rho = float(np.float32(w.gamma)), float(np.float32(w.rho))
+    x_orc = syn.to_numpy_params(w.x)
+    for t in range(steps):
+        Vt = syn.to_numpy_params(ws[t].V)
+        s_orc, f_orc, n_orc = oracle.score(0, 0, w.dims, bias, x_orc, Vt, w.ldv, m, ws[t].features.numpy(), ws[t].targets.numpy(), gamma, rho)
+        P.assert_scores_close(scores[t].cpu().numpy(), s_orc, f_orc, n_orc, rho)
+        got_idx = idx[t].cpu().numpy()
+        P.assert_selection_valid(got_idx, s_orc, b)
+        x_orc = oracle.update(0, x_orc, oracle.aggregate(0, Vt, w.ldv, w.d, m, got_idx), gamma).astype(np.float32)
+    assert P.rel_l2(x.cpu().numpy(), x_orc.astype(np.float64)) <= steps * 1e-6
+
+
+def test_two_launch_loop_with_candidates_and_logits_that_overflow():
+    """A candidate of NaN, one of infinities and one of 1e30 rank last in every iteration; logits of 1e10 keep a finite loss."""
+    w = syn.make_config(1, dims=(50, 10), n_r=4, m=9, b=3, faults=[(3, "signflip")])
+    bad = torch.nonzero(~w.honest).flatten().tolist()
+    w.V[bad[0], 3], w.V[bad[1], 4], w.V[bad[2], :w.d] = float("nan"), float("inf"), 1e30
+    V, f, t = w.V.repeat(5, 1, 1).cuda(), w.features.repeat(5, 1, 1).cuda(), w.targets.repeat(5, 1).cuda()
+    for scale in (1.0, 1e10):
+        x = (w.x * scale).cuda()
+        with zeno.from_workload(w) as z:
+            scores, idx = z.run(x, V, f, t, w.gamma, w.rho, 3)
+            assert z.last_launch_count == 2
+        assert not any(set(row) & set(bad) for row in idx.tolist())
+        assert torch.isfinite(x).all() and torch.isfinite(scores[:, w.honest.cuda()]).all()
+
+
 def test_run_argument_errors():
     w = syn.make_config(1)
     x, V, f, t = P.to_device(w)

@@ -287,8 +287,8 @@ int krum_grid_x(const KrumPlan &p, int sms) {
 }
 
 // Rows in blocks of B: the B that pads m to an even number of blocks with the fewest rows, the largest of those that tie.
-KrumPlan krum_plan(int m) {
-    KrumPlan p = {};
+void krum_size(int m, KrumPlan *plan) {
+    KrumPlan &p = *plan;
     int best = 1 << 30;
     for (int B : {3, 5, 7, 8, 10}) {
         const int nb = (m + 2 * B - 1) / (2 * B) * 2;
@@ -300,6 +300,11 @@ KrumPlan krum_plan(int m) {
     p.tiles = p.nb * p.nb / 2;
     p.ny = (p.tiles + kKrumWarps - 1) / kKrumWarps;
     p.per_y = (p.tiles + p.ny - 1) / p.ny;
+}
+
+KrumPlan krum_plan(int m) {
+    KrumPlan p = {};
+    krum_size(m, &p);
     // neighbouring tiles share row blocks: two of the one against four of the other
     int n = 0;
     for (int i0 = 0; i0 < p.nb; i0 += 2)
@@ -390,8 +395,9 @@ cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b,
 // floats of Krum's workspace for up to m_max candidates: the blocks' sums of every tile's pairs
 size_t krum_part_floats(int m_max, int sms) {
     size_t most = 0;
+    KrumPlan p;
     for (int m = 1; m <= m_max; ++m) {
-        const KrumPlan p = krum_plan(m);
+        krum_size(m, &p);
         const size_t need = (size_t)krum_grid_x(p, sms) * p.tiles * p.B * p.B;
         if (need > most) most = need;
     }

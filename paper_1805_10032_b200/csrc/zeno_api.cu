@@ -201,7 +201,7 @@ zeno_status enqueue_score_cnn(Context *c, const void *x, const void *V, int64_t 
     a.fuse_loss = fuse_loss;
     a.first_in_call = 0;
     tail.used.base[lc] = c->np_base[lc];
-    tail.used.count[lc] = zeno::mlp_norm_slots(a.out);
+    tail.used.count[lc] = zeno::mlp_norm_slots((zeno_dtype)c->desc.param_dtype, a.in, a.out, n_r, m, aligned);
     a.labels = static_cast<const int32_t *>(batch->targets);
     a.losses = loss_buf;
     a.tail = tail;
@@ -442,7 +442,7 @@ zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv,
                          zeno::mlp_mma_usable(a.in, a.out) && is_aligned(x, 16) && is_aligned(V, 16) &&
                          (ldv * esz) % 16 == 0 && (a.offW * esz) % 16 == 0;
         tail.used.base[l] = c->np_base[l];
-        tail.used.count[l] = mma ? zeno::mlp_mma_norm_slots(a.out) : zeno::mlp_norm_slots(a.out);
+        tail.used.count[l] = mma ? zeno::mlp_mma_norm_slots(a.out) : zeno::mlp_norm_slots((zeno_dtype)c->desc.param_dtype, a.in, a.out, n_r, m, aligned);
         a.labels = static_cast<const int32_t *>(batch->targets);
         a.losses = loss_buf;
         a.tail = tail;                               // complete by the time the last layer is reached
@@ -549,7 +549,7 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
             c->offB[l] = desc->has_bias ? off : -1;
             if (desc->has_bias) off += o;
             c->np_base[l] = slots;
-            int layer_slots = zeno::mlp_norm_slots((int)o);
+            int layer_slots = zeno::mlp_norm_slots_most((int)o);
             if (l == 0 && desc->param_dtype == ZENO_F32 && c->use_tc) {
                 // the tensor-core stream may serve the first layer: size its partials and norm slots
                 // for the shortest k-range any plan may pick
@@ -611,7 +611,7 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
         off += classes * c->cnn_flat;
         c->offB[lc] = desc->has_bias ? off : -1;
         c->np_base[lc] = slots;
-        slots += zeno::mlp_norm_slots((int)classes);
+        slots += zeno::mlp_norm_slots_most((int)classes);
         if (classes > widest) widest = classes;
         c->np_slots = slots;
         act_elems = rows * (size_t)n_r_max * (size_t)widest;

@@ -96,6 +96,22 @@ def test_layers_of_unaligned_rows(oracle, dims, n_r, m, dtype, bias):
     P.run_step_parity(oracle, w)
 
 
+# layers by columns: one row and one column short of and beyond a warp's and a block's share, the last stretch of one column
+# and of all but one, every compiled number of samples and tiles of them, both ways the weights are fetched, clusters of
+# blocks, rows of every alignment, bfloat16 rows that start at an odd entry, no bias
+@pytest.mark.parametrize("dims,n_r,m,bias", [
+    ((128, 31, 2), 1, 3, True), ((257, 33, 5), 2, 4, True), ((255, 64, 65, 3), 4, 5, True), ((513, 129, 10), 8, 21, True),
+    ((129, 32, 40), 12, 6, False), ((383, 97, 10), 13, 9, True), ((1025, 161, 10), 17, 5, True), ((767, 45, 131, 7), 24, 37, True),
+    ((640, 100, 9), 25, 4, True), ((2049, 34, 10), 20, 2, False), ((300, 260, 44), 40, 5, True), ((1028, 36, 4), 33, 6, True)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("pad", [0, 1])
+def test_layers_by_columns(oracle, dims, n_r, m, bias, dtype, pad):
+    b = m // 3
+    w = syn.make_config(2, dims=dims, n_r=n_r, m=m, b=b, dtype=dtype, has_bias=bias, ldv=syn.param_count("mlp", dims, bias) + pad,
+                        faults=[(b, "signflip")] if b else [])
+    P.run_step_parity(oracle, w)
+
+
 # the same kernel on rows aligned to four elements (four columns a load), and with half its rows a tile (layers of up to 32
 # rows, up to 64 samples a tile): columns that end inside a slice and inside a load's reach, one and several slices, one
 # row, 32 and 33, every compiled number of samples, clusters

@@ -148,7 +148,7 @@ zeno_status enqueue_score_cnn(Context *c, const void *x, const void *V, int64_t 
     if (c->cnn_net.layers) {
         for (int l = 0; l < lc; ++l) {
             tail.used.base[l] = c->np_base[l];
-            tail.used.count[l] = zeno::cnn_norm_slots((int)c->desc.dims[l + 2]);
+            tail.used.count[l] = zeno::cnn_tc_norm_slots((int)c->desc.dims[l + 1], (int)c->desc.dims[l + 2]);
         }
         e = zeno::launch_cnn_tc(*c, c->cnn_net, x, V, ldv, batch->features, n_r, m, gamma, c->act[(lc - 1) & 1], s, launches);
         if (e != cudaSuccess) return fail_cuda(c, e);
@@ -601,7 +601,8 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
             c->offB[l] = desc->has_bias ? off : -1;
             if (desc->has_bias) off += cout;
             c->np_base[l] = slots;
-            slots += zeno::cnn_norm_slots((int)cout);
+            const int by_pixels = zeno::cnn_norm_slots((int)cout), by_blocks = zeno::cnn_tc_norm_slots((int)cin, (int)cout);
+            slots += by_pixels > by_blocks ? by_pixels : by_blocks;
             if ((l & 1) == 1) side /= 2;                 // the pooling is folded into every second layer
             if (cout * side * side > widest) widest = cout * side * side;
         }

@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kCThreads, 1) cnn_conv_tc_kernel(CnnTcArgs a) 
 // are zero from the allocation on and never written.
 struct CnnPackLayer {
     int64_t offW, offB;
-    int cin, cout, first, nks, n, rows, stages, blocks, np_base;
+    int cin, cout, first, nks, n, rows, stages, splits, blocks, np_base;
     float *w, *bias;
     int64_t w_model, bias_model;
 };
@@ -436,7 +436,8 @@ __global__ void __launch_bounds__(256) cnn_pack_kernel(const __grid_constant__ C
         }
         return;
     }
-    // sixteen output planes of one layer of one model
+    // sixteen output planes of one layer of one model and sixteen of its input planes: a pair a thread, so that no load waits for
+    // another one's use (with all input planes in one block, in turn, the experiment's network took 10.7 us)
     int li = 0, blk = blockIdx.x;
     while (blk >= a.layer[li].blocks) blk -= a.layer[li++].blocks;
     const CnnPackLayer &L = a.layer[li];
@@ -445,10 +446,10 @@ __global__ void __launch_bounds__(256) cnn_pack_kernel(const __grid_constant__ C
     const T *xp = static_cast<const T *>(a.x);
     const T *vp = static_cast<const T *>(a.V) + (has_v ? (int64_t)(model - 1) * a.ldv : 0);
     float nrm = 0.f;
+    const int oblk = blk / L.splits, split = blk - oblk * L.splits;
     // consecutive threads: the four planes of a group, then the output planes, so that the stores are contiguous
-    for (int t = tid; t < (L.cin + 3) / 4 * 64; t += 256) {
-        const int ci = (t >> 6) * 4 + (t & 3), o = blk * 16 + ((t >> 2) & 15);
-        if (ci >= L.cin || o >= L.cout) continue;
+    const int t = split * 256 + tid, ci = (t >> 6) * 4 + (t & 3), o = oblk * 16 + ((t >> 2) & 15);
+    if (ci < L.cin && o < L.cout) {
         const int nb = o / L.n, row = o - nb * L.n;
         const int64_t src = L.offW + ((int64_t)o * L.cin + ci) * 9;
         float xv[9], vv[9];
@@ -475,8 +476,8 @@ __global__ void __launch_bounds__(256) cnn_pack_kernel(const __grid_constant__ C
             }
         }
     }
-    if (tid < 16 && L.offB >= 0 && blk * 16 + tid < L.cout) {
-        const int o = blk * 16 + tid;
+    if (split == 0 && tid < 16 && L.offB >= 0 && oblk * 16 + tid < L.cout) {
+        const int o = oblk * 16 + tid;
         const float bv = has_v ? load_elem(vp + L.offB + o) : 0.f;
         nrm = fmaf(bv, bv, nrm);
         L.bias[(int64_t)c * L.bias_model + o] = candidate_param<T>(load_elem(xp + L.offB + o), bv, a.gamma);
@@ -544,6 +545,9 @@ cudaError_t launch_conv(Context &c, const CnnTcArgs &a, int nb, int blocks, size
 }
 
 }  // namespace
+
+// norm partials of a layer's weights: a slot per warp of every block that packs them
+int cnn_tc_norm_slots(int cin, int cout) { return (cin + 15) / 16 * ((cout + 15) / 16) * 8; }
 
 // Sizes of the layers of a handle's network, and where their parts lie in a workspace for `models` models (floats from
 // its start).
@@ -642,7 +646,8 @@ cudaError_t launch_cnn_tc(Context &c, const CnnTcNet &net, const void *x, const 
         q.n = L.n;
         q.rows = L.rows;
         q.stages = L.stages;
-        q.blocks = (L.cout + 15) / 16;
+        q.splits = (L.cin + 15) / 16;
+        q.blocks = (L.cout + 15) / 16 * q.splits;
         q.np_base = c.np_base[l];
         q.w = c.cnn_ws + L.w;
         q.bias = c.cnn_ws + L.bias;

@@ -236,6 +236,7 @@ struct CnnLayerArgs {
 };
 bool cnn_side_ok(int side);
 int cnn_norm_slots(int cout);
+int cnn_tc_norm_slots(int cin, int cout);
 cudaError_t launch_cnn_conv(Context &c, const CnnLayerArgs &a, cudaStream_t s, int *launches);
 // The same layers on the tensor cores (zeno_cnn_tc.cu): all of them, the dense layer's input into `flat`.
 void cnn_tc_layout(const Context &c, CnnTcNet *net);

@@ -17,11 +17,6 @@ namespace zeno {
 
 namespace {
 
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem, bool valid) {
-    unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    int bytes = valid ? 16 : 0;  // 0 source bytes: the destination is zero-filled
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(bytes));
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
@@ -519,21 +514,23 @@ __global__ void __launch_bounds__(kRowsThreads, 2) mlp_rows_kernel(LayerArgs a, 
 // The last layer when it is small (out <= 32 classes and n_r <= 32 samples, or out <= 16 and
 // n_r <= 64): a cluster of blocks per model computes all of the model's logits and its cross-entropy.
 // Block r of the cluster takes a slice of the input range: it forms w = x - gamma v for its columns of the layer's
-// rows in shared memory (coalesced loads, v^2 accumulated on the way) next to its columns of the model's input
-// activations; warp q multiplies samples SPW q .. SPW q + SPW - 1 against all rows, lanes striding k; the partial
-// logits go to the first block's shared memory, which adds them up and takes the loss, a warp per sample.
-// The work is a chain of latencies (784 x 10 of 21 models: 0.7 MB), so the slices are short enough for all of a
-// block's loads to be in flight at once and everything else a block needs is requested with them.
-constexpr int kHeadCols = 512;                   // columns staged at a time, at most
+// rows in shared memory (coalesced loads, v^2 accumulated on the way), before it waits for the kernel that produces the
+// activations; warp q then multiplies samples SPW q .. SPW q + SPW - 1, whose activations nobody else of the block needs and
+// which come straight from memory, against all rows, lanes striding k; the partial logits go to the first block's shared
+// memory, which adds them up and takes the loss, half a warp per sample where the classes fit.
+// The work is a chain of latencies (784 x 10 of 21 models: 0.7 MB) and, with many samples, of shared-memory reads: every
+// warp reads all rows.  65 models of 4096 x 10 in bfloat16, 64 samples: 30 us a scoring pass (43 with the activations through
+// shared memory, sixteen rows for ten and a warp per sample in the loss); 1029 x 10, binary32: 22 (29).
+constexpr int kHeadSmem = 96 * 1024;             // of the staged rows, at most
 template <typename T, int OUT_T, int SPW, bool VEC>
 __global__ void __launch_bounds__(256) mlp_head_kernel(LayerArgs a, int cluster, int kslice, int KC) {
-    constexpr int NS = 8 * SPW;                  // samples a cluster can hold
-    constexpr int kRows = OUT_T / 8;             // rows a warp stages
-    constexpr int kMaxIter = kHeadCols / 128;    // KC / 128 at most
+    constexpr int NS = 8 * SPW, W = 4;           // samples a cluster can hold; columns of a lane at a time
+    constexpr int kAhead = SPW <= 2 ? 4 : SPW == 4 ? 2 : 1;      // times 128 columns of the samples on their way
+    constexpr int kRows = (OUT_T + 7) / 8;       // rows a warp stages
+    constexpr int kLossLanes = OUT_T <= 16 ? 16 : 32, kLossAt = 256 / kLossLanes, kLossTurns = (NS + kLossAt - 1) / kLossAt;
     extern __shared__ __align__(16) float smem_dyn[];
     float *ws = smem_dyn;                                            // [OUT_T][KC]
-    float *hs = ws + OUT_T * KC;                                     // [NS][KC]
-    float *zp = hs + NS * KC;                                        // [cluster][NS][OUT_T], the first block's is used
+    float *zp = ws + OUT_T * KC;                                     // [cluster][NS][OUT_T], the first block's is used
     float *np = zp + cluster * NS * OUT_T;                           // [cluster][8] sums of v^2, likewise
     __shared__ double loss_s[NS];
 
@@ -559,54 +556,58 @@ __global__ void __launch_bounds__(256) mlp_head_kernel(LayerArgs a, int cluster,
 #pragma unroll
         for (int q = 0; q < SPW; ++q) acc[o][q] = 0.f;
     float nrm = 0.f;
-    // the first block's: a lane's bias entry and the warp's labels, requested now, used at the end
+    // the first block's: a lane's bias entry and the labels of the samples it takes, requested now, used at the end
+    const int cls = lane & (kLossLanes - 1), first_loss = threadIdx.x / kLossLanes;
     float bias_x = 0.f, bias_v = 0.f;
-    int lab[SPW];
+    int lab[kLossTurns];
 #pragma unroll
-    for (int q = 0; q < SPW; ++q) lab[q] = 0;
+    for (int q = 0; q < kLossTurns; ++q) lab[q] = 0;
     if (rank == 0) {
-        if (a.offB >= 0 && lane < a.out) {
-            bias_x = load_elem(static_cast<const T *>(a.x) + a.offB + lane);
-            if (has_v) bias_v = load_elem(vbase + a.offB + lane);
-            if (warp == 0) nrm = bias_v * bias_v;
+        if (a.offB >= 0 && cls < a.out) {
+            bias_x = load_elem(static_cast<const T *>(a.x) + a.offB + cls);
+            if (has_v) bias_v = load_elem(vbase + a.offB + cls);
+            if (threadIdx.x < kLossLanes) nrm = bias_v * bias_v;
         }
 #pragma unroll
-        for (int q = 0; q < SPW; ++q)
-            if (warp + 8 * q < a.n_r) lab[q] = __ldg(a.labels + warp + 8 * q);
+        for (int q = 0; q < kLossTurns; ++q)
+            if (first_loss + kLossAt * q < a.n_r) lab[q] = __ldg(a.labels + first_loss + kLossAt * q);
     }
 
     // w = x - gamma v of the layer's rows for the columns from kb on (zero beyond the rows and the slice)
     auto stage_weights = [&](int kb) {
-        if (VEC) {
-            // all of a thread's loads are issued before the first is used
-            float xv[kRows * kMaxIter][4], vv[kRows * kMaxIter][4];
+        if constexpr (VEC) {
+            constexpr int kBatch = 4;            // of 128 columns: all of a thread's loads of a batch before the first is used
+            for (int k4 = 0; k4 < KC; k4 += kBatch * 128) {
+                float xv[kRows * kBatch][4], vv[kRows * kBatch][4];
 #pragma unroll
-            for (int u = 0; u < kRows * kMaxIter; ++u) {
-                const int o = warp + 8 * (u / kMaxIter), kk = (u % kMaxIter) * 128 + 4 * lane;
+                for (int u = 0; u < kRows * kBatch; ++u) {
+                    const int o = warp + 8 * (u / kBatch), kk = k4 + (u % kBatch) * 128 + 4 * lane;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) xv[u][e] = vv[u][e] = 0.f;
-                if (o < a.out && kk < KC && kb + kk < k1) {
-                    load_vec4(xw + (int64_t)o * K + kb + kk, xv[u]);
-                    if (has_v) load_vec4(vw + (int64_t)o * K + kb + kk, vv[u]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kRows * kMaxIter; ++u) {
-                const int o = warp + 8 * (u / kMaxIter), kk = (u % kMaxIter) * 128 + 4 * lane;
-                if (kk < KC) {
-                    float w4[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        w4[e] = candidate_param<T>(xv[u][e], vv[u][e], a.gamma);
-                        nrm = fmaf(vv[u][e], vv[u][e], nrm);
+                    for (int e = 0; e < 4; ++e) xv[u][e] = vv[u][e] = 0.f;
+                    if (o < a.out && kk < KC && kb + kk < k1) {
+                        load_vec4(xw + (int64_t)o * K + kb + kk, xv[u]);
+                        if (has_v) load_vec4(vw + (int64_t)o * K + kb + kk, vv[u]);
                     }
-                    *reinterpret_cast<float4 *>(ws + o * KC + kk) = make_float4(w4[0], w4[1], w4[2], w4[3]);
+                }
+#pragma unroll
+                for (int u = 0; u < kRows * kBatch; ++u) {
+                    const int o = warp + 8 * (u / kBatch), kk = k4 + (u % kBatch) * 128 + 4 * lane;
+                    if (o < OUT_T && kk < KC) {
+                        float w4[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            w4[e] = candidate_param<T>(xv[u][e], vv[u][e], a.gamma);
+                            nrm = fmaf(vv[u][e], vv[u][e], nrm);
+                        }
+                        *reinterpret_cast<float4 *>(ws + o * KC + kk) = make_float4(w4[0], w4[1], w4[2], w4[3]);
+                    }
                 }
             }
         } else {
 #pragma unroll
             for (int r = 0; r < kRows; ++r) {
                 const int o = warp + 8 * r;
+                if (o >= OUT_T) break;
 #pragma unroll 8
                 for (int kk = lane; kk < KC; kk += 32) {
                     float xv = 0.f, vv = 0.f;
@@ -620,52 +621,61 @@ __global__ void __launch_bounds__(256) mlp_head_kernel(LayerArgs a, int cluster,
             }
         }
     };
-    // the model's input activations for the same columns (asynchronous copies on the vector path)
-    auto stage_acts = [&](int kb) {
-#pragma unroll
-        for (int q = 0; q < SPW; ++q) {
-            const int j = warp + 8 * q;
-            if (VEC) {
-                for (int kk = 4 * lane; kk < KC; kk += 128) {
-                    const bool ok = j < a.n_r && kb + kk < k1;
-                    cp_async16(hs + j * KC + kk, ok ? hin + (int64_t)j * K + kb + kk : a.Hin, ok);
-                }
-            } else {
-#pragma unroll 8
-                for (int kk = lane; kk < KC; kk += 32)
-                    hs[j * KC + kk] = (j < a.n_r && kb + kk < k1) ? __ldg(hin + (int64_t)j * K + kb + kk) : 0.f;
-            }
-        }
-        if (VEC) cp_async_commit();
-    };
 
     if (k0 < k1) stage_weights(k0);
     pdl_wait();
     pdl_launch_dependents();
+    const float *hq[SPW];                        // this warp's samples; beyond the last one it again, its sums are dropped
+#pragma unroll
+    for (int q = 0; q < SPW; ++q) hq[q] = hin + (int64_t)min(warp * SPW + q, a.n_r - 1) * K;
     for (int kb = k0; kb < k1; kb += KC) {
-        if (kb > k0) __syncthreads();
-        stage_acts(kb);                 // in flight while the weights are formed
-        if (kb > k0) stage_weights(kb);
-        if (VEC) cp_async_wait<0>();
+        if (kb > k0) {
+            __syncthreads();
+            stage_weights(kb);
+        }
         __syncthreads();
-        // warp q: its SPW samples against every row; lane l takes k = 4l + 128 i
         if (warp * SPW < a.n_r) {
-#pragma unroll 1
-            for (int kk = 4 * lane; kk < KC; kk += 128) {
-                if (kb + kk - 4 * lane >= k1) break;
-                float4 h4[SPW];
+            const int len = min(KC, k1 - kb);
+            // a lane's columns of 128: four neighbours (VEC), or every 32nd
+            constexpr int kStep = VEC ? 1 : 32;
+            const int at = VEC ? 4 * lane : lane;
+            float h[kAhead][SPW][W];
+            auto load = [&](int k, float (&to)[SPW][W]) {
 #pragma unroll
-                for (int q = 0; q < SPW; ++q) h4[q] = *reinterpret_cast<const float4 *>(hs + (warp * SPW + q) * KC + kk);
+                for (int q = 0; q < SPW; ++q) {
+                    if constexpr (VEC) {
+                        const float4 t = k + at < len ? __ldcg(reinterpret_cast<const float4 *>(hq[q] + kb + k + at)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        to[q][0] = t.x; to[q][1] = t.y; to[q][2] = t.z; to[q][3] = t.w;
+                    } else {
 #pragma unroll
-                for (int o = 0; o < OUT_T; ++o) {
-                    const float4 w4 = *reinterpret_cast<const float4 *>(ws + o * KC + kk);
-#pragma unroll
-                    for (int q = 0; q < SPW; ++q) {
-                        acc[o][q] = fmaf(w4.x, h4[q].x, acc[o][q]);
-                        acc[o][q] = fmaf(w4.y, h4[q].y, acc[o][q]);
-                        acc[o][q] = fmaf(w4.z, h4[q].z, acc[o][q]);
-                        acc[o][q] = fmaf(w4.w, h4[q].w, acc[o][q]);
+                        for (int e = 0; e < W; ++e) to[q][e] = k + at + kStep * e < len ? __ldcg(hq[q] + kb + k + at + kStep * e) : 0.f;
                     }
+                }
+            };
+#pragma unroll
+            for (int d = 0; d < kAhead; ++d) load(128 * d, h[d]);
+#pragma unroll 1
+            for (int k = 0; k < len; k += 128 * kAhead) {
+#pragma unroll
+                for (int d = 0; d < kAhead; ++d) {
+                    const int kd = k + 128 * d;
+                    if (kd >= len) break;
+#pragma unroll
+                    for (int o = 0; o < OUT_T; ++o) {
+                        float w[W];
+                        if constexpr (VEC) {
+                            const float4 t = *reinterpret_cast<const float4 *>(ws + o * KC + kd + at);
+                            w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < W; ++e) w[e] = ws[o * KC + kd + at + kStep * e];
+                        }
+#pragma unroll
+                        for (int q = 0; q < SPW; ++q)
+#pragma unroll
+                            for (int e = 0; e < W; ++e) acc[o][q] = fmaf(w[e], h[d][q][e], acc[o][q]);
+                    }
+                    load(kd + 128 * kAhead, h[d]);
                 }
             }
         }
@@ -686,47 +696,46 @@ __global__ void __launch_bounds__(256) mlp_head_kernel(LayerArgs a, int cluster,
 
     __syncwarp();
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");     // every block runs: its shared memory may be written
-    // lane totals, N (row, sample) pairs at a time; lane l receives pair l of the batch
-    constexpr int N = OUT_T * SPW < 32 ? OUT_T * SPW : 32, kRowsPerBatch = N / SPW;
+    // lane totals, up to 32 (row, sample) pairs at a time; lane l receives pair l of the batch
+    constexpr int kPairs = OUT_T * SPW, N = kPairs < 32 ? (kPairs <= 16 ? 16 : 32) : 32;
     if (warp * SPW < a.n_r) {
         const uint32_t dst = cluster_addr(zp + (size_t)rank * NS * OUT_T, 0);
 #pragma unroll
-        for (int ob = 0; ob < OUT_T; ob += kRowsPerBatch) {
+        for (int e0 = 0; e0 < kPairs; e0 += N) {
             float v[N];
 #pragma unroll
-            for (int o = 0; o < kRowsPerBatch; ++o)
-#pragma unroll
-                for (int q = 0; q < SPW; ++q) v[o * SPW + q] = acc[ob + o][q];
+            for (int e = 0; e < N; ++e) v[e] = e0 + e < kPairs ? acc[e0 + e < kPairs ? (e0 + e) / SPW : 0][(e0 + e) % SPW] : 0.f;
             const float z = warp_transpose_reduce<N>(v, lane);
-            const int o = ob + lane / SPW, j = warp * SPW + lane % SPW;
-            if (lane < N && o < a.out && j < a.n_r) cluster_store(dst + 4 * (j * OUT_T + o), z);
+            const int e = e0 + lane, o = e / SPW, j = warp * SPW + e % SPW;
+            if (lane < N && e < kPairs && o < a.out && j < a.n_r) cluster_store(dst + 4 * (j * OUT_T + o), z);
         }
     }
     nrm = warp_sum(nrm);
     if (lane == 0) cluster_store(cluster_addr(np + rank * 8 + warp, 0), nrm);
     cluster_barrier();
     if (rank != 0) return;
-    // the loss of the samples warp, warp + 8, ..: a lane per class (logits and their differences in double: the
-    // score is a difference of losses that agree in several digits)
+    // the samples' losses: a lane per class (logits and their differences in double: the score is a difference of losses that
+    // agree in several digits)
     const double bias = a.offB >= 0 ? (double)candidate_param<T>(bias_x, bias_v, a.gamma) : 0.0;
 #pragma unroll
-    for (int q = 0; q < SPW; ++q) {
-        const int j = warp + 8 * q;
-        if (j >= a.n_r) break;
+    for (int q = 0; q < kLossTurns; ++q) {
+        const int j = first_loss + kLossAt * q;
+        if (j - (lane / kLossLanes) >= a.n_r) break;             // the whole warp's samples
         double z = 0.0;
-        if (lane < a.out) {
-            for (int r = 0; r < cluster; ++r) z += (double)zp[(r * NS + j) * OUT_T + lane];
+        if (cls < a.out && j < a.n_r) {
+            for (int r = 0; r < cluster; ++r) z += (double)zp[(r * NS + j) * OUT_T + cls];
             z += bias;
         }
-        double zmax = lane < a.out ? z : -INFINITY;      // not rounded: a logit of 1e10 is 512 from its float
+        double zmax = cls < a.out ? z : -INFINITY;       // not rounded: a logit of 1e10 is 512 from its float
 #pragma unroll
-        for (int s = 16; s >= 1; s >>= 1) zmax = fmax(zmax, __shfl_xor_sync(0xffffffffu, zmax, s));
-        const float dz = (float)(z - zmax);
-        const float se = warp_sum(lane < a.out ? expf(dz) : 0.f);           // a NaN logit makes se NaN
+        for (int s = kLossLanes / 2; s >= 1; s >>= 1) zmax = fmax(zmax, __shfl_xor_sync(0xffffffffu, zmax, s));
+        float se = cls < a.out ? expf((float)(z - zmax)) : 0.f;             // a NaN logit makes se NaN
+#pragma unroll
+        for (int s = kLossLanes / 2; s >= 1; s >>= 1) se += __shfl_xor_sync(0xffffffffu, se, s);
         int l = lab[q];
         if (l < 0 || l >= a.out) l = 0;
-        const double zl = __shfl_sync(0xffffffffu, z, l);
-        if (lane == 0) loss_s[j] = (zmax - zl) + (double)logf(se);
+        const double zl = __shfl_sync(0xffffffffu, z, (lane & ~(kLossLanes - 1)) + l);
+        if (cls == 0 && j < a.n_r) loss_s[j] = (zmax - zl) + (double)logf(se);
     }
     __syncthreads();
     if (warp == 0) {
@@ -925,22 +934,22 @@ bool mlp_can_fuse_loss(int out, int n_r) { return (out <= 32 && n_r <= 32) || (o
 
 template <typename T, int OUT_T, int SPW, bool VEC>
 cudaError_t launch_head_sized(Context &c, const LayerArgs &a, cudaStream_t s) {
-    constexpr int NS = 8 * SPW;
+    constexpr int NS = 8 * SPW, kMostCols = kHeadSmem / 4 / OUT_T / 128 * 128;
     // blocks per model: as many as leave a slice of 128 columns and are resident at once (two to an SM up to 16 x 16
     // logits, one beyond: the accumulators).  A second wave costs more than the longer slice (101 models of 512 x 10,
     // 64 samples: 21 us with one block a model, 29 with two)
     const int sms = c.sm_count > 0 ? c.sm_count : 148;
     const int room = a.out <= 16 && a.n_r <= 16 ? 2 * sms : sms;
-    int cluster = 1;
+    int cluster = 1;                             // powers of two: clusters of seven leave a third of the SMs without one
     while (cluster < kMaxCluster && a.in / (2 * cluster) >= 128 && (a.m + 1) * 2 * cluster <= room) cluster *= 2;
     const int kslice = ((a.in + cluster - 1) / cluster + 3) / 4 * 4;
-    const int KC = kslice >= kHeadCols ? kHeadCols : (kslice + 127) / 128 * 128;
-    auto smem = [](int cols, int blocks) { return sizeof(float) * ((size_t)(OUT_T + NS) * cols + (size_t)blocks * (NS * OUT_T + 8)); };
+    const int turns = (kslice + kMostCols - 1) / kMostCols, KC = ((kslice + turns - 1) / turns + 127) / 128 * 128;
+    auto smem = [](int cols, int blocks) { return sizeof(float) * ((size_t)OUT_T * cols + (size_t)blocks * (NS * OUT_T + 8)); };
     // the limit is the function's, for every handle and thread of the process: the most any call asks for, set once
     static PerDeviceOnce attr_set;
     if (attr_set.need(c.device)) {
         cudaError_t e = cudaFuncSetAttribute(mlp_head_kernel<T, OUT_T, SPW, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem(kHeadCols, kMaxCluster));
+                                             (int)smem(kMostCols, kMaxCluster));
         if (e != cudaSuccess) return e;
         attr_set.mark(c.device);
     }
@@ -950,6 +959,12 @@ cudaError_t launch_head_sized(Context &c, const LayerArgs &a, cudaStream_t s) {
 
 template <typename T, bool VEC>
 cudaError_t launch_head(Context &c, const LayerArgs &a, cudaStream_t s) {
+    if (a.out <= 12) {
+        if (a.n_r <= 8) return launch_head_sized<T, 12, 1, VEC>(c, a, s);
+        if (a.n_r <= 16) return launch_head_sized<T, 12, 2, VEC>(c, a, s);
+        if (a.n_r <= 32) return launch_head_sized<T, 12, 4, VEC>(c, a, s);
+        return launch_head_sized<T, 12, 8, VEC>(c, a, s);
+    }
     if (a.out <= 16) {
         if (a.n_r <= 8) return launch_head_sized<T, 16, 1, VEC>(c, a, s);
         if (a.n_r <= 16) return launch_head_sized<T, 16, 2, VEC>(c, a, s);

@@ -83,6 +83,16 @@ def test_small_last_layer_over_its_limits(oracle, dims, n_r, m, dtype, pad):
     P.run_step_parity(oracle, w)
 
 
+# the same by what a cluster stages at once and by its classes and samples: slices in several turns, twelve rows, thirteen and
+# more, samples of a last half warp, one sample more than the warps take
+@pytest.mark.parametrize("dims,n_r,m,dtype,pad", [
+    ((2600, 32), 7, 120, "f32", 0), ((9000, 12), 9, 70, "f32", 1), ((7001, 13), 33, 40, "f32", 0), ((8200, 10), 63, 75, "bf16", 4), ((2051, 11), 1, 9, "bf16", 1)])
+def test_small_last_layer_in_turns(oracle, dims, n_r, m, dtype, pad):
+    d = dims[0] * dims[1] + dims[1]
+    b = m // 3
+    P.run_step_parity(oracle, syn.make_config(1, dims=dims, n_r=n_r, m=m, b=b, dtype=dtype, ldv=d + pad, faults=[(b, "signflip")]))
+
+
 # the layer kernel for rows of any alignment: one row tile and several, slices with remainders, one to eight blocks a tile,
 # every compiled number of samples, several sample tiles, no bias
 @pytest.mark.parametrize("dims,n_r,m,dtype,bias", [

@@ -48,12 +48,6 @@ struct KrumPlan {
 // columns staged at a time: as many as leave room for two blocks an SM (three stages of 28, 70 and 128 binary32 rows)
 inline int krum_cols(int rows, int entry_bytes) { return rows * entry_bytes <= 28 * 4 ? 256 : rows * entry_bytes <= 70 * 4 ? 128 : 64; }
 
-__device__ __forceinline__ void krum_copy(uint32_t dst, const void *src, bool valid, bool wide) {
-    if (wide)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
-}
 __device__ __forceinline__ float krum_value(const float *p) { return *p; }
 __device__ __forceinline__ float krum_value(const __nv_bfloat16 *p) {
     return bf16_bits_to_float(*reinterpret_cast<const unsigned short *>(p));
@@ -106,12 +100,12 @@ krum_pairs_kernel(const T *V, int64_t ldv, int64_t d, int m, const __grid_consta
             const T *row = row_at[r];
             if (!row) continue;
             const bool ok = !last || j0 + q - (kHalves ? late[r] : 0) < d;         // beyond the columns nothing is read
-            krum_copy(dst, ok ? row + j0 + q : row, ok, WIDE);
+            cp_async<WIDE ? 16 : 4>(dst, ok ? row + j0 + q : row, ok);
         }
         if (kHalves && (int)threadIdx.x < rows && late[threadIdx.x]) {             // the last entry of rows that start half a word late
             const T *row = row_at[threadIdx.x];
             const bool ok = j0 + C - 1 < d;
-            if (row) krum_copy((uint32_t)__cvta_generic_to_shared(stage0 + s * stage + threadIdx.x * kPitch + C), ok ? row + j0 + C : row, ok, false);
+            if (row) cp_async<4>((uint32_t)__cvta_generic_to_shared(stage0 + s * stage + threadIdx.x * kPitch + C), ok ? row + j0 + C : row, ok);
         }
     };
     float acc[B * B];
@@ -125,15 +119,15 @@ krum_pairs_kernel(const T *V, int64_t ldv, int64_t d, int m, const __grid_consta
     int64_t ct = blockIdx.x;
     for (int s = 0; s < kKrumStages - 1; ++s) {
         if (ct + (int64_t)s * gridDim.x < tiles_c) load(ct + (int64_t)s * gridDim.x, s);
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        cp_async_commit();
     }
     int s = 0;
     for (; ct < tiles_c; ct += gridDim.x) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(kKrumStages - 2) : "memory");
+        cp_async_wait<kKrumStages - 2>();
         __syncthreads();                      // the stage has landed for every thread; the one before is free
         const int64_t next = ct + (int64_t)(kKrumStages - 1) * gridDim.x;
         if (next < tiles_c) load(next, s == 0 ? kKrumStages - 1 : s - 1);
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        cp_async_commit();
         T *st = stage0 + s * stage;
         if (ct * C + C > d) {                 // beyond the columns whatever the copies brought counts as zero
             const int left = (int)(d - ct * C);
@@ -180,7 +174,7 @@ krum_pairs_kernel(const T *V, int64_t ldv, int64_t d, int m, const __grid_consta
         if (++s == kKrumStages) s = 0;
     }
     // the lanes' sums, 32 pairs at a time (lane l receives pair l of the batch), then the groups'
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    cp_async_wait<0>();
     __syncthreads();
     float *red = reinterpret_cast<float *>(krum_smem);             // [group][tile of the block][B * B]
     if (busy) {

@@ -376,6 +376,23 @@ inline cudaError_t launch_clustered(void (*kernel)(KArgs...), int cluster, dim3 
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Asynchronous copies of 16 or 4 bytes from global into shared memory; one that is not valid reads nothing and writes zeros.
+// All three are barriers to the compiler as well: a thread that waits for its own copies reads what they brought with
+// ordinary loads, which must not move above the wait.
+template <int BYTES>
+__device__ __forceinline__ void cp_async(uint32_t dst, const void *src, bool valid = true) {
+    static_assert(BYTES == 16 || BYTES == 4, "copies of 16 or 4 bytes");
+    if (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t hi16_in_low) {
     return __uint_as_float(hi16_in_low << 16);
 }

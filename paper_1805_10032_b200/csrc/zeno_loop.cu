@@ -55,11 +55,7 @@ struct LoopArgs {
 };
 
 template <int BYTES>
-__device__ __forceinline__ void loop_copy(void *dst, const void *src) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    if (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-}
+__device__ __forceinline__ void loop_copy(void *dst, const void *src) { cp_async<BYTES>((uint32_t)__cvta_generic_to_shared(dst), src); }
 __device__ __forceinline__ void cluster_store_double(uint32_t addr, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
 }
@@ -197,7 +193,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
         float *norm = reinterpret_cast<float *>(sm + p.at_norm + buf * p.norm_bytes);
         for (int i = tid; i < a.m; i += kLoopThreads) loop_copy<4>(norm + i, a.norms + (int64_t)t * a.m + i);
         for (int j = tid; j < a.n_r; j += kLoopThreads) loop_copy<4>(lab_s + buf * a.n_r + j, a.labels + (int64_t)t * a.n_r + j);
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        cp_async_commit();
     };
     load(0, 0);
     for (int q = tid; q < own; q += kLoopThreads) xs[q] = a.x[p0 + q];
@@ -206,7 +202,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
 
     for (int t = 0; t < a.steps; ++t) {
         const int buf = p.bufs == 2 ? t & 1 : 0;
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        cp_async_wait<0>();
         __syncthreads();             // x is updated and this iteration's inputs are here
         TICK(0)
         const float *vs = reinterpret_cast<const float *>(sm + p.at_v + buf * p.v_bytes);

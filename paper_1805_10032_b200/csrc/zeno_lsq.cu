@@ -20,16 +20,6 @@ namespace {
 constexpr int kStageFloats = 8192;   // floats of A per shared-memory stage (32 KB)
 constexpr int kIterK = 128;
 
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem, bool valid) {
-    unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    int bytes = valid ? 16 : 0;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(bytes));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
-}
-
 template <int N>
 __device__ __forceinline__ float warp_transpose_reduce(float (&v)[N], int lane) {
 #pragma unroll
@@ -129,7 +119,7 @@ __global__ void __launch_bounds__(LsqShape<NRT, RB>::kMaxWarps * 32, 1) lsq_stre
                 int j = t / kVecPerRow, kk = (t % kVecPerRow) * 4;
                 bool ok = j < n_valid && kb + kk < K;
                 const float *src = ok ? a.A + (int64_t)(j0 + j) * K + kb + kk : a.A;
-                cp_async16(&dst[j][kk], src, ok);
+                cp_async<16>((uint32_t)__cvta_generic_to_shared(&dst[j][kk]), src, ok);
             }
         } else {
             for (int t = threadIdx.x; t < NRT * kStageK; t += blockDim.x) {

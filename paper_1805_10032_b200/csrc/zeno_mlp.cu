@@ -17,11 +17,6 @@ namespace zeno {
 
 namespace {
 
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
-}
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int s = 16; s >= 1; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
@@ -348,8 +343,8 @@ __global__ void __launch_bounds__(kRowsThreads, 2) mlp_rows_kernel(LayerArgs a, 
             const uint32_t dst = (uint32_t)__cvta_generic_to_shared(mine + u * 2 * R * 32);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + r * 256), "l"(reinterpret_cast<const char *>(xw) + (off[r] + k)) : "memory");
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + r * 256 + 128), "l"(reinterpret_cast<const char *>(vw) + (off[r] + k)) : "memory");
+                cp_async<4>(dst + r * 256, reinterpret_cast<const char *>(xw) + (off[r] + k));
+                cp_async<4>(dst + r * 256 + 128, reinterpret_cast<const char *>(vw) + (off[r] + k));
             }
         } else {
 #pragma unroll
@@ -367,8 +362,7 @@ __global__ void __launch_bounds__(kRowsThreads, 2) mlp_rows_kernel(LayerArgs a, 
 #pragma unroll 4
         for (int j = tid / kLanes; j < N; j += kRowsThreads / kLanes, src += (int64_t)(kRowsThreads / kLanes) * K, dst += 4 * (kRowsThreads / kLanes) * C) {
             const bool ok = k < K && j0 + j < a.n_r;
-            if (W == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(ok ? src : hin), "r"(ok ? 16 : 0) : "memory");
-            else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(ok ? src : hin), "r"(ok ? 4 : 0) : "memory");
+            cp_async<4 * W>(dst, ok ? src : hin, ok);
         }
         if (!ASYNC) cp_async_commit();          // else with the next step's words
     };

@@ -323,6 +323,11 @@ cudaError_t launch_lsq_tc(Context &c, const LsqArgs &a, int max_slabs, int *slab
 int mlp_norm_slots(zeno_dtype dtype, int in, int out, int n_r, int m, bool aligned);
 int mlp_norm_slots_most(int out);
 
+constexpr int kMaxCluster = 8;     // blocks of a cluster in the dense layers' kernels
+// Dense layers by columns (zeno_rows.cu): which layers, and what they take.
+bool layer_by_columns(zeno_dtype dtype, int in, int out, int n_r, int m, bool aligned);
+cudaError_t launch_layer_by_columns(Context &c, const LayerArgs &a, bool aligned, cudaStream_t s);
+
 // ---- device helpers shared by the kernels ------------------------------------------------
 
 #ifdef __CUDACC__
@@ -415,6 +420,18 @@ __device__ __forceinline__ void load_vec4(const __nv_bfloat16 *p, float (&o)[4])
     o[3] = __uint_as_float(t.y & 0xffff0000u);
 }
 
+// elements as they lie in memory: one, or four
+template <typename T> struct RawOf;
+template <> struct RawOf<float> { using One = float; using Four = float4; };
+template <> struct RawOf<__nv_bfloat16> { using One = unsigned short; using Four = uint2; };
+__device__ __forceinline__ float raw_to_float(float v) { return v; }
+__device__ __forceinline__ float raw_to_float(unsigned short v) { return bf16_bits_to_float(v); }
+__device__ __forceinline__ float4 raw_to_float4(float4 v) { return v; }
+__device__ __forceinline__ float4 raw_to_float4(uint2 v) {
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                       __uint_as_float(v.y & 0xffff0000u));
+}
+
 // value rounded to tf32 (10 explicit mantissa bits), ties away from zero in magnitude
 __device__ __forceinline__ float tf32_hi(float a) {
     return __uint_as_float((__float_as_uint(a) + 0x1000u) & 0xffffe000u);
@@ -429,6 +446,18 @@ __device__ __forceinline__ unsigned long long rank_key(float s, int index) {
     unsigned u = __float_as_uint(s);
     u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
     return ((unsigned long long)u << 32) | (unsigned)(0xffffffffu - (unsigned)index);
+}
+
+// the lanes' sum, in every lane
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+    return v;
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+    return v;
 }
 
 // Sum, over the 32 lanes, of each of N per-lane values; lane j (< N) ends up holding the total

@@ -122,6 +122,33 @@ def test_layers_by_columns(oracle, dims, n_r, m, bias, dtype, pad):
     P.run_step_parity(oracle, w)
 
 
+@pytest.mark.parametrize("cols,rows,dtype", [(40001, 33, "f32"), (40001, 33, "bf16"), (40004, 36, "f32")])
+def test_sums_of_long_rows_are_short_sums(cols, rows, dtype):
+    """A logit of 40,000 products of random signs against 64 bits, the layer in as many tiles as leave a lane every 32nd
+    column of whole rows.  An addition to a partial sum of k products errs by 0.41 x 2^-24 of it in the root mean square and
+    the partial sum grows as sqrt(k): a chain of n products is off by 0.41 x 2^-24 sqrt(n / 2) of the result, 6e-7 with all
+    1,250 of a lane and 1.4e-7 with runs of 64, to which the additions of the 32 lanes and of the runs add about as much."""
+    m, n_r, size, gamma = 12, 128, 3e4, 0.125
+    g = torch.Generator().manual_seed(cols + rows)
+    store = torch.bfloat16 if dtype == "bf16" else torch.float32
+    d = rows * cols + rows
+    x = (torch.randn(d, generator=g) * (size / cols ** 0.5)).to(store)
+    V = torch.randn((m, d), generator=g).mul_(0.5 * size / cols ** 0.5 / gamma).to(store)
+    feats = torch.randn((n_r, cols), generator=g)
+    feats[1:] *= 1e-9                                # the first sample's loss is all there is to see
+    labels = torch.randint(0, rows, (n_r,), generator=g, dtype=torch.int32)
+    with zeno.Zeno(zeno.LOSS_SOFTMAX_MLP, zeno.BF16 if dtype == "bf16" else zeno.F32, (cols, rows), True, m, n_r) as z:
+        _, losses, _ = z.score(x.cuda(), V.cuda(), feats.cuda(), labels.cuda(), gamma, 0.0)
+        got = losses.double().cpu()
+    for c in range(m + 1):
+        w = x.double() if c == 0 else x.double() - gamma * V[c - 1].double()
+        w = w.float().to(store).double() if dtype == "bf16" else w
+        z64 = feats.double() @ w[:rows * cols].view(rows, cols).t() + w[rows * cols:]
+        got[c] -= torch.nn.functional.cross_entropy(z64, labels.long())
+    # a loss is the difference of two logits of this size, times 1 / n_r
+    assert (got.square().mean().sqrt() / (size * 2 ** 0.5 / n_r)).item() <= 3.5e-7
+
+
 # the same kernel on rows aligned to four elements (four columns a load), and with half its rows a tile (layers of up to 32
 # rows, up to 64 samples a tile): columns that end inside a slice and inside a load's reach, one and several slices, one
 # row, 32 and 33, every compiled number of samples, clusters

@@ -965,7 +965,8 @@ zeno_status zeno_run(zeno_handle h, void *x, const void *V, int64_t ldv, int64_t
     int launches = 0;
     profile_begin(h);
     zeno_status st = ZENO_OK;
-    if (isfinite(gamma) && isfinite(rho) && rho >= 0.f && zeno::loop_usable(*h, m, n_r, steps)) {
+    const bool rows_aligned = score_rows_aligned(*h, x, V, ldv, features) && step_stride_v % 4 == 0;
+    if (isfinite(gamma) && isfinite(rho) && rho >= 0.f && zeno::loop_usable(*h, m, n_r, steps, rows_aligned)) {
         cudaError_t e = zeno::launch_loop(*h, static_cast<float *>(x), static_cast<const float *>(V), ldv, step_stride_v, m, features,
                                           static_cast<const int32_t *>(targets), n_r, steps, gamma, rho, m - b, scores, idx, s, &launches);
         profile_end(h, s);

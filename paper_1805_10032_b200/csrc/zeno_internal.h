@@ -299,7 +299,7 @@ cudaError_t launch_split_acts(Context &c, const float *H, int models, int n_r, i
 // The server loop of a small binary32 softmax regression in two launches (zeno_loop.cu).  Shorter loops are as many steps.
 constexpr int kLoopMinSteps = 4;
 int64_t loop_workspace(const zeno_model_desc &desc, int64_t d, int device);
-bool loop_usable(const Context &c, int m, int n_r, int steps);
+bool loop_usable(const Context &c, int m, int n_r, int steps, bool aligned);   // rows aligned to four elements
 cudaError_t launch_loop(Context &c, float *x, const float *V, int64_t ldv, int64_t stride_v, int m, const float *features, const int32_t *labels,
                         int n_r, int steps, float gamma, float rho, int keep, float *scores, int32_t *idx, cudaStream_t s, int *launches);
 

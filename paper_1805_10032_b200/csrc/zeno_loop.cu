@@ -85,23 +85,26 @@ __device__ __forceinline__ void loop_wait() {
 #endif
 
 // products[t][c][j][o] = sum_k features[t][j][k] V[t][c][o][k] + the candidate's bias entry o; norms[t][c] = ||v||^2.
-// A block per candidate and iteration, a warp per class, lanes along the columns, NS samples at a time.
+// A block per candidate and iteration, a warp per class and part of the columns, lanes along the columns, NS samples at a time.
+// A part has at most 2,048 columns: a lane's sums are of 64 products however wide the model is.
+constexpr int kProductWarps = 8, kProductCols = 2048, kProductUnits = 128;
 template <int NS>
-__global__ void __launch_bounds__(256) loop_products_kernel(const float *V, int64_t ldv, int64_t stride_v, const float *features, int in,
-                                                            int classes, int has_bias, int m, int n_r, float *products, float *norms) {
-    __shared__ float part[8];
+__global__ void __launch_bounds__(kProductWarps * 32) loop_products_kernel(const float *V, int64_t ldv, int64_t stride_v, const float *features, int in,
+                                                                          int classes, int has_bias, int parts, int m, int n_r, float *products, float *norms) {
+    __shared__ float norm_part[kProductWarps], part[2][kProductUnits][NS];
     pdl_wait();
     pdl_launch_dependents();
     const int c = blockIdx.x, t = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float *v = V + (int64_t)t * stride_v + (int64_t)c * ldv;
     const float *f = features + (int64_t)t * n_r * in;
     float *out = products + ((int64_t)t * m + c) * n_r * classes;
+    const int len = ((in + parts - 1) / parts + 31) / 32 * 32;
     float nrm = 0.f;
-    for (int o = warp; o < classes; o += 8) {
-        const float *row = v + (int64_t)o * in;
-        const float bias = has_bias ? __ldg(v + (int64_t)classes * in + o) : 0.f;
-        if (lane == 0) nrm = fmaf(bias, bias, nrm);
-        for (int j0 = 0; j0 < n_r; j0 += NS) {
+    auto bias_of = [&](int o) { return has_bias ? __ldg(v + (int64_t)classes * in + o) : 0.f; };
+    for (int j0 = 0, b = 0; j0 < n_r; j0 += NS, b ^= 1) {
+        for (int unit = warp; unit < classes * parts; unit += kProductWarps) {
+            const int o = unit / parts, k0 = (unit - o * parts) * len, k1 = min(in, k0 + len);
+            const float *row = v + (int64_t)o * in;
             float acc[NS];
             const float *h[NS];
 #pragma unroll
@@ -110,22 +113,38 @@ __global__ void __launch_bounds__(256) loop_products_kernel(const float *V, int6
                 h[s] = f + (int64_t)min(j0 + s, n_r - 1) * in;
             }
 #pragma unroll 4
-            for (int k = lane; k < in; k += 32) {
+            for (int k = k0 + lane; k < k1; k += 32) {
                 const float vv = __ldg(row + k);
                 if (j0 == 0) nrm = fmaf(vv, vv, nrm);
 #pragma unroll
                 for (int s = 0; s < NS; ++s) acc[s] = fmaf(vv, __ldg(h[s] + k), acc[s]);
             }
             const float z = warp_transpose_reduce<NS>(acc, lane);
-            if (lane < NS && j0 + lane < n_r) out[(j0 + lane) * classes + o] = z + bias;
+            if (parts > 1) {
+                if (lane < NS) part[b][unit][lane] = z;
+            } else {
+                const float bias = bias_of(o);
+                if (lane == 0 && j0 == 0) nrm = fmaf(bias, bias, nrm);
+                if (lane < NS && j0 + lane < n_r) out[(j0 + lane) * classes + o] = z + bias;
+            }
+        }
+        if (parts == 1) continue;
+        __syncthreads();             // the other buffer is written next
+        for (int q = threadIdx.x; q < classes * NS; q += kProductWarps * 32) {
+            const int o = q / NS, s = q - o * NS;
+            float z = 0.f;
+            for (int p = 0; p < parts; ++p) z += part[b][o * parts + p][s];
+            const float bias = bias_of(o);
+            if (j0 + s < n_r) out[(j0 + s) * classes + o] = z + bias;
+            if (j0 == 0 && s == 0) nrm = fmaf(bias, bias, nrm);
         }
     }
     nrm = loop_warp_sum(nrm);
-    if (lane == 0) part[warp] = nrm;
+    if (lane == 0) norm_part[warp] = nrm;
     __syncthreads();
     if (threadIdx.x == 0) {
         float n = 0.f;
-        for (int w = 0; w < 8; ++w) n += part[w];
+        for (int w = 0; w < kProductWarps; ++w) n += norm_part[w];
         norms[(int64_t)t * m + c] = n;
     }
 }
@@ -344,7 +363,22 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
 #endif
 }
 
+// Parts of a class: as few of up to 2,048 columns as leave the eight warps even shares, a part's start and end counting as 384
+// columns.  Iterations whose products fill a warp or two a block wait for them: 16384 x 2 of five candidates, one sample, four
+// iterations take 35 us, with a warp a class 53; 0 where there would be more than a block has room for.
+int product_parts(int in, int classes) {
+    const int least = (in + kProductCols - 1) / kProductCols;
+    int best = 0;
+    int64_t cost = 0;
+    for (int p = least; p < least + 8 && p * classes <= kProductUnits; ++p) {
+        const int64_t len = ((in + p - 1) / p + 31) / 32 * 32, c = (classes * p + kProductWarps - 1) / kProductWarps * (len + 384);
+        if (!best || c < cost) { best = p; cost = c; }
+    }
+    return best;
+}
+
 bool loop_plan(int64_t d, int in, int classes, int m, int n_r, LoopPlan *p) {
+    if (!product_parts(in, classes)) return false;
     if (classes > kLoopMaxClasses || m > kRankMax || d > (int64_t)kLoopSmem * kLoopCluster || n_r > (int)kLoopSmem) return false;
     p->G = kLoopCluster * kLoopParts;
     p->sl = (int)(((d + p->G - 1) / p->G + 7) / 8 * 8);
@@ -431,7 +465,7 @@ int64_t loop_workspace(const zeno_model_desc &desc, int64_t d, int device) {
 // iterations whose products fit the handle's room
 static int64_t loop_batch(const Context &c, int m, int n_r) { return kLoopProducts / ((int64_t)m * ((int64_t)n_r * c.desc.dims[1] + 1)); }
 
-bool loop_usable(const Context &c, int m, int n_r, int steps) {
+bool loop_usable(const Context &c, int m, int n_r, int steps, bool aligned) {
     if (!c.loop_ws || steps < kLoopMinSteps) return false;
     LoopPlan p;
     if (!loop_plan(c.d, (int)c.desc.dims[0], (int)c.desc.dims[1], m, n_r, &p) || loop_batch(c, m, n_r) < kLoopMinSteps) return false;
@@ -439,7 +473,15 @@ bool loop_usable(const Context &c, int m, int n_r, int steps) {
     // by the step's kernels and by these, us: 784 x 10 of 20 candidates 75 and 46 with 4 samples, 85 and 68 with 16, 97 and 125
     // with 32; 4096 x 4 of 12 candidates 70 and 69 with 8 samples, 81 and 106 with 16; 100 x 4 of 64 candidates 76 and 64 with
     // 16 samples, 109 and 130 with 32; 200 x 10 of 128 candidates, 8 samples: 103 and 67
-    return (p.ML * n_r + kLoopWarps - 1) / kLoopWarps <= 5 && n_r * p.n <= 8800;
+    if ((p.ML * n_r + kLoopWarps - 1) / kLoopWarps > 5 || n_r * p.n > 8800) return false;
+    // Wide models whose steps are quick, with loads of four columns and less than 12 us each: few iterations do not pay for the
+    // products and the first candidates' copies, and copies that nothing overlaps take as long as a step.  us, steps and loop:
+    // 4096 x 10 of 5 candidates, one sample, four iterations 31 and 38, eight 62 and 60; 4096 x 4 of 12, 8 samples 33 and 34, 64 and
+    // 54; 1024 x 32 of 20, one copy of 166 KB, eight 73 and 89, twenty with 4 samples 181 and 186.  2395 x 9 of 15, no such loads: four
+    // 52 and 44; 16384 x 2 of 20: four 56 and 51
+    const bool quick_steps = (aligned || m < 3) && c.desc.dims[0] < 8192;
+    if (quick_steps && steps < 8 && (p.n > 1250 || (p.bufs == 1 && n_r * p.n > 8000))) return false;
+    return !quick_steps || p.bufs == 2 || p.n <= 1400;
 }
 
 cudaError_t launch_loop(Context &c, float *x, const float *V, int64_t ldv, int64_t stride_v, int m, const float *features, const int32_t *labels,
@@ -466,6 +508,7 @@ cudaError_t launch_loop(Context &c, float *x, const float *V, int64_t ldv, int64
     // a block's stretch starts at a multiple of eight entries
     a.p.copy = reinterpret_cast<uintptr_t>(V) % 16 == 0 && ldv % 4 == 0 && stride_v % 4 == 0 ? 16 : 4;
     a.p.feature_copy = reinterpret_cast<uintptr_t>(features) % 16 == 0 && a.in % 4 == 0 ? 16 : 4;
+    const int parts = product_parts(a.in, a.classes);
     const int batch = (int)(loop_batch(c, m, n_r) < 32768 ? loop_batch(c, m, n_r) : 32768);
     const int batches = (steps + batch - 1) / batch, each = (steps + batches - 1) / batches;
     profile_mark(c, "server_loop", s);
@@ -481,10 +524,10 @@ cudaError_t launch_loop(Context &c, float *x, const float *V, int64_t ldv, int64
         *launches += 2;
         const dim3 grid(m, a.steps);
         float *norms = c.loop_ws + (int64_t)a.steps * m * n_r * a.classes;
-        cudaError_t e = n_r <= 4 ? launch_chained(loop_products_kernel<4>, grid, dim3(256), 0, s, chain_launches(c), a.V, ldv, stride_v, a.features, a.in,
-                                                  a.classes, (int)c.desc.has_bias, m, n_r, c.loop_ws, norms)
-                                 : launch_chained(loop_products_kernel<8>, grid, dim3(256), 0, s, chain_launches(c), a.V, ldv, stride_v, a.features, a.in,
-                                                  a.classes, (int)c.desc.has_bias, m, n_r, c.loop_ws, norms);
+        cudaError_t e = n_r <= 4 ? launch_chained(loop_products_kernel<4>, grid, dim3(kProductWarps * 32), 0, s, chain_launches(c), a.V, ldv, stride_v, a.features, a.in,
+                                                  a.classes, (int)c.desc.has_bias, parts, m, n_r, c.loop_ws, norms)
+                                 : launch_chained(loop_products_kernel<8>, grid, dim3(kProductWarps * 32), 0, s, chain_launches(c), a.V, ldv, stride_v, a.features, a.in,
+                                                  a.classes, (int)c.desc.has_bias, parts, m, n_r, c.loop_ws, norms);
         if (e != cudaSuccess) return e;
         e = launch_clustered(softmax_loop_kernel, kLoopCluster, dim3(kLoopCluster), dim3(kLoopThreads), (size_t)a.p.bytes, s, chain_launches(c), a);
         if (e != cudaSuccess) return e;

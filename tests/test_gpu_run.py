@@ -142,3 +142,38 @@ def test_run_argument_errors():
         assert st == zeno.ERR_INVALID_ARG                      # no iterations
         scores, idx = z.run(x.clone(), V3, f3, t3, w.gamma, w.rho, w.b)
         assert scores.shape == (2, w.m) and idx.shape == (2, w.m - w.b)
+
+
+@pytest.mark.parametrize("cols,classes,m", [(20001, 2, 4), (9000, 3, 8)])
+def test_loop_of_a_wide_model_adds_up_short_sums(cols, classes, m):
+    """The products of a wide model's candidates against 64 bits: scores that are made of them (x is small beside gamma v).  A
+    chain of n products of random signs is off by 0.41 x 2^-24 sqrt(n / 2) of its result in the root mean square: 4.5e-7 with
+    all 625 of a lane's columns of 20,001, 1.4e-7 with 64 of them; the lanes' and the parts' additions, the rounding of x
+    and of the score to binary32 add as much again."""
+    steps, gamma = 12, 0.5
+    g = torch.Generator().manual_seed(cols)
+    d = cols * classes
+    x = torch.randn(d, generator=g) * (1.0 / cols ** 0.5)
+    V = torch.randn((steps, m, d), generator=g) * (3e4 / cols ** 0.5 / gamma)
+    V[:, 0] = 0                                      # scores higher than candidates with losses of thousands
+    feats = torch.randn((steps, 1, cols), generator=g)
+    labels = torch.zeros((steps, 1), dtype=torch.int32)
+    for t in range(steps):                           # the label: where the candidates' logits are small
+        labels[t] = int((feats[t] @ V[t, 1:].sum(0).view(classes, cols).t()).argmax())
+    xg = x.cuda()
+    with zeno.Zeno(zeno.LOSS_SOFTMAX_MLP, zeno.F32, (cols, classes), False, m, 1) as z:
+        scores, idx = z.run(xg, V.cuda(), feats.cuda(), labels.cuda(), gamma, 0.0, m - 1)
+        assert z.last_launch_count == 2
+    scores, idx = scores.double().cpu(), idx.cpu()
+    err, count = 0.0, 0
+    for t in range(steps):
+        def loss(w):
+            return torch.nn.functional.cross_entropy(feats[t].double() @ w.view(classes, cols).t(), labels[t].long())
+        f0 = loss(x.double())
+        for i in range(1, m):
+            err += (scores[t, i] - (f0 - loss(x.double() - gamma * V[t, i].double()))).item() ** 2
+            count += 1
+        x = (x.double() - gamma * V[t, idx[t, 0]].double()).float()
+    assert torch.allclose(xg.cpu(), x, rtol=1e-6, atol=1e-3)
+    # a loss is the difference of two logits of 3e4, or nothing
+    assert (err / count) ** 0.5 / (3e4 * 2 ** 0.5) <= 3.2e-7

@@ -642,7 +642,7 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     const size_t at_split0 = reserve(split_elems, 4), at_split1 = reserve(split_elems, 4);
     const size_t at_losspart = reserve(rows * 8, 8), at_losssum = reserve(rows, 8);
     const size_t at_headz = reserve(head_elems, 4), at_headt = reserve(rows, 4);
-    const size_t krum_elems = m_max <= ZENO_KRUM_MAX_M ? zeno::krum_part_floats(m_max, c->sm_count > 0 ? c->sm_count : 148) : 0;
+    const size_t krum_elems = m_max <= ZENO_KRUM_MAX_M ? zeno::krum_part_floats(m_max, c->d, c->sm_count > 0 ? c->sm_count : 148) : 0;
     const int64_t loop_elems = zeno::loop_workspace(*desc, c->d, device);
     const size_t at_loop = reserve((size_t)loop_elems, 4);
     const size_t at_krum = reserve(krum_elems, 4), at_krums = reserve(m_max, 4);

@@ -197,25 +197,137 @@ krum_pairs_kernel(const T *V, int64_t ldv, int64_t d, int m, const __grid_consta
     }
 }
 
+// The pairs of fewer columns, or of rows that only copies of 4 bytes bring: 4 x 4 pairs a thread, columns staged by loads of one
+// entry, which need no alignment.  Bound by its reads of shared memory, eight for sixteen pairs, and by the loads, which nothing
+// overlaps; but a block of little code that starts and ends quickly, and one for a stretch of 128 columns.
+constexpr int kSquareCols = 128;              // columns staged per tile
+constexpr int kSquarePitch = kSquareCols + 1; // row pitch in floats: rows of a tile start in different banks
+
+__host__ __device__ inline int square_row_blocks(int m) { return (m + 3) / 4; }
+__host__ __device__ inline int square_tiles(int m) { const int mb = square_row_blocks(m); return mb * (mb + 1) / 2; }
+// groups of threads that share the pair tiles and split a tile's columns between them
+__host__ __device__ inline int square_groups(int m) { const int t = square_tiles(m); return t >= kKrumThreads ? 1 : kKrumThreads / t; }
+// shared memory of the kernel: the staged rows, or the groups' sums when those need more
+inline size_t squares_smem(int m) {
+    const size_t rows = (size_t)square_row_blocks(m) * 4 * kSquarePitch, red = (size_t)square_groups(m) * square_tiles(m) * 16;
+    return (rows > red ? rows : red) * sizeof(float);
+}
+
+// tile index -> (ib, jb) with ib <= jb, row by row of the upper triangle of blocks of four rows
+__device__ __forceinline__ void square_tile_of(int tile, int mb, int &ib, int &jb) {
+    ib = 0;
+    int left = tile;
+    while (left >= mb - ib) { left -= mb - ib; ++ib; }
+    jb = ib + left;
+}
+
+// part[block][tile][4][4]: sums of squared differences of the 4 x 4 pairs (i, j) of a tile over the
+// columns this block took.  With fewer tiles than threads, groups of threads split a staged tile's
+// columns and their sums are added in group order before they are written.
+// kMaxMine: pair tiles a thread may hold (1 while the tiles are fewer than the threads, else 2).
+template <typename T, int kMaxMine>
+__global__ void __launch_bounds__(kKrumThreads, kMaxMine == 1 ? 4 : 3) krum_squares_kernel(const T *V, int64_t ldv, int64_t d, int m, float *part) {
+    extern __shared__ float rows[];           // [m rounded up to 4][kSquarePitch], then [groups][tiles][16]
+    pdl_wait();
+    pdl_launch_dependents();
+    const int mb = square_row_blocks(m), tiles = square_tiles(m), groups = square_groups(m);
+    const int m4 = mb * 4;
+    const int tid = threadIdx.x;
+    const bool shared_tiles = tiles < kKrumThreads;                 // one tile a thread, groups of threads
+    const int group = tid / tiles < groups ? tid / tiles : -1;      // threads beyond groups * tiles idle
+    const int n_mine = shared_tiles ? (group >= 0 ? 1 : 0) : (tiles - tid + kKrumThreads - 1) / kKrumThreads;
+    float acc[kMaxMine][16];
+#pragma unroll
+    for (int q = 0; q < kMaxMine; ++q)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[q][e] = 0.f;
+    for (int64_t j0 = (int64_t)blockIdx.x * kSquareCols; j0 < d; j0 += (int64_t)gridDim.x * kSquareCols) {
+        __syncthreads();
+#pragma unroll 8
+        for (int t = tid; t < m4 * kSquareCols; t += kKrumThreads) {
+            const int r = t / kSquareCols, c = t - r * kSquareCols;
+            rows[r * kSquarePitch + c] = (r < m && j0 + c < d) ? load_elem(V + (int64_t)r * ldv + j0 + c) : 0.f;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kMaxMine; ++q) {
+            if (q >= n_mine) break;
+            const int tile = shared_tiles ? tid - group * tiles : tid + q * kKrumThreads;
+            int ib, jb;
+            square_tile_of(tile, mb, ib, jb);
+            const float *ri = rows + ib * 4 * kSquarePitch, *rj = rows + jb * 4 * kSquarePitch;
+            const int c0 = shared_tiles ? group : 0, cs = shared_tiles ? groups : 1;
+#pragma unroll(kMaxMine == 1 ? 4 : 1)
+            for (int c = c0; c < kSquareCols; c += cs) {
+                float a[4], b[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    a[u] = ri[u * kSquarePitch + c];
+                    b[u] = rj[u * kSquarePitch + c];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) {
+                        const float df = a[u] - b[w];
+                        acc[q][u * 4 + w] = fmaf(df, df, acc[q][u * 4 + w]);
+                    }
+            }
+        }
+    }
+    float *dst = part + (int64_t)blockIdx.x * tiles * 16;
+    if (!shared_tiles) {
+#pragma unroll
+        for (int q = 0; q < kMaxMine; ++q) {
+            if (q >= n_mine) break;
+            float *o = dst + (tid + q * kKrumThreads) * 16;
+#pragma unroll
+            for (int e = 0; e < 16; e += 4) *reinterpret_cast<float4 *>(o + e) = make_float4(acc[q][e], acc[q][e + 1], acc[q][e + 2], acc[q][e + 3]);
+        }
+        return;
+    }
+    __syncthreads();                          // the staged rows are done with: the groups' sums take their place
+    if (group >= 0) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) rows[tid * 16 + e] = acc[0][e];       // tid = group * tiles + tile
+    }
+    __syncthreads();
+    for (int t = tid; t < tiles * 16; t += kKrumThreads) {
+        float sum = 0.f;
+        for (int g = 0; g < groups; ++g) sum += rows[g * tiles * 16 + t];
+        dst[t] = sum;
+    }
+}
+
 // Candidate i = blockIdx.x: its distances to the others, the blocks' partial sums added in a fixed order (a warp an entry:
 // lanes take every 32nd block and their sums meet in a butterfly, in double; a NaN distance counts as plus infinity),
 // then the sum of the m - b - 2 smallest: a distance belongs to it if fewer than that many others are smaller, or equal
 // and of a lower index.
 constexpr int kSumsWarps = 32;                // one round of entries up to 32 candidates
+template <bool SQUARES>
 __global__ void __launch_bounds__(kSumsWarps * 32) krum_sums_kernel(const float *part, int slabs, int m, int b,
                                                                     const __grid_constant__ KrumPlan plan, float *sums_out, float *sums_ws) {
     __shared__ float dist[ZENO_KRUM_MAX_M];
     __shared__ double warp_part[kSumsWarps];
     pdl_wait();
     pdl_launch_dependents();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x, B = plan.B;
-    const int64_t slab = (int64_t)plan.tiles * B * B;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x, B = SQUARES ? 4 : plan.B;
+    const int tiles = SQUARES ? square_tiles(m) : plan.tiles;
+    const int64_t slab = (int64_t)tiles * B * B;
     for (int j = warp; j < m; j += kSumsWarps) {
         const int lo = min(i, j), hi = max(i, j), ia = lo / B, ib = hi / B, r = lo - ia * B, q = hi - ib * B;
-        const int e = ia != ib ? q * B + r : (ia & 1) * (B * (B - 1) / 2) + q * (q - 1) / 2 + r;
-        const float *src = part + (int64_t)plan.at[ia][ib] * B * B + (i == j ? 0 : e);
+        int tile, e;
+        if (SQUARES) {
+            const int mb = square_row_blocks(m);
+            tile = ia * mb - ia * (ia - 1) / 2 + (ib - ia);
+            e = r * B + q;
+        } else {
+            tile = plan.at[ia][ib];
+            e = ia != ib ? q * B + r : (ia & 1) * (B * (B - 1) / 2) + q * (q - 1) / 2 + r;
+        }
+        const float *src = part + (int64_t)tile * B * B + (i == j ? 0 : e);
         double s = 0.0;
-#pragma unroll 4
+#pragma unroll(SQUARES ? 8 : 4)
         for (int q = lane; q < slabs; q += 32) s += (double)__ldcg(src + q * slab);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -365,6 +477,44 @@ cudaError_t launch_pairs_of(Context &c, const KrumPlan &p, const T *V, int64_t l
     }
 }
 
+// Which of the two kernels takes the pairs.  Few columns: less than a stretch of 96 for every SM, 128 where rows are not aligned to 16
+// bytes, are over sooner in little code than register tiles are filled and emptied, with 13 to 48 candidates (42 of aligned bfloat16
+// rows; up to 88 of rows that are not aligned, where most threads have a tile, and 48 columns for every SM).  All three launches, 4 x 4
+// and register tiles: 20 candidates of 6,000 binary32 columns 8.7 us and 10.0, of 400 k 42 and 23; 34 of 8,000, bfloat16 rows of odd
+// pitch 12.6 and 17.3.  Many columns of more than 56 candidates, rows not aligned, where most threads have a tile: a block of the
+// register tiles stages many rows there by copies of 4 bytes, up to nine times over (88 of 300 k: 187 us and 262, bfloat16 183 and
+// 265; 112: 344 and 428, of 30 k 84 and 59).  With few of the last round's threads busy, as at 92, it is the other way.
+bool krum_by_squares(int m, int64_t d, int sms, int entry_bytes, bool wide) {
+    if (m <= 12) return false;
+    const int rounds = (square_tiles(m) + kKrumThreads - 1) / kKrumThreads;
+    const int64_t pairs = (int64_t)m * (m - 1) / 2, places = (int64_t)rounds * kKrumThreads * 16;
+    const bool busy = rounds <= 2 && square_groups(m) * pairs * 100 >= places * 57;
+    const int few = wide ? (m <= (entry_bytes == 4 ? 48 : 42) ? 96 : 0) : m <= 48 ? 128 : m <= 88 && busy ? 48 : 0;
+    if (d <= (int64_t)few * sms) return true;
+    return !wide && m > 56 && busy && d > (int64_t)768 * sms;
+}
+int square_blocks(int m, int64_t d, int sms) {
+    int per_sm = (int)((200u << 10) / squares_smem(m));
+    per_sm = per_sm > 4 ? 4 : per_sm;          // what the registers let be resident
+    const int64_t want = (d + kSquareCols - 1) / kSquareCols, most = (int64_t)per_sm * sms;
+    return (int)(want < most ? want : most);
+}
+
+template <typename T>
+cudaError_t launch_squares(Context &c, const T *V, int64_t ldv, int m, cudaStream_t s, int *blocks) {
+    static PerDeviceOnce attr_set;
+    if (attr_set.need(c.device)) {
+        cudaError_t e = cudaFuncSetAttribute(krum_squares_kernel<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)squares_smem(ZENO_KRUM_MAX_M));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(krum_squares_kernel<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)squares_smem(ZENO_KRUM_MAX_M));
+        if (e != cudaSuccess) return e;
+        attr_set.mark(c.device);
+    }
+    *blocks = square_blocks(m, c.d, c.sm_count > 0 ? c.sm_count : 148);
+    return launch_chained(square_tiles(m) < kKrumThreads ? krum_squares_kernel<T, 1> : krum_squares_kernel<T, 2>, dim3(*blocks), dim3(kKrumThreads),
+                          squares_smem(m), s, chain_launches(c), V, ldv, c.d, m, c.krum_part);
+}
+
 template <typename T>
 cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b, float *out, int32_t *k, float *sums,
                               cudaStream_t s) {
@@ -373,10 +523,13 @@ cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b,
     const KrumPlan p = krum_plan(m);
     int blocks = 0;
     const bool wide = reinterpret_cast<uintptr_t>(V) % 16 == 0 && (ldv * (int64_t)sizeof(T)) % 16 == 0;
-    cudaError_t e = wide ? launch_pairs_of<T, true>(c, p, V, ldv, m, s, &blocks) : launch_pairs_of<T, false>(c, p, V, ldv, m, s, &blocks);
+    cudaError_t e;
+    const bool squares = krum_by_squares(m, d, sms, (int)sizeof(T), wide);
+    if (squares) e = launch_squares(c, V, ldv, m, s, &blocks);
+    else e = wide ? launch_pairs_of<T, true>(c, p, V, ldv, m, s, &blocks) : launch_pairs_of<T, false>(c, p, V, ldv, m, s, &blocks);
     if (e != cudaSuccess) return e;
-    e = launch_chained(krum_sums_kernel, dim3(m), dim3(kSumsWarps * 32), 0, s, chain_launches(c), (const float *)c.krum_part, blocks, m, b, p, sums,
-                       c.krum_sums);
+    e = launch_chained(squares ? krum_sums_kernel<true> : krum_sums_kernel<false>, dim3(m), dim3(kSumsWarps * 32), 0, s, chain_launches(c),
+                       (const float *)c.krum_part, blocks, m, b, p, sums, c.krum_sums);
     if (e != cudaSuccess) return e;
     const int64_t cw = (d + 255) / 256;
     const int cblocks = !out ? 1 : (int)(cw < (int64_t)sms * 8 ? (cw < 1 ? 1 : cw) : (int64_t)sms * 8);
@@ -386,14 +539,18 @@ cudaError_t launch_krum_typed(Context &c, const T *V, int64_t ldv, int m, int b,
 
 }  // namespace
 
-// floats of Krum's workspace for up to m_max candidates: the blocks' sums of every tile's pairs
-size_t krum_part_floats(int m_max, int sms) {
+// floats of Krum's workspace for up to m_max candidates of d columns: the blocks' sums of every tile's pairs
+size_t krum_part_floats(int m_max, int64_t d, int sms) {
     size_t most = 0;
     KrumPlan p;
     for (int m = 1; m <= m_max; ++m) {
         krum_size(m, &p);
         const size_t need = (size_t)krum_grid_x(p, sms) * p.tiles * p.B * p.B;
         if (need > most) most = need;
+        if (krum_by_squares(m, d, sms, 4, false)) {               // and with it the calls of aligned rows and of bfloat16
+            const size_t squares = (size_t)square_blocks(m, d, sms) * square_tiles(m) * 16;
+            if (squares > most) most = squares;
+        }
     }
     return most;
 }

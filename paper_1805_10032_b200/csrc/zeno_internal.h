@@ -304,7 +304,7 @@ cudaError_t launch_loop(Context &c, float *x, const float *V, int64_t ldv, int64
                         int n_r, int steps, float gamma, float rho, int keep, float *scores, int32_t *idx, cudaStream_t s, int *launches);
 
 // The paper's baseline aggregation rules on the same V (zeno_baselines.cu).
-size_t krum_part_floats(int m_max, int sms);
+size_t krum_part_floats(int m_max, int64_t d, int sms);
 cudaError_t launch_median(Context &c, const void *V, int64_t ldv, int m, float *out, cudaStream_t s, int *launches);
 cudaError_t launch_krum(Context &c, const void *V, int64_t ldv, int m, int b, float *out, int32_t *k, float *sums,
                         cudaStream_t s, int *launches);

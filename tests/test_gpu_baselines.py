@@ -183,7 +183,50 @@ def test_krum_over_its_tiles(oracle, m, dtype, d, pad):
     # sums of d squares in binary32: relative error below d / lanes * 2^-24, far within
     assert np.allclose(sums, sums_orc, rtol=2e-5, atol=0)
     assert k.item() == int(np.argmin(sums))
+    assert sums[0] == sums[m - 1]
     assert torch.equal(out.cpu(), V[k.item(), :d].float())
+
+
+# every stage of the ring of staged columns used again and again, the last one ragged: at least five stretches a block, of 64 to
+# 256 columns; few candidates and many; copies of 16 and of 4 bytes, rows of odd pitch and rows that start at an odd entry (bfloat16:
+# in the second half of 4 bytes, in turn or all of them).  Two identical rows are the best ones: the first of them wins
+@pytest.mark.parametrize("m,d,b", [(20, 400004, 6), (42, 130004, 20), (48, 40004, 10), (64, 100004, 21), (96, 60004, 8), (128, 24004, 50)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("pad,start", [(4, 0), (5, 0), (4, 1), (5, 1)])
+def test_krum_of_many_columns(oracle, m, d, b, dtype, pad, start):
+    krum_with_two_best_rows(oracle, m, d, b, dtype, pad, start)
+
+
+# the last sizes 4 x 4 pairs a thread take, and the first beyond, either way: 96 columns for every SM (128 where rows are not aligned,
+# 48 with 49 to 88 candidates; 768 for many), 12, 42, 48, 56, 88, 97, 124 candidates and their neighbours, one and two tiles a thread,
+# stretches with a remainder, one and several groups of threads
+@pytest.mark.parametrize("m,d,pad,start", [(m, *shape) for m in (12, 13, 24, 42, 43, 48, 49) for shape in
+                                           ((300, 0, 0), (1027, 0, 1), (14208, 0, 0), (14216, 0, 0), (18943, 0, 0), (18945, 0, 0))] +
+                         [(m, d, 1, 0) for m in (49, 88, 89) for d in (7104, 7106)] +
+                         [(m, d, 1, 0) for m in (57, 60, 61, 69, 88, 89, 97, 98, 112, 124, 125) for d in (113664, 113666)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_krum_by_either_kernel(oracle, m, dtype, d, pad, start):
+    krum_with_two_best_rows(oracle, m, d, m // 3, dtype, pad, start)
+
+
+def krum_with_two_best_rows(oracle, m, d, b, dtype, pad, start):
+    store = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(m + d)
+    ldv = d + pad
+    room = torch.full((start + m * ldv,), float("nan"), dtype=store, device="cuda")
+    V = room[start:].view(m, ldv)
+    V[:, :d] = torch.randn(d, generator=g, device="cuda").to(store)
+    V[1:m - 1, :d] += (torch.randn((m - 2, d), generator=g, device="cuda") * torch.linspace(0.5, 0.8, m - 2, device="cuda")[:, None]).to(store)
+    kind, dims = (0, ((d - 2) // 2, 2) if d % 2 == 0 else (d - 1, 1)) if dtype == "bf16" else (1, (d, 1))
+    _, sums_orc, _ = oracle.krum(int(dtype == "bf16"), syn.to_numpy_params(V.cpu()), ldv, d, m, b)
+    with zeno.Zeno(kind, int(dtype == "bf16"), dims, True, m, 1) as z:
+        assert z.d == d
+        out, k, sums = z.krum(V, b, ldv=ldv)
+    sums = sums.cpu().numpy().astype(np.float64)
+    # chains of up to d / 32 squares of one sign in binary32: far within
+    assert np.allclose(sums, sums_orc, rtol=2e-5, atol=0)
+    assert sums[0] == sums[m - 1] and k.item() == 0
+    assert torch.equal(out, V[0, :d].float())
 
 
 def test_krum_toy_example_on_the_gpu():

@@ -643,9 +643,8 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     const size_t at_losspart = reserve(rows * 8, 8), at_losssum = reserve(rows, 8);
     const size_t at_headz = reserve(head_elems, 4), at_headt = reserve(rows, 4);
     const size_t krum_elems = m_max <= ZENO_KRUM_MAX_M ? zeno::krum_part_floats(m_max, c->d, c->sm_count > 0 ? c->sm_count : 148) : 0;
-    const int64_t loop_elems = zeno::loop_workspace(*desc, c->d, device);
-    const size_t at_loop = reserve((size_t)loop_elems, 4);
-    const size_t at_krum = reserve(krum_elems, 4), at_krums = reserve(m_max, 4);
+    const size_t loop_elems = (size_t)zeno::loop_workspace(*desc, c->d, m_max, n_r_max);
+    const size_t at_krum = reserve(krum_elems > loop_elems ? krum_elems : loop_elems, 4), at_krums = reserve(m_max, 4);
 
     // Last what depends on where convolutional layers run: on the tensor cores, in a workspace of their own, beside which
     // only the dense layer's input and the logits are kept; with no room for that, on the CUDA cores, between two buffers
@@ -691,7 +690,8 @@ zeno_status zeno_create(zeno_handle *out, const zeno_model_desc *desc, int32_t m
     c->act_split[1] = base + at_split1;
     c->head_zpart = head_elems ? reinterpret_cast<float *>(base + at_headz) : nullptr;
     c->head_tickets = reinterpret_cast<unsigned *>(base + at_headt);
-    c->loop_ws = loop_elems ? reinterpret_cast<float *>(base + at_loop) : nullptr;
+    c->loop_ws = loop_elems ? reinterpret_cast<float *>(base + at_krum) : nullptr;
+    c->loop_floats = (int64_t)loop_elems;
     c->krum_part = krum_elems ? reinterpret_cast<float *>(base + at_krum) : nullptr;
     c->krum_sums = reinterpret_cast<float *>(base + at_krums);
     if (c->cnn_net.layers) c->cnn_ws = reinterpret_cast<float *>(base + at_cnn);

@@ -87,7 +87,8 @@ struct Context {
     // Krum: per-block partial sums of the pairs' squared distances, and the candidates' sums
     float *krum_part;               // NULL when m_max is beyond ZENO_KRUM_MAX_M
     float *krum_sums;               // [m_max]
-    float *loop_ws;                 // the server loop's products of many iterations, or NULL
+    float *loop_ws;                 // the server loop's products of many iterations, in the place of krum_part, or NULL
+    int64_t loop_floats;
     void *host_stage;               // device copies of host inputs (zeno_step_host), grown on demand
     void *tmap_cache;               // encoded tensor maps of the tensor-core kernels (host memory, malloc'ed), or NULL
     size_t host_stage_bytes;
@@ -298,7 +299,7 @@ cudaError_t launch_split_acts(Context &c, const float *H, int models, int n_r, i
 
 // The server loop of a small binary32 softmax regression in two launches (zeno_loop.cu).  Shorter loops are as many steps.
 constexpr int kLoopMinSteps = 4;
-int64_t loop_workspace(const zeno_model_desc &desc, int64_t d, int device);
+int64_t loop_workspace(const zeno_model_desc &desc, int64_t d, int m_max, int n_r_max);
 bool loop_usable(const Context &c, int m, int n_r, int steps, bool aligned);   // rows aligned to four elements
 cudaError_t launch_loop(Context &c, float *x, const float *V, int64_t ldv, int64_t stride_v, int m, const float *features, const int32_t *labels,
                         int n_r, int steps, float gamma, float rho, int keep, float *scores, int32_t *idx, cudaStream_t s, int *launches);

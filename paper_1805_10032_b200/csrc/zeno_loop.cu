@@ -27,7 +27,9 @@ constexpr int kLoopMaxClasses = 32;              // a lane a class
 constexpr int kLoopParts = 4;                    // parts of a block's stretch
 constexpr int kLoopSamples = 4;                  // samples a warp takes at a time
 constexpr size_t kLoopSmem = 220 * 1024;
-constexpr int64_t kLoopProducts = 1 << 20;       // floats of products a handle holds
+constexpr int kLoopLosses = 5;                   // losses a warp takes one after another, at most
+constexpr int kLoopBatch = 32;                   // iterations whose products a handle has room for, at least,
+constexpr int64_t kLoopProducts = 1 << 20;       // but no more floats than this
 
 // How a cluster divides a model, and where a block's shared memory holds what (bytes from its start; x at 0).
 struct LoopPlan {
@@ -428,7 +430,8 @@ cudaError_t set_attributes() {
     return e;
 }
 
-// Whether the device, the current one, holds the cluster: asked once (the answer takes two milliseconds).
+// Whether the device, the current one, holds the cluster: asked once, by the first loop that could use it (the answer takes two
+// milliseconds).  The functions' attributes are set on the way.
 bool cluster_fits(int device) {
     static std::atomic<signed char> known[kMaxDevices];          // 0: not asked, 1: yes, -1: no
     const bool keep = device >= 0 && device < kMaxDevices;
@@ -445,25 +448,30 @@ bool cluster_fits(int device) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    const bool fits = set_attributes() == cudaSuccess && cudaOccupancyMaxActiveClusters(&n, softmax_loop_kernel, &cfg) == cudaSuccess && n >= 1;
-    if (!fits) cudaGetLastError();
-    if (keep) known[device].store(fits ? 1 : -1, std::memory_order_relaxed);
-    return fits;
+    if (set_attributes() != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, softmax_loop_kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();          // no answer: the steps' kernels this time
+        return false;
+    }
+    if (keep) known[device].store(n >= 1 ? 1 : -1, std::memory_order_relaxed);
+    return n >= 1;
 }
 
 }  // namespace
 
-// Floats of the products a handle keeps room for, 0 where it never takes this path: another model, a device that does not
-// hold the cluster, sizes beyond the shared memory with the fewest candidates and samples.
-int64_t loop_workspace(const zeno_model_desc &desc, int64_t d, int device) {
+// Floats of the products a handle keeps room for, 0 where it never takes this path: another model, sizes beyond the shared
+// memory with the fewest candidates and samples.  They lie where Krum's partial sums do: a handle's calls are ordered.
+int64_t loop_workspace(const zeno_model_desc &desc, int64_t d, int m_max, int n_r_max) {
     if (desc.kind != ZENO_LOSS_SOFTMAX_MLP || desc.n_layers != 1 || desc.param_dtype != ZENO_F32) return 0;
     LoopPlan p;
     if (desc.dims[0] > (1 << 20) || desc.dims[1] > kLoopMaxClasses || !loop_plan(d, (int)desc.dims[0], (int)desc.dims[1], 1, 1, &p)) return 0;
-    return cluster_fits(device) ? kLoopProducts : 0;
+    // most of m n_r: the m candidates are less than a block's models times the blocks
+    const int64_t most = kLoopLosses * kLoopWarps * kLoopCluster, rows = (int64_t)m_max * n_r_max < most ? (int64_t)m_max * n_r_max : most;
+    const int64_t need = kLoopBatch * (rows * desc.dims[1] + m_max);
+    return need < kLoopProducts ? need : kLoopProducts;
 }
 
 // iterations whose products fit the handle's room
-static int64_t loop_batch(const Context &c, int m, int n_r) { return kLoopProducts / ((int64_t)m * ((int64_t)n_r * c.desc.dims[1] + 1)); }
+static int64_t loop_batch(const Context &c, int m, int n_r) { return c.loop_floats / ((int64_t)m * ((int64_t)n_r * c.desc.dims[1] + 1)); }
 
 bool loop_usable(const Context &c, int m, int n_r, int steps, bool aligned) {
     if (!c.loop_ws || steps < kLoopMinSteps) return false;
@@ -473,7 +481,7 @@ bool loop_usable(const Context &c, int m, int n_r, int steps, bool aligned) {
     // by the step's kernels and by these, us: 784 x 10 of 20 candidates 75 and 46 with 4 samples, 85 and 68 with 16, 97 and 125
     // with 32; 4096 x 4 of 12 candidates 70 and 69 with 8 samples, 81 and 106 with 16; 100 x 4 of 64 candidates 76 and 64 with
     // 16 samples, 109 and 130 with 32; 200 x 10 of 128 candidates, 8 samples: 103 and 67
-    if ((p.ML * n_r + kLoopWarps - 1) / kLoopWarps > 5 || n_r * p.n > 8800) return false;
+    if ((p.ML * n_r + kLoopWarps - 1) / kLoopWarps > kLoopLosses || n_r * p.n > 8800) return false;
     // Wide models whose steps are quick, with loads of four columns and less than 12 us each: few iterations do not pay for the
     // products and the first candidates' copies, and copies that nothing overlaps take as long as a step.  us, steps and loop:
     // 4096 x 10 of 5 candidates, one sample, four iterations 31 and 38, eight 62 and 60; 4096 x 4 of 12, 8 samples 33 and 34, 64 and
@@ -481,17 +489,11 @@ bool loop_usable(const Context &c, int m, int n_r, int steps, bool aligned) {
     // 52 and 44; 16384 x 2 of 20: four 56 and 51
     const bool quick_steps = (aligned || m < 3) && c.desc.dims[0] < 8192;
     if (quick_steps && steps < 8 && (p.n > 1250 || (p.bufs == 1 && n_r * p.n > 8000))) return false;
-    return !quick_steps || p.bufs == 2 || p.n <= 1400;
+    return (!quick_steps || p.bufs == 2 || p.n <= 1400) && cluster_fits(c.device);
 }
 
 cudaError_t launch_loop(Context &c, float *x, const float *V, int64_t ldv, int64_t stride_v, int m, const float *features, const int32_t *labels,
                         int n_r, int steps, float gamma, float rho, int keep, float *scores, int32_t *idx, cudaStream_t s, int *launches) {
-    static PerDeviceOnce attr_set;
-    if (attr_set.need(c.device)) {
-        cudaError_t e = set_attributes();
-        if (e != cudaSuccess) return e;
-        attr_set.mark(c.device);
-    }
     LoopArgs a;
     a.x = x;
     a.ldv = ldv;

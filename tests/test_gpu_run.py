@@ -177,3 +177,50 @@ def test_loop_of_a_wide_model_adds_up_short_sums(cols, classes, m):
     assert torch.allclose(xg.cpu(), x, rtol=1e-6, atol=1e-3)
     # a loss is the difference of two logits of 3e4, or nothing
     assert (err / count) ** 0.5 / (3e4 * 2 ** 0.5) <= 3.2e-7
+
+
+def test_handles_of_small_models_are_small():
+    """The loop's products have no room of their own beyond a few iterations': 64 handles of the smallest model."""
+    handles = [zeno.Zeno(zeno.LOSS_SOFTMAX_MLP, zeno.F32, (784, 10), True, 20, 4)]
+    before = torch.cuda.mem_get_info()[0]
+    handles += [zeno.Zeno(zeno.LOSS_SOFTMAX_MLP, zeno.F32, (784, 10), True, 20, 4) for _ in range(64)]
+    used = before - torch.cuda.mem_get_info()[0]
+    for z in handles:
+        z.close()
+    assert used <= 64 * (2 << 20)
+
+
+FIRST_CALL = """
+import sys, torch
+sys.path[:0] = [{root!r}, {tests!r}]
+from paper_1805_10032_b200 import synthetic as syn, zeno
+w = syn.make_config(1)
+V, f, t = (v.repeat(6, *([1] * v.dim())).cuda() for v in (w.V, w.features, w.targets))
+with zeno.from_workload(w) as z, zeno.from_workload(w) as other:
+    x, y = w.x.cuda(), w.x.cuda()
+    scores, idx = torch.zeros((6, w.m), device="cuda"), torch.zeros((6, w.m - w.b), dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        z.run(x, V, f, t, w.gamma, w.rho, w.b, scores=scores, idx=idx)
+    assert z.last_launch_count == 2
+    g.replay()
+    want, want_idx = other.run(y, V, f, t, w.gamma, w.rho, w.b)
+    torch.cuda.synchronize()
+    assert torch.equal(x, y) and torch.equal(scores, want) and torch.equal(idx, want_idx)
+    # Krum in between uses the same room
+    other.krum(w.V.cuda(), w.b)
+    y = w.x.cuda()
+    again, _ = other.run(y, V, f, t, w.gamma, w.rho, w.b)
+    assert torch.equal(x, y) and torch.equal(scores, again)
+print("captured")
+"""
+
+
+def test_the_first_loop_of_a_process_can_be_captured():
+    import os
+    import subprocess
+    import sys
+    tests = os.path.dirname(os.path.abspath(__file__))
+    out = subprocess.run([sys.executable, "-c", FIRST_CALL.format(root=os.path.dirname(tests), tests=tests)], capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0 and "captured" in out.stdout, out.stderr[-2000:]

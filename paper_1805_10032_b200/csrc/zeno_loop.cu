@@ -61,11 +61,6 @@ __device__ __forceinline__ void loop_copy(void *dst, const void *src) { cp_async
 __device__ __forceinline__ void cluster_store_double(uint32_t addr, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
 }
-__device__ __forceinline__ float loop_warp_sum(float v) {
-#pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-    return v;
-}
 // the largest of the lanes' values (a NaN with its sign clear counts as larger than all)
 __device__ __forceinline__ float loop_warp_max(float v) {
     const int b = __float_as_int(v), k = __reduce_max_sync(0xffffffffu, b ^ ((b >> 31) & 0x7fffffff));
@@ -80,11 +75,6 @@ __device__ __forceinline__ void loop_wait() {
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-#ifdef LOOP_CLOCK
-#define TICK(i) if (tid == 0 && rank == 0) { const long long now_ = clock64(); ticks[i] += now_ - last_; last_ = now_; }
-#else
-#define TICK(i)
-#endif
 
 // products[t][c][j][o] = sum_k features[t][j][k] V[t][c][o][k] + the candidate's bias entry o; norms[t][c] = ||v||^2.
 // A block per candidate and iteration, a warp per class and part of the columns, lanes along the columns, NS samples at a time.
@@ -141,7 +131,7 @@ __global__ void __launch_bounds__(kProductWarps * 32) loop_products_kernel(const
             if (j0 == 0 && s == 0) nrm = fmaf(bias, bias, nrm);
         }
     }
-    nrm = loop_warp_sum(nrm);
+    nrm = warp_sum(nrm);
     if (lane == 0) norm_part[warp] = nrm;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -176,9 +166,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
     const int f_sample = (kLoopWarps - 1 - warp) / split, f_part = (kLoopWarps - 1 - warp) - f_sample * split;
     // a lane's place in the other blocks when it hands out a warp's four sums: sample lane % 4, blocks lane / 4 and 8 on
     const uint32_t z_a = cluster_addr(zpart, lane >> 2), z_b = cluster_addr(zpart, 8 + (lane >> 2));
-#ifdef LOOP_CLOCK
-    long long ticks[8] = {}, last_ = clock64();
-#endif
 
     pdl_wait();                      // no early trigger: x is written here and read through the read-only path elsewhere
     auto load = [&](int t, int buf) {            // the last warps first: the first ones have products to take
@@ -225,7 +212,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
         const int buf = p.bufs == 2 ? t & 1 : 0;
         cp_async_wait<0>();
         __syncthreads();             // x is updated and this iteration's inputs are here
-        TICK(0)
         const float *vs = reinterpret_cast<const float *>(sm + p.at_v + buf * p.v_bytes);
         const float *hs = reinterpret_cast<const float *>(sm + p.at_h + buf * p.h_bytes);
 
@@ -257,7 +243,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
             for (int u = max(nw - p0, 0) + warp; u < own; u += kLoopWarps)
                 if (lane < kLoopCluster) cluster_store(cluster_addr(biasw + p0 + u - nw, lane), xs[u]);
         }
-        TICK(1)
         loop_arrive();               // what the others wait for is on its way
         if (t + 1 < a.steps) {
             if (p.bufs == 2) {
@@ -269,9 +254,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (int64_t)i * a.ldv * 4 + q));
             }
         }
-        TICK(2)
         loop_wait();
-        TICK(3)
 
         // ---- 2: losses of this block's models
         const float *prod = reinterpret_cast<const float *>(sm + p.at_prod + buf * p.prod_bytes);
@@ -291,7 +274,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
 #pragma unroll
                 for (int s = 16; s >= 1; s >>= 1) ref = fmax(ref, __shfl_xor_sync(0xffffffffu, ref, s));
             }
-            const float se = loop_warp_sum(lane < a.classes ? expf((float)(z - ref)) : 0.f);      // a NaN logit makes se NaN
+            const float se = warp_sum(lane < a.classes ? expf((float)(z - ref)) : 0.f);      // a NaN logit makes se NaN
             int l = lab_s[buf * a.n_r + j];
             if (l < 0 || l >= a.classes) l = 0;
             const double zl = __shfl_sync(0xffffffffu, z, l);
@@ -316,9 +299,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
                 if (lane < kLoopCluster) cluster_store_double(cluster_addr(lossd + lm * kLoopCluster + rank, lane), l);
             }
         }
-        TICK(4)
         cluster_barrier();
-        TICK(5)
 
         // ---- 3: scores, ranking, average, update
         const float *norm = reinterpret_cast<const float *>(sm + p.at_norm + buf * p.norm_bytes);
@@ -344,7 +325,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
             }
         }
         __syncthreads();
-        TICK(6)
         for (int q = tid; q < own; q += kLoopThreads) {
             float acc = 0.f;
 #pragma unroll 8
@@ -355,14 +335,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) softmax_loop_kernel(const __g
             __syncthreads();         // the candidates have been read
             load(t + 1, 0);
         }
-        TICK(7)
     }
     for (int q = tid; q < own; q += kLoopThreads) a.x[p0 + q] = xs[q];
-#ifdef LOOP_CLOCK
-    if (tid == 0 && rank == 0)
-        printf("cycles an iteration: wait %lld products %lld load %lld barrier %lld loss %lld barrier %lld rank %lld average %lld\n", ticks[0] / a.steps, ticks[1] / a.steps,
-               ticks[2] / a.steps, ticks[3] / a.steps, ticks[4] / a.steps, ticks[5] / a.steps, ticks[6] / a.steps, ticks[7] / a.steps);
-#endif
 }
 
 // Parts of a class: as few of up to 2,048 columns as leave the eight warps even shares, a part's start and end counting as 384

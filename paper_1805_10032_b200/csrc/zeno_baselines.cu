@@ -34,7 +34,7 @@ constexpr int kKrumBlocksPerSm = 2;
 constexpr int kKrumMaxBlocks = 16;            // row blocks
 constexpr int kKrumMaxTiles = kKrumMaxBlocks * kKrumMaxBlocks / 2;
 constexpr int kKrumPad = 8;                   // entries between staged rows: rows stay aligned to 16 bytes
-constexpr int kKrumMaxRows = 128;             // staged by a block
+constexpr int kKrumMaxRows = 90;              // staged by a block, of any plan for up to ZENO_KRUM_MAX_M candidates
 
 struct KrumPlan {
     int B, nb;                                // rows of a block, blocks
@@ -45,7 +45,8 @@ struct KrumPlan {
     unsigned char at[kKrumMaxBlocks][kKrumMaxBlocks];          // the tile of two blocks
 };
 
-// columns staged at a time: as many as leave room for two blocks an SM (three stages of 28, 70 and 128 binary32 rows)
+// columns staged at a time: as many as leave room for two blocks an SM (three stages of 28, 70 and 90 binary32 rows).
+// bfloat16 rows always have room for 128 columns, the plans of blocks of three and five rows for 256
 inline int krum_cols(int rows, int entry_bytes) { return rows * entry_bytes <= 28 * 4 ? 256 : rows * entry_bytes <= 70 * 4 ? 128 : 64; }
 
 __device__ __forceinline__ float krum_value(const float *p) { return *p; }
@@ -461,9 +462,13 @@ cudaError_t launch_pairs(Context &c, const KrumPlan &p, const T *V, int64_t ldv,
         if (n > rows) rows = n;
     }
     const int cols = krum_cols(rows, sizeof(T));
-    if (cols == 256) return launch_pairs_cols<T, B, 256, WIDE>(c, p, rows, V, ldv, m, s, blocks);
-    if (B >= 7 && cols == 128) return launch_pairs_cols<T, B < 7 ? 7 : B, 128, WIDE>(c, p, rows, V, ldv, m, s, blocks);
-    return launch_pairs_cols<T, B < 7 ? 7 : B, 64, WIDE>(c, p, rows, V, ldv, m, s, blocks);
+    if constexpr (B >= 7) {
+        if constexpr (B >= 8 && sizeof(T) == 4) {
+            if (cols == 64) return launch_pairs_cols<T, B, 64, WIDE>(c, p, rows, V, ldv, m, s, blocks);
+        }
+        if (cols != 256) return launch_pairs_cols<T, B, 128, WIDE>(c, p, rows, V, ldv, m, s, blocks);
+    }
+    return launch_pairs_cols<T, B, 256, WIDE>(c, p, rows, V, ldv, m, s, blocks);
 }
 
 template <typename T, bool WIDE>

@@ -201,7 +201,7 @@ zeno_status enqueue_score_cnn(Context *c, const void *x, const void *V, int64_t 
     a.fuse_loss = fuse_loss;
     a.first_in_call = 0;
     tail.used.base[lc] = c->np_base[lc];
-    tail.used.count[lc] = zeno::mlp_norm_slots((zeno_dtype)c->desc.param_dtype, a.in, a.out, n_r, m, aligned);
+    tail.used.count[lc] = zeno::mlp_norm_slots(*c, a.in, a.out, n_r, m, aligned);
     a.labels = static_cast<const int32_t *>(batch->targets);
     a.losses = loss_buf;
     a.tail = tail;
@@ -442,7 +442,7 @@ zeno_status enqueue_score(Context *c, const void *x, const void *V, int64_t ldv,
                          zeno::mlp_mma_usable(a.in, a.out) && is_aligned(x, 16) && is_aligned(V, 16) &&
                          (ldv * esz) % 16 == 0 && (a.offW * esz) % 16 == 0;
         tail.used.base[l] = c->np_base[l];
-        tail.used.count[l] = mma ? zeno::mlp_mma_norm_slots(a.out) : zeno::mlp_norm_slots((zeno_dtype)c->desc.param_dtype, a.in, a.out, n_r, m, aligned);
+        tail.used.count[l] = mma ? zeno::mlp_mma_norm_slots(a.out) : zeno::mlp_norm_slots(*c, a.in, a.out, n_r, m, aligned);
         a.labels = static_cast<const int32_t *>(batch->targets);
         a.losses = loss_buf;
         a.tail = tail;                               // complete by the time the last layer is reached

@@ -321,12 +321,12 @@ int lsq_slab_count(const Context &c);
 // Tensor-core version of the least-squares stream (zeno_lsq_tc.cu): one slab per block into a.part.
 bool lsq_tc_usable(const LsqArgs &a, bool aligned);
 cudaError_t launch_lsq_tc(Context &c, const LsqArgs &a, int max_slabs, int *slabs, cudaStream_t s);
-int mlp_norm_slots(zeno_dtype dtype, int in, int out, int n_r, int m, bool aligned);
+int mlp_norm_slots(const Context &c, int in, int out, int n_r, int m, bool aligned);
 int mlp_norm_slots_most(int out);
 
 constexpr int kMaxCluster = 8;     // blocks of a cluster in the dense layers' kernels
 // Dense layers by columns (zeno_rows.cu): which layers, and what they take.
-bool layer_by_columns(zeno_dtype dtype, int in, int out, int n_r, int m, bool aligned);
+bool layer_by_columns(const Context &c, int in, int out, int n_r, int m, bool aligned);
 cudaError_t launch_layer_by_columns(Context &c, const LayerArgs &a, bool aligned, cudaStream_t s);
 
 // ---- device helpers shared by the kernels ------------------------------------------------

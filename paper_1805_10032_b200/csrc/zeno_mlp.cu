@@ -648,7 +648,7 @@ cudaError_t launch_mlp_layer(Context &c, const LayerArgs &a, bool aligned, cudaS
             return aligned ? launch_head<__nv_bfloat16, true>(c, a, s) : launch_head<__nv_bfloat16, false>(c, a, s);
         return aligned ? launch_head<float, true>(c, a, s) : launch_head<float, false>(c, a, s);
     }
-    if (layer_by_columns((zeno_dtype)c.desc.param_dtype, a.in, a.out, a.n_r, a.m, aligned)) return launch_layer_by_columns(c, a, aligned, s);
+    if (layer_by_columns(c, a.in, a.out, a.n_r, a.m, aligned)) return launch_layer_by_columns(c, a, aligned, s);
     if (c.desc.param_dtype == ZENO_BF16)
         return aligned ? launch_layer<__nv_bfloat16, true>(c, a, s) : launch_layer<__nv_bfloat16, false>(c, a, s);
     return aligned ? launch_layer<float, true>(c, a, s) : launch_layer<float, false>(c, a, s);

@@ -203,17 +203,21 @@ __global__ void __launch_bounds__(kRowsThreads, 2) mlp_rows_kernel(LayerArgs a, 
             if ((chunk + 1) * C <= K) steps(std::false_type{});
             else steps(std::true_type{});
         }
-        if (!LONG || chunk >= chunks) break;
+        if constexpr (!LONG) {
+            break;
+        } else {
+            if (chunk >= chunks) break;
 #pragma unroll
-        for (int e0 = 0; e0 < R * N; e0 += kBatch) {
-            const float z = batch_sum(e0);
-            if (lane < kBatch && e0 + lane < R * N) totals[e0] = runs ? totals[e0] + z : z;
+            for (int e0 = 0; e0 < R * N; e0 += kBatch) {
+                const float z = batch_sum(e0);
+                if (lane < kBatch && e0 + lane < R * N) totals[e0] = runs ? totals[e0] + z : z;
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int n = 0; n < N; ++n) acc[r][n] = 0.f;
+            ++runs;
         }
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int n = 0; n < N; ++n) acc[r][n] = 0.f;
-        ++runs;
     }
     // the lanes' sums as [sample][row] where the samples were staged
     if (ASYNC) cp_async_wait<0>();
@@ -332,17 +336,19 @@ cudaError_t launch_rows(Context &c, const LayerArgs &a, cudaStream_t s) {
 // tiles); of aligned rows, whose four columns a lane leave the registers for fewer samples a tile, many samples only
 // where rows are long (300 x 260 in bfloat16 of 64 candidates, 128 samples: 1.15 times as long by columns, 2500 x 2000 of 21
 // candidates 0.91); and within 32-bit offsets.
-bool layer_by_columns(zeno_dtype dtype, int in, int out, int n_r, int m, bool aligned) {
+bool layer_by_columns(const Context &c, int in, int out, int n_r, int m, bool aligned) {
+    const bool f32 = c.desc.param_dtype == ZENO_F32;
+    const int sms = c.sm_count > 0 ? c.sm_count : 148;
     if (in < (n_r <= 8 ? 64 : 128) || (aligned && n_r > 32 && in < 1024)) return false;
     // many binary32 samples of so many tiles that every SM has eight blocks of the other kernel, which reads its samples from
     // shared memory half as often (65 models of 1345 x 1000, 62 samples: 678 us by columns, 630 by tiles)
-    if (dtype == ZENO_F32 && !aligned && n_r > 48 && (int64_t)(m + 1) * ((out + 63) / 64) * ((n_r + 31) / 32) >= 8 * 148) return false;
-    return (int64_t)in * out * (dtype == ZENO_BF16 ? 2 : 4) < (int64_t)1 << 32;
+    if (f32 && !aligned && n_r > 48 && (int64_t)(m + 1) * ((out + 63) / 64) * ((n_r + 31) / 32) >= (int64_t)8 * sms) return false;
+    return (int64_t)in * out * (f32 ? 4 : 2) < (int64_t)1 << 32;
 }
 
 // norm partials of a layer: a slot per warp of every row tile
-int mlp_norm_slots(zeno_dtype dtype, int in, int out, int n_r, int m, bool aligned) {
-    const int rows = layer_by_columns(dtype, in, out, n_r, m, aligned) ? kRowsWarps * rows_of_warp(out, n_r, aligned) : 64;
+int mlp_norm_slots(const Context &c, int in, int out, int n_r, int m, bool aligned) {
+    const int rows = layer_by_columns(c, in, out, n_r, m, aligned) ? kRowsWarps * rows_of_warp(out, n_r, aligned) : 64;
     return (out + rows - 1) / rows * kRowsWarps;
 }
 int mlp_norm_slots_most(int out) { return (out + 31) / 32 * kRowsWarps; }

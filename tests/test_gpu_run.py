@@ -112,6 +112,27 @@ def test_two_launch_loop_over_its_limits(oracle, dims, n_r, m, bias, pad, steps)
     assert P.rel_l2(x.cpu().numpy(), x_orc.astype(np.float64)) <= steps * 1e-6
 
 
+@pytest.mark.parametrize("dims,n_r,m,pad", [((784, 10), 4, 20, 2), ((517, 16), 13, 31, 1), ((1023, 31), 4, 7, 0)])
+def test_two_launch_loop_agrees_with_as_many_steps(dims, n_r, m, pad):
+    """Scores to rounding: a tenth of what the oracle's comparison allows.  The average and the update are the same sums in rank
+    order, so x differs by an addition's rounding where two rows of nearly equal scores change places, and no more."""
+    steps, b = 6, m // 3
+    ov = dict(dims=dims, n_r=n_r, m=m, b=b, ldv=syn.param_count("mlp", dims, True) + pad, faults=[(b, "signflip")])
+    ws = [syn.make_config(1, seed=700 + t, **ov) for t in range(steps)]
+    w = ws[0]
+    x, y = w.x.cuda().clone(), w.x.cuda().clone()
+    V, f, t = (torch.stack([getattr(s, k) for s in ws]).cuda() for k in ("V", "features", "targets"))
+    with zeno.from_workload(w) as z:
+        scores, idx = z.run(x, V, f, t, w.gamma, w.rho, b)
+        assert z.last_launch_count == 2
+        for i in range(steps):
+            _, losses, norms = z.score(y, V[i], f[i], t[i], w.gamma, w.rho)
+            _, want, want_idx = z.step_update(y, V[i], f[i], t[i], w.gamma, w.rho, b, want_out=False)
+            assert torch.all((scores[i] - want).abs() <= 1e-5 * (losses[0].abs() + losses[1:].abs() + w.rho * norms))
+            assert set(idx[i].tolist()) == set(want_idx.tolist())
+    assert P.rel_l2(x.cpu().numpy(), y.double().cpu().numpy()) <= steps * 1e-7
+
+
 def test_two_launch_loop_with_candidates_and_logits_that_overflow():
     """A candidate of NaN, one of infinities and one of 1e30 rank last in every iteration; logits of 1e10 keep a finite loss."""
     w = syn.make_config(1, dims=(50, 10), n_r=4, m=9, b=3, faults=[(3, "signflip")])

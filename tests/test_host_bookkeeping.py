@@ -61,3 +61,35 @@ def test_cnn_param_count_through_the_abi():
         assert zeno.param_count(desc) == syn.param_count("cnn", dims, False)
     for dims in [(16, 3, 8, 10), (34, 3, 8, 8, 10), (6, 3, 8, 8, 8, 8, 10), (15, 3, 8, 8, 10)]:
         assert zeno.param_count(zeno.make_desc(zeno.LOSS_SOFTMAX_CNN, zeno.F32, dims, True)) == 0
+
+
+RULE = textwrap.dedent("""
+    #include <cstdio>
+    #include "zeno_internal.h"
+    int main() {
+        // 65 models of 1345 x 1000 unaligned binary32 rows, 62 samples: 2,080 tiles of the kernel by tiles, 14 for each of 148 SMs, 7 of 296
+        for (int sms : {148, 259, 261, 296, 0}) {
+            zeno::Context c = {};
+            c.sm_count = sms;
+            c.desc.param_dtype = ZENO_F32;
+            std::printf("%d %d ", (int)zeno::layer_by_columns(c, 1345, 1000, 62, 64, false), zeno::mlp_norm_slots(c, 1345, 1000, 62, 64, false));
+        }
+        return 0;
+    }
+""")
+
+
+def test_layers_by_columns_are_chosen_for_the_devices_own_number_of_sms(tmp_path):
+    """A layer goes by tiles where every SM has eight of them, and the norm partials are counted for the kernel that runs."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("no nvcc")
+    lib = zbuild.build()
+    src = tmp_path / "rule.cu"
+    src.write_text(RULE)
+    exe = tmp_path / "rule"
+    subprocess.run([nvcc, "-std=c++17", "-I", os.path.join(ROOT, "paper_1805_10032_b200", "csrc"), "-I", os.path.join(ROOT, "include"),
+                    "-o", str(exe), str(src), lib, "-Xlinker", "-rpath=" + os.path.dirname(lib)], check=True)
+    out = subprocess.run([str(exe)], capture_output=True, text=True, check=True)
+    by_tiles, by_columns = 16 * 8, 32 * 8           # a slot per warp of 16 tiles of 64 rows, of 32 of 32
+    assert [int(v) for v in out.stdout.split()] == [0, by_tiles, 0, by_tiles, 1, by_columns, 1, by_columns, 0, by_tiles]

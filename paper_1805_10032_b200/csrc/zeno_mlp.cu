@@ -259,11 +259,20 @@ __global__ void __launch_bounds__(kLGroups * 64, 2) mlp_layer_kernel(LayerArgs a
 // The work is a chain of latencies (784 x 10 of 21 models: 0.7 MB) and, with many samples, of shared-memory reads: every
 // warp reads all rows.  65 models of 4096 x 10 in bfloat16, 64 samples: 30 us a scoring pass (43 with the activations through
 // shared memory, sixteen rows for ten and a warp per sample in the loss); 1029 x 10, binary32: 22 (29).
-constexpr int kHeadSmem = 96 * 1024;             // of the staged rows, at most
+// Blocks an SM has room for.  Clusters are sized for two an SM with up to 16 x 16 logits, but clusters of four and eight leave places of
+// a GPC's SMs empty: 36 models in clusters of eight are 288 blocks, of which two an SM are 264 at a time and three 384.  Rows of
+// any alignment, whose loads are of one entry, do with the registers for three (35 candidates of 7969 x 13, 5 samples: 27.0 us; with two
+// 39.8; 73 of 10760 x 10, one sample: 55 and 85); of four entries they do not.
+__host__ __device__ constexpr int head_blocks(int out_t, int spw, bool vec) {
+    return out_t <= 16 && spw <= 2 ? (vec ? 2 : 3) : !vec && out_t * spw <= 64 ? 2 : 1;
+}
+// bytes of the staged rows, at most
+__host__ __device__ constexpr int head_rows_bytes(int out_t, int spw, bool vec) { return (head_blocks(out_t, spw, vec) == 3 ? 56 : 96) * 1024; }
 template <typename T, int OUT_T, int SPW, bool VEC>
-__global__ void __launch_bounds__(256) mlp_head_kernel(LayerArgs a, int cluster, int kslice, int KC) {
+__global__ void __launch_bounds__(256, head_blocks(OUT_T, SPW, VEC)) mlp_head_kernel(LayerArgs a, int cluster, int kslice, int KC) {
     constexpr int NS = 8 * SPW, W = 4;           // samples a cluster can hold; columns of a lane at a time
-    constexpr int kAhead = SPW <= 2 ? 4 : SPW == 4 ? 2 : 1;      // times 128 columns of the samples on their way
+    // times 128 columns of the samples on their way: as the registers allow
+    constexpr int kAhead = SPW == 8 || (!VEC && OUT_T > 12 && SPW > 1) ? 1 : SPW == 4 ? 2 : 4;      // times 128 columns of the samples on their way
     constexpr int kRows = (OUT_T + 7) / 8;       // rows a warp stages
     constexpr int kLossLanes = OUT_T <= 16 ? 16 : 32, kLossAt = 256 / kLossLanes, kLossTurns = (NS + kLossAt - 1) / kLossAt;
     extern __shared__ __align__(16) float smem_dyn[];
@@ -597,7 +606,7 @@ bool mlp_can_fuse_loss(int out, int n_r) { return (out <= 32 && n_r <= 32) || (o
 
 template <typename T, int OUT_T, int SPW, bool VEC>
 cudaError_t launch_head_sized(Context &c, const LayerArgs &a, cudaStream_t s) {
-    constexpr int NS = 8 * SPW, kMostCols = kHeadSmem / 4 / OUT_T / 128 * 128;
+    constexpr int NS = 8 * SPW, kMostCols = head_rows_bytes(OUT_T, SPW, VEC) / 4 / OUT_T / 128 * 128;
     // blocks per model: as many as leave a slice of 128 columns and are resident at once (two to an SM up to 16 x 16
     // logits, one beyond: the accumulators).  A second wave costs more than the longer slice (101 models of 512 x 10,
     // 64 samples: 21 us with one block a model, 29 with two)

@@ -482,21 +482,24 @@ cudaError_t launch_pairs_of(Context &c, const KrumPlan &p, const T *V, int64_t l
     }
 }
 
-// Which of the two kernels takes the pairs.  Few columns: less than a stretch of 96 for every SM, 128 where rows are not aligned to 16
-// bytes, are over sooner in little code than register tiles are filled and emptied, with 13 to 48 candidates (42 of aligned bfloat16
-// rows; up to 88 of rows that are not aligned, where most threads have a tile, and 48 columns for every SM).  All three launches, 4 x 4
-// and register tiles: 20 candidates of 6,000 binary32 columns 8.7 us and 10.0, of 400 k 42 and 23; 34 of 8,000, bfloat16 rows of odd
-// pitch 12.6 and 17.3.  Many columns of more than 56 candidates, rows not aligned, where most threads have a tile: a block of the
+// Which of the two kernels takes the pairs.  Few columns: less than so many for every SM are over sooner in little code than register
+// tiles are filled and emptied.  All three launches, 4 x 4 and register tiles, us: 20 candidates of 6,000 binary32 columns 8.7 and 10.0, of 400 k 42
+// and 23; 34 of 8,000, bfloat16 rows of odd pitch 12.6 and 17.3; 12 of 1,074, bfloat16 7.1 and 8.4; 60 of 10,128, binary32 rows not aligned 16.4
+// and 20.8, 57 of 15,454 in bfloat16 21.3 and 26.1, 51 of 11,494 15.2 and 17.8, 59 of 9,520 aligned ones 16.2 and 18.9; up to six candidates fill register tiles of three
+// rows as quickly.  61 to 64 candidates are eight blocks of eight rows without a row too many (61 of 9,890: 20.1 and 19.7).
+// Many columns of more than 56 candidates, rows not aligned, where most threads have a tile: a block of the
 // register tiles stages many rows there by copies of 4 bytes, up to nine times over (88 of 300 k: 187 us and 262, bfloat16 183 and
-// 265; 112: 344 and 428, of 30 k 84 and 59).  With few of the last round's threads busy, as at 92, it is the other way.
+// 265; 112: 344 and 428, of 30 k 84 and 59; 102 of 111,840 133 and 167).  With few of the last round's threads busy, as at 92, it is the other way.
 bool krum_by_squares(int m, int64_t d, int sms, int entry_bytes, bool wide) {
-    if (m <= 12) return false;
+    if (m <= 6) return false;
     const int rounds = (square_tiles(m) + kKrumThreads - 1) / kKrumThreads;
     const int64_t pairs = (int64_t)m * (m - 1) / 2, places = (int64_t)rounds * kKrumThreads * 16;
     const bool busy = rounds <= 2 && square_groups(m) * pairs * 100 >= places * 57;
-    const int few = wide ? (m <= (entry_bytes == 4 ? 48 : 42) ? 96 : 0) : m <= 48 ? 128 : m <= 88 && busy ? 48 : 0;
+    int few;                                  // columns for every SM
+    if (wide) few = m <= 12 ? 16 : m <= (entry_bytes == 4 ? 48 : 42) ? 96 : m <= 64 ? 64 : 0;
+    else few = m <= 10 ? 48 : m <= 12 ? 80 : m <= 48 ? 128 : m >= 57 && m <= 60 ? 112 : m <= 72 && (m < 61 || m > 64) ? 88 : m <= 88 && busy ? 48 : 0;
     if (d <= (int64_t)few * sms) return true;
-    return !wide && m > 56 && busy && d > (int64_t)768 * sms;
+    return !wide && m > 56 && busy && d > (int64_t)(m > 96 && m <= 108 ? 640 : 768) * sms;
 }
 int square_blocks(int m, int64_t d, int sms) {
     int per_sm = (int)((200u << 10) / squares_smem(m));
@@ -552,7 +555,7 @@ size_t krum_part_floats(int m_max, int64_t d, int sms) {
         krum_size(m, &p);
         const size_t need = (size_t)krum_grid_x(p, sms) * p.tiles * p.B * p.B;
         if (need > most) most = need;
-        if (krum_by_squares(m, d, sms, 4, false)) {               // and with it the calls of aligned rows and of bfloat16
+        if (krum_by_squares(m, d, sms, 4, false) || krum_by_squares(m, d, sms, 4, true)) {      // and with them the calls of bfloat16
             const size_t squares = (size_t)square_blocks(m, d, sms) * square_tiles(m) * 16;
             if (squares > most) most = squares;
         }

@@ -209,6 +209,16 @@ def test_krum_by_either_kernel(oracle, m, dtype, d, pad, start):
     krum_with_two_best_rows(oracle, m, d, m // 3, dtype, pad, start)
 
 
+# the same for the fewest candidates and around 48, 64, 72 and 100 of them: 16, 48, 64, 80, 88, 112 and 640 columns for every SM
+@pytest.mark.parametrize("m,d,pad,start", [(m, d, pad, 0) for m in (6, 7, 10, 11, 12) for d, pad in ((2368, 0), (2376, 0), (7103, 0), (7105, 0), (11839, 0), (11841, 0))] +
+                         [(m, d, pad, 0) for m in (43, 49, 56, 61, 64, 65, 72, 73) for d, pad in ((9472, 0), (9480, 0), (13022, 1), (13026, 1))] +
+                         [(m, d, 1, 0) for m in (57, 60) for d in (16574, 16578)] +
+                         [(m, d, 1, 0) for m in (96, 97, 102, 108, 109) for d in (94720, 94722)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_krum_by_either_kernel_with_few_and_many_candidates(oracle, m, dtype, d, pad, start):
+    krum_with_two_best_rows(oracle, m, d, m // 3, dtype, pad, start)
+
+
 def krum_with_two_best_rows(oracle, m, d, b, dtype, pad, start):
     store = torch.bfloat16 if dtype == "bf16" else torch.float32
     g = torch.Generator(device="cuda").manual_seed(m + d)

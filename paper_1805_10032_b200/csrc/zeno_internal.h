@@ -324,6 +324,9 @@ cudaError_t launch_lsq_tc(Context &c, const LsqArgs &a, int max_slabs, int *slab
 int mlp_norm_slots(const Context &c, int in, int out, int n_r, int m, bool aligned);
 int mlp_norm_slots_most(int out);
 
+// The tiles of all models that the kernel by tiles cuts a layer into, and the blocks that share one (zeno_mlp.cu).
+struct LayerTiles { int64_t tiles; int cluster; };
+LayerTiles layer_tiles(const Context &c, int in, int out, int n_r, int m);
 constexpr int kMaxCluster = 8;     // blocks of a cluster in the dense layers' kernels
 // Dense layers by columns (zeno_rows.cu): which layers, and what they take.
 bool layer_by_columns(const Context &c, int in, int out, int n_r, int m, bool aligned);

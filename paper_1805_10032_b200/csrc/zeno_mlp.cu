@@ -271,7 +271,6 @@ __host__ __device__ constexpr int head_rows_bytes(int out_t, int spw, bool vec) 
 template <typename T, int OUT_T, int SPW, bool VEC>
 __global__ void __launch_bounds__(256, head_blocks(OUT_T, SPW, VEC)) mlp_head_kernel(LayerArgs a, int cluster, int kslice, int KC) {
     constexpr int NS = 8 * SPW, W = 4;           // samples a cluster can hold; columns of a lane at a time
-    // times 128 columns of the samples on their way: as the registers allow
     constexpr int kAhead = SPW == 8 || (!VEC && OUT_T > 12 && SPW > 1) ? 1 : SPW == 4 ? 2 : 4;      // times 128 columns of the samples on their way
     constexpr int kRows = (OUT_T + 7) / 8;       // rows a warp stages
     constexpr int kLossLanes = OUT_T <= 16 ? 16 : 32, kLossAt = 256 / kLossLanes, kLossTurns = (NS + kLossAt - 1) / kLossAt;
@@ -558,15 +557,28 @@ __global__ void __launch_bounds__(256) mlp_loss_kernel(const float *logits, cons
     }
 }
 
+// Blocks that share a tile's slices.  Two blocks fit an SM: with fewer than that, clusters, at least two slices a block
+// (evening out a last wave with clusters as well made 190 tiles' kernel 10 % faster and its step 9 % slower).
+int layer_cluster(const Context &c, int64_t tiles, int in) {
+    const int sms = c.sm_count > 0 ? c.sm_count : 148;
+    int cluster = 1;
+    while (cluster < kMaxCluster && tiles * 2 * cluster <= 2 * sms && in >= 2 * kLK * 2 * cluster) cluster *= 2;
+    return cluster;
+}
+
+// Samples in tiles of eight times this: one tile if it holds them all, else the width that pads them least (narrow layers, 33 to 48
+// samples: two tiles of 24; a step of 21 models of 122-507-7-20-11 with 33 takes 39.5 us, with one tile of 64 52).
+int layer_tile_width(int out, int n_r) {
+    if (out <= kLFewRows) return n_r <= 8 ? 1 : n_r <= 16 ? 2 : n_r <= 32 ? 4 : n_r <= 48 ? 3 : 8;
+    const bool by24 = n_r > 32 && (n_r + 23) / 24 <= (n_r + 31) / 32;
+    return n_r <= 8 ? 1 : n_r <= 16 ? 2 : n_r <= 24 || by24 ? 3 : 4;
+}
+
 template <typename T, int R, int TN, bool VEC>
 cudaError_t launch_layer_tiles(Context &c, const LayerArgs &a, cudaStream_t s) {
-    const int sms = c.sm_count > 0 ? c.sm_count : 148;
     const int sample_tiles = (a.n_r + 8 * TN - 1) / (8 * TN);
     const int64_t tiles = (int64_t)((a.out + 8 * R - 1) / (8 * R)) * sample_tiles;
-    // two blocks fit an SM: with fewer than that, clusters of blocks share a tile's slices, at least two slices a block
-    // (evening out a last wave with clusters as well made 190 tiles' kernel 10 % faster and its step 9 % slower)
-    int cluster = 1;
-    while (cluster < kMaxCluster && tiles * (a.m + 1) * 2 * cluster <= 2 * sms && a.in >= 2 * kLK * 2 * cluster) cluster *= 2;
+    const int cluster = layer_cluster(c, tiles * (a.m + 1), a.in);
     // the limit is the function's, for every handle and thread of the process: the most any call asks for, set once
     static PerDeviceOnce attr_set;
     if (attr_set.need(c.device)) {
@@ -580,25 +592,25 @@ cudaError_t launch_layer_tiles(Context &c, const LayerArgs &a, cudaStream_t s) {
                             layer_smem(R, TN, cluster), s, chain_launches(c), a, sample_tiles, cluster);
 }
 
-// samples in tiles of 8 TN: one tile if it holds them all, else the width that pads them least (narrow layers, 33 to 48
-// samples: two tiles of 24; a step of 21 models of 122-507-7-20-11 with 33 takes 39.5 us, with one tile of 64 52)
 template <typename T, bool VEC>
 cudaError_t launch_layer(Context &c, const LayerArgs &a, cudaStream_t s) {
-    if (a.out <= kLFewRows) {
-        if (a.n_r <= 8) return launch_layer_tiles<T, 4, 1, VEC>(c, a, s);
-        if (a.n_r <= 16) return launch_layer_tiles<T, 4, 2, VEC>(c, a, s);
-        if (a.n_r <= 32) return launch_layer_tiles<T, 4, 4, VEC>(c, a, s);
-        if (a.n_r <= 48) return launch_layer_tiles<T, 4, 3, VEC>(c, a, s);
-        return launch_layer_tiles<T, 4, 8, VEC>(c, a, s);
+    const bool narrow = a.out <= kLFewRows;
+    switch (layer_tile_width(a.out, a.n_r)) {
+        case 1: return narrow ? launch_layer_tiles<T, 4, 1, VEC>(c, a, s) : launch_layer_tiles<T, 8, 1, VEC>(c, a, s);
+        case 2: return narrow ? launch_layer_tiles<T, 4, 2, VEC>(c, a, s) : launch_layer_tiles<T, 8, 2, VEC>(c, a, s);
+        case 3: return narrow ? launch_layer_tiles<T, 4, 3, VEC>(c, a, s) : launch_layer_tiles<T, 8, 3, VEC>(c, a, s);
+        case 4: return narrow ? launch_layer_tiles<T, 4, 4, VEC>(c, a, s) : launch_layer_tiles<T, 8, 4, VEC>(c, a, s);
+        default: return launch_layer_tiles<T, 4, 8, VEC>(c, a, s);
     }
-    const bool by24 = a.n_r > 32 && (a.n_r + 23) / 24 <= (a.n_r + 31) / 32;
-    if (a.n_r <= 8) return launch_layer_tiles<T, 8, 1, VEC>(c, a, s);
-    if (a.n_r <= 16) return launch_layer_tiles<T, 8, 2, VEC>(c, a, s);
-    if (a.n_r <= 24 || by24) return launch_layer_tiles<T, 8, 3, VEC>(c, a, s);
-    return launch_layer_tiles<T, 8, 4, VEC>(c, a, s);
 }
 
 }  // namespace
+
+LayerTiles layer_tiles(const Context &c, int in, int out, int n_r, int m) {
+    const int rows = out <= kLFewRows ? kLFewRows : 64, samples = 8 * layer_tile_width(out, n_r);
+    const int64_t tiles = (int64_t)(m + 1) * ((out + rows - 1) / rows) * ((n_r + samples - 1) / samples);
+    return {tiles, layer_cluster(c, tiles, in)};
+}
 
 // The cross-entropy can ride on the last layer's launch when one block sees all of a model's
 // logits: every output row in one block, every sample in one tile.

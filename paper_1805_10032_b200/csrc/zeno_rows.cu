@@ -297,6 +297,17 @@ cudaError_t launch_rows_tiles(Context &c, const LayerArgs &a, cudaStream_t s) {
 // would otherwise have no rows for most of their warps
 __host__ __device__ constexpr int rows_of_warp(int out, int n_r, bool aligned) { return !aligned && n_r <= 8 && out > 32 ? 8 : 4; }
 
+// Many samples in tiles of twelve and more, up to as many as the registers hold the sums of: the fewest padded samples, then the fewest tiles.
+constexpr int kRowsSamples = 24, kRowsAsyncFrom = 512;       // samples of a tile; columns from which one tile's weights come by copies
+int rows_samples(int n_r, int most) {
+    int best = most, least = 1 << 30;
+    for (int n = most; n >= 12; n -= 4) {
+        const int padded = (n_r + n - 1) / n * n;
+        if (padded < least) { least = padded; best = n; }
+    }
+    return best;
+}
+
 template <typename T, int W>
 cudaError_t launch_rows(Context &c, const LayerArgs &a, cudaStream_t s) {
     if (rows_of_warp(a.out, a.n_r, W == 4) == 8) {
@@ -309,18 +320,14 @@ cudaError_t launch_rows(Context &c, const LayerArgs &a, cudaStream_t s) {
     if (a.n_r <= 2) return launch_rows_tiles<T, 4, 2, W>(c, a, s);
     if (a.n_r <= 4) return launch_rows_tiles<T, 4, 4, W>(c, a, s);
     if (a.n_r <= 8) return launch_rows_tiles<T, 4, 8, W>(c, a, s);
-    // tiles of 12 samples and more, as far as the registers hold their sums: the fewest padded samples, then the fewest tiles
-    constexpr int kMost = W == 1 ? 24 : is_bf16<T>::value ? 16 : 12;
-    int best = kMost, least = 1 << 30;
-    for (int n = kMost; n >= 12; n -= 4) {
-        const int padded = (a.n_r + n - 1) / n * n;
-        if (padded < least) { least = padded; best = n; }
-    }
+    constexpr int kMost = W == 1 ? kRowsSamples : is_bf16<T>::value ? 16 : 12;
+    const int best = rows_samples(a.n_r, kMost);
     // one tile of 20 or 24 samples and rows long enough to fill the pipeline: 38 models of 1029 x 301 with 19 samples take 44 us
     // with the copies and 50 without, of 301 x 131 16 and 14; with more tiles the copies and the reads of their words are too
-    // many for the load units (65 models of 1345 x 1000, 62 samples: 794 us and 650)
+    // many for the load units (65 models of 1345 x 1000, 62 samples: 794 us and 650).  40 layers of 17 to 24 samples, 512 to 6000 columns and
+    // 5 to 128 candidates: 0.90 of the time without on average, 0.65 to 1.17 (none of them faster by tiles)
     if constexpr (W == 1 && !is_bf16<T>::value) {
-        if (a.n_r <= 24 && best >= 20 && a.in >= 512)
+        if (a.n_r <= 24 && best >= 20 && a.in >= kRowsAsyncFrom)
             return best == 20 ? launch_rows_tiles<T, 4, 20, 1, true>(c, a, s) : launch_rows_tiles<T, 4, 24, 1, true>(c, a, s);
     }
     if (best == 12) return launch_rows_tiles<T, 4, 12, W>(c, a, s);
@@ -331,6 +338,26 @@ cudaError_t launch_rows(Context &c, const LayerArgs &a, cudaStream_t s) {
 
 }  // namespace
 
+// Whether a layer of many binary32 samples, rows of any alignment, is small enough for the kernel by columns.  The one by tiles reads its
+// samples from shared memory half as often, and does better with more work than fills the device: 12 candidates of 3972 x 930, 94
+// samples 518 us by tiles and 807 by columns; 32 of 4082 x 614, 86 893 and 1,282; 42 of 1166 x 33, 89 (1.2 waves of blocks by columns, one
+// nearly full one by tiles) 63 and 79.  With less the shorter blocks win: 21 of 3512 x 72, 103 samples 225 and 131; 15 of 2288 x 333, 50
+// 154 and 112; tiles of up to sixteen samples, whose sums leave registers to load two steps ahead, even of a few
+// waves: 37 of 1049 x 152, 103 149 and 104, but of short rows not (11 of 168 x 1314, 32 27 and 31).  387 layers of 9 to 128 samples: 0.87 of the time of the kernel by tiles on average, the
+// worst 1.20; by columns wherever rows are long 1.56.
+static bool few_blocks(const Context &c, int in, int out, int n_r, int m) {
+    const int places = 2 * (c.sm_count > 0 ? c.sm_count : 148);          // two blocks an SM of either kernel
+    // narrow layers: 41 to 48 samples are the same tiles either way (73 candidates of 885 x 26, 47 samples: 28 us and 31)
+    if (out <= 32 && n_r <= 48) return n_r <= 40;
+    const LayerTiles t = layer_tiles(c, in, out, n_r, m);
+    const int samples = rows_samples(n_r, kRowsSamples);
+    if (samples <= 16) return t.tiles <= (in < 320 ? places * 3 / 4 : 2 * places);
+    const int64_t blocks = (int64_t)(m + 1) * ((out + 31) / 32) * ((n_r + samples - 1) / samples);
+    const int64_t tile_blocks = t.tiles * t.cluster;
+    const bool one_full_wave = tile_blocks <= places && tile_blocks * 20 >= (int64_t)places * 17;
+    return blocks <= places || (blocks <= 2 * places && !one_full_wave);
+}
+
 // Which of the two kernels takes a layer.  By columns: from 128 columns on, or 64 where few samples leave few sums to add up
 // over the lanes at the end (the layers of 64 x 48 x 1000 of 64 candidates and 128 samples: 245 us by columns, 113 by
 // tiles); of aligned rows, whose four columns a lane leave the registers for fewer samples a tile, many samples only
@@ -338,11 +365,10 @@ cudaError_t launch_rows(Context &c, const LayerArgs &a, cudaStream_t s) {
 // candidates 0.91); and within 32-bit offsets.
 bool layer_by_columns(const Context &c, int in, int out, int n_r, int m, bool aligned) {
     const bool f32 = c.desc.param_dtype == ZENO_F32;
-    const int sms = c.sm_count > 0 ? c.sm_count : 148;
     if (in < (n_r <= 8 ? 64 : 128) || (aligned && n_r > 32 && in < 1024)) return false;
-    // many binary32 samples of so many tiles that every SM has eight blocks of the other kernel, which reads its samples from
-    // shared memory half as often (65 models of 1345 x 1000, 62 samples: 678 us by columns, 630 by tiles)
-    if (f32 && !aligned && n_r > 48 && (int64_t)(m + 1) * ((out + 63) / 64) * ((n_r + 31) / 32) >= (int64_t)8 * sms) return false;
+    // 21 to 24 samples, 25 to 32 and more than 40: 24 a tile, of long rows by asynchronous copies; sixteen; whatever pads least
+    const bool many = n_r > 40 || (n_r > 24 && n_r <= 32) || (n_r > 20 && n_r <= 24 && in < kRowsAsyncFrom);
+    if (f32 && !aligned && many && !few_blocks(c, in, out, n_r, m)) return false;
     return (int64_t)in * out * (f32 ? 4 : 2) < (int64_t)1 << 32;
 }
 

@@ -122,6 +122,16 @@ def test_layers_by_columns(oracle, dims, n_r, m, bias, dtype, pad):
     P.run_step_parity(oracle, w)
 
 
+# many binary32 samples of unaligned rows, either side of the rule that takes a layer by columns or by tiles: 20 and 24, 28, 40 and 41
+# samples, narrow layers of 48 and 49, one wave of blocks and several, tiles of twelve to 24 samples
+@pytest.mark.parametrize("dims,n_r,m", [
+    ((129, 33, 34, 3), 40, 4), ((129, 33, 34, 3), 41, 4), ((244, 20, 9), 48, 5), ((244, 20, 9), 49, 5), ((200, 120, 10), 95, 30), ((200, 330, 10), 95, 30),
+    ((150, 70, 10), 103, 5), ((131, 270, 10), 84, 21), ((150, 300, 10), 20, 70), ((150, 300, 10), 24, 70), ((150, 300, 10), 28, 100), ((150, 300, 10), 28, 130)])
+def test_layers_of_many_samples_of_unaligned_rows(oracle, dims, n_r, m):
+    b = m // 3
+    P.run_step_parity(oracle, syn.make_config(2, dims=dims, n_r=n_r, m=m, b=b, ldv=syn.param_count("mlp", dims, True) + 1, faults=[(b, "signflip")]))
+
+
 @pytest.mark.parametrize("cols,rows,dtype", [(40001, 33, "f32"), (40001, 33, "bf16"), (40004, 36, "f32")])
 def test_sums_of_long_rows_are_short_sums(cols, rows, dtype):
     """A logit of 40,000 products of random signs against 64 bits, the layer in as many tiles as leave a lane every 32nd

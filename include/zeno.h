@@ -255,9 +255,10 @@ zeno_status zeno_step_update(zeno_handle h, void *x, const void *V, int64_t ldv,
  *   features: [steps][n_r x dims[0]] binary32, contiguous;   targets: [steps][n_r] (int32 or float);
  *   scores:   [steps][m] or NULL;   idx: [steps][m - b] or NULL.
  * x is read and updated in place by every iteration.  Four and more iterations of a small binary32 softmax
- * regression go in two launches, which read all candidates ahead; their scores agree with those of as many
- * zeno_step_update calls to rounding, those of other loops bit for bit.  The candidates are inputs: they are what the workers
- * sent for these iterations, however the caller obtained them.  The profiler (zeno_profile) sees the whole
+ * regression may go in two launches for as many iterations as the handle's workspace holds products of, which read all
+ * candidates ahead; their scores agree with those of as many zeno_step_update calls to rounding, those of other loops (so
+ * of all up to three iterations) bit for bit.  The candidates are inputs: they are what the workers sent for these
+ * iterations, however the caller obtained them.  The profiler (zeno_profile) sees the whole
  * run as one call and keeps only the kernels that fit its per-call list.
  * INVALID_ARG: as zeno_step_update, or steps < 1, or step_stride_v < m * ldv. */
 zeno_status zeno_run(zeno_handle h, void *x, const void *V, int64_t ldv, int64_t step_stride_v, int32_t m,

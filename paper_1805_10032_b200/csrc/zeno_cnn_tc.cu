@@ -36,8 +36,8 @@
 //
 // Before the layers, cnn_pack_kernel forms w = x - gamma v of every model in the operand layout (and the sums of
 // v^2); after every second layer cnn_pool_kernel takes the 2 x 2 maxima.  Measured on 21 models of
-// 32 x 32 x 3 -> 32, 32, 64, 64 planes: a step of 4 samples 95 us (with the CUDA-core kernel 353), of 32 samples with
-// bfloat16 weights 384 us (1,268).  What bounds it: an MMA fetches its 128 pixels from shared memory in about 60 cycles
+// 32 x 32 x 3 -> 32, 32, 64, 64 planes: a step of 4 samples 93 us (with the CUDA-core kernel 353), of 32 samples with
+// bfloat16 weights 382 us (1,268).  What bounds it: an MMA fetches its 128 pixels from shared memory in about 60 cycles
 // whatever it multiplies them with (the alignment of a tap makes no difference), and the first layer of 32 samples
 // writes 190 MB in 80 us.
 #include <algorithm>

@@ -17,7 +17,7 @@ namespace zeno {
 
 namespace {
 
-// One dense layer of all models, rows of any alignment, by tiles (the layers layer_by_columns below does not take).  A block
+// One dense layer of all models, rows of any alignment, by tiles (the layers layer_by_columns in zeno_rows.cu does not take).  A block
 // takes 8 R output rows of one model and 8 TN samples and
 // stages slices of 64 input columns in shared memory -- w = x - gamma v formed on the way, v^2 accumulated, all of the
 // next slice's loads in flight during the present one's arithmetic.  Its four groups of 64 threads take sixteen of the

@@ -19,7 +19,7 @@ namespace {
 // 4,095, 40,001 products of random signs: 1.5e-7, 1.8e-7 of it; 2.2e-7, 6.8e-7 in one run; by tiles 1.7e-7, 2.5e-7).  Shorter
 // rows do without the code: with it the step of 1029-301-131-11 takes 2 % longer.
 // Bound by the loads' latency while few are in flight, then by shared-memory reads and additions.  A whole scoring pass by
-// columns and by tiles (the kernel above): 65 models of 2500 x 2000, one sample, binary32 0.51 of the time, bfloat16 0.39; of
+// columns and by tiles (zeno_mlp.cu): 65 models of 2500 x 2000, one sample, binary32 0.51 of the time, bfloat16 0.39; of
 // 1345 x 1000 and 11 samples 0.87 and 0.54; of 1029 x 301 x 131 and 62 samples 0.94 and 0.64.
 constexpr int kRowsAhead = 4;
 constexpr int kRowsWarps = 8, kRowsThreads = kRowsWarps * 32, kRowsCols = 256;

@@ -342,16 +342,17 @@ cudaError_t launch_rows(Context &c, const LayerArgs &a, cudaStream_t s) {
 // samples from shared memory half as often, and does better with more work than fills the device: 12 candidates of 3972 x 930, 94
 // samples 518 us by tiles and 807 by columns; 32 of 4082 x 614, 86 893 and 1,282; 42 of 1166 x 33, 89 (1.2 waves of blocks by columns, one
 // nearly full one by tiles) 63 and 79.  With less the shorter blocks win: 21 of 3512 x 72, 103 samples 225 and 131; 15 of 2288 x 333, 50
-// 154 and 112; tiles of up to sixteen samples, whose sums leave registers to load two steps ahead, even of a few
-// waves: 37 of 1049 x 152, 103 149 and 104, but of short rows not (11 of 168 x 1314, 32 27 and 31).  387 layers of 9 to 128 samples: 0.87 of the time of the kernel by tiles on average, the
-// worst 1.20; by columns wherever rows are long 1.56.
+// 154 and 112; tiles of up to twenty samples, whose sums leave registers to load ahead, even of a few waves: 37 of 1049 x 152, 103
+// samples 149 and 104, 125 of 829 x 57, 97 124 and 103, but of short rows not (11 of 168 x 1314, 32 27 and 31).  380 layers of 17 to 128 samples:
+// 0.87 of the time of the kernel by tiles on average, the worst 1.20; by columns wherever rows are long 1.56.
 static bool few_blocks(const Context &c, int in, int out, int n_r, int m) {
     const int places = 2 * (c.sm_count > 0 ? c.sm_count : 148);          // two blocks an SM of either kernel
     // narrow layers: 41 to 48 samples are the same tiles either way (73 candidates of 885 x 26, 47 samples: 28 us and 31)
     if (out <= 32 && n_r <= 48) return n_r <= 40;
     const LayerTiles t = layer_tiles(c, in, out, n_r, m);
     const int samples = rows_samples(n_r, kRowsSamples);
-    if (samples <= 16) return t.tiles <= (in < 320 ? places * 3 / 4 : 2 * places);
+    if (samples <= 20 && in >= 320) return t.tiles * 2 <= 5 * (int64_t)places;
+    if (samples <= 16) return t.tiles * 4 <= 3 * (int64_t)places;
     const int64_t blocks = (int64_t)(m + 1) * ((out + 31) / 32) * ((n_r + samples - 1) / samples);
     const int64_t tile_blocks = t.tiles * t.cluster;
     const bool one_full_wave = tile_blocks <= places && tile_blocks * 20 >= (int64_t)places * 17;

@@ -484,29 +484,46 @@ cudaError_t launch_pairs_of(Context &c, const KrumPlan &p, const T *V, int64_t l
     }
 }
 
-// Which of the two kernels takes the pairs.  Few columns: less than so many for every SM are over sooner in little code than register
-// tiles are filled and emptied.  All three launches, 4 x 4 and register tiles, us: 20 candidates of 6,000 binary32 columns 8.7 and 10.0, of 400 k 42
-// and 23; 34 of 8,000, bfloat16 rows of odd pitch 12.6 and 17.3; 12 of 1,074, bfloat16 7.1 and 8.4; 60 of 10,128, binary32 rows not aligned 16.4
-// and 20.8, 57 of 15,454 in bfloat16 21.3 and 26.1, 51 of 11,494 15.2 and 17.8, 59 of 9,520 aligned ones 16.2 and 18.9; up to six candidates fill register tiles of three
-// rows as quickly.  61 to 64 candidates are eight blocks of eight rows without a row too many (61 of 9,890: 20.1 and 19.7).
+// blocks of 4 x 4 pairs that are resident at once
+int square_places(int m, int sms) {
+    const int per_sm = (int)((200u << 10) / squares_smem(m));
+    return (per_sm > 4 ? 4 : per_sm) * sms;   // four: what the registers let be resident
+}
+
+// Which of the two kernels takes the pairs.  Few columns are over sooner in little code than register tiles are filled and emptied.
+// All three launches, 4 x 4 and register tiles, us: 20 candidates of 6,000 binary32 columns 8.7 and 10.0, of 400 k 42 and 23; 34 of 8,000, bfloat16
+// rows of odd pitch 12.6 and 17.3; 12 of 1,074, bfloat16 7.1 and 8.4; up to six candidates fill register tiles of three rows as quickly.
+// With 49 to 88 candidates that holds for as many columns as give every SM a block of 4 x 4 pairs, not for fewer, which either kernel leaves SMs
+// without: 60 of 10,128 columns, rows not aligned 16.4 and 20.8, 67 of 11,828 21.2 and 26.1, of 2,616 18.3 and 15.5, 79 of 7,026 20.9 and 24.4, of
+// 1,980 19.1 and 15.5; 61 to 64 are eight blocks of eight rows without a row too many (of 9,890 20.1 and 19.7, of 234 16.4 and 13.0).
 // Many columns of more than 56 candidates, rows not aligned, where most threads have a tile: a block of the
 // register tiles stages many rows there by copies of 4 bytes, up to nine times over (88 of 300 k: 187 us and 262, bfloat16 183 and
-// 265; 112: 344 and 428, of 30 k 84 and 59; 102 of 111,840 133 and 167).  With few of the last round's threads busy, as at 92, it is the other way.
+// 265; 112: 344 and 428, of 30 k 84 and 59; 102 of 111,840 133 and 167, 59 of 242,606
+// in bfloat16 97 and 118; but 83 of 133,650 129 and 109, 80 of 223,762 142 and 130).  With few of the last round's threads busy, as at 92, it is the other way.
 bool krum_by_squares(int m, int64_t d, int sms, int entry_bytes, bool wide) {
     if (m <= 6) return false;
+    int more = 0, most = 0;                   // columns for every SM
+    if (wide) {
+        if (m <= 12) most = 16;
+        else if (m <= (entry_bytes == 4 ? 48 : 42)) most = 96;
+        else if (entry_bytes == 4 && m <= 60) { more = 44; most = 100; }
+    } else {
+        if (m <= 12) most = m <= 10 ? 48 : 80;
+        else if (m <= 48) most = 128;
+        else if (m <= 56) { more = 32; most = 88; }
+        else if (m <= 60) most = 112;
+        else if (m >= 65 && m <= 72) { more = 36; most = 84; }
+        else if (m >= 73 && m <= 88) { more = 40; most = 64; }
+    }
+    if (d > (int64_t)more * sms && d <= (int64_t)most * sms) return true;
     const int rounds = (square_tiles(m) + kKrumThreads - 1) / kKrumThreads;
     const int64_t pairs = (int64_t)m * (m - 1) / 2, places = (int64_t)rounds * kKrumThreads * 16;
     const bool busy = rounds <= 2 && square_groups(m) * pairs * 100 >= places * 57;
-    int few;                                  // columns for every SM
-    if (wide) few = m <= 12 ? 16 : m <= (entry_bytes == 4 ? 48 : 42) ? 96 : m <= 64 ? 64 : 0;
-    else few = m <= 10 ? 48 : m <= 12 ? 80 : m <= 48 ? 128 : m >= 57 && m <= 60 ? 112 : m <= 72 && (m < 61 || m > 64) ? 88 : m <= 88 && busy ? 48 : 0;
-    if (d <= (int64_t)few * sms) return true;
-    return !wide && m > 56 && busy && d > (int64_t)(m > 96 && m <= 108 ? 640 : 768) * sms;
+    const int many = m > 96 && m <= 108 ? 640 : m >= 73 && m <= 80 ? 2048 : 1024;
+    return !wide && m > 56 && busy && d > (int64_t)many * sms;
 }
 int square_blocks(int m, int64_t d, int sms) {
-    int per_sm = (int)((200u << 10) / squares_smem(m));
-    per_sm = per_sm > 4 ? 4 : per_sm;          // what the registers let be resident
-    const int64_t want = (d + kSquareCols - 1) / kSquareCols, most = (int64_t)per_sm * sms;
+    const int64_t want = (d + kSquareCols - 1) / kSquareCols, most = square_places(m, sms);
     return (int)(want < most ? want : most);
 }
 

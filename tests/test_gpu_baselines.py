@@ -209,11 +209,13 @@ def test_krum_by_either_kernel(oracle, m, dtype, d, pad, start):
     krum_with_two_best_rows(oracle, m, d, m // 3, dtype, pad, start)
 
 
-# the same for the fewest candidates and around 48, 64, 72 and 100 of them: 16, 48, 64, 80, 88, 112 and 640 columns for every SM
+# the same for the fewest candidates, for 43 to 89 of them, where few columns go back to the register tiles, and for about 100: the
+# numbers of columns for every SM at which the kernels take turns
 @pytest.mark.parametrize("m,d,pad,start", [(m, d, pad, 0) for m in (6, 7, 10, 11, 12) for d, pad in ((2368, 0), (2376, 0), (7103, 0), (7105, 0), (11839, 0), (11841, 0))] +
-                         [(m, d, pad, 0) for m in (43, 49, 56, 61, 64, 65, 72, 73) for d, pad in ((9472, 0), (9480, 0), (13022, 1), (13026, 1))] +
-                         [(m, d, 1, 0) for m in (57, 60) for d in (16574, 16578)] +
-                         [(m, d, 1, 0) for m in (96, 97, 102, 108, 109) for d in (94720, 94722)])
+                         [(m, d, pad, 0) for m in (43, 49, 60, 61) for d, pad in ((6512, 0), (6520, 0), (14800, 0), (14808, 0))] +
+                         [(m, d, 1, 0) for m, lo, hi in ((49, 32, 88), (56, 32, 88), (57, 0, 112), (60, 0, 112), (64, 36, 84), (65, 36, 84), (72, 36, 84), (73, 40, 64),
+                                                         (88, 40, 64), (89, 40, 64)) for d in (148 * lo, 148 * lo + 2, 148 * hi, 148 * hi + 2) if d >= 4] +
+                         [(m, d, 1, 0) for m in (96, 97, 102, 108, 109) for d in (94720, 94722)] + [(m, d, 1, 0) for m in (57, 88, 109) for d in (151552, 151554)])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_krum_by_either_kernel_with_few_and_many_candidates(oracle, m, dtype, d, pad, start):
     krum_with_two_best_rows(oracle, m, d, m // 3, dtype, pad, start)
